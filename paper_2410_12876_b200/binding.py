@@ -1,11 +1,14 @@
-"""ctypes binding of libag.so: argument marshalling only.
+"""Python binding of libag.so: argument marshalling only.
 
 Each function has the name and argument order of its C counterpart in
-include/ag.h and does nothing but turn torch tensors into device pointers.
+include/ag.h and does nothing but turn torch tensors into device pointers (in
+the extension module _marshal, csrc/py_binding.cpp: marshalled in Python a call
+took longer than a decode step of a short cache).  The structs are ctypes.
 Every step of the layer runs inside the CUDA library; there is no Python or
 CPU fallback, and loading fails loudly when the library has not been built.
 """
 import ctypes
+import importlib
 import os
 
 import torch
@@ -122,16 +125,16 @@ def _ptr(t):
     return t.data_ptr()
 
 
-def _stream(stream):
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
-    return stream if isinstance(stream, int) else stream.cuda_stream
+_m = None
 
 
-def _ws(ws):
-    if ws is None:
-        return None, 0
-    return ws.data_ptr(), ws.numel() * ws.element_size()
+def _marshal():
+    """The extension module that unpacks the arguments and makes the C call (csrc/py_binding.cpp)."""
+    global _m
+    lib()
+    m = importlib.import_module("._marshal", __package__)
+    _m = m
+    return m
 
 
 class RaggedCache:
@@ -193,53 +196,42 @@ def _check(st, where):
 
 
 def ag_gate_forward(desc, X, Wq_g, Wk_g, Wv_g, Wo_g, gamma, scores, flags, ws, stream=None):
-    p, nbytes = _ws(ws)
-    return _check(lib().ag_gate_forward(ctypes.byref(desc), _ptr(X), _ptr(Wq_g), _ptr(Wk_g), _ptr(Wv_g),
-                                        _ptr(Wo_g), _ptr(gamma), _ptr(scores), _ptr(flags), p, nbytes,
-                                        _stream(stream)), "ag_gate_forward")
+    return _check((_m or _marshal()).gate_forward(desc, X, Wq_g, Wk_g, Wv_g, Wo_g, gamma, scores, flags, ws, stream),
+                  "ag_gate_forward")
 
 
 def ag_gate_linear_forward(desc, X, W_lin, gamma, scores, flags, stream=None):
-    return _check(lib().ag_gate_linear_forward(ctypes.byref(desc), _ptr(X), _ptr(W_lin), _ptr(gamma), _ptr(scores),
-                                               _ptr(flags), _stream(stream)), "ag_gate_linear_forward")
+    return _check((_m or _marshal()).gate_linear_forward(desc, X, W_lin, gamma, scores, flags, stream),
+                  "ag_gate_linear_forward")
 
 
 def ag_compact_kv(desc, K, V, flags, cache, prefix, idx, dev_status, ws, stream=None):
-    p, nbytes = _ws(ws)
-    return _check(lib().ag_compact_kv(ctypes.byref(desc), _ptr(K), _ptr(V), _ptr(flags),
-                                      ctypes.byref(cache.struct), _ptr(prefix), _ptr(idx),
-                                      _ptr(dev_status), p, nbytes, _stream(stream)), "ag_compact_kv")
+    return _check((_m or _marshal()).compact_kv(desc, K, V, flags, cache, prefix, idx, dev_status, ws, stream),
+                  "ag_compact_kv")
 
 
 def ag_kv_project_cache(desc, X, Wk, Wv, flags, cache, prefix, idx, K, V, dev_status, stream=None):
-    return _check(lib().ag_kv_project_cache(ctypes.byref(desc), _ptr(X), _ptr(Wk), _ptr(Wv), _ptr(flags),
-                                            ctypes.byref(cache.struct), _ptr(prefix), _ptr(idx), _ptr(K), _ptr(V),
-                                            _ptr(dev_status), _stream(stream)), "ag_kv_project_cache")
+    return _check((_m or _marshal()).kv_project_cache(desc, X, Wk, Wv, flags, cache, prefix, idx, K, V, dev_status,
+                                                      stream), "ag_kv_project_cache")
 
 
 def ag_qkv_project_cache(desc, X, Wq, Wk, Wv, flags, cache, prefix, idx, Q, K, V, dev_status, stream=None):
-    return _check(lib().ag_qkv_project_cache(ctypes.byref(desc), _ptr(X), _ptr(Wq), _ptr(Wk), _ptr(Wv), _ptr(flags),
-                                             ctypes.byref(cache.struct), _ptr(prefix), _ptr(idx), _ptr(Q), _ptr(K),
-                                             _ptr(V), _ptr(dev_status), _stream(stream)), "ag_qkv_project_cache")
+    return _check((_m or _marshal()).qkv_project_cache(desc, X, Wq, Wk, Wv, flags, cache, prefix, idx, Q, K, V,
+                                                       dev_status, stream), "ag_qkv_project_cache")
 
 
 def ag_prefill_attn(desc, Q, K, V, flags, cache, prefix, softmax_scale, O, ws, stream=None):
-    p, nbytes = _ws(ws)
-    return _check(lib().ag_prefill_attn(ctypes.byref(desc), _ptr(Q), _ptr(K), _ptr(V), _ptr(flags),
-                                        ctypes.byref(cache.struct), _ptr(prefix), float(softmax_scale),
-                                        _ptr(O), p, nbytes, _stream(stream)), "ag_prefill_attn")
+    return _check((_m or _marshal()).prefill_attn(desc, Q, K, V, flags, cache, prefix, softmax_scale, O, ws, stream),
+                  "ag_prefill_attn")
 
 
 def ag_out_project(desc, O, Wo, X_res, Y, stream=None):
-    return _check(lib().ag_out_project(ctypes.byref(desc), _ptr(O), _ptr(Wo), _ptr(X_res), _ptr(Y), _stream(stream)),
-                  "ag_out_project")
+    return _check((_m or _marshal()).out_project(desc, O, Wo, X_res, Y, stream), "ag_out_project")
 
 
 def ag_decode_attn(desc, q, k_new, v_new, cache, softmax_scale, o, ws, stream=None):
-    p, nbytes = _ws(ws)
-    return _check(lib().ag_decode_attn(ctypes.byref(desc), _ptr(q), _ptr(k_new), _ptr(v_new),
-                                       ctypes.byref(cache.struct), float(softmax_scale), _ptr(o), p, nbytes,
-                                       _stream(stream)), "ag_decode_attn")
+    return _check((_m or _marshal()).decode_attn(desc, q, k_new, v_new, cache, softmax_scale, o, ws, stream),
+                  "ag_decode_attn")
 
 
 def ag_decode_attn_noalloc(desc, q, k_new, v_new, cache, softmax_scale, o, stream=None):
@@ -247,21 +239,17 @@ def ag_decode_attn_noalloc(desc, q, k_new, v_new, cache, softmax_scale, o, strea
     workspace (see include/ag.h): same result, scratch held inside the library,
     no allocation.  Calls on one device must not overlap; batch * heads is
     limited (1024 at head_dim 128), beyond which AgError(AG_ERR_CAPACITY)."""
-    return _check(lib().ag_decode_attn_noalloc(ctypes.byref(desc), _ptr(q), _ptr(k_new), _ptr(v_new),
-                                               ctypes.byref(cache.struct), float(softmax_scale), _ptr(o),
-                                               _stream(stream)), "ag_decode_attn_noalloc")
+    return _check((_m or _marshal()).decode_attn_noalloc(desc, q, k_new, v_new, cache, softmax_scale, o, stream),
+                  "ag_decode_attn_noalloc")
 
 
 def ag_decode_step(desc, q, k_new, v_new, flag_new, cache, softmax_scale, o, dev_status, ws, stream=None):
-    p, nbytes = _ws(ws)
-    return _check(lib().ag_decode_step(ctypes.byref(desc), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(flag_new),
-                                       ctypes.byref(cache.struct), float(softmax_scale), _ptr(o), _ptr(dev_status),
-                                       p, nbytes, _stream(stream)), "ag_decode_step")
+    return _check((_m or _marshal()).decode_step(desc, q, k_new, v_new, flag_new, cache, softmax_scale, o, dev_status,
+                                                 ws, stream), "ag_decode_step")
 
 
 def ag_cache_append(desc, k_new, v_new, flag_new, cache, dev_status, stream=None):
-    return _check(lib().ag_cache_append(ctypes.byref(desc), _ptr(k_new), _ptr(v_new), _ptr(flag_new),
-                                        ctypes.byref(cache.struct), _ptr(dev_status), _stream(stream)),
+    return _check((_m or _marshal()).cache_append(desc, k_new, v_new, flag_new, cache, dev_status, stream),
                   "ag_cache_append")
 
 
