@@ -31,13 +31,18 @@ namespace ag {
 using namespace umma;
 
 constexpr int kGaThreads = 192;
-constexpr int kGaBM = 128, kGaBN = 64, kGaD = 128;
+constexpr int kGaBM = 128, kGaBN = 64;
 constexpr int kGaPanel = 128 * 128;                  // Q: [128 rows][64 bf16]
-constexpr int kGaTile = 2 * kGaPanel;                // 32 KB: Q hi or Q lo
 constexpr int kGaKvPanel = kGaBN * 128;              // K / V: [64 rows][64 bf16] = 8 KB
-constexpr int kGaKvTile = 2 * kGaKvPanel;            // 16 KB: one of hi / lo
-constexpr int kGaKvStage = 2 * kGaKvTile;            // 32 KB: hi + lo
-constexpr int kGaSmemBytes = 2 * kGaTile + 4 * kGaKvStage + 1024 + 256;   // Q + 2 K stages + 2 V stages
+// Tiles of gate heads of width D (64 or 128): one or two 64-column panels.
+template <int D>
+struct GaCfg {
+  static constexpr int kPanels = D / 64;
+  static constexpr int kTile = kPanels * kGaPanel;        // Q hi or Q lo
+  static constexpr int kKvTile = kPanels * kGaKvPanel;    // K or V, one of hi / lo
+  static constexpr int kKvStage = 2 * kKvTile;            // hi + lo
+  static constexpr int kSmemBytes = 2 * kTile + 4 * kKvStage + 1024 + 256;   // Q + 2 K stages + 2 V stages
+};
 constexpr uint32_t kGaColS = 0, kGaColO = 256, kGaColPhi = 384, kGaColPlo = 448, kGaTmemCols = 512;
 constexpr float kGaRescaleThreshold = 8.f;
 
@@ -46,7 +51,7 @@ constexpr int kGaPieceCost = 3;      // set-up + epilogue of a piece, in half ti
 
 struct GateAttnArgs {
   const int32_t *seq_lens;  // [B] or NULL: tokens past seq_lens[b] are padding
-  float *part_o;            // [items, 128, 128] un-normalised partial outputs
+  float *part_o;            // [items, 128, D] un-normalised partial outputs
   float *part_ml;           // [items, 128, 2]   running max (log2 units) and sum per row
   int n, n_qtiles, gate_heads, problems, GD, causal;
   int steps_per_prob;       // (query tile, key tile) steps of one (sequence, head)
@@ -109,10 +114,13 @@ __host__ __device__ inline int ga_slot(int prob, int qt, int n_qtiles, int seg) 
   return prob * n_qtiles + qt + seg;
 }
 
+template <int kGaD>
 __global__ void __launch_bounds__(kGaThreads, 1)
 gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__ CUtensorMap tmLo,
                     const __grid_constant__ CUtensorMap tmHiKv, const __grid_constant__ CUtensorMap tmLoKv,
                     const __grid_constant__ GateAttnArgs a) {
+  using C = GaCfg<kGaD>;
+  constexpr int kGaTile = C::kTile, kGaKvTile = C::kKvTile, kGaKvStage = C::kKvStage;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sQ = smem;                    // [hi | lo]
@@ -171,16 +179,18 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
         ok = mbar_wait(q_empty, (pc & 1) ^ 1);       // the previous piece's last Q K^T has read Q
         if (!ok) break;
         mbar_arrive_expect_tx(q_full, 2 * kGaTile);
-        tma_load_3d(sQ, &tmHi, q_full, xq, j0, b);
-        tma_load_3d(sQ + kGaPanel, &tmHi, q_full, xq + 64, j0, b);
-        tma_load_3d(sQ + kGaTile, &tmLo, q_full, xq, j0, b);
-        tma_load_3d(sQ + kGaTile + kGaPanel, &tmLo, q_full, xq + 64, j0, b);
+#pragma unroll
+        for (int p = 0; p < C::kPanels; ++p) {
+          tma_load_3d(sQ + p * kGaPanel, &tmHi, q_full, xq + p * 64, j0, b);
+          tma_load_3d(sQ + kGaTile + p * kGaPanel, &tmLo, q_full, xq + p * 64, j0, b);
+        }
         auto load_kv = [&](uint8_t *dst, uint64_t *bar, int xc, int y) {
           mbar_arrive_expect_tx(bar, kGaKvStage);
-          tma_load_3d(dst, &tmHiKv, bar, xc, y, b);
-          tma_load_3d(dst + kGaKvPanel, &tmHiKv, bar, xc + 64, y, b);
-          tma_load_3d(dst + kGaKvTile, &tmLoKv, bar, xc, y, b);
-          tma_load_3d(dst + kGaKvTile + kGaKvPanel, &tmLoKv, bar, xc + 64, y, b);
+#pragma unroll
+          for (int p = 0; p < C::kPanels; ++p) {
+            tma_load_3d(dst + p * kGaKvPanel, &tmHiKv, bar, xc + p * 64, y, b);
+            tma_load_3d(dst + kGaKvTile + p * kGaKvPanel, &tmLoKv, bar, xc + p * 64, y, b);
+          }
         };
         for (int i = 0; i < pz.n_kv; ++i, ++t) {
           const int st = t & 1;
@@ -337,7 +347,7 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
         if (!ok) break;
         tc_fence_after_sync();
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < kGaD / 32; ++c) {
           uint32_t r[32];
           tmem_ld_x32_sync(tm_lane + kGaColO + c * 32, r);
 #pragma unroll
@@ -386,10 +396,10 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
       const size_t it = (size_t)ga_slot(pz.prob, pz.qt, a.n_qtiles, (int)blockIdx.x);
       float *op = a.part_o + (it * kGaBM + row) * kGaD;
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < kGaD / 32; ++c) {
         uint32_t r[32];
         tmem_ld_x32_sync(tm_lane + kGaColO + c * 32, r);
-        if (c == 3) {                                // O is in registers: the next piece may overwrite it
+        if (c + 1 == kGaD / 32) {                                // O is in registers: the next piece may overwrite it
           tc_fence_before_sync();
           mbar_arrive(o_free);
         }
@@ -412,18 +422,21 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
 
 bool gate_attn_tc_supported(const ag_layer_desc &d) {
   const int GD = d.gate_heads * d.gate_head_dim;
-  return d.dtype == AG_BF16 && d.gate_head_dim == 128 && gate_proj_tc_supported(d.hidden, GD);
+  return d.dtype == AG_BF16 && (d.gate_head_dim == 128 || d.gate_head_dim == 64) && gate_proj_tc_supported(d.hidden, GD);
 }
 
 // The split-K merge of MHA' and the gate's output layer in one pass (Eq. 3, Eq. 4):
-//   H'[t, g * 128 + c] = sum_s w_s O_s[r, c] / sum_s w_s l_s,  w_s = 2^(m_s - max_s m_s)
+//   H'[t, g * D + c] = sum_s w_s O_s[r, c] / sum_s w_s l_s,  w_s = 2^(m_s - max_s m_s)
 //   s[t, i] = H'[t, :] Wo_g[:, i];  flag = s + gamma_i > logit(tau)
 // One CTA = 16 tokens, one warp per token.  A warp merges the token's row of every gate head
-// (a lane per four columns: every access is one 512-byte row) into shared memory; then warp w
+// (a lane per D / 32 columns: every access is one whole row) into shared memory; then warp w
 // takes four tokens and a quarter of the reduction, a lane per head, in rounds of 32 heads,
 // against a [GD][32] slice of Wo staged in shared memory.  H' never goes to global memory.
 constexpr int kMoTokens = 16, kMoThreads = kMoTokens * 32;
-template <typename T>
+template <int N> struct FloatVec;
+template <> struct FloatVec<2> { using type = float2; };
+template <> struct FloatVec<4> { using type = float4; };
+template <typename T, int kGaD>
 __global__ void __launch_bounds__(kMoThreads)
 gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const T *__restrict__ Wo, const float *__restrict__ gamma,
                       float logit_tau, int h, float *__restrict__ scores, uint8_t *__restrict__ flags) {
@@ -471,20 +484,28 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const T *__restric
       for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) mmax[u] = fmaxf(mmax[u], __shfl_xor_sync(0xffffffffu, mmax[u], off));
-      float4 acc[4];
+      constexpr int kV = kGaD / 32;                  // columns per lane
+      using Vec = typename FloatVec<kV>::type;
+      float acc[4][kV];
       float lsum[4];
       int ns_max = 0;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) { acc[u] = make_float4(0.f, 0.f, 0.f, 0.f); lsum[u] = 0.f; ns_max = max(ns_max, ns[u]); }
+      for (int u = 0; u < 4; ++u) {
+#pragma unroll
+        for (int e = 0; e < kV; ++e) acc[u][e] = 0.f;
+        lsum[u] = 0.f;
+        ns_max = max(ns_max, ns[u]);
+      }
       for (int s = 0; s < ns_max; ++s) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           if (s < ns[u]) {
             const float2 ml = *reinterpret_cast<const float2 *>(a.part_ml + (row0[u] + (size_t)s * kGaBM) * 2);
-            const float4 o = *reinterpret_cast<const float4 *>(a.part_o + (row0[u] + (size_t)s * kGaBM) * kGaD + lane * 4);
+            const Vec o4 = *reinterpret_cast<const Vec *>(a.part_o + (row0[u] + (size_t)s * kGaBM) * kGaD + lane * kV);
+            const float *o = reinterpret_cast<const float *>(&o4);
             const float w = fast_exp2(ml.x - mmax[u]);
-            acc[u].x = fmaf(w, o.x, acc[u].x); acc[u].y = fmaf(w, o.y, acc[u].y);
-            acc[u].z = fmaf(w, o.z, acc[u].z); acc[u].w = fmaf(w, o.w, acc[u].w);
+#pragma unroll
+            for (int e = 0; e < kV; ++e) acc[u][e] = fmaf(w, o[e], acc[u][e]);
             lsum[u] = fmaf(w, ml.y, lsum[u]);
           }
         }
@@ -493,8 +514,10 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const T *__restric
       for (int u = 0; u < 4; ++u) {
         if (g0 + u < a.gate_heads) {
           const float inv = 1.f / lsum[u];
-          *reinterpret_cast<float4 *>(hrow + (g0 + u) * kGaD + lane * 4) =
-              make_float4(acc[u].x * inv, acc[u].y * inv, acc[u].z * inv, acc[u].w * inv);
+          Vec hv;
+#pragma unroll
+          for (int e = 0; e < kV; ++e) reinterpret_cast<float *>(&hv)[e] = acc[u][e] * inv;
+          *reinterpret_cast<Vec *>(hrow + (g0 + u) * kGaD + lane * kV) = hv;
         }
       }
     }
@@ -622,12 +645,14 @@ size_t gate_attn_partial_bytes(const ag_layer_desc &d) {
   // one slot per piece: query tiles + segments, whatever the device (no device is asked here)
   const size_t nq = (d.seq + kGaBM - 1) / kGaBM;
   const size_t slots = (size_t)d.batch * d.gate_heads * nq + kGaMaxSeg;
-  return align_up(slots * kGaBM * kGaD * sizeof(float), 256) + align_up(slots * kGaBM * 2 * sizeof(float), 256);
+  return align_up(slots * kGaBM * d.gate_head_dim * sizeof(float), 256) + align_up(slots * kGaBM * 2 * sizeof(float), 256);
 }
 
-int launch_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const void *qkv_lo, void *partials,
-                        const void *Wo, const float *gamma, float logit_tau, float *scores, uint8_t *flags,
-                        cudaStream_t st) {
+template <int kGaD>
+static int run_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const void *qkv_lo, void *partials,
+                            const void *Wo, const float *gamma, float logit_tau, float *scores, uint8_t *flags,
+                            cudaStream_t st) {
+  constexpr int kGaSmemBytes = GaCfg<kGaD>::kSmemBytes;
   const int GD = d.gate_heads * d.gate_head_dim;
   CUtensorMap tmHi, tmLo;
   int rc = make_tmap_3d_bf16(&tmHi, qkv_hi, d.batch, d.seq, 3 * GD, kGaBM, 64);
@@ -650,17 +675,24 @@ int launch_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const void *
   a.part_ml = reinterpret_cast<float *>(static_cast<char *>(partials) +
                                         align_up(slots * kGaBM * kGaD * sizeof(float), 256));
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)kGaD));
-  AG_CUDA_TRY(cudaFuncSetAttribute(gate_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGaSmemBytes));
-  gate_attn_tc_kernel<<<(unsigned)plan.n_seg, kGaThreads, kGaSmemBytes, st>>>(tmHi, tmLo, tmHiKv, tmLoKv, a);
+  AG_CUDA_TRY(cudaFuncSetAttribute(gate_attn_tc_kernel<kGaD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGaSmemBytes));
+  gate_attn_tc_kernel<kGaD><<<(unsigned)plan.n_seg, kGaThreads, kGaSmemBytes, st>>>(tmHi, tmLo, tmHiKv, tmLoKv, a);
   AG_LAUNCH_CHECK();
   const size_t mo_smem = sizeof(float) * kMoTokens * GD + sizeof(__nv_bfloat16) * GD * 32 + sizeof(float) * 4 * kMoTokens * 32;
-  auto mo = gate_merge_out_kernel<__nv_bfloat16>;
+  auto mo = gate_merge_out_kernel<__nv_bfloat16, kGaD>;
   AG_CUDA_TRY(cudaFuncSetAttribute(mo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mo_smem));
   const int blocks = d.batch * ((d.seq + kMoTokens - 1) / kMoTokens);
   mo<<<blocks, kMoThreads, mo_smem, st>>>(a, static_cast<const __nv_bfloat16 *>(Wo), gamma, logit_tau, kv_heads_of(d),
                                           scores, flags);
   AG_LAUNCH_CHECK();
   return AG_OK;
+}
+
+int launch_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const void *qkv_lo, void *partials,
+                        const void *Wo, const float *gamma, float logit_tau, float *scores, uint8_t *flags,
+                        cudaStream_t st) {
+  return d.gate_head_dim == 64 ? run_gate_attn_tc<64>(d, qkv_hi, qkv_lo, partials, Wo, gamma, logit_tau, scores, flags, st)
+                               : run_gate_attn_tc<128>(d, qkv_hi, qkv_lo, partials, Wo, gamma, logit_tau, scores, flags, st);
 }
 
 int gate_attn_tc_wait_timeouts() {

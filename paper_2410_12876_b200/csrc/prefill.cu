@@ -155,6 +155,7 @@ int launch_prefill(const ag_layer_desc &d, const void *Q, const void *K, const v
   if (prefill_tc_supported(d, c)) {
     int rc = launch_prefill_tc(d, Q, K, V, c, prefix, scale, O, lse, st);
     if (rc || !lse) return rc;
+    if (d.head_dim == 64) return run_prefill_band<__nv_bfloat16, 64>(d, Q, K, V, flags, lse, scale, O, st);
     return launch_prefill_band_mma(d, Q, K, V, flags, lse, scale, O, st);
   }
   if (d.dtype == AG_F32) {

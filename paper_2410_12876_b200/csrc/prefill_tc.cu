@@ -1,5 +1,5 @@
 // Prefill attention under the eviction mask (Eq. 2 with M_i of Eq. 5) on the
-// Blackwell tensor cores, bf16, head_dim 128.
+// Blackwell tensor cores, bf16, head_dim 64 or 128.
 //
 // One CTA handles 128 consecutive queries of one slab s = (sequence, head).
 // Query j attends to cache rows r < prefix[s, j] (exactly the retained tokens
@@ -14,7 +14,7 @@
 //               P written back to TMEM as bf16, O rescaled only when the running
 //               maximum grows by more than 2^8, final normalisation and store
 //
-// TMEM columns: S0 [0,64) S1 [64,128), each overwritten in place by its P (bf16 pairs); O [128,256).
+// TMEM columns: S0 [0,64) S1 [64,128), each overwritten in place by its P (bf16 pairs); O [128,128 + D).
 // The self term seeds the running softmax (m = s_jj, l = 1) and its value row
 // is added in the epilogue: O_j = (sum_r p_r v_r + w_self v_j) / l.  Every byte
 // that enters or leaves the CTA travels by TMA.
@@ -26,18 +26,23 @@ namespace ag {
 using namespace umma;
 
 constexpr int kPfThreads = 192;
-constexpr int kPfBM = 128, kPfD = 128;
+constexpr int kPfBM = 128;
 constexpr int kPfPanel = 128 * 128;                   // [128 rows][64 bf16] = 16 KB (Q, dense K / V, O)
-constexpr int kPfTile = 2 * kPfPanel;                 // 32 KB
 constexpr float kRescaleThreshold = 8.f;              // log2 units
 
 // Key tiles of 64 cache rows; two CTAs per SM (256 TMEM columns, 97 KB of shared memory each).
 // 128-row tiles with one CTA per SM measured slower on 4096-token heads (131 us against 100 us).
 constexpr int kPfBN = 64;
 constexpr int kPfKvPanel = kPfBN * 128;               // [64 rows][64 bf16] = 8 KB
-constexpr int kPfKvTile = 2 * kPfKvPanel;             // 16 KB
-constexpr int kPfKvBuf = 2 * kPfKvTile;               // two stages = one 32 KB dense tile
-constexpr int kPfSmemBytes = kPfTile + 2 * kPfKvBuf + 1024 + 256;
+// A tile is one 64-column panel (head_dim 64) or two (128).
+template <int D>
+struct PfCfg {
+  static constexpr int kPanels = D / 64;
+  static constexpr int kTile = kPanels * kPfPanel;    // Q, dense K / V, O: 16 or 32 KB
+  static constexpr int kKvTile = kPanels * kPfKvPanel;
+  static constexpr int kKvBuf = 2 * kKvTile;          // two stages = one dense tile
+  static constexpr int kSmemBytes = kTile + 2 * kKvBuf + 1024 + 256;
+};
 constexpr uint32_t kColS = 0, kColO = 2 * kPfBN, kTmemCols = 256;
 constexpr int kPfCtasPerSm = 2;
 
@@ -68,11 +73,14 @@ __device__ __forceinline__ uint32_t tile_chunk_offset(int row, int chunk) {
 // CTA's own 128 rows, of which only the diagonal (q_j . k_j) is read.  Last,
 // the dense V tile is brought in for the self term of the output, and the O
 // tile leaves through shared memory with one TMA store.
+template <int kPfD>
 __global__ void __launch_bounds__(kPfThreads, kPfCtasPerSm)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKd,
                   const __grid_constant__ CUtensorMap tmVd, const __grid_constant__ CUtensorMap tmO,
                   const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                   const PrefillTcArgs a) {
+  using C = PfCfg<kPfD>;
+  constexpr int kPfTile = C::kTile, kPfKvTile = C::kKvTile, kPfKvBuf = C::kKvBuf;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sQ = smem;
@@ -137,26 +145,28 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       bool ok = true;
       if (n_kv > 0) {
         mbar_arrive_expect_tx(q_full, kPfTile);
-        tma_load_3d(sQ, &tmQ, q_full, 0, j0, slab);
-        tma_load_3d(sQ + kPfPanel, &tmQ, q_full, 64, j0, slab);
+#pragma unroll
+        for (int p = 0; p < C::kPanels; ++p) tma_load_3d(sQ + p * kPfPanel, &tmQ, q_full, p * 64, j0, slab);
         // self tile: dense K rows j0 .. j0 + 127 across both V stages, which no P V needs before
         // the first softmax is done; the first cache tiles of K load alongside it
         mbar_arrive_expect_tx(&v_full[0], kPfTile);
-        tma_load_3d(sV, &tmKd, &v_full[0], 0, j0, kv_slab);
-        tma_load_3d(sV + kPfPanel, &tmKd, &v_full[0], 64, j0, kv_slab);
+#pragma unroll
+        for (int p = 0; p < C::kPanels; ++p) tma_load_3d(sV + p * kPfPanel, &tmKd, &v_full[0], p * 64, j0, kv_slab);
         for (int i = 0; i < n_kv && ok; ++i) {
           const int st = i & 1;
           const int y = row0 + i * kPfBN;
           ok = mbar_wait(&k_empty[st], ((i >> 1) & 1) ^ 1);     // earlier uses of the stage: i >> 1
           if (!ok) break;
           mbar_arrive_expect_tx(&k_full[st], kPfKvTile);
-          tma_load_2d(sK + st * kPfKvTile, &tmK, &k_full[st], 0, y);
-          tma_load_2d(sK + st * kPfKvTile + kPfKvPanel, &tmK, &k_full[st], 64, y);
+#pragma unroll
+          for (int p = 0; p < C::kPanels; ++p)
+            tma_load_2d(sK + st * kPfKvTile + p * kPfKvPanel, &tmK, &k_full[st], p * 64, y);
           ok = mbar_wait(&v_empty[st], (i >> 1) & 1);           // the self tile + i >> 1 earlier tiles
           if (!ok) break;
           mbar_arrive_expect_tx(&v_full[st], kPfKvTile);
-          tma_load_2d(sV + st * kPfKvTile, &tmV, &v_full[st], 0, y);
-          tma_load_2d(sV + st * kPfKvTile + kPfKvPanel, &tmV, &v_full[st], 64, y);
+#pragma unroll
+          for (int p = 0; p < C::kPanels; ++p)
+            tma_load_2d(sV + st * kPfKvTile + p * kPfKvPanel, &tmV, &v_full[st], p * 64, y);
         }
       }
       // dense V rows for the self term of the output, into the K buffer once both stages are free
@@ -164,8 +174,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       if (ok && k1_uses > 0) ok = mbar_wait(&k_empty[1], (k1_uses & 1) ^ 1);
       if (ok) {
         mbar_arrive_expect_tx(&k_full[0], kPfTile);
-        tma_load_3d(sK, &tmVd, &k_full[0], 0, j0, kv_slab);
-        tma_load_3d(sK + kPfPanel, &tmVd, &k_full[0], 64, j0, kv_slab);
+#pragma unroll
+        for (int p = 0; p < C::kPanels; ++p) tma_load_3d(sK + p * kPfPanel, &tmVd, &k_full[0], p * 64, j0, kv_slab);
       }
     }
   } else if (warp == 1) {
@@ -338,7 +348,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         if (!ok) break;
         tc_fence_after_sync();
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < kPfD / 32; ++c) {
           uint32_t o[32];
           tmem_ld_x32_sync(tm_lane + kColO + c * 32, o);
 #pragma unroll
@@ -353,12 +363,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       if ((i + 1) * kPfBN > L) {
         ok = mbar_wait(&v_full[st], ((i >> 1) + (st == 0 ? 1 : 0)) & 1);
         if (!ok) break;
-        const int vr = tid >> 1;                      // two threads per row, one panel each
+        const int vr = tid >> 1;                      // two threads per row, one half each
         if (i * kPfBN + vr >= L) {
           uint4 z = make_uint4(0, 0, 0, 0);
-          uint8_t *v0 = sV + st * kPfKvTile + (tid & 1) * kPfKvPanel + vr * 128;
+          uint8_t *v0 = sV + st * kPfKvTile + vr * 128 + (tid & 1) * (kPfD == 128 ? kPfKvPanel : 64);
 #pragma unroll
-          for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4 *>(v0 + c * 16) = z;
+          for (int c = 0; c < kPfD / 16; ++c) *reinterpret_cast<uint4 *>(v0 + c * 16) = z;
         }
         fence_proxy_async_smem();
       }
@@ -379,7 +389,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       const float inv = 1.f / l;
       if (a.lse != nullptr && valid) a.lse[(size_t)slab * a.n + j] = n_kv > 0 ? m + log2f(l) : -INFINITY;
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < kPfD / 32; ++c) {
         uint32_t r[32];
         if (n_kv > 0) {
           tmem_ld_x32_sync(tm_lane + kColO + c * 32, r);
@@ -406,8 +416,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     }
     named_barrier_sync(1, 128);
     if (ok && threadIdx.x == 64) {
-      tma_store_3d(&tmO, sV, 0, j0, slab);           // rows past n are dropped by the tensor map
-      tma_store_3d(&tmO, sV + kPfPanel, 64, j0, slab);
+#pragma unroll
+      for (int p = 0; p < C::kPanels; ++p)           // rows past n are dropped by the tensor map
+        tma_store_3d(&tmO, sV + p * kPfPanel, p * 64, j0, slab);
       tma_store_commit();
       tma_store_wait_read();
     }
@@ -418,12 +429,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 }
 
 bool prefill_tc_supported(const ag_layer_desc &d, const ag_cache &c) {
-  return d.dtype == AG_BF16 && d.head_dim == 128 && c.pool_rows < ((int64_t)1 << 31) &&
+  return d.dtype == AG_BF16 && c.pool_rows < ((int64_t)1 << 31) &&
          (int64_t)d.batch * d.heads * ((d.seq + kPfBM - 1) / kPfBM) < ((int64_t)1 << 31);
 }
 
-int launch_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const ag_cache &c,
-                      const int32_t *prefix, float scale, void *O, float *lse, cudaStream_t st) {
+template <int kPfD>
+static int run_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const ag_cache &c,
+                          const int32_t *prefix, float scale, void *O, float *lse, cudaStream_t st) {
   const int slabs = d.batch * d.heads;
   CUtensorMap tmQ, tmKd, tmVd, tmO, tmK, tmV;
   int rc;
@@ -445,10 +457,17 @@ int launch_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, cons
   a.scale_log2 = scale * 1.4426950408889634f;
   a.lse = lse;
   a.seq_lens = d.seq_lens;
-  AG_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmemBytes));
-  prefill_tc_kernel<<<a.n_qtiles * slabs, kPfThreads, kPfSmemBytes, st>>>(tmQ, tmKd, tmVd, tmO, tmK, tmV, a);
+  constexpr int smem = PfCfg<kPfD>::kSmemBytes;
+  AG_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel<kPfD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  prefill_tc_kernel<kPfD><<<a.n_qtiles * slabs, kPfThreads, smem, st>>>(tmQ, tmKd, tmVd, tmO, tmK, tmV, a);
   AG_LAUNCH_CHECK();
   return AG_OK;
+}
+
+int launch_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const ag_cache &c,
+                      const int32_t *prefix, float scale, void *O, float *lse, cudaStream_t st) {
+  return d.head_dim == 64 ? run_prefill_tc<64>(d, Q, K, V, c, prefix, scale, O, lse, st)
+                          : run_prefill_tc<128>(d, Q, K, V, c, prefix, scale, O, lse, st);
 }
 
 int prefill_tc_wait_timeouts() {
