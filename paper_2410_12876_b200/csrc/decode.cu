@@ -71,13 +71,13 @@ __device__ __forceinline__ void append_new_row(const AppendArgs &ap, int slab, i
   if (vec == 0) ap.len[slab] = L + 1;
 }
 
-// Recent-token window: scores of the query against the ring of its key/value slab, by every warp
-// of the CTA: sm_s[r] = scale_log2 * q . k_r for a live slot (an evicted token the query still
+// Recent-token window: scores of the query against the ring of its key/value slab, by warps 0 .. n_warps - 1
+// of those that call: sm_s[r] = scale_log2 * q . k_r for a live slot (an evicted token the query still
 // sees), -inf otherwise.  The caller synchronises the CTA before reading sm_s.
 template <typename T, int D>
-__device__ __forceinline__ void ring_scores(const RecentRing &rg, int kv, const T *__restrict__ q_row,
-                                            float scale_log2, float *sm_s) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
+__device__ __forceinline__ void ring_scores_part(const RecentRing &rg, int kv, const T *__restrict__ q_row,
+                                                 float scale_log2, float *sm_s, int warp, int n_warps) {
+  const int lane = threadIdx.x & 31;
   for (int r = warp; r < rg.R; r += n_warps) {
     const T *kr = static_cast<const T *>(rg.k) + ((size_t)kv * rg.R + r) * D;
     float a = 0.f;
@@ -87,6 +87,12 @@ __device__ __forceinline__ void ring_scores(const RecentRing &rg, int kv, const 
     for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
     if (lane == 0) sm_s[r] = rg.live[(size_t)kv * rg.R + r] != 0 ? a * scale_log2 : -INFINITY;
   }
+}
+
+template <typename T, int D>
+__device__ __forceinline__ void ring_scores(const RecentRing &rg, int kv, const T *__restrict__ q_row,
+                                            float scale_log2, float *sm_s) {
+  ring_scores_part<T, D>(rg, kv, q_row, scale_log2, sm_s, threadIdx.x >> 5, blockDim.x >> 5);
 }
 
 // Rows [r_begin, r_end) of one slab, streamed by a whole CTA of kThreads threads: thread (g, v) =
@@ -169,6 +175,8 @@ decode_partial_kernel(const T *__restrict__ q, const T *__restrict__ k_rows,
   constexpr int kGroups = kPartThreads / kLanes;
   const int slab = blockIdx.y, chunk = blockIdx.x;
   const int kv = hm.kv_slab(slab);
+  pdl_launch_dependents();
+  pdl_wait();
   const int L = len[kv];
   const int r_begin = chunk * chunk_rows;
   if (r_begin >= L) return;
@@ -218,6 +226,8 @@ decode_partial_gqa_kernel(const T *__restrict__ q, const T *__restrict__ k_rows,
   constexpr int kGroups = kPartThreads / kLanes;
   const int kv = blockIdx.y, chunk = blockIdx.x;
   const int slab0 = (kv / kv_heads) * kv_heads * G + (kv % kv_heads) * G;   // first query slab of the group
+  pdl_launch_dependents();
+  pdl_wait();
   const int L = len[kv];
   const int r_begin = chunk * chunk_rows;
   if (r_begin >= L) return;
@@ -312,61 +322,88 @@ decode_partial_gqa_kernel(const T *__restrict__ q, const T *__restrict__ k_rows,
   }
 }
 
-// One CTA of D threads per slab: thread d owns output dimension d.
+// Merges the chunks' triples of every query slab with the self term.  One CTA per key/value slab: D threads
+// (thread d owns output dimension d) for each of blockDim.y query heads of the group, in rounds, so that the
+// CTA that appends to the slab is the only one that reads its length.  The chunks' weights are computed
+// side by side, a chunk per lane, and the partial outputs are loaded eight at a time: one chunk after the
+// other, each load waiting for its turn, took 11.5 us for 1024 query slabs of 17 chunks.
 template <typename T, int D>
-__global__ void __launch_bounds__(D)
+__global__ void __launch_bounds__(512)
 decode_combine_kernel(const T *__restrict__ q, const T *__restrict__ k_new,
                       const T *__restrict__ v_new, const int32_t *len,
                       float scale_log2, int chunk_rows, const float *__restrict__ part_o,
                       const float *__restrict__ part_ml, T *__restrict__ o,
-                      const int64_t *__restrict__ row_off, const AppendArgs ap, const HeadMap hm,
-                      const RecentRing rg) {
-  const int slab = blockIdx.x, d = threadIdx.x;
-  const int kv = hm.kv_slab(slab);
+                      const int64_t *__restrict__ row_off, int G, const AppendArgs ap, const RecentRing rg) {
+  static_assert(kMaxSplits == 32, "a lane per chunk");
+  const int kv = blockIdx.x, d = threadIdx.x, y = threadIdx.y, lane = d & 31;
+  constexpr int kMaxHeads = 512 / D;
+  __shared__ float red[kMaxHeads][D / 32];
+  __shared__ float ring_s[kMaxHeads][kMaxRecent];
+  __shared__ float wgt[kMaxHeads][kMaxSplits];       // weight of every chunk
+  __shared__ float lsum_s[kMaxHeads][2];             // maximum and sum over chunks, self and ring
+  pdl_launch_dependents();
+  pdl_wait();
+  const float kn = Elem<T>::load(k_new + (size_t)kv * D + d), vn = Elem<T>::load(v_new + (size_t)kv * D + d);
   const int L = len[kv];
   const int n_chunks = (L + chunk_rows - 1) / chunk_rows;
-  __shared__ float red[D / 32];
-  __shared__ float ring_s[kMaxRecent];
-  float a = Elem<T>::load(q + (size_t)slab * D + d) * Elem<T>::load(k_new + (size_t)kv * D + d);
+  for (int h0 = 0; h0 < G; h0 += blockDim.y) {
+    const int h = h0 + y;
+    const bool on = h < G;                           // whole warps: D is a multiple of 32
+    const int slab = kv * G + min(h, G - 1);
+    float a = Elem<T>::load(q + (size_t)slab * D + d) * kn;
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-  if ((d & 31) == 0) red[d >> 5] = a;
-  ring_scores<T, D>(rg, kv, q + (size_t)slab * D, scale_log2, ring_s);
-  __syncthreads();
-  // Every thread of the CTA has read the slab's length (above the barrier), and the chunk pass, the
-  // only reader of the slab's rows, has completed: the new row may go in and the length may move.
-  // (Never asked for when query heads share a slab: another head's CTA may still be reading its length.)
-  append_new_row<T, D>(ap, kv, L, row_off[kv], k_new, v_new);
-  float s_self = 0.f;
-#pragma unroll
-  for (int i = 0; i < D / 32; ++i) s_self += red[i];
-  s_self *= scale_log2;
-  const float *pml = part_ml + (size_t)slab * kMaxSplits * 2;
-  float m = s_self;
-  for (int c = 0; c < n_chunks; ++c) m = fmaxf(m, pml[2 * c]);
-  for (int r = 0; r < rg.R; ++r) m = fmaxf(m, ring_s[r]);
-  const float w_self = exp2f(s_self - m);
-  float acc = w_self * Elem<T>::load(v_new + (size_t)kv * D + d);
-  float l = w_self;
-  const float *po = part_o + (size_t)slab * kMaxSplits * D + d;
-  for (int c = 0; c < n_chunks; ++c) {
-    const float w = exp2f(pml[2 * c] - m);
-    acc = fmaf(w, po[(size_t)c * D], acc);
-    l = fmaf(w, pml[2 * c + 1], l);
-  }
-  // the evicted tokens of the recent-token window
-  for (int r = 0; r < rg.R; ++r) {
-    if (ring_s[r] == -INFINITY) continue;
-    const float w = exp2f(ring_s[r] - m);
-    acc = fmaf(w, Elem<T>::load(static_cast<const T *>(rg.v) + ((size_t)kv * rg.R + r) * D + d), acc);
-    l += w;
-  }
-  Elem<T>::store(o + (size_t)slab * D + d, acc / l);
-  if (rg.R > 0 && ap.flag_new != nullptr) {
-    // the step carries the append: the new token joins the ring once every thread has read it
-    constexpr int kVecs = D * (int)sizeof(T) / 16;
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    if (lane == 0) red[y][d >> 5] = a;
+    ring_scores_part<T, D>(rg, kv, q + (size_t)slab * D, scale_log2, ring_s[y], d >> 5, D / 32);
     __syncthreads();
-    if (d < kVecs)
+    if (d < 32) {
+      // one warp per head: the chunks' maxima and sums, one per lane
+      float s_self = 0.f;
+#pragma unroll
+      for (int i = 0; i < D / 32; ++i) s_self += red[y][i];
+      s_self *= scale_log2;
+      const float2 ml = lane < n_chunks ? *reinterpret_cast<const float2 *>(part_ml + ((size_t)slab * kMaxSplits + lane) * 2)
+                                        : make_float2(-INFINITY, 0.f);
+      const float rs = lane < rg.R ? ring_s[y][lane] : -INFINITY;
+      float m = fmaxf(fmaxf(ml.x, rs), s_self);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+      const float w = exp2f(ml.x - m), wr = exp2f(rs - m);      // 2^-inf = 0
+      float l = fmaf(w, ml.y, wr);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+      wgt[y][lane] = w;
+      if (lane < rg.R) ring_s[y][lane] = wr;
+      if (lane == 0) {
+        const float w_self = exp2f(s_self - m);
+        lsum_s[y][0] = w_self;
+        lsum_s[y][1] = l + w_self;
+      }
+    }
+    __syncthreads();
+    float acc = lsum_s[y][0] * vn;
+    const float *po = part_o + (size_t)slab * kMaxSplits * D + d;
+    for (int c0 = 0; c0 < n_chunks; c0 += 8) {
+      float x[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) x[c] = c0 + c < n_chunks ? po[(size_t)(c0 + c) * D] : 0.f;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) acc = fmaf(wgt[y][c0 + c], x[c], acc);
+    }
+    // the evicted tokens of the recent-token window
+    for (int r = 0; r < rg.R; ++r) {
+      const float w = ring_s[y][r];
+      if (w > 0.f) acc = fmaf(w, Elem<T>::load(static_cast<const T *>(rg.v) + ((size_t)kv * rg.R + r) * D + d), acc);
+    }
+    if (on) Elem<T>::store(o + (size_t)slab * D + d, acc / lsum_s[y][1]);
+    __syncthreads();                                 // shared memory of this round has been read
+  }
+  // Every thread of the CTA has read the slab's length, and the chunk pass, the only reader of the slab's
+  // rows, has completed: the new row may go in and the length may move; the ring has been read too.
+  if (y == 0) {
+    append_new_row<T, D>(ap, kv, L, row_off[kv], k_new, v_new);
+    constexpr int kVecs = D * (int)sizeof(T) / 16;
+    if (rg.R > 0 && ap.flag_new != nullptr && d < kVecs)
       ring_put<kVecs>(rg, kv, d, reinterpret_cast<const uint8_t *>(k_new + (size_t)kv * D),
                       reinterpret_cast<const uint8_t *>(v_new + (size_t)kv * D), ap.flag_new[kv] != 0);
   }
@@ -496,27 +533,32 @@ decode_cluster_kernel(const T *__restrict__ q, const T *__restrict__ k_new, cons
   cluster.sync();
 }
 
-// The cluster form for bf16, head_dim 128, with the rows streamed through shared memory and the
-// scores and weighted sums on warp-level MMAs (decode_mma_core.cuh; the query is row 0 of the 16-row
-// operand): per row a fraction of the instructions of the CUDA-core form, which at these sizes is
-// bound by instruction issue and by what one SM can take in, not by latency alone.  CTA `rank`
-// takes whole 64-row tiles; everything after the streaming is as in decode_cluster_kernel.
+// The cluster form for bf16, with the rows streamed through shared memory and the scores and weighted sums
+// on warp-level MMAs (decode_mma_core.cuh): per row a fraction of the instructions of the CUDA-core form,
+// which at these sizes is bound by instruction issue and by what one SM can take in, not by latency alone.
+// One cluster per run of G <= 16 query slabs that share a key/value slab (G = 1 without grouped-query
+// attention): the G queries are rows of one MMA operand, so the slab is read once for all of them, and the
+// one cluster that reads it may append to it.  CTA `rank` takes whole 64-row tiles; after the cluster
+// barrier rank r merges the heads r, r + 8 of the group.
 // three stages: a CTA has few tiles and no neighbour to hide behind, so two of them are kept in flight
 constexpr int kCmStages = 3;
+// kMaxG: 1 (one query per slab), 8 or 16.
+template <int D, int kMaxG>
 __global__ void __launch_bounds__(kGqThreads, 2)
 decode_cluster_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k_new,
                           const __nv_bfloat16 *__restrict__ v_new, const __nv_bfloat16 *__restrict__ k_rows,
                           const __nv_bfloat16 *__restrict__ v_rows, const int64_t *__restrict__ row_off,
-                          const int32_t *len, float scale_log2, __nv_bfloat16 *__restrict__ out,
+                          const int32_t *len, float scale_log2, __nv_bfloat16 *__restrict__ out, int group,
                           const AppendArgs ap, const HeadMap hm, const RecentRing rg) {
   namespace cg = cooperative_groups;
   using T = __nv_bfloat16;
-  constexpr int D = kGqD;
-  static_assert(kGqThreads == D, "one thread per output dimension in the merge");
+  static_assert(kGqThreads >= D, "one thread per output dimension in the merge");
+  constexpr int kHeads = (kMaxG + kClusterSize - 1) / kClusterSize;    // heads a rank merges, at most
+  const int G = kMaxG == 1 ? 1 : group;
   extern __shared__ __align__(128) uint8_t gq_smem[];
   cg::cluster_group cluster = cg::this_cluster();
-  const int slab = blockIdx.y, rank = (int)cluster.block_rank();
-  const int kv = hm.kv_slab(slab);
+  const int slab0 = blockIdx.y * G, rank = (int)cluster.block_rank();
+  const int kv = hm.kv_slab(slab0);
   const int d = threadIdx.x;
   pdl_launch_dependents();
   // the slab's first row never changes once the cache is laid out: read ahead of the wait for the
@@ -527,56 +569,70 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat
   const int per = ((L + kClusterSize - 1) / kClusterSize + kGqTile - 1) / kGqTile * kGqTile;
   const int r_begin = min(L, rank * per), r_end = min(L, r_begin + per);
 
-  __shared__ float cta_o[D];          // this CTA's triple, read by the first CTA of the cluster
-  __shared__ float cta_ml[2];
-  __shared__ float red[D / 32];
-  __shared__ float ring_s[kMaxRecent];
+  // this CTA's triples [G][D] and [G][2], read by the merging ranks: behind the warps' triples in the ring's memory
+  float *cta_o = reinterpret_cast<float *>(gq_smem + gq_smem_bytes(D, kCmStages) - kGqMaxGroup * (D + 2) * 4);
+  float *cta_ml = cta_o + kGqMaxGroup * D;
+  __shared__ float red[kHeads][D / 32];
+  __shared__ float ring_s[kHeads][kMaxRecent];
 
-  // self score q . k_new and the new value: only the first CTA needs them; in flight with the stream
-  float prod = 0.f, v_self = 0.f;
-  if (rank == 0) {
-    prod = Elem<T>::load(q + (size_t)slab * D + d) * Elem<T>::load(k_new + (size_t)kv * D + d);
-    v_self = Elem<T>::load(v_new + (size_t)kv * D + d);
+  // self scores q . k_new of the heads this rank merges, and the new value: in flight with the stream
+  float prod[kHeads], v_self = 0.f;
+#pragma unroll
+  for (int u = 0; u < kHeads; ++u) {
+    const int h = rank + u * kClusterSize;
+    prod[u] = (h < G && d < D) ? Elem<T>::load(q + (size_t)(slab0 + h) * D + d) * Elem<T>::load(k_new + (size_t)kv * D + d) : 0.f;
   }
+  if (rank < G && d < D) v_self = Elem<T>::load(v_new + (size_t)kv * D + d);
 
   if (r_begin < r_end) {              // the same for the whole CTA
-    const size_t row0 = (size_t)slab_row0 * kGqRowBytes;
-    const GqWarpTriples w = gq_stream_rows<kCmStages>(gq_smem, q + (size_t)slab * D, 1,
+    const size_t row0 = (size_t)slab_row0 * (D * 2);
+    const GqWarpTriples w = gq_stream_rows<D, kCmStages, (kMaxG + 7) / 8>(gq_smem, q + (size_t)slab0 * D, G,
                                            reinterpret_cast<const uint8_t *>(k_rows) + row0,
                                            reinterpret_cast<const uint8_t *>(v_rows) + row0, r_begin, r_end, scale_log2);
-    float acc, mc, lc;
-    gq_combine(w, 0, d, acc, mc, lc);
-    cta_o[d] = acc;
-    if (d == 0) { cta_ml[0] = mc; cta_ml[1] = lc; }
+    for (int x = d; x < G * D; x += kGqThreads) {
+      const int h = x / D, e = x % D;
+      float acc, mc, lc;
+      gq_combine<D>(w, h, e, acc, mc, lc);
+      cta_o[x] = acc;
+      if (e == 0) { cta_ml[2 * h] = mc; cta_ml[2 * h + 1] = lc; }
+    }
   } else {
-    cta_o[d] = 0.f;
-    if (d == 0) { cta_ml[0] = -INFINITY; cta_ml[1] = 0.f; }
+    for (int x = d; x < G * D; x += kGqThreads) cta_o[x] = 0.f;
+    if (d < G) { cta_ml[2 * d] = -INFINITY; cta_ml[2 * d + 1] = 0.f; }
   }
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) prod += __shfl_xor_sync(0xffffffffu, prod, off);
-  if ((d & 31) == 0) red[d >> 5] = prod;
-  if (rank == 0) ring_scores<T, D>(rg, kv, q + (size_t)slab * D, scale_log2, ring_s);
+  for (int u = 0; u < kHeads; ++u) {
+    const int h = rank + u * kClusterSize;
+    if (h >= G) break;                // the same for the whole CTA
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) prod[u] += __shfl_xor_sync(0xffffffffu, prod[u], off);
+    if ((d & 31) == 0 && d < D) red[u][d >> 5] = prod[u];
+    ring_scores<T, D>(rg, kv, q + (size_t)(slab0 + h) * D, scale_log2, ring_s[u]);
+  }
   cluster.sync();
   // every CTA of the cluster has read the length and its rows: the new row may go in
-  // (never asked for when query heads share a slab: another head's cluster may still be reading its length)
+  // (never asked for when a query slab outside this cluster shares the slab)
   if (rank == 0) append_new_row<T, D>(ap, kv, L, slab_row0, k_new, v_new);
-  if (rank == 0) {
+#pragma unroll
+  for (int u = 0; u < kHeads; ++u) {
+    const int h = rank + u * kClusterSize;
+    if (h >= G || d >= D) break;
     float s_self = 0.f;
 #pragma unroll
-    for (int i = 0; i < D / 32; ++i) s_self += red[i];
+    for (int i = 0; i < D / 32; ++i) s_self += red[u][i];
     s_self *= scale_log2;
     float mr[kClusterSize], lr[kClusterSize], orr[kClusterSize];
 #pragma unroll
     for (int r = 0; r < kClusterSize; ++r) {
-      const float *ml = cluster.map_shared_rank(cta_ml, r);
+      const float *ml = cluster.map_shared_rank(cta_ml, r) + 2 * h;
       mr[r] = ml[0];
       lr[r] = ml[1];
-      orr[r] = cluster.map_shared_rank(cta_o, r)[d];
+      orr[r] = cluster.map_shared_rank(cta_o, r)[h * D + d];
     }
     float mm = s_self;
 #pragma unroll
     for (int r = 0; r < kClusterSize; ++r) mm = fmaxf(mm, mr[r]);
-    for (int r = 0; r < rg.R; ++r) mm = fmaxf(mm, ring_s[r]);
+    for (int r = 0; r < rg.R; ++r) mm = fmaxf(mm, ring_s[u][r]);
     const float w_self = exp2f(s_self - mm);
     float acc = w_self * v_self;
     float lsum = w_self;
@@ -588,34 +644,35 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat
     }
     // the evicted tokens of the recent-token window
     for (int r = 0; r < rg.R; ++r) {
-      if (ring_s[r] == -INFINITY) continue;
-      const float w = exp2f(ring_s[r] - mm);
+      if (ring_s[u][r] == -INFINITY) continue;
+      const float w = exp2f(ring_s[u][r] - mm);
       acc = fmaf(w, Elem<T>::load(static_cast<const T *>(rg.v) + ((size_t)kv * rg.R + r) * D + d), acc);
       lsum += w;
     }
-    Elem<T>::store(out + (size_t)slab * D + d, acc / lsum);
+    Elem<T>::store(out + (size_t)(slab0 + h) * D + d, acc / lsum);
   }
+  cluster.sync();
   if (rank == 0 && rg.R > 0 && ap.flag_new != nullptr) {
-    // the step carries the append: the new token joins the ring once every thread has read it
+    // the step carries the append: the new token joins the ring once every rank has read it
     constexpr int kVecs = D * (int)sizeof(T) / 16;
-    __syncthreads();
     if (d < kVecs)
       ring_put<kVecs>(rg, kv, d, reinterpret_cast<const uint8_t *>(k_new + (size_t)kv * D),
                       reinterpret_cast<const uint8_t *>(v_new + (size_t)kv * D), ap.flag_new[kv] != 0);
   }
-  cluster.sync();
 }
 
-static int launch_decode_cluster_mma(int slabs, const void *q, const void *k_new, const void *v_new,
+// groups: clusters (runs of G query slabs on one key/value slab each)
+template <int D, int kMaxG>
+static int launch_decode_cluster_mma(int groups, int G, const void *q, const void *k_new, const void *v_new,
                                      const ag_cache &c, float scale_log2, void *o, const AppendArgs &ap,
                                      const HeadMap &hm, const RecentRing &rg, cudaStream_t st) {
   using T = __nv_bfloat16;
-  AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   gq_smem_bytes(kCmStages)));
+  constexpr int smem = gq_smem_bytes(D, kCmStages);
+  AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kClusterSize, slabs);
+  cfg.gridDim = dim3(kClusterSize, groups);
   cfg.blockDim = dim3(kGqThreads);
-  cfg.dynamicSmemBytes = gq_smem_bytes(kCmStages);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -623,10 +680,10 @@ static int launch_decode_cluster_mma(int slabs, const void *q, const void *k_new
   attr[1] = pdl_attribute();
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_mma_kernel, static_cast<const T *>(q),
+  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_mma_kernel<D, kMaxG>, static_cast<const T *>(q),
                                  static_cast<const T *>(k_new), static_cast<const T *>(v_new),
                                  static_cast<const T *>(c.k_rows), static_cast<const T *>(c.v_rows),
-                                 c.row_off, c.len, scale_log2, static_cast<T *>(o), ap, hm, rg));
+                                 c.row_off, c.len, scale_log2, static_cast<T *>(o), G, ap, hm, rg));
   return AG_OK;
 }
 
@@ -656,53 +713,70 @@ size_t decode_workspace_bytes(const ag_layer_desc &d) {
   return align_up(slabs * kMaxSplits * (d.head_dim + 2) * sizeof(float), 256);
 }
 
+// A launch that may overlap its set-up with the tail of its predecessor (the kernel calls pdl_wait()).
+template <typename... Params, typename... Args>
+static int launch_pdl(void (*kern)(Params...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = pdl_attribute();
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...));
+  return AG_OK;
+}
+
+// Whether the kernels a decode step of this layer takes can carry the append: whichever CTA or cluster
+// appends to a slab has to be the only one that reads it.  Not so where query heads that share a slab go to
+// clusters of their own.
+static bool decode_carries_append(const ag_layer_desc &d) {
+  if (kv_heads_of(d) == d.heads || d.batch * d.heads > kClusterMaxSlabs) return true;
+  return d.dtype == AG_BF16 && d.heads / kv_heads_of(d) <= kGqMaxGroup;
+}
+
 template <typename T, int D>
 static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, const void *v_new,
                       const ag_cache &c, float scale, void *o, void *ws, const AppendArgs &ap, cudaStream_t st) {
   const int slabs = d.batch * d.heads;              // one per (sequence, query head)
   const HeadMap hm{d.heads, kv_heads_of(d)};
+  const int group = hm.heads / hm.kv_heads, kv_slabs = d.batch * hm.kv_heads;
   const RecentRing rg = ring_of(d, c);
   const float scale_log2 = scale * 1.4426950408889634f;
-  if constexpr (std::is_same_v<T, __nv_bfloat16> && D == kGqD) {
+  if constexpr (std::is_same_v<T, __nv_bfloat16>) {
+    // grouped-query attention: one cluster per key/value slab reads it for all its query heads
+    if (group <= kGqMaxGroup && kv_slabs <= kClusterMaxSlabs)
+      return (group == 1 ? launch_decode_cluster_mma<D, 1> : group <= 8 ? launch_decode_cluster_mma<D, 8> :
+              launch_decode_cluster_mma<D, 16>)(kv_slabs, group, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
     if (slabs <= kClusterMaxSlabs)
-      return launch_decode_cluster_mma(slabs, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
+      return launch_decode_cluster_mma<D, 1>(slabs, 1, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
+  } else {
+    if (slabs <= kClusterMaxSlabs)
+      return launch_decode_cluster<T, D, kClusterThreads>(slabs, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
   }
-  if (slabs <= kClusterMaxSlabs)
-    return launch_decode_cluster<T, D, kClusterThreads>(slabs, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
   int chunk_rows = (c.max_cap + kMaxSplits - 1) / kMaxSplits;
   chunk_rows = (chunk_rows + 127) / 128 * 128;   // whole iterations of the partial kernel (bf16, D = 128)
   const int n_chunks = c.max_cap > 0 ? (c.max_cap + chunk_rows - 1) / chunk_rows : 0;
   float *part_o = static_cast<float *>(ws);
   float *part_ml = part_o + (size_t)slabs * kMaxSplits * D;
-  const int group = hm.heads / hm.kv_heads;
+  auto qp = static_cast<const T *>(q), kn = static_cast<const T *>(k_new), vn = static_cast<const T *>(v_new);
+  auto kr = static_cast<const T *>(c.k_rows), vr = static_cast<const T *>(c.v_rows);
+  int rc = AG_OK;
   if (n_chunks > 0 && decode_gqa_mma_supported(d)) {
     // grouped-query attention, bf16: the group's heads are the rows of a tensor-core tile
-    int rc = launch_decode_partial_gqa_mma(d, q, c, scale_log2, chunk_rows, n_chunks, part_o, part_ml, kMaxSplits, st);
-    if (rc) return rc;
+    rc = launch_decode_partial_gqa_mma(d, q, c, scale_log2, chunk_rows, n_chunks, part_o, part_ml, kMaxSplits, st);
   } else if (n_chunks > 0 && (group == 2 || group == 4)) {
     // grouped-query attention: the rows of a key/value slab are read once for its query heads
-    dim3 grid(n_chunks, d.batch * hm.kv_heads);
-    auto qp = static_cast<const T *>(q);
-    auto kr = static_cast<const T *>(c.k_rows), vr = static_cast<const T *>(c.v_rows);
-    if (group == 2)
-      decode_partial_gqa_kernel<T, D, 2><<<grid, kPartThreads, 0, st>>>(qp, kr, vr, c.row_off, c.len, scale_log2,
-                                                                         chunk_rows, part_o, part_ml, hm.kv_heads);
-    else
-      decode_partial_gqa_kernel<T, D, 4><<<grid, kPartThreads, 0, st>>>(qp, kr, vr, c.row_off, c.len, scale_log2,
-                                                                         chunk_rows, part_o, part_ml, hm.kv_heads);
-    AG_LAUNCH_CHECK();
+    rc = launch_pdl(group == 2 ? decode_partial_gqa_kernel<T, D, 2> : decode_partial_gqa_kernel<T, D, 4>,
+                    dim3(n_chunks, kv_slabs), dim3(kPartThreads), st, qp, kr, vr, c.row_off, c.len, scale_log2,
+                    chunk_rows, part_o, part_ml, hm.kv_heads);
   } else if (n_chunks > 0) {
-    dim3 grid(n_chunks, slabs);
-    decode_partial_kernel<T, D><<<grid, kPartThreads, 0, st>>>(
-        static_cast<const T *>(q), static_cast<const T *>(c.k_rows),
-        static_cast<const T *>(c.v_rows), c.row_off, c.len, scale_log2, chunk_rows, part_o, part_ml, hm);
-    AG_LAUNCH_CHECK();
+    rc = launch_pdl(decode_partial_kernel<T, D>, dim3(n_chunks, slabs), dim3(kPartThreads), st, qp, kr, vr, c.row_off,
+                    c.len, scale_log2, chunk_rows, part_o, part_ml, hm);
   }
-  decode_combine_kernel<T, D><<<slabs, D, 0, st>>>(
-      static_cast<const T *>(q), static_cast<const T *>(k_new), static_cast<const T *>(v_new),
-      c.len, scale_log2, chunk_rows, part_o, part_ml, static_cast<T *>(o), c.row_off, ap, hm, rg);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  if (rc) return rc;
+  return launch_pdl(decode_combine_kernel<T, D>, dim3(kv_slabs), dim3(D, group < 512 / D ? group : 512 / D), st, qp, kn,
+                    vn, c.len, scale_log2, chunk_rows, part_o, part_ml, static_cast<T *>(o), c.row_off, group, ap, rg);
 }
 
 static int dispatch_decode(const ag_layer_desc &d, const void *q, const void *k_new, const void *v_new,
@@ -725,7 +799,7 @@ int launch_decode(const ag_layer_desc &d, const void *q, const void *k_new, cons
 int launch_decode_step(const ag_layer_desc &d, const void *q, const void *k_new, const void *v_new,
                        const uint8_t *flag_new, const ag_cache &c, float scale, void *o,
                        int32_t *dev_status, void *ws, cudaStream_t st) {
-  if (kv_heads_of(d) != d.heads) {
+  if (!decode_carries_append(d)) {
     // query heads share a slab: the append waits for all of them, in a launch of its own
     int rc = dispatch_decode(d, q, k_new, v_new, c, scale, o, ws, AppendArgs{}, st);
     if (rc) return rc;

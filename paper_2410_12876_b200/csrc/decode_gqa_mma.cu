@@ -13,6 +13,7 @@ namespace ag {
 
 // two stages x three CTAs per SM measured better here than deeper rings in fewer CTAs
 constexpr int kGqChunkStages = 2;
+template <int kGqD, int kHalves>
 __global__ void __launch_bounds__(kGqThreads, 3)
 decode_partial_gqa_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k_rows,
                               const __nv_bfloat16 *__restrict__ v_rows, const int64_t *__restrict__ row_off,
@@ -20,19 +21,22 @@ decode_partial_gqa_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bf
                               float *__restrict__ part_o, float *__restrict__ part_ml, int kv_heads, int G,
                               int max_splits) {
   extern __shared__ __align__(128) uint8_t gq_smem[];
+  constexpr int kGqRowBytes = kGqD * 2;
   const int kv = blockIdx.y, chunk = blockIdx.x;
   const int slab0 = (kv / kv_heads) * kv_heads * G + (kv % kv_heads) * G;     // first query slab of the group
+  pdl_launch_dependents();
+  pdl_wait();
   const int L = len[kv];
   const int r_begin = chunk * chunk_rows;
   if (r_begin >= L) return;                                                    // the whole CTA, before any barrier
   const int r_end = min(L, r_begin + chunk_rows);
   const uint8_t *Kg = reinterpret_cast<const uint8_t *>(k_rows) + (size_t)row_off[kv] * kGqRowBytes;
   const uint8_t *Vg = reinterpret_cast<const uint8_t *>(v_rows) + (size_t)row_off[kv] * kGqRowBytes;
-  const GqWarpTriples w = gq_stream_rows<kGqChunkStages>(gq_smem, q + (size_t)slab0 * kGqD, G, Kg, Vg, r_begin, r_end, scale_log2);
+  const GqWarpTriples w = gq_stream_rows<kGqD, kGqChunkStages, kHalves>(gq_smem, q + (size_t)slab0 * kGqD, G, Kg, Vg, r_begin, r_end, scale_log2);
   for (int x = threadIdx.x; x < G * kGqD; x += kGqThreads) {     // one (head, output dimension) at a time
     const int h = x / kGqD, d = x % kGqD;
     float acc, mc, lc;
-    gq_combine(w, h, d, acc, mc, lc);
+    gq_combine<kGqD>(w, h, d, acc, mc, lc);
     const size_t slot = (size_t)(slab0 + h) * max_splits + chunk;
     part_o[slot * kGqD + d] = acc;
     if (d == 0) {
@@ -44,22 +48,39 @@ decode_partial_gqa_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bf
 
 bool decode_gqa_mma_supported(const ag_layer_desc &d) {
   const int group = d.heads / kv_heads_of(d);
-  return d.dtype == AG_BF16 && d.head_dim == kGqD && group >= 2 && group <= kGqMaxGroup;
+  return d.dtype == AG_BF16 && group >= 2 && group <= kGqMaxGroup;
+}
+
+template <int D, int kHalves>
+static int run_partial(const ag_layer_desc &d, const void *q, const ag_cache &c, float scale_log2, int chunk_rows,
+                       int n_chunks, float *part_o, float *part_ml, int max_splits, cudaStream_t st) {
+  const int kvh = kv_heads_of(d);
+  constexpr int smem = gq_smem_bytes(D, kGqChunkStages);
+  AG_CUDA_TRY(cudaFuncSetAttribute(decode_partial_gqa_mma_kernel<D, kHalves>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  dim3 grid(n_chunks, d.batch * kvh);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kGqThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = pdl_attribute();
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_partial_gqa_mma_kernel<D, kHalves>, static_cast<const __nv_bfloat16 *>(q),
+                                 static_cast<const __nv_bfloat16 *>(c.k_rows),
+                                 static_cast<const __nv_bfloat16 *>(c.v_rows), static_cast<const int64_t *>(c.row_off),
+                                 static_cast<const int32_t *>(c.len), scale_log2, chunk_rows, part_o, part_ml, kvh,
+                                 d.heads / kvh, max_splits));
+  return AG_OK;
 }
 
 int launch_decode_partial_gqa_mma(const ag_layer_desc &d, const void *q, const ag_cache &c, float scale_log2,
                                   int chunk_rows, int n_chunks, float *part_o, float *part_ml, int max_splits,
                                   cudaStream_t st) {
-  const int kvh = kv_heads_of(d);
-  AG_CUDA_TRY(cudaFuncSetAttribute(decode_partial_gqa_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   gq_smem_bytes(kGqChunkStages)));
-  dim3 grid(n_chunks, d.batch * kvh);
-  decode_partial_gqa_mma_kernel<<<grid, kGqThreads, gq_smem_bytes(kGqChunkStages), st>>>(
-      static_cast<const __nv_bfloat16 *>(q), static_cast<const __nv_bfloat16 *>(c.k_rows),
-      static_cast<const __nv_bfloat16 *>(c.v_rows), c.row_off, c.len, scale_log2, chunk_rows, part_o, part_ml,
-      kvh, d.heads / kvh, max_splits);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  const bool small = d.heads / kv_heads_of(d) <= 8;
+  auto run = d.head_dim == 64 ? (small ? run_partial<64, 1> : run_partial<64, 2>)
+                              : (small ? run_partial<128, 1> : run_partial<128, 2>);
+  return run(d, q, c, scale_log2, chunk_rows, n_chunks, part_o, part_ml, max_splits, st);
 }
 
 }  // namespace ag

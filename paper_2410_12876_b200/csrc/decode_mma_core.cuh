@@ -14,14 +14,17 @@
 
 namespace ag {
 
-constexpr int kGqD = 128;                 // head_dim (bf16)
 constexpr int kGqWarps = 4, kGqThreads = kGqWarps * 32;
 constexpr int kGqTile = kGqWarps * 16;    // rows per tile: 16 per warp
-constexpr int kGqRowBytes = kGqD * 2;
-constexpr int kGqTileBytes = kGqTile * kGqRowBytes;           // 16 KB
-// dynamic shared memory of a kernel that streams with a ring of `stages` (K tile, V tile) pairs
-constexpr int gq_smem_bytes(int stages) { return stages * 2 * kGqTileBytes; }
+// dynamic shared memory of a kernel that streams rows of D bf16 with a ring of `stages` (K tile, V tile) pairs
+__host__ __device__ constexpr int gq_tile_bytes(int D) { return kGqTile * D * 2; }           // 16 KB at D = 128
+__host__ __device__ constexpr int gq_smem_bytes(int D, int stages) { return stages * 2 * gq_tile_bytes(D); }
 constexpr int kGqMaxGroup = 16;
+// Byte offset of 16-byte piece `piece` of row `row` in a shared-memory tile of D bf16 per row.
+template <int D>
+__device__ __forceinline__ uint32_t gq_tile_off(int row, int piece) {
+  return D == 128 ? tile256_off(row, piece) : (uint32_t)(row * 128 + ((piece ^ (row & 7)) << 4));
+}
 
 // Per-warp triples in shared memory, laid over the tile ring once the rows have been consumed.
 struct GqWarpTriples {
@@ -30,12 +33,15 @@ struct GqWarpTriples {
 
 // Every thread of the CTA (kGqThreads of them) calls this with the same arguments; r_begin < r_end.
 // q: G consecutive query vectors [G][D]; Kg, Vg: first row of the slab.  Returns after a CTA barrier
-// with the warps' triples in shared memory (gq_smem: gq_smem_bytes(kGqStages) of dynamic shared memory;
+// with the warps' triples in shared memory (gq_smem: gq_smem_bytes(D, kGqStages) of dynamic shared memory;
 // kGqStages - 1 tiles are in flight while one is worked on).
-template <int kGqStages>
+// kHalves: 1 for G <= 8 (rows 8..15 of the operand are zero and their softmax is left out), 2 for G <= 16.
+template <int kGqD, int kGqStages, int kHalves>
 __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const __nv_bfloat16 *__restrict__ q, int G,
                                                         const uint8_t *__restrict__ Kg, const uint8_t *__restrict__ Vg,
                                                         int r_begin, int r_end, float scale_log2) {
+  static_assert(kGqD == 64 || kGqD == 128, "head_dim");
+  constexpr int kGqRowBytes = kGqD * 2, kGqTileBytes = gq_tile_bytes(kGqD), kPieces = kGqD / 8;
   const int n_tiles = (r_end - r_begin + kGqTile - 1) / kGqTile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;                                       // fragment row, column pair
@@ -46,11 +52,11 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
     const uint32_t sk = smem0 + (i % kGqStages) * 2 * kGqTileBytes, sv = sk + kGqTileBytes;
     const int r0 = r_begin + i * kGqTile;
 #pragma unroll
-    for (int x = 0; x < kGqTile * 16 / kGqThreads; ++x) {
-      const int idx = threadIdx.x + x * kGqThreads, r = idx >> 4, c = idx & 15;
+    for (int x = 0; x < kGqTile * kPieces / kGqThreads; ++x) {
+      const int idx = threadIdx.x + x * kGqThreads, r = idx / kPieces, c = idx % kPieces;
       const size_t src = (size_t)min(r0 + r, r_end - 1) * kGqRowBytes + c * 16;
-      cp_async16(sk + tile256_off(r, c), Kg + src);
-      cp_async16(sv + tile256_off(r, c), Vg + src);
+      cp_async16(sk + gq_tile_off<kGqD>(r, c), Kg + src);
+      cp_async16(sv + gq_tile_off<kGqD>(r, c), Vg + src);
     }
   };
 #pragma unroll
@@ -66,12 +72,11 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
     const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + (size_t)min(g, G - 1) * kGqD);
     const uint32_t lo = qrow[ks * 8 + t], hi = qrow[ks * 8 + 4 + t];
     qa[ks][0] = g < G ? lo : 0u;
-    qa[ks][1] = 0u;                                     // rows 8..15: G <= 8 is all this kernel is asked for
+    qa[ks][1] = 0u;
     qa[ks][2] = g < G ? hi : 0u;
     qa[ks][3] = 0u;
   }
-  const bool two_halves = G > 8;
-  if (two_halves) {
+  if (kHalves == 2) {
 #pragma unroll
     for (int ks = 0; ks < kGqD / 16; ++ks) {
       const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + (size_t)min(g + 8, G - 1) * kGqD);
@@ -85,7 +90,9 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
   for (int nt = 0; nt < kGqD / 8; ++nt)
 #pragma unroll
     for (int e = 0; e < 4; ++e) o[nt][e] = 0.f;
-  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};       // rows g and g + 8
+  float m[kHalves], l[kHalves];                                 // rows g (and g + 8)
+#pragma unroll
+  for (int h = 0; h < kHalves; ++h) { m[h] = -INFINITY; l[h] = 0.f; }
 
   for (int i = 0; i < n_tiles; ++i) {
     if (i + kGqStages - 1 < n_tiles) load_tile(i + kGqStages - 1);
@@ -103,14 +110,14 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
         uint32_t b[4];
         // matrices: (keys 0-7, dims lo), (keys 0-7, dims hi), (keys 8-15, dims lo), (keys 8-15, dims hi)
         const int mi = lane >> 3, row = warp * 16 + (mi >> 1) * 8 + (lane & 7);
-        ldmatrix_x4(b, sk + tile256_off(row, ks * 2 + (mi & 1)));
+        ldmatrix_x4(b, sk + gq_tile_off<kGqD>(row, ks * 2 + (mi & 1)));
         mma_16816(s0, qa[ks], b[0], b[1]);
         mma_16816(s1, qa[ks], b[2], b[3]);
       }
       // online softmax of rows g (and g + 8): this thread holds keys 2t, 2t+1 of each column tile
-      uint32_t pa[4];
+      uint32_t pa[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < kHalves; ++h) {
         float sv4[4] = {s0[2 * h], s0[2 * h + 1], s1[2 * h], s1[2 * h + 1]};
         const int kcol[4] = {2 * t, 2 * t + 1, 8 + 2 * t, 9 + 2 * t};
         float tmax = -INFINITY;
@@ -143,7 +150,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
         uint32_t b[4];
         // matrices: (keys 0-7, dims lo), (keys 8-15, dims lo), (keys 0-7, dims hi), (keys 8-15, dims hi)
         const int mi = lane >> 3, row = warp * 16 + (mi & 1) * 8 + (lane & 7);
-        ldmatrix_x4_trans(b, sv + tile256_off(row, nt2 * 2 + (mi >> 1)));
+        ldmatrix_x4_trans(b, sv + gq_tile_off<kGqD>(row, nt2 * 2 + (mi >> 1)));
         mma_16816(o[2 * nt2], pa, b[0], b[1]);
         mma_16816(o[2 * nt2 + 1], pa, b[2], b[3]);
       }
@@ -154,7 +161,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
 
   // merge the four warps' triples through shared memory (the tiles are no longer needed)
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < kHalves; ++h) {
     l[h] += __shfl_xor_sync(0xffffffffu, l[h], 1);
     l[h] += __shfl_xor_sync(0xffffffffu, l[h], 2);
   }
@@ -162,7 +169,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
   float *sm_m = sm_o + kGqWarps * kGqMaxGroup * kGqD;           // [warps][16]
   float *sm_l = sm_m + kGqWarps * kGqMaxGroup;
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < kHalves; ++h) {
     const int row = g + 8 * h;
     if (row < G) {
 #pragma unroll
@@ -182,6 +189,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
 }
 
 // The CTA's triple for query h, output dimension d, from the warps' triples.
+template <int kGqD>
 __device__ __forceinline__ void gq_combine(const GqWarpTriples &w, int h, int d, float &acc, float &mc, float &lc) {
   mc = -INFINITY;
 #pragma unroll
