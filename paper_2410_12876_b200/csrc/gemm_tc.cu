@@ -13,6 +13,7 @@
 // Products of bf16 inputs are exact in the f32 accumulator, so the result
 // differs from an exact evaluation only by f32 summation error.
 #include "ag_common.cuh"
+#include "gemm_splitk.cuh"
 #include "umma.cuh"
 
 namespace ag {
@@ -490,11 +491,78 @@ static int run_gemm_pair(const void *X, const void *W0, const void *W1, const vo
   return AG_OK;
 }
 
+// The gate's projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
+template <int BN>
+struct GateProjSplit {
+  CUtensorMap tmA, tmB[3];
+  float *C;
+  __nv_bfloat16 *hi, *lo;
+  int M, GD, n_tiles_n;
+  struct Shared {};
+  struct Row {};
+  __device__ void prefetch() const { prefetch_tensormap(&tmA); prefetch_tensormap(&tmB[0]); }
+  __device__ void load_a(uint8_t *dst, uint64_t *bar, int tile, int kb) const {
+    tma_load_2d(dst, &tmA, bar, kb * kTcBK, tile / n_tiles_n * kTcBM);        // rows past M are filled with zeros
+  }
+  __device__ void load_b(uint8_t *dst, uint64_t *bar, int tile, int panel, int kb) const {
+    const int col = tile % n_tiles_n * BN + panel * 64;                       // a panel lies in one weight
+    tma_load_2d(dst, &tmB[col / GD], bar, col % GD, kb * kTcBK);
+  }
+  __device__ void prepare(Shared &, int, int, int) const {}
+  __device__ Row load_row(int, int, int) const { return {}; }
+  __device__ void row(Shared &, int tile, int r, int col, const float (&acc)[BN / 32], const Row &) const {
+    const int m = tile / n_tiles_n * kTcBM + r;
+    if (m >= M) return;
+#pragma unroll
+    for (int c = 0; c < BN / 128; ++c) {
+      const size_t at = (size_t)m * 3 * GD + tile % n_tiles_n * BN + c * 128 + col;
+      const float *x = acc + c * 4;
+      if (hi != nullptr) {
+        float h[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) split_bf16(x[e], h[e], l[e]);
+        *reinterpret_cast<uint2 *>(hi + at) = make_uint2(pack_bf16x2(h[0], h[1]), pack_bf16x2(h[2], h[3]));
+        *reinterpret_cast<uint2 *>(lo + at) = make_uint2(pack_bf16x2(l[0], l[1]), pack_bf16x2(l[2], l[3]));
+      } else {
+        *reinterpret_cast<float4 *>(C + at) = make_float4(x[0], x[1], x[2], x[3]);
+      }
+    }
+  }
+};
+
+// Runs the projection split over clusters if that is the faster way (*done), else does nothing.
+template <int BN>
+static int try_gemm_split(const void *X, const void *W0, const void *W1, const void *W2, float *C, __nv_bfloat16 *Chi,
+                          __nv_bfloat16 *Clo, int M, int K, int GD, cudaStream_t st, bool *done) {
+  const int *cap;
+  int rc = splitk::splitk_capacity<BN, GateProjSplit<BN>>(&cap);
+  if (rc) return rc;
+  const int n_tiles_n = 3 * GD / BN, num_kb = (K + kTcBK - 1) / kTcBK;
+  const long long tiles = (long long)n_tiles_n * ((M + kTcBM - 1) / kTcBM);
+  const int splits = splitk::choose_split(tiles, num_kb, cap);
+  *done = splits > 1;
+  if (splits == 1) return AG_OK;
+  GateProjSplit<BN> p;
+  if ((rc = make_tmap_2d_bf16(&p.tmA, X, M, K, (uint64_t)K * 2, kTcBM, kTcBK))) return rc;
+  const void *Ws[3] = {W0, W1, W2};
+  for (int i = 0; i < 3; ++i)
+    if ((rc = make_tmap_2d_bf16(&p.tmB[i], Ws[i], K, GD, (uint64_t)GD * 2, kTcBK, 64))) return rc;
+  p.C = C; p.hi = Chi; p.lo = Clo; p.M = M; p.GD = GD; p.n_tiles_n = n_tiles_n;
+  return splitk::launch_splitk<BN>(p, tiles, num_kb, splits, st);
+}
+
 bool gate_proj_tc_supported(int K, int GD) { return GD % 128 == 0 && K % 8 == 0; }
 
 int launch_gate_proj_tc(const void *X, const void *W0, const void *W1, const void *W2, float *C, void *Chi,
                         void *Clo, int M, int K, int GD, cudaStream_t st) {
   auto hi = static_cast<__nv_bfloat16 *>(Chi), lo = static_cast<__nv_bfloat16 *>(Clo);
+  // less than two waves of 128-column tiles: the reduction split over clusters where that fills the chip
+  if ((long long)((M + kTcBM - 1) / kTcBM) * (3 * GD / 128) <= 2 * gemm_sm_count()) {
+    bool done = false;
+    const int rc = GD % 256 == 0 ? try_gemm_split<256>(X, W0, W1, W2, C, hi, lo, M, K, GD, st, &done)
+                                 : try_gemm_split<128>(X, W0, W1, W2, C, hi, lo, M, K, GD, st, &done);
+    if (rc || done) return rc;
+  }
   // at least half a wave of pair tiles (256 x 384): CTA pairs
   if ((long long)(3 * GD / kGpBN) * ((M + 2 * kTcBM - 1) / (2 * kTcBM)) * 4 >= gemm_sm_count())
     return run_gemm_pair(X, W0, W1, W2, C, hi, lo, M, K, GD, st);

@@ -17,6 +17,7 @@
 // TMA store, the dense copy leaves by TMA stores, and the retained rows are copied from the
 // same staging area, one 256-byte row per half-warp.
 #include "ag_common.cuh"
+#include "gemm_splitk.cuh"
 #include "umma.cuh"
 
 namespace ag {
@@ -55,6 +56,63 @@ struct KvEpilogue {
   int n_sub, tps, n, kv_heads, heads;
 };
 
+// The rank of token t = t0 + r_in among the retained tokens of key/value slab `slab`, by 128 threads (r_in = 0 ..
+// 127, warps quad = 0 .. 3): the slab's flag row is a few KB and is counted whole, as 16-byte vectors, for the
+// number retained before the tile and in the slab; the tile's own tokens are ranked by warp ballot + popc.
+// Returns the token's row in the ragged cache (-1: evicted, or the slab is too small).  write: also prefix (and
+// idx), and, from the tile that holds a sequence's first token, the slab's length.
+__device__ __forceinline__ long long kv_rank_token(const KvEpilogue &e, size_t slab, int t0, int quad, int lane,
+                                                   int *red, bool write) {
+  const int n = e.n, r_in = quad * 32 + lane, t = t0 + r_in;
+  const uint8_t *f = e.flags + slab * n;
+  int before = 0, total = 0;
+  if ((n & 15) == 0) {                                      // flag rows start on 16-byte boundaries
+    const uint4 *fv = reinterpret_cast<const uint4 *>(f);
+    for (int x = r_in; x < n / 16; x += kBM) {
+      const uint4 w = ldg128(fv + x);
+      const int c = nonzero_bytes(w.x) + nonzero_bytes(w.y) + nonzero_bytes(w.z) + nonzero_bytes(w.w);
+      total += c;
+      if (x * 16 < t0) before += c;                         // t0 is a multiple of 16: a vector lies on one side
+    }
+  } else {
+    for (int x = r_in; x < n; x += kBM) {
+      const int c = f[x] != 0;
+      total += c;
+      if (x < t0) before += c;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    before += __shfl_xor_sync(0xffffffffu, before, o);
+    total += __shfl_xor_sync(0xffffffffu, total, o);
+  }
+  const bool in_seq = t < n;                                // a sequence may end inside its last sub-tile
+  const bool keep = in_seq && f[t] != 0;
+  const unsigned word = __ballot_sync(0xffffffffu, keep);
+  const int in_warp = __popc(word & ((1u << lane) - 1u));
+  if (lane == 0) { red[quad] = before; red[4 + quad] = total; red[8 + quad] = __popc(word); }
+  named_barrier_sync(2, 128);
+  before = red[0] + red[1] + red[2] + red[3];
+  total = red[4] + red[5] + red[6] + red[7];
+  int excl = 0;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) excl += q < quad ? red[8 + q] : 0;
+  named_barrier_sync(2, 128);                             // red is free for the next head
+  const int p = before + excl + in_warp;                  // rank within the slab
+  const bool fits = total <= e.cap[slab];
+  if (write && in_seq) {
+    int32_t *pre = e.prefix + slab * (n + 1);
+    pre[t] = p;
+    if (keep && e.idx) e.idx[slab * n + p] = t;
+    if (t == 0) {
+      pre[n] = total;
+      e.len[slab] = fits ? total : 0;
+      if (!fits && e.dev_status) atomicOr(e.dev_status, AG_DEV_OVERFLOW);
+    }
+  }
+  return fits && keep ? (long long)e.row_off[slab] + p : -1;
+}
+
 // Warps 2..9 of a CTA: rank the tile's tokens while the MMAs run, then drain the CTA's mts sub-tiles
 // (first sub-tile sub0, columns [nw, nw + BN) of weight `which`) from tensor memory at tmem_acc.
 template <int BN, int MT>
@@ -62,77 +120,22 @@ __device__ __forceinline__ void kv_epilogue(const KvEpilogue &e, uint8_t *smem, 
                                             uint64_t *acc_full, uint32_t tmem_acc, int sub0, int mts, int which, int nw,
                                             int num_kb, int warp, int lane) {
   constexpr int kHeads = BN / kD;
-  const uint8_t *flags = e.flags;
-  int32_t *prefix = e.prefix, *idx = e.idx, *len = e.len, *dev_status = e.dev_status;
-  const int64_t *row_off = e.row_off;
-  const int32_t *cap = e.cap;
-  const int n_sub = e.n_sub, tps = e.tps, n = e.n, kv_heads = e.kv_heads;
+  const int n_sub = e.n_sub, tps = e.tps, kv_heads = e.kv_heads;
   const int out_heads = which == 2 ? e.heads : e.kv_heads;
   // epilogue warps: warp w may touch TMEM lanes [32 * (w % 4), +32); warps 2..5 drain the first
   // half of a sub-tile's columns, warps 6..9 the second
   const int quad = warp & 3, half = (warp - 2) >> 2;
   const int r_in = quad * 32 + lane;           // token of the sub-tile this thread drains
-  // While the MMAs run: the rank of every token of the tile among the retained tokens of its slab
-  // (the slab's flag row is a few KB: counted whole, as 16-byte vectors, for the number retained
-  // before the tile and in the slab; the tile's own tokens ranked by warp ballot + popc), hence its
-  // row in the ragged cache (-1: evicted, or the slab is too small).  The key tiles also write
-  // prefix (and idx), and the one that holds a sequence's first token the slab's length.
+  // While the MMAs run: the cache row of every token of the tile.
 #pragma unroll
   for (int mt = 0; mt < (half == 0 ? MT : 0); ++mt) {           // warps 2..5 only
     const int sub = sub0 + mt;
-    const int b = sub / tps, t0 = (sub % tps) * kBM, t = t0 + r_in;
+    const int b = sub / tps, t0 = (sub % tps) * kBM;
 #pragma unroll
     for (int hh = 0; hh < kHeads; ++hh) {
       long long d = -1;
       if (sub < n_sub && mt < mts && which != 2) {                // the same for all 128 threads
-        const size_t slab = (size_t)b * kv_heads + nw / kD + hh;
-        const uint8_t *f = flags + slab * n;
-        int before = 0, total = 0;
-        if ((n & 15) == 0) {                                      // flag rows start on 16-byte boundaries
-          const uint4 *fv = reinterpret_cast<const uint4 *>(f);
-          for (int x = r_in; x < n / 16; x += kBM) {
-            const uint4 w = ldg128(fv + x);
-            const int c = nonzero_bytes(w.x) + nonzero_bytes(w.y) + nonzero_bytes(w.z) + nonzero_bytes(w.w);
-            total += c;
-            if (x * 16 < t0) before += c;                         // t0 is a multiple of 16: a vector lies on one side
-          }
-        } else {
-          for (int x = r_in; x < n; x += kBM) {
-            const int c = f[x] != 0;
-            total += c;
-            if (x < t0) before += c;
-          }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          before += __shfl_xor_sync(0xffffffffu, before, o);
-          total += __shfl_xor_sync(0xffffffffu, total, o);
-        }
-        const bool in_seq = t < n;                                // a single sequence may end inside its last sub-tile
-        const bool keep = in_seq && f[t] != 0;
-        const unsigned word = __ballot_sync(0xffffffffu, keep);
-        const int in_warp = __popc(word & ((1u << lane) - 1u));
-        if (lane == 0) { red[quad] = before; red[4 + quad] = total; red[8 + quad] = __popc(word); }
-        named_barrier_sync(2, 128);
-        before = red[0] + red[1] + red[2] + red[3];
-        total = red[4] + red[5] + red[6] + red[7];
-        int excl = 0;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) excl += q < quad ? red[8 + q] : 0;
-        named_barrier_sync(2, 128);                             // red is free for the next head
-        const int p = before + excl + in_warp;                  // rank within the slab
-        const bool fits = total <= cap[slab];
-        if (fits && keep) d = row_off[slab] + p;
-        if (which == 0 && in_seq) {
-          int32_t *pre = prefix + slab * (n + 1);
-          pre[t] = p;
-          if (keep && idx) idx[slab * n + p] = t;
-          if (t == 0) {
-            pre[n] = total;
-            len[slab] = fits ? total : 0;
-            if (!fits && dev_status) atomicOr(dev_status, AG_DEV_OVERFLOW);
-          }
-        }
+        d = kv_rank_token(e, (size_t)b * kv_heads + nw / kD + hh, t0, quad, lane, red, which == 0);
       }
       dst_row[(mt * kHeads + hh) * kBM + r_in] = d;
     }
@@ -453,6 +456,87 @@ int sm_count() {
   return sms;
 }
 
+// The same projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
+template <int BN>
+struct KvProjSplit {
+  CUtensorMap tmA, tmB[3];                        // weights of keys, values, queries
+  KvEpilogue e;
+  __nv_bfloat16 *out[3];                          // dense K, V, Q
+  int GD, n_tiles_n;
+  struct Shared {
+    long long dst[BN / kD][kBM];
+    int red[12];
+  };
+  struct Row {};
+  __device__ void prefetch() const { prefetch_tensormap(&tmA); prefetch_tensormap(&tmB[0]); }
+  __device__ int column(int tile) const { return tile % n_tiles_n * BN; }       // in the packed output [K | V | Q]
+  __device__ int which(int tile) const { return min(column(tile) / GD, 2); }    // a tile lies in one weight
+  __device__ int head(int tile) const { return (column(tile) - which(tile) * GD) / kD; }
+  __device__ void load_a(uint8_t *dst, uint64_t *bar, int tile, int kb) const {
+    const int sub = tile / n_tiles_n;                        // 128 tokens of one sequence; zeros past its end
+    tma_load_3d(dst, &tmA, bar, kb * kBK, sub % e.tps * kBM, sub / e.tps);
+  }
+  __device__ void load_b(uint8_t *dst, uint64_t *bar, int tile, int panel, int kb) const {
+    tma_load_2d(dst, &tmB[which(tile)], bar, head(tile) * kD + panel * 64, kb * kBK);
+  }
+  __device__ void prepare(Shared &sh, int tile, int rank, int) const {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, sub = tile / n_tiles_n;
+    if (warp >= 6) return;
+    for (int hh = 0; hh < BN / kD; ++hh)
+      sh.dst[hh][quad * 32 + lane] =
+          which(tile) == 2 ? -1
+                           : kv_rank_token(e, (size_t)(sub / e.tps) * e.kv_heads + head(tile) + hh, sub % e.tps * kBM, quad,
+                                           lane, sh.red, which(tile) == 0 && rank == 0);
+  }
+  __device__ Row load_row(int, int, int) const { return {}; }
+  __device__ void row(Shared &sh, int tile, int r, int col, const float (&acc)[BN / 32], const Row &) const {
+    const int sub = tile / n_tiles_n, t = sub % e.tps * kBM + r, w = which(tile);
+    if (t >= e.n) return;
+    const int heads = w == 2 ? e.heads : e.kv_heads;
+#pragma unroll
+    for (int hh = 0; hh < BN / kD; ++hh) {
+      const uint2 v = make_uint2(pack_bf16x2(acc[4 * hh], acc[4 * hh + 1]), pack_bf16x2(acc[4 * hh + 2], acc[4 * hh + 3]));
+      const size_t slab = (size_t)(sub / e.tps) * heads + head(tile) + hh;
+      *reinterpret_cast<uint2 *>(out[w] + (slab * e.n + t) * kD + col) = v;
+      const long long d = sh.dst[hh][r];
+      if (d >= 0) *reinterpret_cast<uint2 *>((w == 0 ? e.k_rows : e.v_rows) + (size_t)d * (kD * 2) + col * 2) = v;
+    }
+  }
+};
+
+// Runs the projection split over clusters if that is the faster way (*done), else does nothing.
+template <int BN>
+int try_split(const ag_layer_desc &d, const void *X, const void *Wq, const void *Wk, const void *Wv, const uint8_t *flags,
+              const ag_cache &c, int32_t *prefix, int32_t *idx, void *Q, void *K, void *V, int32_t *dev_status,
+              cudaStream_t st, bool *done) {
+  const int *cap;
+  int rc = splitk::splitk_capacity<BN, KvProjSplit<BN>>(&cap);
+  if (rc) return rc;
+  const int hk = kv_heads_of(d), GD = hk * kD, QD = Wq ? d.heads * kD : 0, num_kb = (d.hidden + kBK - 1) / kBK;
+  KvProjSplit<BN> p;
+  p.n_tiles_n = (2 * GD + QD) / BN;
+  p.GD = GD;
+  p.e = KvEpilogue{};
+  p.e.tps = (d.seq + kBM - 1) / kBM;
+  p.e.n_sub = d.batch * p.e.tps;
+  const long long tiles = (long long)p.n_tiles_n * p.e.n_sub;
+  const int splits = splitk::choose_split(tiles, num_kb, cap);
+  *done = splits > 1;
+  if (splits == 1) return AG_OK;
+  if ((rc = make_tmap_3d_bf16(&p.tmA, X, d.batch, d.seq, d.hidden, kBM, kBK))) return rc;
+  if ((rc = make_tmap_2d_bf16(&p.tmB[0], Wk, d.hidden, GD, (uint64_t)GD * 2, kBK, 64))) return rc;
+  if ((rc = make_tmap_2d_bf16(&p.tmB[1], Wv, d.hidden, GD, (uint64_t)GD * 2, kBK, 64))) return rc;
+  p.tmB[2] = p.tmB[0];                            // stand-in when there is no query projection
+  if (Wq && (rc = make_tmap_2d_bf16(&p.tmB[2], Wq, d.hidden, QD, (uint64_t)QD * 2, kBK, 64))) return rc;
+  p.e.flags = flags; p.e.prefix = prefix; p.e.idx = idx;
+  p.e.row_off = c.row_off; p.e.cap = c.cap; p.e.len = c.len;
+  p.e.k_rows = static_cast<uint8_t *>(c.k_rows); p.e.v_rows = static_cast<uint8_t *>(c.v_rows);
+  p.e.dev_status = dev_status; p.e.n = d.seq; p.e.kv_heads = hk; p.e.heads = d.heads;
+  p.out[0] = static_cast<__nv_bfloat16 *>(K); p.out[1] = static_cast<__nv_bfloat16 *>(V);
+  p.out[2] = static_cast<__nv_bfloat16 *>(Q);
+  return splitk::launch_splitk<BN>(p, tiles, num_kb, splits, st);
+}
+
 template <int BN, int MT>
 int run(const ag_layer_desc &d, const void *X, const void *Wq, const void *Wk, const void *Wv, const uint8_t *flags,
         const ag_cache &c, int32_t *prefix, int32_t *idx, void *Q, void *K, void *V, int32_t *dev_status,
@@ -516,8 +600,16 @@ int launch_kv_proj_cache(const ag_layer_desc &d, const void *X, const void *Wq, 
                          void *V, int32_t *dev_status, cudaStream_t st) {
   const int hk = kv_heads_of(d), hq = Wq ? d.heads : 0;
   const long long tiles128 = (long long)(2 * hk + hq) * d.batch * ((d.seq + kBM - 1) / kBM);
-  int rc;
-  if (hk % 2 == 0 && hq % 2 == 0) {
+  const bool wide = hk % 2 == 0 && hq % 2 == 0;
+  int rc = AG_OK;
+  bool done = false;
+  // less than a wave of tiles: the reduction split over clusters where that fills the chip
+  if (tiles128 <= (wide ? 2 : 1) * sm_count()) {
+    rc = (wide ? try_split<256> : try_split<128>)(d, X, Wq, Wk, Wv, flags, c, prefix, idx, Q, K, V, dev_status, st, &done);
+    if (rc) return rc;
+  }
+  if (done) {
+  } else if (wide) {
     // more than one wave: CTA pairs on 512 x 256 tiles
     if (tiles128 > 2 * sm_count()) rc = run<256, 1>(d, X, Wq, Wk, Wv, flags, c, prefix, idx, Q, K, V, dev_status, st, true);
     else rc = run<256, 1>(d, X, Wq, Wk, Wv, flags, c, prefix, idx, Q, K, V, dev_status, st);

@@ -19,6 +19,7 @@
 // SMs more than once.  out_proj_simt_kernel is the CUDA-core form for float32 layers, head_dim 64
 // and shapes the tiles do not cover.
 #include "ag_common.cuh"
+#include "gemm_splitk.cuh"
 #include "umma.cuh"
 
 namespace ag {
@@ -484,6 +485,80 @@ int run_pair(const ag_layer_desc &dsc, const void *O, const void *Wo, const void
   return AG_OK;
 }
 
+// The same projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
+template <int BN>
+struct OutProjSplit {
+  CUtensorMap tmO, tmW;
+  const __nv_bfloat16 *X_res;
+  __nv_bfloat16 *Y;
+  int tps, n, heads, d, n_tiles_n;
+  struct Shared {};
+  struct Row { uint2 x[BN / 128]; };                         // skip connection
+  __device__ void prefetch() const { prefetch_tensormap(&tmO); prefetch_tensormap(&tmW); }
+  __device__ void load_a(uint8_t *dst, uint64_t *bar, int tile, int kb) const {
+    const int sub = tile / n_tiles_n;                        // 128 tokens of one sequence; zeros past its end
+    tma_load_3d(dst, &tmO, bar, kb % (kD / kBK) * kBK, sub % tps * kBM, sub / tps * heads + kb / (kD / kBK));
+  }
+  __device__ void load_b(uint8_t *dst, uint64_t *bar, int tile, int panel, int kb) const {
+    tma_load_2d(dst, &tmW, bar, tile % n_tiles_n * BN + panel * 64, kb * kBK);
+  }
+  // Offset of column `col` of row r in X_res and Y, or -1 past the sequence's end.
+  __device__ long long offset(int tile, int r, int col) const {
+    const int sub = tile / n_tiles_n, t = sub % tps * kBM + r;
+    return t < n ? ((long long)(sub / tps) * n + t) * d + tile % n_tiles_n * BN + col : -1;
+  }
+  // the CTA's rows of the skip connection on their way into L2 while the MMAs run
+  __device__ void prepare(Shared &, int tile, int rank, int splits) const {
+    if (X_res == nullptr) return;
+    const int first = rank * kBM / splits, count = (rank + 1) * kBM / splits - first;
+    for (int i = (int)threadIdx.x - 64; i < count * (BN / 64); i += 256) {
+      const long long at = offset(tile, first + i / (BN / 64), i % (BN / 64) * 64);
+      if (at >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(X_res + at));
+    }
+  }
+  __device__ Row load_row(int tile, int r, int col) const {
+    Row v;
+    const long long at = offset(tile, r, col);
+#pragma unroll
+    for (int c = 0; c < BN / 128; ++c)
+      v.x[c] = X_res != nullptr && at >= 0 ? *reinterpret_cast<const uint2 *>(X_res + at + c * 128) : make_uint2(0u, 0u);
+    return v;
+  }
+  __device__ void row(Shared &, int tile, int r, int col, const float (&acc)[BN / 32], const Row &res) const {
+    const long long at = offset(tile, r, col);
+    if (at < 0) return;
+#pragma unroll
+    for (int c = 0; c < BN / 128; ++c) {
+      const float *a = acc + c * 4;
+      const uint2 x = res.x[c];
+      *reinterpret_cast<uint2 *>(Y + at + c * 128) =
+          make_uint2(pack_bf16x2(a[0] + __uint_as_float(x.x << 16), a[1] + __uint_as_float(x.x & 0xffff0000u)),
+                     pack_bf16x2(a[2] + __uint_as_float(x.y << 16), a[3] + __uint_as_float(x.y & 0xffff0000u)));
+    }
+  }
+};
+
+// Runs the projection split over clusters if that is the faster way (*done), else does nothing.
+template <int BN>
+int try_split(const ag_layer_desc &dsc, const void *O, const void *Wo, const void *X_res, void *Y, cudaStream_t st,
+              bool *done) {
+  const int *cap;
+  int rc = splitk::splitk_capacity<BN, OutProjSplit<BN>>(&cap);
+  if (rc) return rc;
+  const int d = dsc.hidden, num_kb = dsc.heads * (kD / kBK), tps = (dsc.seq + kBM - 1) / kBM;
+  const long long tiles = (long long)(d / BN) * dsc.batch * tps;
+  const int splits = splitk::choose_split(tiles, num_kb, cap);
+  *done = splits > 1;
+  if (splits == 1) return AG_OK;
+  OutProjSplit<BN> p;
+  if ((rc = make_tmap_3d_bf16(&p.tmO, O, (uint64_t)dsc.batch * dsc.heads, dsc.seq, kD, kBM, kBK))) return rc;
+  if ((rc = make_tmap_2d_bf16(&p.tmW, Wo, dsc.heads * kD, d, (uint64_t)d * 2, kBK, 64))) return rc;
+  p.X_res = static_cast<const __nv_bfloat16 *>(X_res);
+  p.Y = static_cast<__nv_bfloat16 *>(Y);
+  p.tps = tps; p.n = dsc.seq; p.heads = dsc.heads; p.d = d; p.n_tiles_n = d / BN;
+  return splitk::launch_splitk<BN>(p, tiles, num_kb, splits, st);
+}
+
 template <typename T>
 int run_simt(const ag_layer_desc &dsc, const void *O, const void *Wo, const void *X_res, void *Y, cudaStream_t st) {
   dim3 grid((dsc.hidden + 255) / 256, dsc.batch * dsc.seq);
@@ -509,7 +584,16 @@ int launch_out_proj(const ag_layer_desc &d, const void *O, const void *Wo, const
       // stage, which keeps the tensor pipe fed from shared memory (a single CTA on a 256 x 256 tile reads 12 KB of
       // operands per MMA while TMA writes the next stage, more than shared memory's 128 B a clock)
       if (tiles128 > 2 * sm_count()) return run_pair(d, O, Wo, X_res, Y, st);
+      // less than a wave: the reduction split over clusters where that fills the chip
+      bool done = false;
+      const int rc = try_split<256>(d, O, Wo, X_res, Y, st, &done);
+      if (rc || done) return rc;
       return run_tc<256, 1>(d, O, Wo, X_res, Y, st);
+    }
+    if (tiles128 <= sm_count()) {
+      bool done = false;
+      const int rc = try_split<128>(d, O, Wo, X_res, Y, st, &done);
+      if (rc || done) return rc;
     }
     return run_tc<128, 1>(d, O, Wo, X_res, Y, st);
   }
