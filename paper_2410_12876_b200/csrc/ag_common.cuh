@@ -33,6 +33,22 @@ inline cudaLaunchAttribute pdl_attribute() {
   at.val.programmaticStreamSerializationAllowed = 1;
   return at;
 }
+#ifdef __CUDACC__
+// A launch that may overlap its set-up with the tail of its predecessor (the kernel calls pdl_wait()).
+template <typename... Params, typename... Args>
+inline int launch_pdl(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args &...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = pdl_attribute();
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...));
+  return AG_OK;
+}
+#endif
 // Recent-token window: the ring of a slab holds the last recent_window - 1 tokens (0 = no ring).
 constexpr int kMaxRecent = 16;
 inline int recent_rows(const ag_layer_desc &d) { return d.recent_window > 1 ? d.recent_window - 1 : 0; }
@@ -196,10 +212,13 @@ __device__ __forceinline__ void ring_put(const RecentRing &rg, int slab, int vec
 __device__ __forceinline__ uint4 ldg128(const void *p) {
   return __ldg(reinterpret_cast<const uint4 *>(p));
 }
+// For kernels that start with pdl_wait(): a plain load stays behind the wait, where one through the non-coherent
+// path (__ldg, or a const __restrict__ argument) may be moved ahead of it.
+__device__ __forceinline__ uint4 ld128(const void *p) { return *reinterpret_cast<const uint4 *>(p); }
 // Streaming 16-byte load that does not allocate in L1 (data used once).
 __device__ __forceinline__ uint4 ldg128_stream(const void *p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }

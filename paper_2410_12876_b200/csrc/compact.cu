@@ -21,11 +21,11 @@ __device__ __forceinline__ int nonzero_bytes(uint32_t w) { return __popc(__vcmpn
 // one row of K and one row of V.  kRowBytes = 0: count pass, no rows move.
 template <int kRowBytes>
 __global__ void __launch_bounds__(kCompactThreads)
-compact_kernel(const uint8_t *__restrict__ flags, int n, const int32_t *__restrict__ cap,
-               int32_t *__restrict__ len, int32_t *__restrict__ prefix, int32_t *__restrict__ idx,
-               int32_t *__restrict__ dev_status, const uint8_t *__restrict__ K,
-               const uint8_t *__restrict__ V, const int64_t *__restrict__ row_off,
-               uint8_t *__restrict__ k_rows, uint8_t *__restrict__ v_rows) {
+compact_kernel(const uint8_t *flags, int n, const int32_t *cap,
+               int32_t *len, int32_t *prefix, int32_t *idx,
+               int32_t *dev_status, const uint8_t *K,
+               const uint8_t *V, const int64_t *row_off,
+               uint8_t *k_rows, uint8_t *v_rows) {
   const int slab = blockIdx.y, t0 = blockIdx.x * kCompactThreads;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint8_t *f = flags + (size_t)slab * n;
@@ -33,12 +33,14 @@ compact_kernel(const uint8_t *__restrict__ flags, int n, const int32_t *__restri
   __shared__ int warp_excl[kCompactThreads / 32];
   __shared__ int tok_list[kCompactThreads];
 
+  pdl_wait();
+  pdl_launch_dependents();
   // retained tokens before this chunk, and in the slab
   int before = 0, total = 0;
   if ((n & 15) == 0) {                       // rows of the flag array start on 16-byte boundaries
     const uint4 *fv = reinterpret_cast<const uint4 *>(f);
     for (int x = threadIdx.x; x < n / 16; x += kCompactThreads) {
-      const uint4 w = ldg128(fv + x);
+      const uint4 w = ld128(fv + x);
       const int c = nonzero_bytes(w.x) + nonzero_bytes(w.y) + nonzero_bytes(w.z) + nonzero_bytes(w.w);
       total += c;
       if (x * 16 < t0) before += c;          // t0 is a multiple of 16: a vector lies on one side
@@ -119,11 +121,11 @@ compact_kernel(const uint8_t *__restrict__ flags, int n, const int32_t *__restri
 
 template <int kRowBytes>
 __global__ void __launch_bounds__(256)
-append_rows_kernel(const uint8_t *__restrict__ k_new, const uint8_t *__restrict__ v_new,
-                   const uint8_t *__restrict__ flag_new, int n_slabs,
-                   const int64_t *__restrict__ row_off, const int32_t *__restrict__ cap,
-                   int32_t *__restrict__ len, uint8_t *__restrict__ k_rows,
-                   uint8_t *__restrict__ v_rows, int32_t *__restrict__ dev_status, const RecentRing ring) {
+append_rows_kernel(const uint8_t *k_new, const uint8_t *v_new,
+                   const uint8_t *flag_new, int n_slabs,
+                   const int64_t *row_off, const int32_t *cap,
+                   int32_t *len, uint8_t *k_rows,
+                   uint8_t *v_rows, int32_t *dev_status, const RecentRing ring) {
   constexpr int kVecs = kRowBytes / 16;
   constexpr int kGroups = 256 / kVecs;
   const int slab = blockIdx.x * kGroups + threadIdx.x / kVecs;
@@ -153,8 +155,8 @@ append_rows_kernel(const uint8_t *__restrict__ k_new, const uint8_t *__restrict_
 // With per-sequence lengths the prompt of a slab is the first seq_lens[b] of its n positions.
 // One CTA per slab, thread (slot, 16-byte piece).
 template <int kRowBytes>
-__global__ void recent_fill_kernel(const uint8_t *__restrict__ K, const uint8_t *__restrict__ V,
-                                   const uint8_t *__restrict__ flags, int n, const int32_t *__restrict__ seq_lens,
+__global__ void recent_fill_kernel(const uint8_t *K, const uint8_t *V,
+                                   const uint8_t *flags, int n, const int32_t *seq_lens,
                                    int kv_heads, const RecentRing ring) {
   constexpr int kVecs = kRowBytes / 16;
   const int slab = blockIdx.x, slot = threadIdx.x / kVecs, v = threadIdx.x % kVecs;
@@ -192,23 +194,17 @@ int launch_compact(const ag_layer_desc &d, const void *K, const void *V, const u
   auto Vb = static_cast<const uint8_t *>(V);
   auto kr = static_cast<uint8_t *>(c.k_rows);
   auto vr = static_cast<uint8_t *>(c.v_rows);
+  decltype(&compact_kernel<0>) kern;
   switch (K ? row_bytes(d) : 0) {
-    case 0:
-      compact_kernel<0><<<grid, kCompactThreads, 0, st>>>(flags, d.seq, c.cap, c.len, prefix, ix, dev_status, Kb, Vb, c.row_off, kr, vr);
-      break;
-    case 128:
-      compact_kernel<128><<<grid, kCompactThreads, 0, st>>>(flags, d.seq, c.cap, c.len, prefix, ix, dev_status, Kb, Vb, c.row_off, kr, vr);
-      break;
-    case 256:
-      compact_kernel<256><<<grid, kCompactThreads, 0, st>>>(flags, d.seq, c.cap, c.len, prefix, ix, dev_status, Kb, Vb, c.row_off, kr, vr);
-      break;
-    case 512:
-      compact_kernel<512><<<grid, kCompactThreads, 0, st>>>(flags, d.seq, c.cap, c.len, prefix, ix, dev_status, Kb, Vb, c.row_off, kr, vr);
-      break;
-    default:
-      return AG_ERR_UNSUPPORTED;
+    case 0: kern = compact_kernel<0>; break;
+    case 128: kern = compact_kernel<128>; break;
+    case 256: kern = compact_kernel<256>; break;
+    case 512: kern = compact_kernel<512>; break;
+    default: return AG_ERR_UNSUPPORTED;
   }
-  AG_LAUNCH_CHECK();
+  const int rc = launch_pdl(kern, grid, dim3(kCompactThreads), 0, st, flags, d.seq, c.cap, c.len, prefix, ix, dev_status, Kb,
+                            Vb, c.row_off, kr, vr);
+  if (rc) return rc;
   const RecentRing ring = ring_of(d, c);
   if (K && ring.R > 0) return launch_recent_fill(d, K, V, flags, c, st);
   return AG_OK;

@@ -53,7 +53,7 @@ struct AppendArgs {
 // completed.  L = the length those reads saw.
 template <typename T, int D>
 __device__ __forceinline__ void append_new_row(const AppendArgs &ap, int slab, int L, int64_t row0,
-                                               const T *__restrict__ k_new, const T *__restrict__ v_new,
+                                               const T *k_new, const T *v_new,
                                                int first = 0) {
   constexpr int kVecs = D * (int)sizeof(T) / 16;
   const int vec = (int)threadIdx.x - first;
@@ -75,7 +75,7 @@ __device__ __forceinline__ void append_new_row(const AppendArgs &ap, int slab, i
 // of those that call: sm_s[r] = scale_log2 * q . k_r for a live slot (an evicted token the query still
 // sees), -inf otherwise.  The caller synchronises the CTA before reading sm_s.
 template <typename T, int D>
-__device__ __forceinline__ void ring_scores_part(const RecentRing &rg, int kv, const T *__restrict__ q_row,
+__device__ __forceinline__ void ring_scores_part(const RecentRing &rg, int kv, const T *q_row,
                                                  float scale_log2, float *sm_s, int warp, int n_warps) {
   const int lane = threadIdx.x & 31;
   for (int r = warp; r < rg.R; r += n_warps) {
@@ -90,7 +90,7 @@ __device__ __forceinline__ void ring_scores_part(const RecentRing &rg, int kv, c
 }
 
 template <typename T, int D>
-__device__ __forceinline__ void ring_scores(const RecentRing &rg, int kv, const T *__restrict__ q_row,
+__device__ __forceinline__ void ring_scores(const RecentRing &rg, int kv, const T *q_row,
                                             float scale_log2, float *sm_s) {
   ring_scores_part<T, D>(rg, kv, q_row, scale_log2, sm_s, threadIdx.x >> 5, blockDim.x >> 5);
 }
@@ -99,8 +99,8 @@ __device__ __forceinline__ void ring_scores(const RecentRing &rg, int kv, const 
 // (row group, 16-byte slice of the row) ends with its group's running maximum m, sum l and slice
 // of o (log2 domain).
 template <typename T, int D, int kThreads>
-__device__ __forceinline__ void decode_stream_rows(const T *__restrict__ q, const T *__restrict__ k_rows,
-                                                   const T *__restrict__ v_rows, int64_t row0, int slab,
+__device__ __forceinline__ void decode_stream_rows(const T *q, const T *k_rows,
+                                                   const T *v_rows, int64_t row0, int slab,
                                                    int r_begin, int r_end, float scale_log2, float &m,
                                                    float &l, float (&o)[Elem<T>::kPerVec]) {
   constexpr int kEpl = Elem<T>::kPerVec;        // elements per lane
@@ -109,7 +109,7 @@ __device__ __forceinline__ void decode_stream_rows(const T *__restrict__ q, cons
   const int g = threadIdx.x / kLanes, v = threadIdx.x % kLanes;
 
   float qf[kEpl];
-  Elem<T>::unpack(ldg128(q + (size_t)slab * D + v * kEpl), qf);
+  Elem<T>::unpack(ld128(q + (size_t)slab * D + v * kEpl), qf);
 #pragma unroll
   for (int e = 0; e < kEpl; ++e) qf[e] *= scale_log2;
 
@@ -166,10 +166,10 @@ __device__ __forceinline__ void decode_stream_rows(const T *__restrict__ q, cons
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kPartThreads)
-decode_partial_kernel(const T *__restrict__ q, const T *__restrict__ k_rows,
-                      const T *__restrict__ v_rows, const int64_t *__restrict__ row_off,
-                      const int32_t *__restrict__ len, float scale_log2, int chunk_rows,
-                      float *__restrict__ part_o, float *__restrict__ part_ml, const HeadMap hm) {
+decode_partial_kernel(const T *q, const T *k_rows,
+                      const T *v_rows, const int64_t *row_off,
+                      const int32_t *len, float scale_log2, int chunk_rows,
+                      float *part_o, float *part_ml, const HeadMap hm) {
   constexpr int kEpl = Elem<T>::kPerVec;
   constexpr int kLanes = D / kEpl;
   constexpr int kGroups = kPartThreads / kLanes;
@@ -217,10 +217,10 @@ decode_partial_kernel(const T *__restrict__ q, const T *__restrict__ k_rows,
 constexpr int kUnrollGqa = 4;
 template <typename T, int D, int G>
 __global__ void __launch_bounds__(kPartThreads)
-decode_partial_gqa_kernel(const T *__restrict__ q, const T *__restrict__ k_rows,
-                          const T *__restrict__ v_rows, const int64_t *__restrict__ row_off,
-                          const int32_t *__restrict__ len, float scale_log2, int chunk_rows,
-                          float *__restrict__ part_o, float *__restrict__ part_ml, int kv_heads) {
+decode_partial_gqa_kernel(const T *q, const T *k_rows,
+                          const T *v_rows, const int64_t *row_off,
+                          const int32_t *len, float scale_log2, int chunk_rows,
+                          float *part_o, float *part_ml, int kv_heads) {
   constexpr int kEpl = Elem<T>::kPerVec;
   constexpr int kLanes = D / kEpl;
   constexpr int kGroups = kPartThreads / kLanes;
@@ -237,7 +237,7 @@ decode_partial_gqa_kernel(const T *__restrict__ q, const T *__restrict__ k_rows,
   float qf[G][kEpl], o[G][kEpl], m[G], l[G];
 #pragma unroll
   for (int h = 0; h < G; ++h) {
-    Elem<T>::unpack(ldg128(q + (size_t)(slab0 + h) * D + v * kEpl), qf[h]);
+    Elem<T>::unpack(ld128(q + (size_t)(slab0 + h) * D + v * kEpl), qf[h]);
     m[h] = -INFINITY; l[h] = 0.f;
 #pragma unroll
     for (int e = 0; e < kEpl; ++e) { qf[h][e] *= scale_log2; o[h][e] = 0.f; }
@@ -329,11 +329,11 @@ decode_partial_gqa_kernel(const T *__restrict__ q, const T *__restrict__ k_rows,
 // other, each load waiting for its turn, took 11.5 us for 1024 query slabs of 17 chunks.
 template <typename T, int D>
 __global__ void __launch_bounds__(512)
-decode_combine_kernel(const T *__restrict__ q, const T *__restrict__ k_new,
-                      const T *__restrict__ v_new, const int32_t *len,
-                      float scale_log2, int chunk_rows, const float *__restrict__ part_o,
-                      const float *__restrict__ part_ml, T *__restrict__ o,
-                      const int64_t *__restrict__ row_off, int G, const AppendArgs ap, const RecentRing rg) {
+decode_combine_kernel(const T *q, const T *k_new,
+                      const T *v_new, const int32_t *len,
+                      float scale_log2, int chunk_rows, const float *part_o,
+                      const float *part_ml, T *o,
+                      const int64_t *row_off, int G, const AppendArgs ap, const RecentRing rg) {
   static_assert(kMaxSplits == 32, "a lane per chunk");
   const int kv = blockIdx.x, d = threadIdx.x, y = threadIdx.y, lane = d & 31;
   constexpr int kMaxHeads = 512 / D;
@@ -417,10 +417,10 @@ decode_combine_kernel(const T *__restrict__ q, const T *__restrict__ k_new,
 constexpr int kClusterSize = 8;
 template <typename T, int D, int kThreads>
 __global__ void __launch_bounds__(kThreads)
-decode_cluster_kernel(const T *__restrict__ q, const T *__restrict__ k_new, const T *__restrict__ v_new,
-                      const T *__restrict__ k_rows, const T *__restrict__ v_rows,
-                      const int64_t *__restrict__ row_off, const int32_t *len,
-                      float scale_log2, T *__restrict__ out, const AppendArgs ap, const HeadMap hm,
+decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
+                      const T *k_rows, const T *v_rows,
+                      const int64_t *row_off, const int32_t *len,
+                      float scale_log2, T *out, const AppendArgs ap, const HeadMap hm,
                       const RecentRing rg) {
   namespace cg = cooperative_groups;
   constexpr int kEpl = Elem<T>::kPerVec;
@@ -445,10 +445,11 @@ decode_cluster_kernel(const T *__restrict__ q, const T *__restrict__ k_new, cons
 
   // self score q . k_new: only the first CTA needs it; its loads are in flight with the stream's
   // (and the new value, which the merge after the cluster barrier would otherwise wait for)
-  float prod = 0.f, v_self = 0.f;
+  T q_raw = T(0.f), k_raw = T(0.f), v_raw = T(0.f);    // (not used before the stream is done)
   if (rank == 0 && threadIdx.x < D) {
-    prod = Elem<T>::load(q + (size_t)slab * D + threadIdx.x) * Elem<T>::load(k_new + (size_t)kv * D + threadIdx.x);
-    v_self = Elem<T>::load(v_new + (size_t)kv * D + threadIdx.x);
+    q_raw = q[(size_t)slab * D + threadIdx.x];
+    k_raw = k_new[(size_t)kv * D + threadIdx.x];
+    v_raw = v_new[(size_t)kv * D + threadIdx.x];
   }
 
   float m, l, o[kEpl];
@@ -457,7 +458,9 @@ decode_cluster_kernel(const T *__restrict__ q, const T *__restrict__ k_new, cons
   if (v == 0) { sm_m[g] = m; sm_l[g] = l; }
 #pragma unroll
   for (int e = 0; e < kEpl; ++e) sm_o[g][v * kEpl + e] = o[e];
+  const float v_self = Elem<T>::load(&v_raw);
   if (threadIdx.x < D) {              // whole warps: D is a multiple of 32
+    float prod = Elem<T>::load(&q_raw) * Elem<T>::load(&k_raw);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) prod += __shfl_xor_sync(0xffffffffu, prod, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = prod;
@@ -545,10 +548,10 @@ constexpr int kCmStages = 3;
 // kMaxG: 1 (one query per slab), 8 or 16.
 template <int D, int kMaxG>
 __global__ void __launch_bounds__(kGqThreads, 2)
-decode_cluster_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k_new,
-                          const __nv_bfloat16 *__restrict__ v_new, const __nv_bfloat16 *__restrict__ k_rows,
-                          const __nv_bfloat16 *__restrict__ v_rows, const int64_t *__restrict__ row_off,
-                          const int32_t *len, float scale_log2, __nv_bfloat16 *__restrict__ out, int group,
+decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
+                          const __nv_bfloat16 *v_new, const __nv_bfloat16 *k_rows,
+                          const __nv_bfloat16 *v_rows, const int64_t *row_off,
+                          const int32_t *len, float scale_log2, __nv_bfloat16 *out, int group,
                           const AppendArgs ap, const HeadMap hm, const RecentRing rg) {
   namespace cg = cooperative_groups;
   using T = __nv_bfloat16;
@@ -576,13 +579,16 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat
   __shared__ float ring_s[kHeads][kMaxRecent];
 
   // self scores q . k_new of the heads this rank merges, and the new value: in flight with the stream
-  float prod[kHeads], v_self = 0.f;
+  T q_raw[kHeads], k_raw = T(0.f), v_raw = T(0.f);           // (not used before the stream is done)
 #pragma unroll
   for (int u = 0; u < kHeads; ++u) {
     const int h = rank + u * kClusterSize;
-    prod[u] = (h < G && d < D) ? Elem<T>::load(q + (size_t)(slab0 + h) * D + d) * Elem<T>::load(k_new + (size_t)kv * D + d) : 0.f;
+    q_raw[u] = (h < G && d < D) ? q[(size_t)(slab0 + h) * D + d] : T(0.f);
   }
-  if (rank < G && d < D) v_self = Elem<T>::load(v_new + (size_t)kv * D + d);
+  if (rank < G && d < D) {
+    k_raw = k_new[(size_t)kv * D + d];
+    v_raw = v_new[(size_t)kv * D + d];
+  }
 
   if (r_begin < r_end) {              // the same for the whole CTA
     const size_t row0 = (size_t)slab_row0 * (D * 2);
@@ -604,11 +610,13 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat
   for (int u = 0; u < kHeads; ++u) {
     const int h = rank + u * kClusterSize;
     if (h >= G) break;                // the same for the whole CTA
+    float prod = Elem<T>::load(&q_raw[u]) * Elem<T>::load(&k_raw);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) prod[u] += __shfl_xor_sync(0xffffffffu, prod[u], off);
-    if ((d & 31) == 0 && d < D) red[u][d >> 5] = prod[u];
+    for (int off = 16; off > 0; off >>= 1) prod += __shfl_xor_sync(0xffffffffu, prod, off);
+    if ((d & 31) == 0 && d < D) red[u][d >> 5] = prod;
     ring_scores<T, D>(rg, kv, q + (size_t)(slab0 + h) * D, scale_log2, ring_s[u]);
   }
+  const float v_self = Elem<T>::load(&v_raw);
   cluster.sync();
   // every CTA of the cluster has read the length and its rows: the new row may go in
   // (never asked for when a query slab outside this cluster shares the slab)
@@ -713,20 +721,6 @@ size_t decode_workspace_bytes(const ag_layer_desc &d) {
   return align_up(slabs * kMaxSplits * (d.head_dim + 2) * sizeof(float), 256);
 }
 
-// A launch that may overlap its set-up with the tail of its predecessor (the kernel calls pdl_wait()).
-template <typename... Params, typename... Args>
-static int launch_pdl(void (*kern)(Params...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = st;
-  cudaLaunchAttribute attr = pdl_attribute();
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...));
-  return AG_OK;
-}
-
 // Whether the kernels a decode step of this layer takes can carry the append: whichever CTA or cluster
 // appends to a slab has to be the only one that reads it.  Not so where query heads that share a slab go to
 // clusters of their own.
@@ -768,14 +762,14 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
   } else if (n_chunks > 0 && (group == 2 || group == 4)) {
     // grouped-query attention: the rows of a key/value slab are read once for its query heads
     rc = launch_pdl(group == 2 ? decode_partial_gqa_kernel<T, D, 2> : decode_partial_gqa_kernel<T, D, 4>,
-                    dim3(n_chunks, kv_slabs), dim3(kPartThreads), st, qp, kr, vr, c.row_off, c.len, scale_log2,
+                    dim3(n_chunks, kv_slabs), dim3(kPartThreads), 0, st, qp, kr, vr, c.row_off, c.len, scale_log2,
                     chunk_rows, part_o, part_ml, hm.kv_heads);
   } else if (n_chunks > 0) {
-    rc = launch_pdl(decode_partial_kernel<T, D>, dim3(n_chunks, slabs), dim3(kPartThreads), st, qp, kr, vr, c.row_off,
+    rc = launch_pdl(decode_partial_kernel<T, D>, dim3(n_chunks, slabs), dim3(kPartThreads), 0, st, qp, kr, vr, c.row_off,
                     c.len, scale_log2, chunk_rows, part_o, part_ml, hm);
   }
   if (rc) return rc;
-  return launch_pdl(decode_combine_kernel<T, D>, dim3(kv_slabs), dim3(D, group < 512 / D ? group : 512 / D), st, qp, kn,
+  return launch_pdl(decode_combine_kernel<T, D>, dim3(kv_slabs), dim3(D, group < 512 / D ? group : 512 / D), 0, st, qp, kn,
                     vn, c.len, scale_log2, chunk_rows, part_o, part_ml, static_cast<T *>(o), c.row_off, group, ap, rg);
 }
 

@@ -15,10 +15,10 @@ namespace ag {
 constexpr int kGqChunkStages = 2;
 template <int kGqD, int kHalves>
 __global__ void __launch_bounds__(kGqThreads, 3)
-decode_partial_gqa_mma_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k_rows,
-                              const __nv_bfloat16 *__restrict__ v_rows, const int64_t *__restrict__ row_off,
-                              const int32_t *__restrict__ len, float scale_log2, int chunk_rows,
-                              float *__restrict__ part_o, float *__restrict__ part_ml, int kv_heads, int G,
+decode_partial_gqa_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_rows,
+                              const __nv_bfloat16 *v_rows, const int64_t *row_off,
+                              const int32_t *len, float scale_log2, int chunk_rows,
+                              float *part_o, float *part_ml, int kv_heads, int G,
                               int max_splits) {
   extern __shared__ __align__(128) uint8_t gq_smem[];
   constexpr int kGqRowBytes = kGqD * 2;
@@ -58,20 +58,10 @@ static int run_partial(const ag_layer_desc &d, const void *q, const ag_cache &c,
   constexpr int smem = gq_smem_bytes(D, kGqChunkStages);
   AG_CUDA_TRY(cudaFuncSetAttribute(decode_partial_gqa_mma_kernel<D, kHalves>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   dim3 grid(n_chunks, d.batch * kvh);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(kGqThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr = pdl_attribute();
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_partial_gqa_mma_kernel<D, kHalves>, static_cast<const __nv_bfloat16 *>(q),
-                                 static_cast<const __nv_bfloat16 *>(c.k_rows),
-                                 static_cast<const __nv_bfloat16 *>(c.v_rows), static_cast<const int64_t *>(c.row_off),
-                                 static_cast<const int32_t *>(c.len), scale_log2, chunk_rows, part_o, part_ml, kvh,
-                                 d.heads / kvh, max_splits));
-  return AG_OK;
+  return launch_pdl(decode_partial_gqa_mma_kernel<D, kHalves>, grid, dim3(kGqThreads), smem, st,
+                    static_cast<const __nv_bfloat16 *>(q), static_cast<const __nv_bfloat16 *>(c.k_rows),
+                    static_cast<const __nv_bfloat16 *>(c.v_rows), c.row_off, c.len, scale_log2, chunk_rows, part_o, part_ml,
+                    kvh, d.heads / kvh, max_splits);
 }
 
 int launch_decode_partial_gqa_mma(const ag_layer_desc &d, const void *q, const ag_cache &c, float scale_log2,

@@ -37,8 +37,8 @@ struct GqWarpTriples {
 // kGqStages - 1 tiles are in flight while one is worked on).
 // kHalves: 1 for G <= 8 (rows 8..15 of the operand are zero and their softmax is left out), 2 for G <= 16.
 template <int kGqD, int kGqStages, int kHalves>
-__device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const __nv_bfloat16 *__restrict__ q, int G,
-                                                        const uint8_t *__restrict__ Kg, const uint8_t *__restrict__ Vg,
+__device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const __nv_bfloat16 *q, int G,
+                                                        const uint8_t *Kg, const uint8_t *Vg,
                                                         int r_begin, int r_end, float scale_log2) {
   static_assert(kGqD == 64 || kGqD == 128, "head_dim");
   constexpr int kGqRowBytes = kGqD * 2, kGqTileBytes = gq_tile_bytes(kGqD), kPieces = kGqD / 8;
@@ -59,12 +59,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
       cp_async16(sv + gq_tile_off<kGqD>(r, c), Vg + src);
     }
   };
-#pragma unroll
-  for (int i = 0; i < kGqStages - 1; ++i) {
-    if (i < n_tiles) load_tile(i);
-    cp_async_commit();
-  }
-
+  // (Q is asked for first: these loads cannot move ahead of the asynchronous copies by themselves)
   // A fragments of Q: row g = query head g of the group (rows >= G are zero), 8 steps of 16 dims
   uint32_t qa[kGqD / 16][4];
 #pragma unroll
@@ -83,6 +78,12 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
       qa[ks][1] = g + 8 < G ? qrow[ks * 8 + t] : 0u;
       qa[ks][3] = g + 8 < G ? qrow[ks * 8 + 4 + t] : 0u;
     }
+  }
+
+#pragma unroll
+  for (int i = 0; i < kGqStages - 1; ++i) {
+    if (i < n_tiles) load_tile(i);
+    cp_async_commit();
   }
 
   float o[kGqD / 8][4];

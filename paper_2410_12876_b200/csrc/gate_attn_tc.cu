@@ -24,6 +24,7 @@
 // TMEM columns: S0 [0,64) S1 [128,192) O [256,384) Phi [384,448) Plo [448,512), each P half holding two
 // tiles' weights (32 columns per tile).
 #include "ag_common.cuh"
+#include "mma_sync.cuh"
 #include "umma.cuh"
 
 namespace ag {
@@ -41,7 +42,10 @@ struct GaCfg {
   static constexpr int kTile = kPanels * kGaPanel;        // Q hi or Q lo
   static constexpr int kKvTile = kPanels * kGaKvPanel;    // K or V, one of hi / lo
   static constexpr int kKvStage = 2 * kKvTile;            // hi + lo
-  static constexpr int kSmemBytes = 2 * kTile + 4 * kKvStage + 1024 + 256;   // Q + 2 K stages + 2 V stages
+  static constexpr int kUsedBytes = 2 * kTile + 4 * kKvStage + 1024 + 256;   // Q + 2 K stages + 2 V stages
+  // one CTA per SM whatever D (each takes all of tensor memory: a second one on the SM would wait for the first
+  // to end while other SMs stand idle)
+  static constexpr int kSmemBytes = kUsedBytes > 120 * 1024 ? kUsedBytes : 120 * 1024;
 };
 constexpr uint32_t kGaColS = 0, kGaColO = 256, kGaColPhi = 384, kGaColPlo = 448, kGaTmemCols = 512;
 constexpr float kGaRescaleThreshold = 8.f;
@@ -166,6 +170,8 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();                                        // the projections are there
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -429,29 +435,61 @@ bool gate_attn_tc_supported(const ag_layer_desc &d) {
 //   H'[t, g * D + c] = sum_s w_s O_s[r, c] / sum_s w_s l_s,  w_s = 2^(m_s - max_s m_s)
 //   s[t, i] = H'[t, :] Wo_g[:, i];  flag = s + gamma_i > logit(tau)
 // One CTA = 16 tokens, one warp per token.  A warp merges the token's row of every gate head
-// (a lane per D / 32 columns: every access is one whole row) into shared memory; then warp w
-// takes four tokens and a quarter of the reduction, a lane per head, in rounds of 32 heads,
-// against a [GD][32] slice of Wo staged in shared memory.  H' never goes to global memory.
+// (a lane per D / 32 columns: every access is one whole row) into shared memory; then the warps share the
+// reduction, 16 columns of H' at a time, as m16n8k16 MMAs of the 16 tokens against 32 heads of Wo.
+// Every float32 of H' enters as three bf16 (8 + 8 + 8 mantissa bits: exactly its value), so nothing of it
+// is lost, and Wo is bf16 as it comes.  The warps' sums are added in a fixed order.  H' never goes to global
+// memory.  (With the products on CUDA cores, operands from shared memory, this was 18 us at 4,096 tokens
+// and 141 us at 8 x 4,096.)  Wo is fetched before the wait for MHA', which it does not depend on.
 constexpr int kMoTokens = 16, kMoThreads = kMoTokens * 32;
 template <int N> struct FloatVec;
 template <> struct FloatVec<2> { using type = float2; };
 template <> struct FloatVec<4> { using type = float4; };
-template <typename T, int kGaD>
+constexpr int kMoRedPitch = 33;                                  // floats per token of a warp's sums (32 heads)
+constexpr int kMoRedBytes = kMoTokens * kMoTokens * kMoRedPitch * 4;
+__host__ __device__ constexpr int mo_w_bytes(int GD) { return GD * 64 > kMoRedBytes ? GD * 64 : kMoRedBytes; }
+__host__ __device__ constexpr int mo_smem_bytes(int GD) { return mo_w_bytes(GD) + kMoTokens * (GD + 8) * 4; }
+// Byte offset of 16-byte piece `piece` (8 heads) of row `c` of the staged slice of Wo: 64-byte rows, pieces XOR-ed so
+// that the eight rows one ldmatrix reads fall into different banks.
+__device__ __forceinline__ uint32_t mo_w_off(int c, int piece) { return (uint32_t)(c * 64 + ((piece ^ ((c >> 1) & 3)) << 4)); }
+
+template <int kGaD>
 __global__ void __launch_bounds__(kMoThreads)
-gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const T *__restrict__ Wo, const float *__restrict__ gamma,
-                      float logit_tau, int h, float *__restrict__ scores, uint8_t *__restrict__ flags) {
+gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat16 *__restrict__ Wo,
+                      const float *__restrict__ gamma, float logit_tau, int h, float *__restrict__ scores,
+                      uint8_t *__restrict__ flags) {
   extern __shared__ __align__(16) unsigned char mo_smem[];
-  float *Hs = reinterpret_cast<float *>(mo_smem);                                   // [16][GD]
-  T *Ws = reinterpret_cast<T *>(mo_smem + sizeof(float) * kMoTokens * a.GD);       // [GD][32]
-  float *red = reinterpret_cast<float *>(mo_smem + sizeof(float) * kMoTokens * a.GD + sizeof(T) * a.GD * 32);  // [4][16][32]
+  unsigned char *Ws = mo_smem;                                   // [GD][32] bf16, then the warps' sums
+  float *red = reinterpret_cast<float *>(mo_smem);               // [16 warps][16 tokens][33]
+  float *Hs = reinterpret_cast<float *>(mo_smem + mo_w_bytes(a.GD));     // [16][GD + 8]
+  const int pitch = a.GD + 8;
+  __shared__ int seg_first[2][kMoThreads];           // per gate head: first segment, number of pieces
   const int tiles_per_seq = (a.n + kMoTokens - 1) / kMoTokens;
   const int b = blockIdx.x / tiles_per_seq, t0 = (blockIdx.x % tiles_per_seq) * kMoTokens;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = t0 + warp;
-  float *hrow = Hs + warp * a.GD;
+  float *hrow = Hs + warp * pitch;
+  // heads i0 .. i0 + 31 of Wo
+  auto stage_wo = [&](int i0) {
+    const uint32_t ws = smem_u32(Ws);
+    for (int x = threadIdx.x; x < a.GD * 4; x += kMoThreads) {
+      const int c = x >> 2, i = i0 + (x & 3) * 8;
+      const uint32_t off = mo_w_off(c, x & 3);
+      if ((h & 7) == 0 && i < h) {
+        cp_async16(ws + off, Wo + (size_t)c * h + i);
+      } else {
+        __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(Ws + off);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) dst[e] = i + e < h ? Wo[(size_t)c * h + i + e] : __float2bfloat16_rn(0.f);
+      }
+    }
+    cp_async_commit();
+  };
+  stage_wo(0);
+  pdl_wait();
+  pdl_launch_dependents();
   // The CTA's 16 tokens lie in one query tile: which segments hold its pieces is looked up once per
   // gate head (a binary search over the boundaries in constant memory), by one thread each.
-  int *seg_first = reinterpret_cast<int *>(red);     // [gate_heads] first segment, then [gate_heads] piece count
   {
     const int qt = t0 / kGaBM;
     const int y0 = ga_first_step(qt, a.n_qtiles, a.causal), y1 = y0 + ga_key_tiles(qt, a.n_qtiles, a.causal);
@@ -460,8 +498,8 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const T *__restric
       // the query tile's steps [x0, x1) of the list lie in segments seg0 .. seg1, one piece in each
       const int x0 = prob * a.steps_per_prob + y0, x1 = prob * a.steps_per_prob + y1;
       const int seg0 = ga_segment_of(a, x0);
-      seg_first[g] = seg0;
-      seg_first[a.gate_heads + g] = ga_segment_of(a, x1 - 1) - seg0 + 1;
+      seg_first[0][g] = seg0;
+      seg_first[1][g] = ga_segment_of(a, x1 - 1) - seg0 + 1;
     }
   }
   __syncthreads();
@@ -475,8 +513,8 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const T *__restric
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int g = min(g0 + u, a.gate_heads - 1), prob = b * a.gate_heads + g;
-        ns[u] = seg_first[a.gate_heads + g];
-        row0[u] = (size_t)ga_slot(prob, qt, a.n_qtiles, seg_first[g]) * kGaBM + r;   // + s * 128 per piece
+        ns[u] = seg_first[1][g];
+        row0[u] = (size_t)ga_slot(prob, qt, a.n_qtiles, seg_first[0][g]) * kGaBM + r;   // + s * 128 per piece
         mmax[u] = -INFINITY;
         for (int s = lane; s < ns[u]; s += 32) mmax[u] = fmaxf(mmax[u], a.part_ml[(row0[u] + (size_t)s * kGaBM) * 2]);
       }
@@ -496,6 +534,7 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const T *__restric
         lsum[u] = 0.f;
         ns_max = max(ns_max, ns[u]);
       }
+#pragma unroll 2
       for (int s = 0; s < ns_max; ++s) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -521,57 +560,64 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const T *__restric
         }
       }
     }
+  } else {
+    for (int c = lane; c < a.GD; c += 32) hrow[c] = 0.f;         // a token past the end: its row is an MMA operand all the same
   }
+  const int g = lane >> 2, tq = lane & 3, mi = lane >> 3;
   for (int i0 = 0; i0 < h; i0 += 32) {
-    __syncthreads();                                 // H' rows complete; previous slice of Wo consumed
-    if (sizeof(T) == 2 && (h & 7) == 0) {            // 16-byte pieces of the rows of Wo
-      for (int x = threadIdx.x; x < a.GD * 4; x += kMoThreads) {
-        const int c = x >> 2, i = i0 + (x & 3) * 8;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (i < h) v = ldg128(Wo + (size_t)c * h + i);
-        *reinterpret_cast<uint4 *>(Ws + c * 32 + (x & 3) * 8) = v;
-      }
-    } else {
-      for (int x = threadIdx.x; x < a.GD * 32; x += kMoThreads) {
-        const int c = x >> 5, i = i0 + (x & 31);
-        Ws[x] = i < h ? Wo[(size_t)c * h + i] : T(0.f);
-      }
+    if (i0 > 0) {
+      __syncthreads();                               // the previous round's sums have been read
+      stage_wo(i0);
     }
-    __syncthreads();
-    {
-      // warp w: tokens 4 (w & 3) .. + 3 against head `lane` over a quarter of the reduction,
-      // c in [cq, cq + 1) GD / 4; per four steps four broadcast float4 of H' and four values of Wo
-      // feed sixteen FMAs.  The quarters are added in a fixed order below.
-      const int tq = warp & 3, cq = warp >> 2;
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      const float *h4 = Hs + tq * 4 * a.GD;
-      const int c_begin = cq * (a.GD / 4), c_end = c_begin + a.GD / 4;    // GD is a multiple of 128
-#pragma unroll 4
-      for (int c = c_begin; c < c_end; c += 4) {
-        float w[4];
+    cp_async_wait<0>();
+    __syncthreads();                                 // H' rows and this slice of Wo are complete
+    float c[4][4];                                   // 16 tokens x 32 heads, this warp's share of the reduction
 #pragma unroll
-        for (int k = 0; k < 4; ++k) w[k] = Elem<T>::load(Ws + (c + k) * 32 + lane);
+    for (int nb = 0; nb < 4; ++nb)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float4 x = *reinterpret_cast<const float4 *>(h4 + q * a.GD + c);
-          acc[q] = fmaf(x.x, w[0], acc[q]);
-          acc[q] = fmaf(x.y, w[1], acc[q]);
-          acc[q] = fmaf(x.z, w[2], acc[q]);
-          acc[q] = fmaf(x.w, w[3], acc[q]);
+      for (int e = 0; e < 4; ++e) c[nb][e] = 0.f;
+    const uint32_t ws = smem_u32(Ws);
+    for (int k0 = warp * 16; k0 < a.GD; k0 += kMoTokens * 16) {
+      uint32_t ah[3][4];                             // the three bf16 parts of the fragment of H'
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        float2 x = *reinterpret_cast<const float2 *>(Hs + (g + (f & 1) * 8) * pitch + k0 + (f >> 1) * 8 + 2 * tq);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          float h0, h1;
+          split_bf16(x.x, h0, x.x);
+          split_bf16(x.y, h1, x.y);
+          ah[q][f] = pack_bf16x2(h0, h1);
         }
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) red[(cq * kMoTokens + tq * 4 + q) * 32 + lane] = acc[q];
+      for (int nb2 = 0; nb2 < 2; ++nb2) {
+        uint32_t bw[4];
+        // matrices: (k 0-7, heads lo), (k 8-15, heads lo), (k 0-7, heads hi), (k 8-15, heads hi)
+        ldmatrix_x4_trans(bw, ws + mo_w_off(k0 + (mi & 1) * 8 + (lane & 7), nb2 * 2 + (mi >> 1)));
+#pragma unroll
+        for (int q = 2; q >= 0; --q) {
+          mma_16816(c[2 * nb2], ah[q], bw[0], bw[1]);
+          mma_16816(c[2 * nb2 + 1], ah[q], bw[2], bw[3]);
+        }
+      }
     }
+    __syncthreads();                                 // Wo has been read: the sums may take its place
+#pragma unroll
+    for (int nb = 0; nb < 4; ++nb)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        red[(warp * kMoTokens + g + (e >> 1) * 8) * kMoRedPitch + nb * 8 + 2 * tq + (e & 1)] = c[nb][e];
     __syncthreads();
     {
-      // thread (token = warp, head = lane): the four quarters in order
-      const float *rp = red + warp * 32 + lane;
-      const float sc = ((rp[0] + rp[kMoTokens * 32]) + rp[2 * kMoTokens * 32]) + rp[3 * kMoTokens * 32];
-      const int i = i0 + lane;
-      if (i < h && t < a.n) {
-        const size_t o = ((size_t)b * h + i) * a.n + t;
-        const bool padding = a.seq_lens && t >= a.seq_lens[b];
+      // 16 consecutive threads: one head's 16 tokens, which lie side by side in scores and flags
+      const int tok = threadIdx.x & 15, i = i0 + (threadIdx.x >> 4), tt = t0 + tok;
+      float sc = 0.f;
+#pragma unroll
+      for (int w = 0; w < kMoTokens; ++w) sc += red[(w * kMoTokens + tok) * kMoRedPitch + (threadIdx.x >> 4)];
+      if (i < h && tt < a.n) {
+        const size_t o = ((size_t)b * h + i) * a.n + tt;
+        const bool padding = a.seq_lens && tt >= a.seq_lens[b];
         if (scores) scores[o] = sc;
         flags[o] = !padding && (sc + (gamma ? gamma[i] : 0.f)) > logit_tau ? 1 : 0;
       }
@@ -676,16 +722,14 @@ static int run_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const vo
                                         align_up(slots * kGaBM * kGaD * sizeof(float), 256));
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)kGaD));
   AG_CUDA_TRY(cudaFuncSetAttribute(gate_attn_tc_kernel<kGaD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGaSmemBytes));
-  gate_attn_tc_kernel<kGaD><<<(unsigned)plan.n_seg, kGaThreads, kGaSmemBytes, st>>>(tmHi, tmLo, tmHiKv, tmLoKv, a);
-  AG_LAUNCH_CHECK();
-  const size_t mo_smem = sizeof(float) * kMoTokens * GD + sizeof(__nv_bfloat16) * GD * 32 + sizeof(float) * 4 * kMoTokens * 32;
-  auto mo = gate_merge_out_kernel<__nv_bfloat16, kGaD>;
-  AG_CUDA_TRY(cudaFuncSetAttribute(mo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mo_smem));
+  rc = launch_pdl(gate_attn_tc_kernel<kGaD>, dim3(plan.n_seg), dim3(kGaThreads), kGaSmemBytes, st, tmHi, tmLo, tmHiKv,
+                  tmLoKv, a);
+  if (rc) return rc;
+  auto mo = gate_merge_out_kernel<kGaD>;
+  AG_CUDA_TRY(cudaFuncSetAttribute(mo, cudaFuncAttributeMaxDynamicSharedMemorySize, mo_smem_bytes(GD)));
   const int blocks = d.batch * ((d.seq + kMoTokens - 1) / kMoTokens);
-  mo<<<blocks, kMoThreads, mo_smem, st>>>(a, static_cast<const __nv_bfloat16 *>(Wo), gamma, logit_tau, kv_heads_of(d),
-                                          scores, flags);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  return launch_pdl(mo, dim3(blocks), dim3(kMoThreads), mo_smem_bytes(GD), st, a, static_cast<const __nv_bfloat16 *>(Wo),
+                    gamma, logit_tau, kv_heads_of(d), scores, flags);
 }
 
 int launch_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const void *qkv_lo, void *partials,

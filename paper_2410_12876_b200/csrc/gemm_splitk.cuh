@@ -74,6 +74,7 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_launch_dependents();                           // a kernel that waits for this grid may set itself up
 
   if (warp == 0) {
     if (lane == 0) {

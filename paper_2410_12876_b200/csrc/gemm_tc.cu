@@ -77,6 +77,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_launch_dependents();                           // MHA' may set itself up (it waits for this grid's end)
 
   if (warp == 0) {
     if (lane == 0) {
@@ -255,6 +256,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   cluster_arrive_wait();                           // both CTAs' barriers are initialised, tensor memory is allocated
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_launch_dependents();                           // MHA' may set itself up (it waits for this grid's end)
 
   if (warp == 0) {
     if (lane == 0) {

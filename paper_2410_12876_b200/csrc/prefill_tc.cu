@@ -51,6 +51,7 @@ struct PrefillTcArgs {
   const int64_t *row_off;
   const int32_t *len;
   int n, n_qtiles, slabs;           // slabs: (sequence, query head) pairs
+  int band_slabs;                   // slabs per band of the tile order
   int heads, kv_heads;              // query heads share key/value heads in groups of heads / kv_heads
   float scale_log2;
   float *lse;                       // NULL, or [slabs, n]: m + log2(l) of every row (see launch_prefill_tc)
@@ -97,9 +98,29 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 16);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // heaviest query tiles first
-  const int qt = a.n_qtiles - 1 - (int)(blockIdx.x / a.slabs);
-  const int slab = blockIdx.x % a.slabs;           // Q and O live here
+  // Slabs in bands whose keys and values stay in L2 while the band's query tiles pass over them; inside a
+  // band the heaviest query tiles first.  (With all slabs in one band, 8 x 32 heads of 4096 tokens swept
+  // their 300 MB of cache rows through the 126 MB of L2 once per query tile.)
+  const int band = (int)blockIdx.x / (a.band_slabs * a.n_qtiles), in_band = (int)blockIdx.x % (a.band_slabs * a.n_qtiles);
+  const int slabs_here = min(a.band_slabs, a.slabs - band * a.band_slabs);
+  const int qt = a.n_qtiles - 1 - in_band / slabs_here;
+  const int slab = band * a.band_slabs + in_band % slabs_here;   // Q and O live here
+  if (threadIdx.x == 0) {
+    mbar_init(q_full, 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], 1);
+      mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1);
+      mbar_init(&s_full[s], 1);
+    }
+    mbar_init(&p_ready[0], 128); mbar_init(&p_ready[1], 128);
+    mbar_init(&pv_done[0], 1); mbar_init(&pv_done[1], 1);
+    mbar_init(self_full, 1);
+    fence_barrier_init();
+    prefetch_tensormap(&tmQ); prefetch_tensormap(&tmKd); prefetch_tensormap(&tmVd);
+    prefetch_tensormap(&tmK); prefetch_tensormap(&tmV); prefetch_tensormap(&tmO);
+  }
+  pdl_wait();                                       // the cache, prefix and lengths are there
+  pdl_launch_dependents();
   // a query tile past its sequence's end holds padding only: its outputs are unspecified, nothing to do
   if (a.seq_lens != nullptr && qt * kPfBM >= a.seq_lens[slab / a.heads]) return;
   // K, V, the flags' prefix counts and the cache belong to the key/value head (grouped-query attention)
@@ -116,20 +137,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   // uses of K stage 0 / 1 before the dense V tile: even / odd cache tiles
   const int k0_uses = (n_kv + 1) / 2, k1_uses = n_kv / 2;
 
-  if (threadIdx.x == 0) {
-    mbar_init(q_full, 1);
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], 1);
-      mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1);
-      mbar_init(&s_full[s], 1);
-    }
-    mbar_init(&p_ready[0], 128); mbar_init(&p_ready[1], 128);
-    mbar_init(&pv_done[0], 1); mbar_init(&pv_done[1], 1);
-    mbar_init(self_full, 1);
-    fence_barrier_init();
-    prefetch_tensormap(&tmQ); prefetch_tensormap(&tmKd); prefetch_tensormap(&tmVd);
-    prefetch_tensormap(&tmK); prefetch_tensormap(&tmV); prefetch_tensormap(&tmO);
-  }
   if (warp == 1) {
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
@@ -454,14 +461,19 @@ static int run_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, 
   a.prefix = prefix; a.row_off = c.row_off; a.len = c.len;
   a.n = d.seq; a.n_qtiles = (d.seq + kPfBM - 1) / kPfBM; a.slabs = slabs;
   a.heads = d.heads; a.kv_heads = kv_heads_of(d);
+  // Cache rows of a band: at most 32 MB of keys and 32 MB of values if every token were kept (half of L2 with
+  // what else passes through it), but enough tiles for a full round of the chip at the lightest query tiles' end.
+  const long long slab_bytes = (long long)d.seq * kPfD * 2 / (d.heads / a.kv_heads);
+  a.band_slabs = (int)((32LL << 20) / (slab_bytes > 0 ? slab_bytes : 1));
+  if (a.band_slabs < 32) a.band_slabs = 32;
+  if (a.band_slabs > slabs) a.band_slabs = slabs;
   a.scale_log2 = scale * 1.4426950408889634f;
   a.lse = lse;
   a.seq_lens = d.seq_lens;
   constexpr int smem = PfCfg<kPfD>::kSmemBytes;
   AG_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel<kPfD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  prefill_tc_kernel<kPfD><<<a.n_qtiles * slabs, kPfThreads, smem, st>>>(tmQ, tmKd, tmVd, tmO, tmK, tmV, a);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  return launch_pdl(prefill_tc_kernel<kPfD>, dim3(a.n_qtiles * slabs), dim3(kPfThreads), smem, st, tmQ, tmKd, tmVd, tmO, tmK,
+                    tmV, a);
 }
 
 int launch_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const ag_cache &c,
