@@ -542,7 +542,9 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
 // One cluster per run of G <= 16 query slabs that share a key/value slab (G = 1 without grouped-query
 // attention): the G queries are rows of one MMA operand, so the slab is read once for all of them, and the
 // one cluster that reads it may append to it.  CTA `rank` takes whole 64-row tiles; after the cluster
-// barrier rank r merges the heads r, r + 8 of the group.
+// barrier rank r merges the heads r, r + 8 of the group.  The tiles go round the ranks, so a rank's first tile does
+// not depend on the slab's length and its rows are asked for together with the length (before it is known
+// they are only known to lie inside the slab): one trip to L2 less on the path of a step.
 // three stages: a CTA has few tiles and no neighbour to hide behind, so two of them are kept in flight
 constexpr int kCmStages = 3;
 // kMaxG: 1 (one query per slab), 8 or 16.
@@ -550,7 +552,7 @@ template <int D, int kMaxG>
 __global__ void __launch_bounds__(kGqThreads, 2)
 decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
                           const __nv_bfloat16 *v_new, const __nv_bfloat16 *k_rows,
-                          const __nv_bfloat16 *v_rows, const int64_t *row_off,
+                          const __nv_bfloat16 *v_rows, const int64_t *row_off, const int32_t *cap,
                           const int32_t *len, float scale_log2, __nv_bfloat16 *out, int group,
                           const AppendArgs ap, const HeadMap hm, const RecentRing rg) {
   namespace cg = cooperative_groups;
@@ -564,13 +566,17 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   const int kv = hm.kv_slab(slab0);
   const int d = threadIdx.x;
   pdl_launch_dependents();
-  // the slab's first row never changes once the cache is laid out: read ahead of the wait for the
-  // preceding kernel, so that only the length is on the critical path after it
+  // the slab's first row and capacity never change once the cache is laid out: read ahead of the wait for the
+  // preceding kernel
   const int64_t slab_row0 = row_off[kv];
+  const int slab_cap = cap[kv];
   pdl_wait();
   const int L = len[kv];
-  const int per = ((L + kClusterSize - 1) / kClusterSize + kGqTile - 1) / kGqTile * kGqTile;
-  const int r_begin = min(L, rank * per), r_end = min(L, r_begin + per);
+  const int r_first = rank * kGqTile;
+  const uint8_t *Kg = reinterpret_cast<const uint8_t *>(k_rows) + (size_t)slab_row0 * (D * 2);
+  const uint8_t *Vg = reinterpret_cast<const uint8_t *>(v_rows) + (size_t)slab_row0 * (D * 2);
+  if (r_first < slab_cap) gq_load_tile<D>((uint32_t)__cvta_generic_to_shared(gq_smem), Kg, Vg, r_first, slab_cap);
+  cp_async_commit();
 
   // this CTA's triples [G][D] and [G][2], read by the merging ranks: behind the warps' triples in the ring's memory
   float *cta_o = reinterpret_cast<float *>(gq_smem + gq_smem_bytes(D, kCmStages) - kGqMaxGroup * (D + 2) * 4);
@@ -590,11 +596,9 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
     v_raw = v_new[(size_t)kv * D + d];
   }
 
-  if (r_begin < r_end) {              // the same for the whole CTA
-    const size_t row0 = (size_t)slab_row0 * (D * 2);
-    const GqWarpTriples w = gq_stream_rows<D, kCmStages, (kMaxG + 7) / 8>(gq_smem, q + (size_t)slab0 * D, G,
-                                           reinterpret_cast<const uint8_t *>(k_rows) + row0,
-                                           reinterpret_cast<const uint8_t *>(v_rows) + row0, r_begin, r_end, scale_log2);
+  if (r_first < L) {                  // the same for the whole CTA
+    const GqWarpTriples w = gq_stream_rows<D, kCmStages, (kMaxG + 7) / 8, true>(
+        gq_smem, q + (size_t)slab0 * D, G, Kg, Vg, r_first, kClusterSize * kGqTile, L, scale_log2);
     for (int x = d; x < G * D; x += kGqThreads) {
       const int h = x / D, e = x % D;
       float acc, mc, lc;
@@ -605,6 +609,7 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   } else {
     for (int x = d; x < G * D; x += kGqThreads) cta_o[x] = 0.f;
     if (d < G) { cta_ml[2 * d] = -INFINITY; cta_ml[2 * d + 1] = 0.f; }
+    cp_async_wait<0>();               // (the first tile, asked for in vain)
   }
 #pragma unroll
   for (int u = 0; u < kHeads; ++u) {
@@ -691,7 +696,7 @@ static int launch_decode_cluster_mma(int groups, int G, const void *q, const voi
   AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_mma_kernel<D, kMaxG>, static_cast<const T *>(q),
                                  static_cast<const T *>(k_new), static_cast<const T *>(v_new),
                                  static_cast<const T *>(c.k_rows), static_cast<const T *>(c.v_rows),
-                                 c.row_off, c.len, scale_log2, static_cast<T *>(o), G, ap, hm, rg));
+                                 c.row_off, c.cap, c.len, scale_log2, static_cast<T *>(o), G, ap, hm, rg));
   return AG_OK;
 }
 

@@ -31,34 +31,42 @@ struct GqWarpTriples {
   float *o, *m, *l;     // [warps][16][D], [warps][16], [warps][16]
 };
 
-// Every thread of the CTA (kGqThreads of them) calls this with the same arguments; r_begin < r_end.
+// One tile of K and of V (64 rows from r0; rows from r_end on are replaced by the last one before it) on its way to
+// the ring stage at smem address `stage`.
+template <int kGqD>
+__device__ __forceinline__ void gq_load_tile(uint32_t stage, const uint8_t *Kg, const uint8_t *Vg, int r0, int r_end) {
+  constexpr int kPieces = kGqD / 8;
+#pragma unroll
+  for (int x = 0; x < kGqTile * kPieces / kGqThreads; ++x) {
+    const int idx = threadIdx.x + x * kGqThreads, r = idx / kPieces, c = idx % kPieces;
+    const size_t src = (size_t)min(r0 + r, r_end - 1) * (kGqD * 2) + c * 16;
+    cp_async16(stage + gq_tile_off<kGqD>(r, c), Kg + src);
+    cp_async16(stage + gq_tile_bytes(kGqD) + gq_tile_off<kGqD>(r, c), Vg + src);
+  }
+}
+
+// Every thread of the CTA (kGqThreads of them) calls this with the same arguments.  The CTA's tiles are the 64
+// rows from r_first + i * r_step for i = 0, 1, ... while that is below r_end (at least one).
 // q: G consecutive query vectors [G][D]; Kg, Vg: first row of the slab.  Returns after a CTA barrier
 // with the warps' triples in shared memory (gq_smem: gq_smem_bytes(D, kGqStages) of dynamic shared memory;
 // kGqStages - 1 tiles are in flight while one is worked on).
+// kFirstLoaded: the caller has issued tile 0 into stage 0 and committed it, perhaps before it knew r_end: its rows
+// past r_end may then hold anything.  Their scores are masked; their values are masked too (0 * NaN is NaN).
 // kHalves: 1 for G <= 8 (rows 8..15 of the operand are zero and their softmax is left out), 2 for G <= 16.
-template <int kGqD, int kGqStages, int kHalves>
+template <int kGqD, int kGqStages, int kHalves, bool kFirstLoaded>
 __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const __nv_bfloat16 *q, int G,
-                                                        const uint8_t *Kg, const uint8_t *Vg,
-                                                        int r_begin, int r_end, float scale_log2) {
+                                                        const uint8_t *Kg, const uint8_t *Vg, int r_first, int r_step,
+                                                        int r_end, float scale_log2) {
   static_assert(kGqD == 64 || kGqD == 128, "head_dim");
-  constexpr int kGqRowBytes = kGqD * 2, kGqTileBytes = gq_tile_bytes(kGqD), kPieces = kGqD / 8;
-  const int n_tiles = (r_end - r_begin + kGqTile - 1) / kGqTile;
+  constexpr int kGqTileBytes = gq_tile_bytes(kGqD);
+  const int n_tiles = (r_end - r_first + r_step - 1) / r_step;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;                                       // fragment row, column pair
   const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(gq_smem);
-
-  // tile i -> stage i % kGqStages; rows past r_end are clamped to the last valid row (weight 0 below)
-  auto load_tile = [&](int i) {
-    const uint32_t sk = smem0 + (i % kGqStages) * 2 * kGqTileBytes, sv = sk + kGqTileBytes;
-    const int r0 = r_begin + i * kGqTile;
-#pragma unroll
-    for (int x = 0; x < kGqTile * kPieces / kGqThreads; ++x) {
-      const int idx = threadIdx.x + x * kGqThreads, r = idx / kPieces, c = idx % kPieces;
-      const size_t src = (size_t)min(r0 + r, r_end - 1) * kGqRowBytes + c * 16;
-      cp_async16(sk + gq_tile_off<kGqD>(r, c), Kg + src);
-      cp_async16(sv + gq_tile_off<kGqD>(r, c), Vg + src);
-    }
+  auto load_tile = [&](int i) {                                                // tile i -> stage i % kGqStages
+    gq_load_tile<kGqD>(smem0 + (i % kGqStages) * 2 * kGqTileBytes, Kg, Vg, r_first + i * r_step, r_end);
   };
+
   // (Q is asked for first: these loads cannot move ahead of the asynchronous copies by themselves)
   // A fragments of Q: row g = query head g of the group (rows >= G are zero), 8 steps of 16 dims
   uint32_t qa[kGqD / 16][4];
@@ -81,7 +89,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
   }
 
 #pragma unroll
-  for (int i = 0; i < kGqStages - 1; ++i) {
+  for (int i = kFirstLoaded ? 1 : 0; i < kGqStages - 1; ++i) {
     if (i < n_tiles) load_tile(i);
     cp_async_commit();
   }
@@ -101,7 +109,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
     cp_async_wait<kGqStages - 1>();                             // tile i has landed (this thread's pieces)
     __syncthreads();                                            // ... and everybody's
     const uint32_t sk = smem0 + (i % kGqStages) * 2 * kGqTileBytes, sv = sk + kGqTileBytes;
-    const int key0 = r_begin + i * kGqTile + warp * 16;         // this warp's 16 rows of the tile
+    const int key0 = r_first + i * r_step + warp * 16;          // this warp's 16 rows of the tile
 
     if (key0 < r_end) {
       // S = Q K^T for 16 keys: two 8-key column tiles
@@ -145,13 +153,23 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
           o[nt][2 * h + 1] *= alpha;
         }
       }
-      // O += P V: 16 keys x 128 dims, two 8-dim column tiles per ldmatrix
+      // O += P V: 16 keys x D dims, two 8-dim column tiles per ldmatrix
+      uint32_t vmask[2];                                        // valid keys among 2t, 2t + 1 | 2t + 8, 2t + 9
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int k = key0 + e * 8 + 2 * t;
+        vmask[e] = k + 1 < r_end ? 0xffffffffu : (k < r_end ? 0xffffu : 0u);
+      }
 #pragma unroll
       for (int nt2 = 0; nt2 < kGqD / 16; ++nt2) {
         uint32_t b[4];
         // matrices: (keys 0-7, dims lo), (keys 8-15, dims lo), (keys 0-7, dims hi), (keys 8-15, dims hi)
         const int mi = lane >> 3, row = warp * 16 + (mi & 1) * 8 + (lane & 7);
         ldmatrix_x4_trans(b, sv + gq_tile_off<kGqD>(row, nt2 * 2 + (mi >> 1)));
+        if (kFirstLoaded && i == 0) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) b[e] &= vmask[e & 1];
+        }
         mma_16816(o[2 * nt2], pa, b[0], b[1]);
         mma_16816(o[2 * nt2 + 1], pa, b[2], b[3]);
       }
