@@ -2,9 +2,15 @@
 // the fp32 layer (tcgen05 has no true-fp32 MMA) and the fp32 internals of the
 // gate (MHA' of Sec. 3.3 evaluated on float32 Q', K', V').
 //
-// One CTA = 64 query rows x one problem (sequence, head); keys are visited in
-// tiles of 64 with an online softmax.  Row j sees the first bound(j) rows of
-// the key array, where bound is
+// One CTA = BM (64, 32 or 16) query rows x one problem (sequence, head); keys are visited in
+// tiles of 64 with an online softmax, whatever BM, so a row's result does not depend on it.  Thread
+// (tx, ty) of 16 x 16 holds rows ty * BM / 16 .. and keys tx, tx + 16, tx + 32, tx + 48 of a tile.  K and V
+// lie row-major in shared memory (rows of D + 4 floats: the 16-byte reads of eight lanes fall into
+// different banks) and arrive by 16-byte asynchronous copies: the next K while the weighted sum runs, V
+// while the scores are computed.  Inner loops read 16 bytes of every operand per four steps.
+// Few query tiles (a short prompt) get small BM, so that more SMs work: 128 tokens of 4 heads of 64 (8 CTAs at
+// BM = 64) 25 -> 10.6 us.
+// Row j sees the first bound(j) rows of the key array, where bound is
 //   kGateCausal : j + 1            (lower-triangular mask inside MHA')
 //   kGateFull   : n                (every token sees the whole sequence)
 //   kPrefill    : prefix[s, j]     (retained tokens before j, read from the
@@ -12,6 +18,7 @@
 //                                   v_j) from the dense K, V: Eq. 5.
 #pragma once
 #include "ag_common.cuh"
+#include "mma_sync.cuh"
 
 namespace ag {
 
@@ -39,32 +46,34 @@ struct SimtAttnArgs {
   const int32_t *seq_lens;
 };
 
-constexpr int kSimtBM = 64, kSimtBN = 64, kSimtThreads = 256;
+constexpr int kSimtBN = 64, kSimtThreads = 256;
 
-template <int D>
+template <int D, int BM>
 constexpr size_t simt_attn_smem_bytes() {
-  return sizeof(float) * ((size_t)kSimtBM * D + (size_t)D * (kSimtBN + 4) + (size_t)kSimtBN * D +
-                          (size_t)kSimtBM * (kSimtBN + 4));
+  return sizeof(float) * ((size_t)(BM + kSimtBN) * (D + 4) + (size_t)kSimtBN * D + (size_t)BM * (kSimtBN + 4));
 }
 
-template <typename TIn, typename TOut, int D, int MODE>
+template <typename TIn, typename TOut, int D, int MODE, int BM>
 __global__ void __launch_bounds__(kSimtThreads)
 simt_attn_kernel(const SimtAttnArgs a) {
   extern __shared__ __align__(16) float smem[];
-  float *Qs = smem;                               // [BM][D]
-  float *Kt = Qs + kSimtBM * D;                   // [D][BN + 4]  (transposed)
-  float *Vs = Kt + D * (kSimtBN + 4);             // [BN][D]
-  float *Ps = Vs + kSimtBN * D;                   // [BM][BN + 4]
-  constexpr int KP = kSimtBN + 4;
+  constexpr int QP = D + 4, PP = kSimtBN + 4;     // row pitches
+  float *Qs = smem;                               // [BM][QP]
+  float *Ks = Qs + BM * QP;                       // [BN][QP]
+  float *Vs = Ks + kSimtBN * QP;                  // [BN][D]
+  float *Ps = Vs + kSimtBN * D;                   // [BM][PP]
+  constexpr int RM = BM / 16;                     // rows per thread
   constexpr int kEpl = Elem<TIn>::kPerVec;
   constexpr int kVecPerRow = D / kEpl;
   constexpr int kOC = D / 64;                     // float4 column groups per thread
 
   const int prob = blockIdx.y;
   const int b = prob / a.inner, i = prob % a.inner;
-  const int j0 = blockIdx.x * kSimtBM;
+  const int j0 = (gridDim.x - 1 - blockIdx.x) * BM;   // the tiles with the most keys first
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
 
+  pdl_wait();
+  pdl_launch_dependents();
   const TIn *Qp = static_cast<const TIn *>(a.Q) + b * a.q_batch + i * a.q_inner;
   // grouped-query attention: query head i reads key/value head ik, cache slab prob_kv
   const int group = a.kv_group > 1 ? a.kv_group : 1;
@@ -86,49 +95,63 @@ simt_attn_kernel(const SimtAttnArgs a) {
   // prefill: a query tile past its sequence's end holds padding only (outputs unspecified): nothing to do
   if (MODE == kPrefill && a.seq_lens && j0 >= a.seq_lens[prob / a.inner]) return;
 
-  // Q tile -> shared (rows past n are clamped; they are never stored)
-  for (int x = tid; x < kSimtBM * kVecPerRow; x += kSimtThreads) {
-    const int r = x / kVecPerRow, c = x % kVecPerRow;
-    const int j = min(j0 + r, a.n - 1);
-    float f[kEpl];
-    Elem<TIn>::unpack(ldg128(Qp + j * a.q_row + c * kEpl), f);
+  // rows r0 .. of src -> shared rows of `pitch` floats; rows past `last` are clamped (masked below, or never stored)
+  auto load_rows = [&](float *dst, int pitch, const TIn *src, long long row_stride, int r0, int count, int last) {
+    for (int x = tid; x < count * kVecPerRow; x += kSimtThreads) {
+      const int r = x / kVecPerRow, c = x % kVecPerRow;
+      const TIn *from = src + min(r0 + r, last) * row_stride + c * kEpl;
+      float *to = dst + r * pitch + c * kEpl;
+      if constexpr (sizeof(TIn) == 4) {
+        cp_async16((uint32_t)__cvta_generic_to_shared(to), from);
+      } else {
+        float f[kEpl];
+        Elem<TIn>::unpack(ld128(from), f);
 #pragma unroll
-    for (int e = 0; e < kEpl; ++e) Qs[r * D + c * kEpl + e] = f[e];
-  }
+        for (int e = 0; e < kEpl; ++e) to[e] = f[e];
+      }
+    }
+    cp_async_commit();
+  };
 
-  int bound[4];
-  bool valid[4];
+  int bound[RM];
+  bool valid[RM];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int j = j0 + ty * 4 + r;
+  for (int r = 0; r < RM; ++r) {
+    const int j = j0 + ty * RM + r;
     valid[r] = j < a.n;
     const int jc = min(j, a.n - 1);
     bound[r] = MODE == kGateCausal ? jc + 1 : (MODE == kGateFull ? n_keys : min(pre[jc], slab_len));
     if (!valid[r]) bound[r] = 0;
   }
-  const int j_last = min(j0 + kSimtBM, a.n) - 1;
+  const int j_last = min(j0 + BM, a.n) - 1;
   const int max_bound = MODE == kGateCausal ? j_last + 1 : (MODE == kGateFull ? n_keys : min(pre[j_last], slab_len));
   const int n_tiles = (max_bound + kSimtBN - 1) / kSimtBN;
+  const int t_last = max_bound - 1;                 // rows past it are masked for every query
+  load_rows(Qs, QP, Qp, a.q_row, j0, BM, a.n - 1);
+  if (n_tiles > 0) {
+    load_rows(Ks, QP, Kp, kp_row, 0, kSimtBN, t_last);
+    load_rows(Vs, D, Vp, vp_row, 0, kSimtBN, t_last);
+  }
 
-  float m[4], l[4], o[4][kOC][4];
+  float m[RM], l[RM], o[RM][kOC][4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < RM; ++r) {
     m[r] = -INFINITY; l[r] = 0.f;
 #pragma unroll
     for (int c = 0; c < kOC; ++c)
 #pragma unroll
       for (int e = 0; e < 4; ++e) o[r][c][e] = 0.f;
   }
-  __syncthreads();
 
   if (MODE == kPrefill) {
     // self term: the diagonal of Eq. 5 seeds the running softmax (m = s_jj, l = 1, o = v_j)
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = ty * 4 + r;
-      const int j = min(j0 + row, a.n - 1);
+    for (int r = 0; r < RM; ++r) {
+      const int j = min(j0 + ty * RM + r, a.n - 1);
       float acc = 0.f;
-      for (int d = tx; d < D; d += 16) acc = fmaf(Qs[row * D + d], Elem<TIn>::load(Kd + j * a.k_row + d), acc);
+#pragma unroll
+      for (int d = 0; d < D; d += 16)
+        acc = fmaf(Elem<TIn>::load(Qp + j * a.q_row + d + tx), Elem<TIn>::load(Kd + j * a.k_row + d + tx), acc);
 #pragma unroll
       for (int off = 8; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
       m[r] = acc * a.scale_log2;
@@ -142,46 +165,36 @@ simt_attn_kernel(const SimtAttnArgs a) {
 
   for (int kt = 0; kt < n_tiles; ++kt) {
     const int t0 = kt * kSimtBN;
-    const int t_last = max_bound - 1;   // clamp: rows past max_bound are masked for every query
-    __syncthreads();
-    for (int x = tid; x < kSimtBN * kVecPerRow; x += kSimtThreads) {
-      const int r = x / kVecPerRow, c = x % kVecPerRow;
-      const int t = min(t0 + r, t_last);
-      float f[kEpl];
-      Elem<TIn>::unpack(ldg128(Kp + t * kp_row + c * kEpl), f);
+    cp_async_wait<1>();                             // Q and this K (this thread's pieces)
+    __syncthreads();                                // ... and everybody's
+    float s[RM][4];
 #pragma unroll
-      for (int e = 0; e < kEpl; ++e) Kt[(c * kEpl + e) * KP + r] = f[e];
-      Elem<TIn>::unpack(ldg128(Vp + t * vp_row + c * kEpl), f);
-#pragma unroll
-      for (int e = 0; e < kEpl; ++e) Vs[r * D + c * kEpl + e] = f[e];
-    }
-    __syncthreads();
-
-    float s[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < RM; ++r)
 #pragma unroll
       for (int c = 0; c < 4; ++c) s[r][c] = 0.f;
 #pragma unroll 4
-    for (int d = 0; d < D; ++d) {
-      const float4 kv = *reinterpret_cast<const float4 *>(&Kt[d * KP + tx * 4]);
-      float qv[4];
+    for (int d = 0; d < D; d += 4) {
+      float4 qv[RM];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) qv[r] = Qs[(ty * 4 + r) * D + d];
+      for (int r = 0; r < RM; ++r) qv[r] = *reinterpret_cast<const float4 *>(&Qs[(ty * RM + r) * QP + d]);
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        s[r][0] = fmaf(qv[r], kv.x, s[r][0]);
-        s[r][1] = fmaf(qv[r], kv.y, s[r][1]);
-        s[r][2] = fmaf(qv[r], kv.z, s[r][2]);
-        s[r][3] = fmaf(qv[r], kv.w, s[r][3]);
+      for (int c = 0; c < 4; ++c) {
+        const float4 kv = *reinterpret_cast<const float4 *>(&Ks[(tx + 16 * c) * QP + d]);
+#pragma unroll
+        for (int r = 0; r < RM; ++r) {
+          s[r][c] = fmaf(qv[r].x, kv.x, s[r][c]);
+          s[r][c] = fmaf(qv[r].y, kv.y, s[r][c]);
+          s[r][c] = fmaf(qv[r].z, kv.z, s[r][c]);
+          s[r][c] = fmaf(qv[r].w, kv.w, s[r][c]);
+        }
       }
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < RM; ++r) {
       float mx = -INFINITY;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const bool vis = t0 + tx * 4 + c < bound[r];
+        const bool vis = t0 + tx + 16 * c < bound[r];
         s[r][c] = vis ? s[r][c] * a.scale_log2 : -INFINITY;
         mx = fmaxf(mx, s[r][c]);
       }
@@ -204,33 +217,44 @@ simt_attn_kernel(const SimtAttnArgs a) {
       for (int c = 0; c < kOC; ++c)
 #pragma unroll
         for (int e = 0; e < 4; ++e) o[r][c][e] *= alpha;
-      *reinterpret_cast<float4 *>(&Ps[(ty * 4 + r) * KP + tx * 4]) = make_float4(p[0], p[1], p[2], p[3]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) Ps[(ty * RM + r) * PP + tx + 16 * c] = p[c];
     }
-    __syncthreads();
-#pragma unroll 2
-    for (int t = 0; t < kSimtBN; ++t) {
-      float pv[4];
+    cp_async_wait<0>();                             // this V
+    __syncthreads();                                // V and P complete; K has been read
+    if (kt + 1 < n_tiles) load_rows(Ks, QP, Kp, kp_row, t0 + kSimtBN, kSimtBN, t_last);
+#pragma unroll 4
+    for (int t = 0; t < kSimtBN; t += 4) {
+      float4 pv[RM];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) pv[r] = Ps[(ty * 4 + r) * KP + t];
+      for (int r = 0; r < RM; ++r) pv[r] = *reinterpret_cast<const float4 *>(&Ps[(ty * RM + r) * PP + t]);
 #pragma unroll
-      for (int c = 0; c < kOC; ++c) {
-        const float4 vv = *reinterpret_cast<const float4 *>(&Vs[t * D + c * 64 + tx * 4]);
+      for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          o[r][c][0] = fmaf(pv[r], vv.x, o[r][c][0]);
-          o[r][c][1] = fmaf(pv[r], vv.y, o[r][c][1]);
-          o[r][c][2] = fmaf(pv[r], vv.z, o[r][c][2]);
-          o[r][c][3] = fmaf(pv[r], vv.w, o[r][c][3]);
+        for (int c = 0; c < kOC; ++c) {
+          const float4 vv = *reinterpret_cast<const float4 *>(&Vs[(t + u) * D + c * 64 + tx * 4]);
+#pragma unroll
+          for (int r = 0; r < RM; ++r) {
+            const float w = u == 0 ? pv[r].x : u == 1 ? pv[r].y : u == 2 ? pv[r].z : pv[r].w;
+            o[r][c][0] = fmaf(w, vv.x, o[r][c][0]);
+            o[r][c][1] = fmaf(w, vv.y, o[r][c][1]);
+            o[r][c][2] = fmaf(w, vv.z, o[r][c][2]);
+            o[r][c][3] = fmaf(w, vv.w, o[r][c][3]);
+          }
         }
-      }
+    }
+    if (kt + 1 < n_tiles) {
+      __syncthreads();                              // V and P have been read
+      load_rows(Vs, D, Vp, vp_row, t0 + kSimtBN, kSimtBN, t_last);
     }
   }
+  cp_async_wait<0>();                               // (Q alone, where there was no tile)
 
   TOut *Op = static_cast<TOut *>(a.O) + b * a.o_batch + i * a.o_inner;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < RM; ++r) {
     if (!valid[r]) continue;
-    const int j = j0 + ty * 4 + r;
+    const int j = j0 + ty * RM + r;
     const float inv = 1.f / l[r];
     if (MODE == kPrefill && a.lse != nullptr && tx == 0) a.lse[(size_t)prob * a.n + j] = m[r] + log2f(l[r]);
 #pragma unroll
@@ -241,15 +265,24 @@ simt_attn_kernel(const SimtAttnArgs a) {
   }
 }
 
+template <typename TIn, typename TOut, int D, int MODE, int BM>
+int launch_simt_attn_bm(const SimtAttnArgs &a, int problems, cudaStream_t st) {
+  constexpr size_t smem = simt_attn_smem_bytes<D, BM>();
+  auto kern = simt_attn_kernel<TIn, TOut, D, MODE, BM>;
+  AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  return launch_pdl(kern, dim3((a.n + BM - 1) / BM, problems), dim3(kSimtThreads), smem, st, a);
+}
+
+// BM by the number of CTAs it gives.  A key tile costs a CTA about 4,500, 5,000 or 9,000 cycles at BM = 16, 32, 64
+// (D = 128: the first two are bound by shared-memory reads, the last by FMA issue), so 32 is nearly as
+// quick per CTA as 16 and 64 the cheapest per row only once every SM has two.
 template <typename TIn, typename TOut, int D, int MODE>
 int launch_simt_attn(const SimtAttnArgs &a, int problems, cudaStream_t st) {
-  constexpr size_t smem = simt_attn_smem_bytes<D>();
-  auto kern = simt_attn_kernel<TIn, TOut, D, MODE>;
-  AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dim3 grid((a.n + kSimtBM - 1) / kSimtBM, problems);
-  kern<<<grid, kSimtThreads, smem, st>>>(a);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  constexpr long long kSms = 148;
+  auto ctas = [&](int bm) { return (long long)((a.n + bm - 1) / bm) * problems; };
+  if (ctas(64) >= 2 * kSms) return launch_simt_attn_bm<TIn, TOut, D, MODE, 64>(a, problems, st);
+  if (ctas(32) >= kSms / 2) return launch_simt_attn_bm<TIn, TOut, D, MODE, 32>(a, problems, st);
+  return launch_simt_attn_bm<TIn, TOut, D, MODE, 16>(a, problems, st);
 }
 
 }  // namespace ag

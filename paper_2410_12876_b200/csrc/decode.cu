@@ -415,7 +415,9 @@ decode_combine_kernel(const T *q, const T *k_new,
 // second barrier keeps every CTA's shared memory alive until it has been read.  No CTA leaves
 // early: the cluster barriers need all of them.
 constexpr int kClusterSize = 8;
-template <typename T, int D, int kThreads>
+//
+// kCtas = 1: a cluster of one, for caches that one CTA streams in a round or two (its barriers are the CTA's own).
+template <typename T, int D, int kThreads, int kCtas>
 __global__ void __launch_bounds__(kThreads)
 decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
                       const T *k_rows, const T *v_rows,
@@ -427,12 +429,12 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
   constexpr int kLanes = D / kEpl;
   constexpr int kGroups = kThreads / kLanes;
   cg::cluster_group cluster = cg::this_cluster();
-  const int slab = blockIdx.y, rank = (int)cluster.block_rank();
+  const int slab = blockIdx.y, rank = kCtas == 1 ? 0 : (int)cluster.block_rank();
   const int kv = hm.kv_slab(slab);
   pdl_launch_dependents();
   pdl_wait();
   const int L = len[kv];
-  const int per = ((L + kClusterSize - 1) / kClusterSize + kGroups - 1) / kGroups * kGroups;
+  const int per = ((L + kCtas - 1) / kCtas + kGroups - 1) / kGroups * kGroups;
   const int r_begin = min(L, rank * per), r_end = min(L, r_begin + per);
   const int g = threadIdx.x / kLanes, v = threadIdx.x % kLanes;
 
@@ -484,7 +486,8 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
     cta_ml[0] = mc;
     cta_ml[1] = lc;
   }
-  cluster.sync();
+  if constexpr (kCtas > 1) cluster.sync();
+  else __syncthreads();
   // every CTA of the cluster has read the length and its rows: the new row may go in
   // (never asked for when query heads share a slab: another head's cluster may still be reading its length)
   // by threads that have no part in the merge below, so that the two run side by side
@@ -495,23 +498,23 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
 #pragma unroll
     for (int i = 0; i < D / 32; ++i) s_self += red[i];
     s_self *= scale_log2;
-    float mr[kClusterSize], lr[kClusterSize], orr[kClusterSize];
+    float mr[kCtas], lr[kCtas], orr[kCtas];
 #pragma unroll
-    for (int r = 0; r < kClusterSize; ++r) {
-      const float *ml = cluster.map_shared_rank(cta_ml, r);
+    for (int r = 0; r < kCtas; ++r) {
+      const float *ml = kCtas == 1 ? cta_ml : cluster.map_shared_rank(cta_ml, r);
       mr[r] = ml[0];
       lr[r] = ml[1];
-      orr[r] = cluster.map_shared_rank(cta_o, r)[d];
+      orr[r] = (kCtas == 1 ? cta_o : cluster.map_shared_rank(cta_o, r))[d];
     }
     float mm = s_self;
 #pragma unroll
-    for (int r = 0; r < kClusterSize; ++r) mm = fmaxf(mm, mr[r]);
+    for (int r = 0; r < kCtas; ++r) mm = fmaxf(mm, mr[r]);
     for (int r = 0; r < rg.R; ++r) mm = fmaxf(mm, ring_s[r]);
     const float w_self = exp2f(s_self - mm);
     float acc = w_self * v_self;
     float lsum = w_self;
 #pragma unroll
-    for (int r = 0; r < kClusterSize; ++r) {
+    for (int r = 0; r < kCtas; ++r) {
       const float w = mr[r] == -INFINITY ? 0.f : exp2f(mr[r] - mm);
       acc = fmaf(w, orr[r], acc);
       lsum = fmaf(w, lr[r], lsum);
@@ -533,7 +536,7 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
       ring_put<kVecs>(rg, kv, threadIdx.x, reinterpret_cast<const uint8_t *>(k_new + (size_t)kv * D),
                       reinterpret_cast<const uint8_t *>(v_new + (size_t)kv * D), ap.flag_new[kv] != 0);
   }
-  cluster.sync();
+  if constexpr (kCtas > 1) cluster.sync();
 }
 
 // The cluster form for bf16, with the rows streamed through shared memory and the scores and weighted sums
@@ -700,21 +703,21 @@ static int launch_decode_cluster_mma(int groups, int G, const void *q, const voi
   return AG_OK;
 }
 
-template <typename T, int D, int kThreads>
+template <typename T, int D, int kThreads, int kCtas>
 static int launch_decode_cluster(int slabs, const void *q, const void *k_new, const void *v_new,
                                  const ag_cache &c, float scale_log2, void *o, const AppendArgs &ap,
                                  const HeadMap &hm, const RecentRing &rg, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kClusterSize, slabs);
+  cfg.gridDim = dim3(kCtas, slabs);
   cfg.blockDim = dim3(kThreads);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kClusterSize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[0].val.clusterDim.x = kCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1] = pdl_attribute();
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_kernel<T, D, kThreads>, static_cast<const T *>(q),
+  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_kernel<T, D, kThreads, kCtas>, static_cast<const T *>(q),
                                  static_cast<const T *>(k_new), static_cast<const T *>(v_new),
                                  static_cast<const T *>(c.k_rows), static_cast<const T *>(c.v_rows),
                                  c.row_off, c.len, scale_log2, static_cast<T *>(o), ap, hm, rg));
@@ -750,8 +753,11 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     if (slabs <= kClusterMaxSlabs)
       return launch_decode_cluster_mma<D, 1>(slabs, 1, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
   } else {
+    // caches of at most two rounds of one CTA's rows (host-known bound): no cluster
+    constexpr int kRound = kUnroll * kClusterThreads / (D / Elem<T>::kPerVec);
     if (slabs <= kClusterMaxSlabs)
-      return launch_decode_cluster<T, D, kClusterThreads>(slabs, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
+      return (c.max_cap <= 2 * kRound ? launch_decode_cluster<T, D, kClusterThreads, 1>
+                                      : launch_decode_cluster<T, D, kClusterThreads, kClusterSize>)(slabs, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
   }
   int chunk_rows = (c.max_cap + kMaxSplits - 1) / kMaxSplits;
   chunk_rows = (chunk_rows + 127) / 128 * 128;   // whole iterations of the partial kernel (bf16, D = 128)

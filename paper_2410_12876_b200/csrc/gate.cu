@@ -17,73 +17,106 @@
 
 namespace ag {
 
-constexpr int kGemmBM = 64, kGemmBN = 64, kGemmBK = 16;
+constexpr int kGemmBK = 32;
 
-// C[M, 3*GD] (float32) = A[M, Kd] * [W0 | W1 | W2], each W [Kd, GD] row-major.
-template <typename T>
+// C[M, 3*GD] (float32) = A[M, Kd] * [W0 | W1 | W2], each W [Kd, GD] row-major: the CUDA-core form.
+// One CTA of 256 threads = BT x BT outputs (64: 4 x 4 per thread; 32: 2 x 2, for few tokens, so that more SMs
+// work).  k-blocks of 32 arrive by asynchronous copies, the next one while one is worked on; A is read four k
+// at a time.  Bound by arithmetic and, at few tokens, by the length of the chain over K: 16 k at a time with
+// scalar loads behind the barrier took 16.9 us for 128 x 256 x 384.
+template <typename T, int BT>
 __global__ void __launch_bounds__(256)
-gate_proj_kernel(const T *__restrict__ A, const T *__restrict__ W0, const T *__restrict__ W1,
-                 const T *__restrict__ W2, float *__restrict__ C, int M, int Kd, int GD) {
-  __shared__ __align__(16) float As[kGemmBK][kGemmBM + 4];
-  __shared__ __align__(16) float Ws[kGemmBK][kGemmBN];
+gate_proj_kernel(const T *A, const T *W0, const T *W1, const T *W2, float *C, int M, int Kd, int GD) {
+  constexpr int TM = BT / 16, AP = kGemmBK + 4, kEpl = Elem<T>::kPerVec;
+  __shared__ __align__(16) float As[2][BT][AP];
+  __shared__ __align__(16) float Ws[2][kGemmBK][BT];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * kGemmBM;
-  const int n0 = blockIdx.x * kGemmBN;           // column in the packed [3*GD] output
+  const int m0 = blockIdx.y * BT;
+  const int n0 = blockIdx.x * BT;                // column in the packed [3*GD] output
   const int which = n0 / GD, nw = n0 % GD;       // GD is a multiple of 64: a tile never straddles
   const T *W = which == 0 ? W0 : (which == 1 ? W1 : W2);
-  float acc[4][4];
+  pdl_launch_dependents();
+  // k-block kb -> buffer kb & 1; rows past M are clamped (never stored), k past Kd is zero (Kd is a multiple of 8)
+  auto load_block = [&](int kb) {
+    const int k0 = kb * kGemmBK, buf = kb & 1;
+    for (int x = tid; x < BT * kGemmBK / kEpl; x += 256) {
+      const int ar = x / (kGemmBK / kEpl), ak = x % (kGemmBK / kEpl) * kEpl;
+      const int wr = x / (BT / kEpl), wc = x % (BT / kEpl) * kEpl;
+      const bool a_in = k0 + ak < Kd, w_in = k0 + wr < Kd;
+      const T *from_a = A + (size_t)min(m0 + ar, M - 1) * Kd + (a_in ? k0 + ak : 0);
+      const T *from_w = W + (size_t)(w_in ? k0 + wr : 0) * GD + nw + wc;
+      if constexpr (sizeof(T) == 4) {
+        cp_async16_zfill((uint32_t)__cvta_generic_to_shared(&As[buf][ar][ak]), from_a, a_in ? 16 : 0);
+        cp_async16_zfill((uint32_t)__cvta_generic_to_shared(&Ws[buf][wr][wc]), from_w, w_in ? 16 : 0);
+      } else {
+        float fa[kEpl], fw[kEpl];
+        Elem<T>::unpack(a_in ? ld128(from_a) : make_uint4(0u, 0u, 0u, 0u), fa);
+        Elem<T>::unpack(w_in ? ld128(from_w) : make_uint4(0u, 0u, 0u, 0u), fw);
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-  for (int k0 = 0; k0 < Kd; k0 += kGemmBK) {
-    {
-      const int r = tid >> 2, kq = (tid & 3) * 4;
-      const int row = min(m0 + r, M - 1);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int k = k0 + kq + e;
-        As[kq + e][r] = k < Kd ? Elem<T>::load(A + (size_t)row * Kd + k) : 0.f;
+        for (int e = 0; e < kEpl; ++e) { As[buf][ar][ak + e] = fa[e]; Ws[buf][wr][wc + e] = fw[e]; }
       }
-      const int kr = tid >> 4, c4 = (tid & 15) * 4;
-      const int k = k0 + kr;
+    }
+    cp_async_commit();
+  };
+  float acc[TM][TM];
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        Ws[kr][c4 + e] = k < Kd ? Elem<T>::load(W + (size_t)k * GD + nw + c4 + e) : 0.f;
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TM; ++j) acc[i][j] = 0.f;
+
+  const int n_blocks = (Kd + kGemmBK - 1) / kGemmBK;
+  load_block(0);
+  for (int kb = 0; kb < n_blocks; ++kb) {
+    if (kb + 1 < n_blocks) {
+      load_block(kb + 1);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
     }
     __syncthreads();
+    const int buf = kb & 1;
 #pragma unroll
-    for (int k = 0; k < kGemmBK; ++k) {
-      const float4 a = *reinterpret_cast<const float4 *>(&As[k][ty * 4]);
-      const float4 w = *reinterpret_cast<const float4 *>(&Ws[k][tx * 4]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, wv[4] = {w.x, w.y, w.z, w.w};
+    for (int k = 0; k < kGemmBK; k += 4) {
+      float4 av[TM];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4 *>(&As[buf][ty * TM + i][k]);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], wv[j], acc[i][j]);
+      for (int u = 0; u < 4; ++u) {
+        float w[TM];
+#pragma unroll
+        for (int j = 0; j < TM; ++j) w[j] = Ws[buf][k + u][tx * TM + j];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const float x = u == 0 ? av[i].x : u == 1 ? av[i].y : u == 2 ? av[i].z : av[i].w;
+#pragma unroll
+          for (int j = 0; j < TM; ++j) acc[i][j] = fmaf(x, w[j], acc[i][j]);
+        }
+      }
     }
-    __syncthreads();
+    __syncthreads();                             // the buffer may be refilled
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int row = m0 + ty * 4 + i;
-    if (row < M)
-      *reinterpret_cast<float4 *>(C + (size_t)row * 3 * GD + n0 + tx * 4) =
-          make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  for (int i = 0; i < TM; ++i) {
+    const int row = m0 + ty * TM + i;
+    if (row < M) {
+#pragma unroll
+      for (int j = 0; j < TM; ++j) C[(size_t)row * 3 * GD + n0 + tx * TM + j] = acc[i][j];
+    }
   }
 }
 
-// s = [H'_1 .. H'_h'] Wo_g and the threshold of Eq. 4.  One CTA = 16 tokens, one
-// warp = 4 of them, lane = head (in rounds of 32 heads).  The 16 rows of H and a
+// s = [H'_1 .. H'_h'] Wo_g and the threshold of Eq. 4.  One CTA = kTokens tokens, one
+// warp = kTokens / 4 of them, lane = head (in rounds of 32 heads).  The rows of H and a
 // [GD][32] slice of Wo are staged in shared memory: per step of the reduction a
-// warp reads one conflict-free row of Wo and four broadcast values of H.
-constexpr int kOutTokens = 16, kOutThreads = 128;
-template <typename T>
+// warp reads one conflict-free row of Wo and a broadcast value of H per token.  4 tokens where 16 would leave
+// most SMs without a CTA.
+constexpr int kOutThreads = 128;
+template <typename T, int kOutTokens>
 __global__ void __launch_bounds__(kOutThreads)
-gate_out_kernel(const float *__restrict__ H, const T *__restrict__ Wo,
+gate_out_kernel(const float *H, const T *__restrict__ Wo,
                 const float *__restrict__ gamma, float logit_tau, int B, int n, int GD, int h,
                 const int32_t *__restrict__ seq_lens, float *__restrict__ scores, uint8_t *__restrict__ flags) {
+  constexpr int kPer = kOutTokens / 4;           // tokens per warp
   extern __shared__ __align__(16) unsigned char sh_raw[];
   float *Hs = reinterpret_cast<float *>(sh_raw);                       // [16][GD]
   T *Ws = reinterpret_cast<T *>(sh_raw + sizeof(float) * kOutTokens * GD);   // [GD][32]
@@ -91,6 +124,8 @@ gate_out_kernel(const float *__restrict__ H, const T *__restrict__ Wo,
   const int b = blockIdx.x / tiles_per_seq, t0 = (blockIdx.x % tiles_per_seq) * kOutTokens;
   const int nt = min(kOutTokens, n - t0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
+  pdl_launch_dependents();
   const float *Hg = H + ((size_t)b * n + t0) * GD;                     // rows are contiguous
   for (int x = threadIdx.x; x < kOutTokens * GD; x += kOutThreads) Hs[x] = x < nt * GD ? Hg[x] : 0.f;
   for (int i0 = 0; i0 < h; i0 += 32) {
@@ -100,20 +135,22 @@ gate_out_kernel(const float *__restrict__ H, const T *__restrict__ Wo,
       Ws[x] = i < h ? Wo[(size_t)c * h + i] : T(0.f);
     }
     __syncthreads();
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    const float *hr = Hs + warp * 4 * GD;
+    float acc[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) acc[q] = 0.f;
+    const float *hr = Hs + warp * kPer * GD;
 #pragma unroll 8
     for (int c = 0; c < GD; ++c) {
       const float w = Elem<T>::load(Ws + c * 32 + lane);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fmaf(hr[q * GD + c], w, acc[q]);
+      for (int q = 0; q < kPer; ++q) acc[q] = fmaf(hr[q * GD + c], w, acc[q]);
     }
     const int i = i0 + lane;
     if (i < h) {
       const float gm = gamma ? gamma[i] : 0.f;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int tt = warp * 4 + q;
+      for (int q = 0; q < kPer; ++q) {
+        const int tt = warp * kPer + q;
         if (tt < nt) {
           const size_t o = ((size_t)b * h + i) * n + t0 + tt;
           const bool padding = seq_lens && t0 + tt >= seq_lens[b];
@@ -157,10 +194,12 @@ static int run_gate(const ag_layer_desc &d, const void *X, const void *Wq, const
       int rc = launch_gate_proj_tc(X, Wq, Wk, Wv, qkv, nullptr, nullptr, M, d.hidden, GD, st);
       if (rc) return rc;
     } else {
-      dim3 grid(3 * GD / kGemmBN, (M + kGemmBM - 1) / kGemmBM);
-      gate_proj_kernel<T><<<grid, 256, 0, st>>>(static_cast<const T *>(X), static_cast<const T *>(Wq),
-                                                static_cast<const T *>(Wk), static_cast<const T *>(Wv),
-                                                qkv, M, d.hidden, GD);
+      auto p = [](const void *x) { return static_cast<const T *>(x); };
+      // 64 x 64 outputs per CTA, or 32 x 32 where that leaves SMs without a CTA
+      if ((long long)(3 * GD / 64) * ((M + 63) / 64) >= 148)
+        gate_proj_kernel<T, 64><<<dim3(3 * GD / 64, (M + 63) / 64), 256, 0, st>>>(p(X), p(Wq), p(Wk), p(Wv), qkv, M, d.hidden, GD);
+      else
+        gate_proj_kernel<T, 32><<<dim3(3 * GD / 32, (M + 31) / 32), 256, 0, st>>>(p(X), p(Wq), p(Wk), p(Wv), qkv, M, d.hidden, GD);
       AG_LAUNCH_CHECK();
     }
     SimtAttnArgs a{};
@@ -183,14 +222,13 @@ static int run_gate(const ag_layer_desc &d, const void *X, const void *Wq, const
     if (rc) return rc;
   }
 
-  const size_t out_smem = sizeof(float) * (size_t)kOutTokens * GD + sizeof(T) * (size_t)GD * 32;
-  auto out_kern = gate_out_kernel<T>;
+  const int tokens = d.batch * d.seq <= 16 * 148 ? 4 : 16;
+  const size_t out_smem = sizeof(float) * (size_t)tokens * GD + sizeof(T) * (size_t)GD * 32;
+  auto out_kern = tokens == 4 ? gate_out_kernel<T, 4> : gate_out_kernel<T, 16>;
   AG_CUDA_TRY(cudaFuncSetAttribute(out_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out_smem));
-  const int blocks = d.batch * ((d.seq + kOutTokens - 1) / kOutTokens);
-  out_kern<<<blocks, kOutThreads, out_smem, st>>>(hcat, static_cast<const T *>(Wo), gamma, logit_tau,
-                                                 d.batch, d.seq, GD, kv_heads_of(d), d.seq_lens, scores, flags);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  const int blocks = d.batch * ((d.seq + tokens - 1) / tokens);
+  return launch_pdl(out_kern, dim3(blocks), dim3(kOutThreads), out_smem, st, hcat, static_cast<const T *>(Wo), gamma,
+                    logit_tau, d.batch, d.seq, GD, kv_heads_of(d), d.seq_lens, scores, flags);
 }
 
 int launch_gate(const ag_layer_desc &d, const void *X, const void *Wq, const void *Wk,
