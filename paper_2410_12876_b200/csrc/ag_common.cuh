@@ -80,15 +80,19 @@ int launch_gate(const ag_layer_desc &d, const void *X, const void *Wq, const voi
                 uint8_t *flags, void *ws, cudaStream_t st);
 
 // Tensor-core (tcgen05) projection GEMM for bf16 inputs: [M, 3*GD] = X [W0 | W1 | W2], written
-// either as float32 (C) or, when Chi / Clo are given, as the bf16 pair hi + lo of each float32 value.
+// as float32 (parts = 0) or as the sum of 2 or 3 bf16 parts of each float32 value: out holds that many
+// planes [M, 3*GD], the largest part first (two parts: 2^-17 of the value is lost; three: nothing).
+// seq_lens (or NULL): M = batch * n rows; tiles of which no row lies in the first align_up(seq_lens[b], 128)
+// tokens of its sequence are left out.
 bool gate_proj_tc_supported(int K, int GD);
-int launch_gate_proj_tc(const void *X, const void *W0, const void *W1, const void *W2, float *C, void *Chi,
-                        void *Clo, int M, int K, int GD, cudaStream_t st);
-// Tensor-core MHA' (Sec. 3.3) on the hi / lo pairs, then the split-K merge fused with the gate's
+int launch_gate_proj_tc(const void *X, const void *W0, const void *W1, const void *W2, void *out, int parts,
+                        int M, int K, int GD, const int32_t *seq_lens, int n, cudaStream_t st);
+// Tensor-core MHA' (Sec. 3.3) on the bf16 parts, then the split-K merge fused with the gate's
 // output layer and threshold (Eq. 3, Eq. 4): scores (optional) and flags [B, h, n].
 bool gate_attn_tc_supported(const ag_layer_desc &d);
 size_t gate_attn_partial_bytes(const ag_layer_desc &d);   // split-K partials (workspace)
-int launch_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const void *qkv_lo, void *partials,
+int gate_attn_parts(const ag_layer_desc &d);              // bf16 parts per float32 value it takes
+int launch_gate_attn_tc(const ag_layer_desc &d, const void *qkv, void *partials,
                         const void *Wo, const float *gamma, float logit_tau, float *scores, uint8_t *flags,
                         cudaStream_t st);
 int gate_attn_tc_wait_timeouts();
@@ -207,6 +211,16 @@ __device__ __forceinline__ void ring_put(const RecentRing &rg, int slab, int vec
     rg.live[(size_t)slab * rg.R + slot] = kept ? 0 : 1;
     rg.pos[slab] = p + 1;
   }
+}
+
+// Rows [m0, m1) of a batch of sequences of n tokens each, flattened: whether none of them is among the first
+// align_up(seq_lens[b], align) tokens of its sequence.  (The lengths are read behind the wait for the kernel before.)
+__device__ __forceinline__ bool padding_rows(const int32_t *seq_lens, int n, int m0, int m1, int align) {
+  if (seq_lens == nullptr) return false;
+  pdl_wait();
+  for (int b = m0 / n; b * n < m1; ++b)
+    if (max(m0 - b * n, 0) < (seq_lens[b] + align - 1) / align * align) return false;
+  return true;
 }
 
 __device__ __forceinline__ uint4 ldg128(const void *p) {

@@ -164,11 +164,11 @@ gate_out_kernel(const float *H, const T *__restrict__ Wo,
 
 size_t gate_workspace_bytes(const ag_layer_desc &d) {
   const size_t rows = (size_t)d.batch * d.seq, GD = (size_t)d.gate_heads * d.gate_head_dim;
-  // [Q' | K' | V'] (float32, or the bf16 hi and lo halves), then H' (CUDA-core path) or the split-K
+  // [Q' | K' | V'] (float32, or its bf16 parts), then H' (CUDA-core path) or the split-K
   // partials of MHA' (tensor-core path, where H' stays on chip)
-  const size_t qkv = align_up(rows * 3 * GD * sizeof(float), 256);
-  if (d.dtype == AG_BF16 && gate_attn_tc_supported(d)) return qkv + gate_attn_partial_bytes(d);
-  return qkv + align_up(rows * GD * sizeof(float), 256);
+  if (d.dtype == AG_BF16 && gate_attn_tc_supported(d))
+    return align_up(rows * 3 * GD * 2 * gate_attn_parts(d), 256) + gate_attn_partial_bytes(d);
+  return align_up(rows * 3 * GD * sizeof(float), 256) + align_up(rows * GD * sizeof(float), 256);
 }
 
 template <typename T>
@@ -181,17 +181,18 @@ static int run_gate(const ag_layer_desc &d, const void *X, const void *Wq, const
                                           align_up((size_t)M * 3 * GD * sizeof(float), 256));
   const float logit_tau = (float)log((double)d.tau / (1.0 - (double)d.tau));
   if (sizeof(T) == 2 && gate_attn_tc_supported(d)) {
-    // tensor-core path: projections as bf16 hi/lo pairs, MHA' on tcgen05 with three products per term
-    void *hi = ws;
-    void *lo = static_cast<char *>(ws) + (size_t)M * 3 * GD * sizeof(__nv_bfloat16);
-    int rc = launch_gate_proj_tc(X, Wq, Wk, Wv, nullptr, hi, lo, M, d.hidden, GD, st);
+    // tensor-core path: projections as bf16 parts, MHA' on tcgen05 with a product per pair of parts that matters.
+    // Padding is projected only as far as MHA' reads it: the causal one stops at the query tile (128 tokens)
+    // that holds a sequence's end, the bidirectional one visits every key tile.
+    const int parts = gate_attn_parts(d);
+    int rc = launch_gate_proj_tc(X, Wq, Wk, Wv, ws, parts, M, d.hidden, GD, d.gate_causal ? d.seq_lens : nullptr, d.seq, st);
     if (rc) return rc;
-    void *partials = hcat;                           // H' stays on chip: the partials take its place
+    void *partials = static_cast<char *>(ws) + align_up((size_t)M * 3 * GD * 2 * parts, 256);   // H' stays on chip
     // the merge of the split-K partials carries the output layer and the threshold with it
-    return launch_gate_attn_tc(d, hi, lo, partials, Wo, gamma, logit_tau, scores, flags, st);
+    return launch_gate_attn_tc(d, ws, partials, Wo, gamma, logit_tau, scores, flags, st);
   } else {
     if (sizeof(T) == 2 && gate_proj_tc_supported(d.hidden, GD)) {
-      int rc = launch_gate_proj_tc(X, Wq, Wk, Wv, qkv, nullptr, nullptr, M, d.hidden, GD, st);
+      int rc = launch_gate_proj_tc(X, Wq, Wk, Wv, qkv, 0, M, d.hidden, GD, nullptr, d.seq, st);
       if (rc) return rc;
     } else {
       auto p = [](const void *x) { return static_cast<const T *>(x); };

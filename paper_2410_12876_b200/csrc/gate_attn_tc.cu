@@ -5,7 +5,8 @@
 // V' or of the attention weights would flip flags.  Every float32 operand x is
 // therefore carried as a bf16 pair x = hi + lo (|x - hi - lo| <= 2^-17 |x|) and
 // each product A B is evaluated as  Ahi Bhi + Ahi Blo + Alo Bhi  in the float32
-// accumulator (the dropped lo*lo term is 2^-16 relative).
+// accumulator (the dropped lo*lo term is 2^-16 relative).  Gate heads of 64 take three parts (their sum is exactly
+// x) and the six products down to 2^-16: with half the columns that costs about what two parts cost at 128.
 //
 // Structure as in the prefill kernel: warp 0 TMA, warp 1 tcgen05.mma issue,
 // warps 2..5 softmax with one row per thread.  A query tile is 128 queries of
@@ -21,7 +22,7 @@
 // (O, m, l); gate_merge_out_kernel combines the pieces of a query tile and
 // applies the gate's output layer and threshold.
 //
-// TMEM columns: S0 [0,64) S1 [128,192) O [256,384) Phi [384,448) Plo [448,512), each P half holding two
+// TMEM columns: S0 [0,64) S1 [128,192) O [256,256 + D) then 64 columns per part of P, each holding two
 // tiles' weights (32 columns per tile).
 #include "ag_common.cuh"
 #include "mma_sync.cuh"
@@ -39,15 +40,22 @@ constexpr int kGaKvPanel = kGaBN * 128;              // K / V: [64 rows][64 bf16
 template <int D>
 struct GaCfg {
   static constexpr int kPanels = D / 64;
-  static constexpr int kTile = kPanels * kGaPanel;        // Q hi or Q lo
-  static constexpr int kKvTile = kPanels * kGaKvPanel;    // K or V, one of hi / lo
-  static constexpr int kKvStage = 2 * kKvTile;            // hi + lo
-  static constexpr int kUsedBytes = 2 * kTile + 4 * kKvStage + 1024 + 256;   // Q + 2 K stages + 2 V stages
+  static constexpr int kParts = D == 64 ? 3 : 2;          // bf16 parts per float32 value
+  static constexpr int kProducts = kParts == 3 ? 6 : 3;   // products of parts (i, j), i + j < kParts
+  static constexpr int kTile = kPanels * kGaPanel;        // one part of Q
+  static constexpr int kKvTile = kPanels * kGaKvPanel;    // one part of K or V
+  static constexpr int kKvStage = kParts * kKvTile;
+  static constexpr int kUsedBytes = kParts * kTile + 4 * kKvStage + 1024 + 256;   // Q + 2 K stages + 2 V stages
+  static constexpr uint32_t kColO = 256, kColP = kColO + D;
+  static_assert(kColP + 64 * kParts <= 512, "tensor memory");
+  // parts of the first and of the second operand of product t
+  __host__ __device__ static constexpr int first(int t) { return t == 0 || t == 1 || t == 3 ? 0 : (t == 2 || t == 5 ? 1 : 2); }
+  __host__ __device__ static constexpr int second(int t) { return t == 0 || t == 2 || t == 4 ? 0 : (t == 1 || t == 5 ? 1 : 2); }
   // one CTA per SM whatever D (each takes all of tensor memory: a second one on the SM would wait for the first
   // to end while other SMs stand idle)
   static constexpr int kSmemBytes = kUsedBytes > 120 * 1024 ? kUsedBytes : 120 * 1024;
 };
-constexpr uint32_t kGaColS = 0, kGaColO = 256, kGaColPhi = 384, kGaColPlo = 448, kGaTmemCols = 512;
+constexpr uint32_t kGaColS = 0, kGaTmemCols = 512;
 constexpr float kGaRescaleThreshold = 8.f;
 
 constexpr int kGaMaxSeg = 256;       // segments at most (one per SM)
@@ -67,6 +75,9 @@ struct GateAttnArgs {
   int seg_begin[kGaMaxSeg + 1];
   float scale_log2;
 };
+
+// One map per part (all 3 encoded): boxes of a query tile's rows and of a key tile's.
+struct GateAttnMaps { CUtensorMap q[3], kv[3]; };
 
 // Key tiles query tile qt attends to, and the work items they are cut into.
 // (key tiles hold 64 keys, query tiles 128 queries)
@@ -120,15 +131,13 @@ __host__ __device__ inline int ga_slot(int prob, int qt, int n_qtiles, int seg) 
 
 template <int kGaD>
 __global__ void __launch_bounds__(kGaThreads, 1)
-gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__ CUtensorMap tmLo,
-                    const __grid_constant__ CUtensorMap tmHiKv, const __grid_constant__ CUtensorMap tmLoKv,
-                    const __grid_constant__ GateAttnArgs a) {
+gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_constant__ GateAttnArgs a) {
   using C = GaCfg<kGaD>;
   constexpr int kGaTile = C::kTile, kGaKvTile = C::kKvTile, kGaKvStage = C::kKvStage;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t *sQ = smem;                    // [hi | lo]
-  uint8_t *sK = sQ + 2 * kGaTile;        // [stage][hi | lo]
+  uint8_t *sQ = smem;                    // [part]
+  uint8_t *sK = sQ + C::kParts * kGaTile;      // [stage][part]
   uint8_t *sV = sK + 2 * kGaKvStage;
   uint64_t *bars = reinterpret_cast<uint64_t *>(sV + 2 * kGaKvStage);
   uint64_t *q_full = bars, *k_full = bars + 1, *k_empty = bars + 3, *v_full = bars + 5, *v_empty = bars + 7;  // [2]
@@ -159,8 +168,8 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
     mbar_init(q_empty, 1);
     mbar_init(o_free, 128);
     fence_barrier_init();
-    prefetch_tensormap(&tmHi); prefetch_tensormap(&tmLo);
-    prefetch_tensormap(&tmHiKv); prefetch_tensormap(&tmLoKv);
+#pragma unroll
+    for (int i = 0; i < C::kParts; ++i) { prefetch_tensormap(&tm.q[i]); prefetch_tensormap(&tm.kv[i]); }
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, kGaTmemCols);
@@ -184,19 +193,19 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
         const int xq = g * kGaD, xk = a.GD + g * kGaD, xv = 2 * a.GD + g * kGaD;   // columns in [Q' | K' | V']
         ok = mbar_wait(q_empty, (pc & 1) ^ 1);       // the previous piece's last Q K^T has read Q
         if (!ok) break;
-        mbar_arrive_expect_tx(q_full, 2 * kGaTile);
+        mbar_arrive_expect_tx(q_full, C::kParts * kGaTile);
 #pragma unroll
-        for (int p = 0; p < C::kPanels; ++p) {
-          tma_load_3d(sQ + p * kGaPanel, &tmHi, q_full, xq + p * 64, j0, b);
-          tma_load_3d(sQ + kGaTile + p * kGaPanel, &tmLo, q_full, xq + p * 64, j0, b);
-        }
+        for (int i = 0; i < C::kParts; ++i)
+#pragma unroll
+          for (int p = 0; p < C::kPanels; ++p)
+            tma_load_3d(sQ + i * kGaTile + p * kGaPanel, &tm.q[i], q_full, xq + p * 64, j0, b);
         auto load_kv = [&](uint8_t *dst, uint64_t *bar, int xc, int y) {
           mbar_arrive_expect_tx(bar, kGaKvStage);
 #pragma unroll
-          for (int p = 0; p < C::kPanels; ++p) {
-            tma_load_3d(dst + p * kGaKvPanel, &tmHiKv, bar, xc + p * 64, y, b);
-            tma_load_3d(dst + kGaKvTile + p * kGaKvPanel, &tmLoKv, bar, xc + p * 64, y, b);
-          }
+          for (int i = 0; i < C::kParts; ++i)
+#pragma unroll
+            for (int p = 0; p < C::kPanels; ++p)
+              tma_load_3d(dst + i * kGaKvTile + p * kGaKvPanel, &tm.kv[i], bar, xc + p * 64, y, b);
         };
         for (int i = 0; i < pz.n_kv; ++i, ++t) {
           const int st = t & 1;
@@ -226,10 +235,9 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
       const uint32_t d = tmem + kGaColS + st * 128;
       const uint32_t kb = k_lo + ((st * kGaKvStage) >> 4);
       if (elect_one()) {
-        // Qhi Khi + Qhi Klo + Qlo Khi
 #pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          const uint32_t qa = q_lo + ((t == 2 ? kGaTile : 0) >> 4), ka = kb + ((t == 1 ? kGaKvTile : 0) >> 4);
+        for (int t = 0; t < C::kProducts; ++t) {
+          const uint32_t qa = q_lo + ((C::first(t) * kGaTile) >> 4), ka = kb + ((C::second(t) * kGaKvTile) >> 4);
 #pragma unroll
           for (int k = 0; k < kGaD / 16; ++k)
             mma_ss_lohi(d, qa + (((k >> 2) * kGaPanel + (k & 3) * 32) >> 4), q_hi,
@@ -262,13 +270,13 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
       tc_fence_after_sync();
       const uint32_t vb = v_lo + ((st * kGaKvStage) >> 4);
       if (elect_one()) {
-        // Phi Vhi + Phi Vlo + Plo Vhi
 #pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          const uint32_t pa = tmem + (t == 2 ? kGaColPlo : kGaColPhi) + st * (kGaBN / 2), va = vb + ((t == 1 ? kGaKvTile : 0) >> 4);
+        for (int t = 0; t < C::kProducts; ++t) {
+          const uint32_t pa = tmem + C::kColP + C::first(t) * 64 + st * (kGaBN / 2);
+          const uint32_t va = vb + ((C::second(t) * kGaKvTile) >> 4);
 #pragma unroll
           for (int k = 0; k < kGaBN / 16; ++k)
-            mma_ts_lohi(tmem + kGaColO, pa + k * 8, va + ((k * 2048) >> 4), v_hi, idesc_pv, (i | t | k) != 0);
+            mma_ts_lohi(tmem + C::kColO, pa + k * 8, va + ((k * 2048) >> 4), v_hi, idesc_pv, (i | t | k) != 0);
         }
         mma_commit(&v_empty[st]);
         mma_commit(&pv_done[st]);
@@ -355,10 +363,10 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
 #pragma unroll 1
         for (int c = 0; c < kGaD / 32; ++c) {
           uint32_t r[32];
-          tmem_ld_x32_sync(tm_lane + kGaColO + c * 32, r);
+          tmem_ld_x32_sync(tm_lane + C::kColO + c * 32, r);
 #pragma unroll
           for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
-          tmem_st_x32(tm_lane + kGaColO + c * 32, r);
+          tmem_st_x32(tm_lane + C::kColO + c * 32, r);
         }
       }
       // this tile's P buffer was last read by the P V of tile t - 2
@@ -371,20 +379,23 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
       float rs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int c = 0; c < kGaBN / 16; ++c) {
-        uint32_t ph[8], pl[8];
+        uint32_t pk[C::kParts][8];
 #pragma unroll
         for (int e = 0; e < 16; e += 2) {
-          const float p0 = fast_exp2(fmaf(__uint_as_float(r[c * 16 + e]), a.scale_log2, -m_exp));
-          const float p1 = fast_exp2(fmaf(__uint_as_float(r[c * 16 + e + 1]), a.scale_log2, -m_exp));
+          float p0 = fast_exp2(fmaf(__uint_as_float(r[c * 16 + e]), a.scale_log2, -m_exp));
+          float p1 = fast_exp2(fmaf(__uint_as_float(r[c * 16 + e + 1]), a.scale_log2, -m_exp));
           rs[(e >> 1) & 3] += p0 + p1;
-          float h0, l0, h1, l1;
-          split_bf16(p0, h0, l0);
-          split_bf16(p1, h1, l1);
-          ph[e >> 1] = pack_bf16x2(h0, h1);
-          pl[e >> 1] = pack_bf16x2(l0, l1);
+#pragma unroll
+          for (int i = 0; i < C::kParts; ++i) {
+            float h0, h1;
+            split_bf16(p0, h0, p0);
+            split_bf16(p1, h1, p1);
+            pk[i][e >> 1] = pack_bf16x2(h0, h1);
+          }
         }
-        tmem_st_x8(tm_lane + kGaColPhi + (t & 1) * (kGaBN / 2) + c * 8, ph);
-        tmem_st_x8(tm_lane + kGaColPlo + (t & 1) * (kGaBN / 2) + c * 8, pl);
+#pragma unroll
+        for (int i = 0; i < C::kParts; ++i)
+          tmem_st_x8(tm_lane + C::kColP + i * 64 + (t & 1) * (kGaBN / 2) + c * 8, pk[i]);
       }
       const float rowsum = (rs[0] + rs[1]) + (rs[2] + rs[3]);
       l += rowsum;
@@ -404,7 +415,7 @@ gate_attn_tc_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_const
 #pragma unroll 1
       for (int c = 0; c < kGaD / 32; ++c) {
         uint32_t r[32];
-        tmem_ld_x32_sync(tm_lane + kGaColO + c * 32, r);
+        tmem_ld_x32_sync(tm_lane + C::kColO + c * 32, r);
         if (c + 1 == kGaD / 32) {                                // O is in registers: the next piece may overwrite it
           tc_fence_before_sync();
           mbar_arrive(o_free);
@@ -488,6 +499,14 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
   stage_wo(0);
   pdl_wait();
   pdl_launch_dependents();
+  if (a.seq_lens != nullptr && t0 >= a.seq_lens[b]) {
+    // padding only: flags 0, scores left as they are
+    cp_async_wait<0>();
+    const int tok = threadIdx.x & 15;
+    for (int i = threadIdx.x >> 4; i < h; i += kMoThreads / kMoTokens)
+      if (t0 + tok < a.n) flags[((size_t)b * h + i) * a.n + t0 + tok] = 0;
+    return;
+  }
   // The CTA's 16 tokens lie in one query tile: which segments hold its pieces is looked up once per
   // gate head (a binary search over the boundaries in constant memory), by one thread each.
   {
@@ -695,19 +714,19 @@ size_t gate_attn_partial_bytes(const ag_layer_desc &d) {
 }
 
 template <int kGaD>
-static int run_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const void *qkv_lo, void *partials,
+static int run_gate_attn_tc(const ag_layer_desc &d, const void *qkv, void *partials,
                             const void *Wo, const float *gamma, float logit_tau, float *scores, uint8_t *flags,
                             cudaStream_t st) {
   constexpr int kGaSmemBytes = GaCfg<kGaD>::kSmemBytes;
   const int GD = d.gate_heads * d.gate_head_dim;
-  CUtensorMap tmHi, tmLo;
-  int rc = make_tmap_3d_bf16(&tmHi, qkv_hi, d.batch, d.seq, 3 * GD, kGaBM, 64);
-  if (rc) return rc;
-  rc = make_tmap_3d_bf16(&tmLo, qkv_lo, d.batch, d.seq, 3 * GD, kGaBM, 64);
-  if (rc) return rc;
-  CUtensorMap tmHiKv, tmLoKv;
-  if ((rc = make_tmap_3d_bf16(&tmHiKv, qkv_hi, d.batch, d.seq, 3 * GD, kGaBN, 64))) return rc;
-  if ((rc = make_tmap_3d_bf16(&tmLoKv, qkv_lo, d.batch, d.seq, 3 * GD, kGaBN, 64))) return rc;
+  GateAttnMaps tm;
+  int rc;
+  const size_t plane = (size_t)d.batch * d.seq * 3 * GD;
+  for (int i = 0; i < 3; ++i) {
+    const void *part = static_cast<const __nv_bfloat16 *>(qkv) + (i < GaCfg<kGaD>::kParts ? i : 0) * plane;
+    if ((rc = make_tmap_3d_bf16(&tm.q[i], part, d.batch, d.seq, 3 * GD, kGaBM, 64))) return rc;
+    if ((rc = make_tmap_3d_bf16(&tm.kv[i], part, d.batch, d.seq, 3 * GD, kGaBN, 64))) return rc;
+  }
   GateAttnArgs a;
   a.seq_lens = d.seq_lens;
   a.n = d.seq; a.n_qtiles = (d.seq + kGaBM - 1) / kGaBM;
@@ -722,8 +741,7 @@ static int run_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const vo
                                         align_up(slots * kGaBM * kGaD * sizeof(float), 256));
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)kGaD));
   AG_CUDA_TRY(cudaFuncSetAttribute(gate_attn_tc_kernel<kGaD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGaSmemBytes));
-  rc = launch_pdl(gate_attn_tc_kernel<kGaD>, dim3(plan.n_seg), dim3(kGaThreads), kGaSmemBytes, st, tmHi, tmLo, tmHiKv,
-                  tmLoKv, a);
+  rc = launch_pdl(gate_attn_tc_kernel<kGaD>, dim3(plan.n_seg), dim3(kGaThreads), kGaSmemBytes, st, tm, a);
   if (rc) return rc;
   auto mo = gate_merge_out_kernel<kGaD>;
   AG_CUDA_TRY(cudaFuncSetAttribute(mo, cudaFuncAttributeMaxDynamicSharedMemorySize, mo_smem_bytes(GD)));
@@ -732,11 +750,13 @@ static int run_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const vo
                     gamma, logit_tau, kv_heads_of(d), scores, flags);
 }
 
-int launch_gate_attn_tc(const ag_layer_desc &d, const void *qkv_hi, const void *qkv_lo, void *partials,
+int gate_attn_parts(const ag_layer_desc &d) { return d.gate_head_dim == 64 ? GaCfg<64>::kParts : GaCfg<128>::kParts; }
+
+int launch_gate_attn_tc(const ag_layer_desc &d, const void *qkv, void *partials,
                         const void *Wo, const float *gamma, float logit_tau, float *scores, uint8_t *flags,
                         cudaStream_t st) {
-  return d.gate_head_dim == 64 ? run_gate_attn_tc<64>(d, qkv_hi, qkv_lo, partials, Wo, gamma, logit_tau, scores, flags, st)
-                               : run_gate_attn_tc<128>(d, qkv_hi, qkv_lo, partials, Wo, gamma, logit_tau, scores, flags, st);
+  return d.gate_head_dim == 64 ? run_gate_attn_tc<64>(d, qkv, partials, Wo, gamma, logit_tau, scores, flags, st)
+                               : run_gate_attn_tc<128>(d, qkv, partials, Wo, gamma, logit_tau, scores, flags, st);
 }
 
 int gate_attn_tc_wait_timeouts() {

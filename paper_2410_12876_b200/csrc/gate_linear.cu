@@ -60,7 +60,8 @@ gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * kGlBM;
   const int kb_begin = rank * a.kb_per_cta;
-  const int num_kb = max(0, min(a.kb_total, kb_begin + a.kb_per_cta) - kb_begin);
+  // a tile that holds padding only: no scores to compute, flags 0
+  const int num_kb = padding_rows(a.seq_lens, a.n, m0, min(m0 + kGlBM, a.M), 1) ? 0 : max(0, min(a.kb_total, kb_begin + a.kb_per_cta) - kb_begin);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kGlStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -77,6 +78,8 @@ gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -225,11 +228,12 @@ static int run_gate_linear_tc(const ag_layer_desc &d, const void *X, const void 
   cfg.blockDim = dim3(kGlThreads);
   cfg.dynamicSmemBytes = kGlSmemBytes;
   cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = split; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1] = pdl_attribute();
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tmX, tmW, a));
   return AG_OK;
 }

@@ -8,7 +8,7 @@
 // r adds up rows [r 128 / S, (r + 1) 128 / S) of the tile through distributed shared memory
 // and hands them to the projection's epilogue, a warp per row.
 //
-// P (the projection) supplies: args; load_a / load_b (the TMA boxes of a k-block); prepare (work of the
+// P (the projection) supplies: args; skip (a tile nobody wants); load_a / load_b (the TMA boxes of a k-block); prepare (work of the
 // epilogue warps while the MMAs run); load_row (what the row's epilogue reads from memory, asked for together
 // with the sums) and row (one finished row of BN columns: lane l has columns 4 l .. 4 l + 3 of every group of 128).
 #pragma once
@@ -59,6 +59,7 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
   const int rank = (int)cluster_ctarank(), tile = blockIdx.x / splits;
   const int kb_begin = rank * num_kb / splits, kb_end = (rank + 1) * num_kb / splits;    // never empty: splits <= num_kb
 
+  if (p.skip(tile)) return;                          // the whole cluster
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     mbar_init(acc_full, 1);
@@ -74,7 +75,8 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
-  pdl_launch_dependents();                           // a kernel that waits for this grid may set itself up
+  pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -202,8 +204,9 @@ cudaLaunchConfig_t splitk_config(int ctas, int splits, cudaStream_t st, cudaLaun
   cfg.stream = st;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = splits; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1] = pdl_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cfg;
 }
 
@@ -232,7 +235,7 @@ int splitk_capacity(const int **out) {
     for (int s = 2; s <= kMaxSplit; ++s) {
       auto kern = kernel_of<BN, P>(s);
       AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmemBytes));
-      cudaLaunchAttribute attr[1];
+      cudaLaunchAttribute attr[2];
       cudaLaunchConfig_t cfg = splitk_config<BN, P>(s, s, nullptr, attr);
       int n = 0;
       AG_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, kern, &cfg));
@@ -248,7 +251,7 @@ template <int BN, class P>
 int launch_splitk(const P &p, long long tiles, int num_kb, int splits, cudaStream_t st) {
   auto kern = kernel_of<BN, P>(splits);
   AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmemBytes));
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = splitk_config<BN, P>((int)(tiles * splits), splits, st, attr);
   AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, p, num_kb));
   return AG_OK;

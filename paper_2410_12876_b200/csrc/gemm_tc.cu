@@ -33,12 +33,40 @@ template <int BN, int MT> struct GemmTcCfg {
   static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*align*/ + 256 /*barriers*/;
 };
 
+// Stages the third bf16 part of columns [c_begin, c_end) of one accumulator row per thread (row r_in = 32 quad +
+// lane), in the layout of a swizzled TMA store.
+__device__ __forceinline__ void stage_third(uint8_t *smem, uint32_t tmem, int quad, int r_in, int c_begin, int c_end) {
+#pragma unroll 1
+  for (int c = c_begin; c < c_end; c += 32) {
+    uint32_t r[32];
+    tmem_ld_x32_sync(tmem + ((uint32_t)(quad * 32) << 16) + c, r);
+    const uint32_t panel = (uint32_t)(c >> 6) * kTcBM * 128 + r_in * 128;
+#pragma unroll
+    for (int e = 0; e < 32; e += 8) {
+      uint32_t t[4];
+#pragma unroll
+      for (int q = 0; q < 8; q += 2) {
+        float part, x0 = __uint_as_float(r[e + q]), x1 = __uint_as_float(r[e + q + 1]);
+        split_bf16(x0, part, x0);
+        split_bf16(x0, part, x0);
+        split_bf16(x1, part, x1);
+        split_bf16(x1, part, x1);
+        t[q >> 1] = pack_bf16x2(x0, x1);
+      }
+      const uint32_t chunk = (uint32_t)(((c & 32) >> 3) + (e >> 3));
+      *reinterpret_cast<uint4 *>(smem + panel + ((chunk ^ (r_in & 7)) << 4)) = make_uint4(t[0], t[1], t[2], t[3]);
+    }
+  }
+  fence_proxy_async_smem();
+}
+
 template <int BN, int MT>
 __global__ void __launch_bounds__(kTcThreads, 1)
 gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                     const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
                     const __grid_constant__ CUtensorMap tmChi, const __grid_constant__ CUtensorMap tmClo,
-                    float *__restrict__ C, bool split, int M, int K, int GD, int n_tiles_n, int halved_from) {
+                    const __grid_constant__ CUtensorMap tmC3, float *__restrict__ C, int parts, int M, int K, int GD,
+                    int n_tiles_n, int halved_from, const int32_t *seq_lens, int n) {
   using Cfg = GemmTcCfg<BN, MT>;
   constexpr uint32_t kTmemCols = MT * Cfg::kAccCols;
   static_assert(kTmemCols == 128 || kTmemCols == 256 || kTmemCols == 512, "TMEM columns: a power of two");
@@ -58,6 +86,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   const int bn = halved ? BN / 2 : BN;         // columns of this CTA (a multiple of 64)
   const int m0 = (tile / n_tiles_n) * (MT * kTcBM);
   const int n0 = (tile % n_tiles_n) * BN + (halved ? ((cta - halved_from) & 1) * (BN / 2) : 0);   // in the packed [3 * GD] output
+  if (padding_rows(seq_lens, n, m0, min(m0 + MT * kTcBM, M), kTcBM)) return;
   // a 64-column panel of B lies in one weight (64 divides GD); a tile may straddle two
   const int num_kb = (K + kTcBK - 1) / kTcBK;
 
@@ -77,7 +106,8 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
-  pdl_launch_dependents();                           // MHA' may set itself up (it waits for this grid's end)
+  pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -141,7 +171,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     for (int mt = 0; mt < MT; ++mt) {
     const int row = m0 + mt * kTcBM + quad * 32 + lane;
     const uint32_t tmem_sub = tmem_acc + mt * Cfg::kAccCols;
-    if (ok && num_kb > 0 && split) {
+    if (ok && num_kb > 0 && parts > 0) {
       // x = hi + lo in bf16 pairs, for consumers that rebuild float32 precision from three
       // products.  Every MMA has completed, so every stage has been read: the tile is staged
       // over them as panels of [128 rows][64 bf16] (128-byte rows, 16-byte chunks XOR-swizzled by
@@ -180,6 +210,16 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
         tma_store_commit();
         tma_store_wait_read();
+      }
+      if (parts == 3) {                                // what the first two parts leave, over the same staging area
+        named_barrier_sync(1, 256);
+        stage_third(smem, tmem_sub, quad, r_in, c_begin, c_end);
+        named_barrier_sync(1, 256);
+        if (threadIdx.x == 64) {
+          for (int p = 0; p < bn / 64; ++p) tma_store_2d(&tmC3, smem + p * kTcBM * 128, n0 + p * 64, m0 + mt * kTcBM);
+          tma_store_commit();
+          tma_store_wait_read();
+        }
       }
       if (MT > 1) named_barrier_sync(1, 256);          // the staging area is free for the next sub-tile
     } else if (ok && num_kb > 0) {
@@ -221,7 +261,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
 gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                       const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
                       const __grid_constant__ CUtensorMap tmChi, const __grid_constant__ CUtensorMap tmClo,
-                      float *__restrict__ C, bool split, int M, int K, int GD, int n_tiles_n) {
+                      const __grid_constant__ CUtensorMap tmC3, float *__restrict__ C, int parts, int M, int K, int GD,
+                      int n_tiles_n, const int32_t *seq_lens, int n) {
   constexpr uint32_t kTmemCols = 512;              // 384 used: columns [0, 256) of the wide MMA, [256, 384) of the narrow
   static_assert(2 * (kGpBN / 64) * kTcBM * 128 <= kGpStages * kGpStageBytes, "staging fits the stages");
   extern __shared__ uint8_t smem_raw[];
@@ -237,6 +278,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   const int tile = blockIdx.x >> 1;
   const int m0 = (tile / n_tiles_n) * (2 * kTcBM) + (int)rank * kTcBM;   // this CTA's rows
   const int n0 = (tile % n_tiles_n) * kGpBN;                              // in the packed [3 * GD] output
+  if (padding_rows(seq_lens, n, m0 - (int)rank * kTcBM, min(m0 + (2 - (int)rank) * kTcBM, M), kTcBM)) return;   // both CTAs
   const int num_kb = (K + kTcBK - 1) / kTcBK;
 
   if (threadIdx.x == 0) {
@@ -256,7 +298,8 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   cluster_arrive_wait();                           // both CTAs' barriers are initialised, tensor memory is allocated
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
-  pdl_launch_dependents();                           // MHA' may set itself up (it waits for this grid's end)
+  pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -318,7 +361,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     const bool ok = *gave_up == 0;
     tc_fence_after_sync();
     const int r_in = quad * 32 + lane, row = m0 + r_in;
-    if (ok && num_kb > 0 && split) {
+    if (ok && num_kb > 0 && parts > 0) {
       // x = hi + lo in bf16 pairs.  Every MMA of both CTAs has completed, so every stage has been read: the
       // tile is staged over them as panels of [128 rows][64 bf16] (128-byte rows, 16-byte chunks
       // XOR-swizzled by the row): six hi panels, then six lo panels.
@@ -354,6 +397,16 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         }
         tma_store_commit();
         tma_store_wait_read();
+      }
+      if (parts == 3) {
+        named_barrier_sync(1, 256);
+        stage_third(smem, tmem_acc, quad, r_in, c_begin, c_end);
+        named_barrier_sync(1, 256);
+        if (threadIdx.x == 64) {
+          for (int p = 0; p < kGpBN / 64; ++p) tma_store_2d(&tmC3, smem + p * kTcBM * 128, n0 + p * 64, m0);
+          tma_store_commit();
+          tma_store_wait_read();
+        }
       }
     } else if (ok && num_kb > 0) {
       const size_t crow = (size_t)row * 3 * GD + n0;
@@ -434,9 +487,29 @@ static int gemm_sm_count() {
   return sms;
 }
 
+// Where the projection goes, and which rows of it are wanted (see launch_gate_proj_tc).
+struct GemmOut {
+  void *out;
+  int parts;
+  const int32_t *seq_lens;
+  int n;
+  float *f32() const { return parts == 0 ? static_cast<float *>(out) : nullptr; }
+  __nv_bfloat16 *part(int i, size_t plane) const { return i < parts ? static_cast<__nv_bfloat16 *>(out) + i * plane : nullptr; }
+  // output maps of the bf16 parts (a weight stands in for those not asked for)
+  int maps(CUtensorMap *tmC, const void *stand_in, int M, int GD) const {
+    for (int i = 0; i < 3; ++i) {
+      const void *p = part(i, (size_t)M * 3 * GD);
+      const int rc = p ? make_tmap_2d_bf16(&tmC[i], p, M, 3 * (uint64_t)GD, 3 * (uint64_t)GD * 2, kTcBM, 64)
+                       : make_tmap_2d_bf16(&tmC[i], stand_in, 1, GD, (uint64_t)GD * 2, 1, 64);
+      if (rc) return rc;
+    }
+    return AG_OK;
+  }
+};
+
 template <int BN, int MT>
-static int run_gemm_tc(const void *X, const void *W0, const void *W1, const void *W2, float *C,
-                       __nv_bfloat16 *Chi, __nv_bfloat16 *Clo, int M, int K, int GD, cudaStream_t st) {
+static int run_gemm_tc(const void *X, const void *W0, const void *W1, const void *W2, const GemmOut &o, int M, int K,
+                       int GD, cudaStream_t st) {
   using Cfg = GemmTcCfg<BN, MT>;
   CUtensorMap tmA, tmB[3];
   int rc = make_tmap_2d_bf16(&tmA, X, M, K, (uint64_t)K * 2, kTcBM, kTcBK);
@@ -446,14 +519,8 @@ static int run_gemm_tc(const void *X, const void *W0, const void *W1, const void
     rc = make_tmap_2d_bf16(&tmB[i], Ws[i], K, GD, (uint64_t)GD * 2, kTcBK, 64);
     if (rc) return rc;
   }
-  // output maps of the hi / lo form (one row of a weight stands in when that form is not asked for)
-  CUtensorMap tmC[2];
-  const void *outs[2] = {Chi ? (const void *)Chi : W0, Clo ? (const void *)Clo : W0};
-  for (int i = 0; i < 2; ++i) {
-    rc = Chi ? make_tmap_2d_bf16(&tmC[i], outs[i], M, 3 * (uint64_t)GD, 3 * (uint64_t)GD * 2, kTcBM, 64)
-             : make_tmap_2d_bf16(&tmC[i], outs[i], 1, GD, (uint64_t)GD * 2, 1, 64);
-    if (rc) return rc;
-  }
+  CUtensorMap tmC[3];
+  if ((rc = o.maps(tmC, W0, M, GD))) return rc;
   auto kern = gemm_bf16_tc_kernel<BN, MT>;
   AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
   const int n_tiles_n = 3 * GD / BN, n_tiles = n_tiles_n * ((M + MT * kTcBM - 1) / (MT * kTcBM));
@@ -462,14 +529,12 @@ static int run_gemm_tc(const void *X, const void *W0, const void *W1, const void
   const int tail = n_tiles % sms;
   const int halved_from = (BN % 128 == 0 && tail > 0 && 2 * tail <= sms) ? n_tiles - tail : n_tiles;   // (any MT)
   const int ctas = halved_from + 2 * (n_tiles - halved_from);
-  kern<<<ctas, kTcThreads, Cfg::kSmemBytes, st>>>(tmA, tmB[0], tmB[1], tmB[2], tmC[0], tmC[1], C, Chi != nullptr, M, K,
-                                                  GD, n_tiles_n, halved_from);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  return launch_pdl(kern, dim3(ctas), dim3(kTcThreads), Cfg::kSmemBytes, st, tmA, tmB[0], tmB[1], tmB[2], tmC[0], tmC[1],
+                    tmC[2], o.f32(), o.parts, M, K, GD, n_tiles_n, halved_from, o.seq_lens, o.n);
 }
 
-static int run_gemm_pair(const void *X, const void *W0, const void *W1, const void *W2, float *C, __nv_bfloat16 *Chi,
-                         __nv_bfloat16 *Clo, int M, int K, int GD, cudaStream_t st) {
+static int run_gemm_pair(const void *X, const void *W0, const void *W1, const void *W2, const GemmOut &o, int M, int K,
+                         int GD, cudaStream_t st) {
   CUtensorMap tmA, tmB[3];
   int rc = make_tmap_2d_bf16(&tmA, X, M, K, (uint64_t)K * 2, kTcBM, kTcBK);
   if (rc) return rc;
@@ -478,19 +543,12 @@ static int run_gemm_pair(const void *X, const void *W0, const void *W1, const vo
     rc = make_tmap_2d_bf16(&tmB[i], Ws[i], K, GD, (uint64_t)GD * 2, kTcBK, 64);
     if (rc) return rc;
   }
-  CUtensorMap tmC[2];
-  const void *outs[2] = {Chi ? (const void *)Chi : W0, Clo ? (const void *)Clo : W0};
-  for (int i = 0; i < 2; ++i) {
-    rc = Chi ? make_tmap_2d_bf16(&tmC[i], outs[i], M, 3 * (uint64_t)GD, 3 * (uint64_t)GD * 2, kTcBM, 64)
-             : make_tmap_2d_bf16(&tmC[i], outs[i], 1, GD, (uint64_t)GD * 2, 1, 64);
-    if (rc) return rc;
-  }
+  CUtensorMap tmC[3];
+  if ((rc = o.maps(tmC, W0, M, GD))) return rc;
   AG_CUDA_TRY(cudaFuncSetAttribute(gemm_bf16_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGpSmemBytes));
   const int n_tiles_n = 3 * GD / kGpBN, n_tiles_m = (M + 2 * kTcBM - 1) / (2 * kTcBM);
-  gemm_bf16_pair_kernel<<<2 * n_tiles_n * n_tiles_m, kTcThreads, kGpSmemBytes, st>>>(
-      tmA, tmB[0], tmB[1], tmB[2], tmC[0], tmC[1], C, Chi != nullptr, M, K, GD, n_tiles_n);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  return launch_pdl(gemm_bf16_pair_kernel, dim3(2 * n_tiles_n * n_tiles_m), dim3(kTcThreads), kGpSmemBytes, st, tmA, tmB[0],
+                    tmB[1], tmB[2], tmC[0], tmC[1], tmC[2], o.f32(), o.parts, M, K, GD, n_tiles_n, o.seq_lens, o.n);
 }
 
 // The gate's projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
@@ -498,10 +556,16 @@ template <int BN>
 struct GateProjSplit {
   CUtensorMap tmA, tmB[3];
   float *C;
-  __nv_bfloat16 *hi, *lo;
+  __nv_bfloat16 *part[3];
   int M, GD, n_tiles_n;
+  const int32_t *seq_lens;
+  int n;
   struct Shared {};
   struct Row {};
+  __device__ bool skip(int tile) const {
+    const int m0 = tile / n_tiles_n * kTcBM;
+    return padding_rows(seq_lens, n, m0, min(m0 + kTcBM, M), kTcBM);
+  }
   __device__ void prefetch() const { prefetch_tensormap(&tmA); prefetch_tensormap(&tmB[0]); }
   __device__ void load_a(uint8_t *dst, uint64_t *bar, int tile, int kb) const {
     tma_load_2d(dst, &tmA, bar, kb * kTcBK, tile / n_tiles_n * kTcBM);        // rows past M are filled with zeros
@@ -519,12 +583,16 @@ struct GateProjSplit {
     for (int c = 0; c < BN / 128; ++c) {
       const size_t at = (size_t)m * 3 * GD + tile % n_tiles_n * BN + c * 128 + col;
       const float *x = acc + c * 4;
-      if (hi != nullptr) {
-        float h[4], l[4];
+      if (part[0] != nullptr) {
+        float rest[4] = {x[0], x[1], x[2], x[3]};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) split_bf16(x[e], h[e], l[e]);
-        *reinterpret_cast<uint2 *>(hi + at) = make_uint2(pack_bf16x2(h[0], h[1]), pack_bf16x2(h[2], h[3]));
-        *reinterpret_cast<uint2 *>(lo + at) = make_uint2(pack_bf16x2(l[0], l[1]), pack_bf16x2(l[2], l[3]));
+        for (int q = 0; q < 3; ++q) {
+          if (part[q] == nullptr) break;
+          float h[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) split_bf16(rest[e], h[e], rest[e]);
+          *reinterpret_cast<uint2 *>(part[q] + at) = make_uint2(pack_bf16x2(h[0], h[1]), pack_bf16x2(h[2], h[3]));
+        }
       } else {
         *reinterpret_cast<float4 *>(C + at) = make_float4(x[0], x[1], x[2], x[3]);
       }
@@ -534,8 +602,8 @@ struct GateProjSplit {
 
 // Runs the projection split over clusters if that is the faster way (*done), else does nothing.
 template <int BN>
-static int try_gemm_split(const void *X, const void *W0, const void *W1, const void *W2, float *C, __nv_bfloat16 *Chi,
-                          __nv_bfloat16 *Clo, int M, int K, int GD, cudaStream_t st, bool *done) {
+static int try_gemm_split(const void *X, const void *W0, const void *W1, const void *W2, const GemmOut &o, int M, int K,
+                          int GD, cudaStream_t st, bool *done) {
   const int *cap;
   int rc = splitk::splitk_capacity<BN, GateProjSplit<BN>>(&cap);
   if (rc) return rc;
@@ -549,25 +617,27 @@ static int try_gemm_split(const void *X, const void *W0, const void *W1, const v
   const void *Ws[3] = {W0, W1, W2};
   for (int i = 0; i < 3; ++i)
     if ((rc = make_tmap_2d_bf16(&p.tmB[i], Ws[i], K, GD, (uint64_t)GD * 2, kTcBK, 64))) return rc;
-  p.C = C; p.hi = Chi; p.lo = Clo; p.M = M; p.GD = GD; p.n_tiles_n = n_tiles_n;
+  p.C = o.f32();
+  for (int i = 0; i < 3; ++i) p.part[i] = o.part(i, (size_t)M * 3 * GD);
+  p.seq_lens = o.seq_lens; p.n = o.n; p.M = M; p.GD = GD; p.n_tiles_n = n_tiles_n;
   return splitk::launch_splitk<BN>(p, tiles, num_kb, splits, st);
 }
 
 bool gate_proj_tc_supported(int K, int GD) { return GD % 128 == 0 && K % 8 == 0; }
 
-int launch_gate_proj_tc(const void *X, const void *W0, const void *W1, const void *W2, float *C, void *Chi,
-                        void *Clo, int M, int K, int GD, cudaStream_t st) {
-  auto hi = static_cast<__nv_bfloat16 *>(Chi), lo = static_cast<__nv_bfloat16 *>(Clo);
+int launch_gate_proj_tc(const void *X, const void *W0, const void *W1, const void *W2, void *out, int parts,
+                        int M, int K, int GD, const int32_t *seq_lens, int n, cudaStream_t st) {
+  const GemmOut o{out, parts, seq_lens, n};
   // less than two waves of 128-column tiles: the reduction split over clusters where that fills the chip
   if ((long long)((M + kTcBM - 1) / kTcBM) * (3 * GD / 128) <= 2 * gemm_sm_count()) {
     bool done = false;
-    const int rc = GD % 256 == 0 ? try_gemm_split<256>(X, W0, W1, W2, C, hi, lo, M, K, GD, st, &done)
-                                 : try_gemm_split<128>(X, W0, W1, W2, C, hi, lo, M, K, GD, st, &done);
+    const int rc = GD % 256 == 0 ? try_gemm_split<256>(X, W0, W1, W2, o, M, K, GD, st, &done)
+                                 : try_gemm_split<128>(X, W0, W1, W2, o, M, K, GD, st, &done);
     if (rc || done) return rc;
   }
   // at least half a wave of pair tiles (256 x 384): CTA pairs
   if ((long long)(3 * GD / kGpBN) * ((M + 2 * kTcBM - 1) / (2 * kTcBM)) * 4 >= gemm_sm_count())
-    return run_gemm_pair(X, W0, W1, W2, C, hi, lo, M, K, GD, st);
+    return run_gemm_pair(X, W0, W1, W2, o, M, K, GD, st);
   if (GD % 256 == 0) {
     // more than one wave of 128 x 256 tiles: 256 x 256 tiles, whose two row sub-tiles share every
     // stage of W (a third less operand traffic per FLOP; the kernel is bound by feeding the SMs)
@@ -578,12 +648,12 @@ int launch_gate_proj_tc(const void *X, const void *W0, const void *W1, const voi
       // operand loads, not the MMAs, set it), so with several rounds the fewer, wider tiles stay.
       const long long row_tiles = (M + 2 * kTcBM - 1) / (2 * kTcBM);
       if (GD % 64 == 0 && row_tiles * (3 * GD / 192) <= gemm_sm_count())
-        return run_gemm_tc<192, 2>(X, W0, W1, W2, C, hi, lo, M, K, GD, st);
-      return run_gemm_tc<256, 2>(X, W0, W1, W2, C, hi, lo, M, K, GD, st);
+        return run_gemm_tc<192, 2>(X, W0, W1, W2, o, M, K, GD, st);
+      return run_gemm_tc<256, 2>(X, W0, W1, W2, o, M, K, GD, st);
     }
-    return run_gemm_tc<256, 1>(X, W0, W1, W2, C, hi, lo, M, K, GD, st);
+    return run_gemm_tc<256, 1>(X, W0, W1, W2, o, M, K, GD, st);
   }
-  return run_gemm_tc<128, 1>(X, W0, W1, W2, C, hi, lo, M, K, GD, st);
+  return run_gemm_tc<128, 1>(X, W0, W1, W2, o, M, K, GD, st);
 }
 
 int gemm_tc_wait_timeouts() {

@@ -69,7 +69,7 @@ __device__ __forceinline__ long long kv_rank_token(const KvEpilogue &e, size_t s
   if ((n & 15) == 0) {                                      // flag rows start on 16-byte boundaries
     const uint4 *fv = reinterpret_cast<const uint4 *>(f);
     for (int x = r_in; x < n / 16; x += kBM) {
-      const uint4 w = ldg128(fv + x);
+      const uint4 w = ld128(fv + x);
       const int c = nonzero_bytes(w.x) + nonzero_bytes(w.y) + nonzero_bytes(w.z) + nonzero_bytes(w.w);
       total += c;
       if (x * 16 < t0) before += c;                         // t0 is a multiple of 16: a vector lies on one side
@@ -205,10 +205,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 kv_proj_cache_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBk,
                      const __grid_constant__ CUtensorMap tmBv, const __grid_constant__ CUtensorMap tmBq,
                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                     const __grid_constant__ CUtensorMap tmQ, const uint8_t *__restrict__ flags,
-                     int32_t *__restrict__ prefix, int32_t *__restrict__ idx, const int64_t *__restrict__ row_off,
-                     const int32_t *__restrict__ cap, int32_t *__restrict__ len, uint8_t *__restrict__ k_rows,
-                     uint8_t *__restrict__ v_rows, int32_t *__restrict__ dev_status, int n_sub, int tps, int Kdim, int GD,
+                     const __grid_constant__ CUtensorMap tmQ, const uint8_t *flags,
+                     int32_t *prefix, int32_t *idx, const int64_t *row_off,
+                     const int32_t *cap, int32_t *len, uint8_t *k_rows,
+                     uint8_t *v_rows, int32_t *dev_status, int n_sub, int tps, int Kdim, int GD,
                      int n, int kv_heads, int heads, int n_tiles_m, int n_tiles_n) {
   using Cfg = KvCfg<BN, MT>;
   constexpr uint32_t kTmemCols = MT * BN;
@@ -259,6 +259,8 @@ kv_proj_cache_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -333,10 +335,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 kv_proj_cache_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBk,
                           const __grid_constant__ CUtensorMap tmBv, const __grid_constant__ CUtensorMap tmBq,
                           const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                          const __grid_constant__ CUtensorMap tmQ, const uint8_t *__restrict__ flags,
-                          int32_t *__restrict__ prefix, int32_t *__restrict__ idx, const int64_t *__restrict__ row_off,
-                          const int32_t *__restrict__ cap, int32_t *__restrict__ len, uint8_t *__restrict__ k_rows,
-                          uint8_t *__restrict__ v_rows, int32_t *__restrict__ dev_status, int n_sub, int tps, int Kdim,
+                          const __grid_constant__ CUtensorMap tmQ, const uint8_t *flags,
+                          int32_t *prefix, int32_t *idx, const int64_t *row_off,
+                          const int32_t *cap, int32_t *len, uint8_t *k_rows,
+                          uint8_t *v_rows, int32_t *dev_status, int n_sub, int tps, int Kdim,
                           int GD, int n, int kv_heads, int heads, int n_tiles_m, int n_tiles_n, int split_from) {
   constexpr int BN = kPairBN, MT = kPairMT;
   constexpr uint32_t kTmemCols = MT * BN;          // 512: two accumulators of 128 rows x 256 columns per CTA
@@ -385,6 +387,8 @@ kv_proj_cache_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
   cluster_arrive_wait();                           // both CTAs' barriers are initialised, tensor memory is allocated
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
+  pdl_launch_dependents();
   const uint32_t stage_tx = (uint32_t)(mts * (kBM * kBK * 2) + kPairBBytes);
 
   if (warp == 0) {
@@ -468,6 +472,7 @@ struct KvProjSplit {
     int red[12];
   };
   struct Row {};
+  __device__ bool skip(int) const { return false; }
   __device__ void prefetch() const { prefetch_tensormap(&tmA); prefetch_tensormap(&tmB[0]); }
   __device__ int column(int tile) const { return tile % n_tiles_n * BN; }       // in the packed output [K | V | Q]
   __device__ int which(int tile) const { return min(column(tile) / GD, 2); }    // a tile lies in one weight
@@ -572,20 +577,17 @@ int run(const ag_layer_desc &d, const void *X, const void *Wq, const void *Wk, c
     const int tail = n_tiles % n_pairs;
     const int split_from = (tail > 0 && 2 * tail <= n_pairs) ? n_tiles - tail : n_tiles;
     const int ctas = 2 * (split_from + 2 * (n_tiles - split_from));
-    kv_proj_cache_pair_kernel<<<ctas, kThreads, kPairSmemBytes, st>>>(
+    return launch_pdl(kv_proj_cache_pair_kernel, dim3(ctas), dim3(kThreads), kPairSmemBytes, st,
         tmA, tmBk, tmBv, tmBq, tmK, tmV, tmQ, flags, prefix, idx, c.row_off, c.cap, c.len, static_cast<uint8_t *>(c.k_rows),
         static_cast<uint8_t *>(c.v_rows), dev_status, n_sub, tps, Kdim, GD, d.seq, hk, d.heads, n_tiles_m, n_tiles_n, split_from);
-    AG_LAUNCH_CHECK();
-    return AG_OK;
   }
   auto kern = kv_proj_cache_kernel<BN, MT>;
   AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
   const int n_tiles_n = (2 * GD + QD) / BN, n_tiles_m = (n_sub + MT - 1) / MT, n_tiles = n_tiles_n * n_tiles_m;
-  kern<<<n_tiles, kThreads, Cfg::kSmemBytes, st>>>(tmA, tmBk, tmBv, tmBq, tmK, tmV, tmQ, flags, prefix, idx, c.row_off, c.cap, c.len,
-                                                   static_cast<uint8_t *>(c.k_rows), static_cast<uint8_t *>(c.v_rows),
-                                                   dev_status, n_sub, tps, Kdim, GD, d.seq, hk, d.heads, n_tiles_m, n_tiles_n);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  return launch_pdl(kern, dim3(n_tiles), dim3(kThreads), Cfg::kSmemBytes, st, tmA, tmBk, tmBv, tmBq, tmK, tmV, tmQ, flags,
+                    prefix, idx, c.row_off, c.cap, c.len, static_cast<uint8_t *>(c.k_rows),
+                    static_cast<uint8_t *>(c.v_rows), dev_status, n_sub, tps, Kdim, GD, d.seq, hk, d.heads, n_tiles_m,
+                    n_tiles_n);
 }
 
 }  // namespace

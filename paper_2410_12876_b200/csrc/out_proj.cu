@@ -47,7 +47,7 @@ template <int BN, int MT> struct OpCfg {
 template <int BN, int MT>
 __global__ void __launch_bounds__(kThreads, 1)
 out_proj_tc_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmW,
-                   const __grid_constant__ CUtensorMap tmY, const __nv_bfloat16 *__restrict__ X_res, int n_sub, int tps,
+                   const __grid_constant__ CUtensorMap tmY, const __nv_bfloat16 *X_res, int n_sub, int tps,
                    int n, int heads, int d, int n_tiles_m, int n_tiles_n) {
   using Cfg = OpCfg<BN, MT>;
   constexpr uint32_t kTmemCols = MT * BN;
@@ -93,6 +93,8 @@ out_proj_tc_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constan
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -242,7 +244,7 @@ constexpr int kPairSmemBytes = kPairStages * kPairStageBytes + 1024 + 256;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 out_proj_pair_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmW,
-                     const __grid_constant__ CUtensorMap tmY, const __nv_bfloat16 *__restrict__ X_res, int n_sub, int tps,
+                     const __grid_constant__ CUtensorMap tmY, const __nv_bfloat16 *X_res, int n_sub, int tps,
                      int n, int heads, int d, int n_tiles_m, int n_tiles_n) {
   constexpr int BN = kPairBN, MT = kPairMT;
   constexpr uint32_t kTmemCols = MT * BN;          // 512: two accumulators of 128 rows x 256 columns per CTA
@@ -286,6 +288,8 @@ out_proj_pair_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_const
   cluster_arrive_wait();                           // both CTAs' barriers are initialised, tensor memory is allocated
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
+  pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -442,17 +446,15 @@ int run_tc(const ag_layer_desc &dsc, const void *O, const void *Wo, const void *
   auto kern = out_proj_tc_kernel<BN, MT>;
   AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
   const int n_tiles_n = d / BN, n_tiles_m = (n_sub + MT - 1) / MT, n_tiles = n_tiles_n * n_tiles_m;
-  kern<<<n_tiles, kThreads, Cfg::kSmemBytes, st>>>(tmO, tmW, tmY, static_cast<const __nv_bfloat16 *>(X_res), n_sub, tps,
+  return launch_pdl(kern, dim3(n_tiles), dim3(kThreads), Cfg::kSmemBytes, st, tmO, tmW, tmY, static_cast<const __nv_bfloat16 *>(X_res), n_sub, tps,
                                                    dsc.seq, dsc.heads, d, n_tiles_m, n_tiles_n);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
 }
 
 // CUDA-core form: one thread per (token, output column); consecutive threads take consecutive
 // columns, so the rows of W^O are read coalesced and the token's head outputs are broadcast.
 template <typename T>
 __global__ void __launch_bounds__(256)
-out_proj_simt_kernel(const T *__restrict__ O, const T *__restrict__ Wo, const T *__restrict__ X_res, T *__restrict__ Y,
+out_proj_simt_kernel(const T *O, const T *Wo, const T *X_res, T *Y,
                      int n, int heads, int D, int d) {
   const int tok = blockIdx.y, c = blockIdx.x * 256 + threadIdx.x;   // tok = b n + t
   if (c >= d) return;
@@ -479,10 +481,7 @@ int run_pair(const ag_layer_desc &dsc, const void *O, const void *Wo, const void
   if (rc) return rc;
   AG_CUDA_TRY(cudaFuncSetAttribute(out_proj_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes));
   const int n_tiles_n = d / kPairBN, n_tiles_m = (n_sub + 2 * kPairMT - 1) / (2 * kPairMT);
-  out_proj_pair_kernel<<<2 * n_tiles_n * n_tiles_m, kThreads, kPairSmemBytes, st>>>(
-      tmO, tmW, tmY, static_cast<const __nv_bfloat16 *>(X_res), n_sub, tps, dsc.seq, dsc.heads, d, n_tiles_m, n_tiles_n);
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  return launch_pdl(out_proj_pair_kernel, dim3(2 * n_tiles_n * n_tiles_m), dim3(kThreads), kPairSmemBytes, st, tmO, tmW, tmY, static_cast<const __nv_bfloat16 *>(X_res), n_sub, tps, dsc.seq, dsc.heads, d, n_tiles_m, n_tiles_n);
 }
 
 // The same projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
@@ -494,6 +493,7 @@ struct OutProjSplit {
   int tps, n, heads, d, n_tiles_n;
   struct Shared {};
   struct Row { uint2 x[BN / 128]; };                         // skip connection
+  __device__ bool skip(int) const { return false; }
   __device__ void prefetch() const { prefetch_tensormap(&tmO); prefetch_tensormap(&tmW); }
   __device__ void load_a(uint8_t *dst, uint64_t *bar, int tile, int kb) const {
     const int sub = tile / n_tiles_n;                        // 128 tokens of one sequence; zeros past its end

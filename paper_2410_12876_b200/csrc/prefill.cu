@@ -28,11 +28,13 @@ template <typename T, int D>
 __global__ void __launch_bounds__(kBandThreads)
 prefill_band_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
                     const uint8_t *__restrict__ flags, const float *__restrict__ lse, T *__restrict__ O,
-                    int n, int heads, int kv_heads, int R, float scale_log2) {
+                    int n, int heads, int kv_heads, int R, float scale_log2, const int32_t *seq_lens) {
   constexpr int kEpl = Elem<T>::kPerVec;
   constexpr int kLanes = D / kEpl;                 // lanes per query
   constexpr int kRowsPerCta = kBandThreads / kLanes;
   const int slab = blockIdx.y;
+  // padding only: outputs unspecified, nothing to do
+  if (seq_lens != nullptr && (int)blockIdx.x * kRowsPerCta >= seq_lens[slab / heads]) return;
   const int kv = (slab / heads) * kv_heads + (slab % heads) / (heads / kv_heads);
   const int g = threadIdx.x / kLanes, v = threadIdx.x % kLanes;
   const int j = min(blockIdx.x * kRowsPerCta + g, n - 1);     // clamped rows recompute row n - 1, store nothing
@@ -115,7 +117,7 @@ static int run_prefill_band(const ag_layer_desc &d, const void *Q, const void *K
   dim3 grid((d.seq + kRowsPerCta - 1) / kRowsPerCta, d.batch * d.heads);
   prefill_band_kernel<T, D><<<grid, kBandThreads, 0, st>>>(
       static_cast<const T *>(Q), static_cast<const T *>(K), static_cast<const T *>(V), flags, lse,
-      static_cast<T *>(O), d.seq, d.heads, kv_heads_of(d), recent_rows(d), scale * 1.4426950408889634f);
+      static_cast<T *>(O), d.seq, d.heads, kv_heads_of(d), recent_rows(d), scale * 1.4426950408889634f, d.seq_lens);
   AG_LAUNCH_CHECK();
   return AG_OK;
 }

@@ -23,9 +23,10 @@ __global__ void __launch_bounds__(kBmThreads, 3)
 prefill_band_mma_kernel(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restrict__ K,
                         const __nv_bfloat16 *__restrict__ V, const uint8_t *__restrict__ flags,
                         const float *__restrict__ lse, __nv_bfloat16 *__restrict__ O, int n, int heads,
-                        int kv_heads, int R, float scale_log2) {
+                        int kv_heads, int R, float scale_log2, const int32_t *seq_lens) {
   extern __shared__ __align__(128) uint8_t bm_smem[];
   const int slab = blockIdx.y, j0 = blockIdx.x * kBmQ;
+  if (seq_lens != nullptr && j0 >= seq_lens[slab / heads]) return;     // padding only: outputs unspecified
   const int kv = (slab / heads) * kv_heads + (slab % heads) / (heads / kv_heads);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const uint32_t sQ = (uint32_t)__cvta_generic_to_shared(bm_smem), sO = sQ + kBmQ * 256;
@@ -174,7 +175,7 @@ int launch_prefill_band_mma(const ag_layer_desc &d, const void *Q, const void *K
   prefill_band_mma_kernel<<<grid, kBmThreads, kBmSmemBytes, st>>>(
       static_cast<const __nv_bfloat16 *>(Q), static_cast<const __nv_bfloat16 *>(K),
       static_cast<const __nv_bfloat16 *>(V), flags, lse, static_cast<__nv_bfloat16 *>(O), d.seq, d.heads,
-      kv_heads_of(d), recent_rows(d), scale * 1.4426950408889634f);
+      kv_heads_of(d), recent_rows(d), scale * 1.4426950408889634f, d.seq_lens);
   AG_LAUNCH_CHECK();
   return AG_OK;
 }
