@@ -386,12 +386,8 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
           float p1 = fast_exp2(fmaf(__uint_as_float(r[c * 16 + e + 1]), a.scale_log2, -m_exp));
           rs[(e >> 1) & 3] += p0 + p1;
 #pragma unroll
-          for (int i = 0; i < C::kParts; ++i) {
-            float h0, h1;
-            split_bf16(p0, h0, p0);
-            split_bf16(p1, h1, p1);
-            pk[i][e >> 1] = pack_bf16x2(h0, h1);
-          }
+          for (int i = 0; i + 1 < C::kParts; ++i) pk[i][e >> 1] = take_bf16x2(p0, p1);
+          pk[C::kParts - 1][e >> 1] = pack_bf16x2(p0, p1);
         }
 #pragma unroll
         for (int i = 0; i < C::kParts; ++i)
@@ -601,13 +597,9 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         float2 x = *reinterpret_cast<const float2 *>(Hs + (g + (f & 1) * 8) * pitch + k0 + (f >> 1) * 8 + 2 * tq);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          float h0, h1;
-          split_bf16(x.x, h0, x.x);
-          split_bf16(x.y, h1, x.y);
-          ah[q][f] = pack_bf16x2(h0, h1);
-        }
+        ah[0][f] = take_bf16x2(x.x, x.y);
+        ah[1][f] = take_bf16x2(x.x, x.y);
+        ah[2][f] = pack_bf16x2(x.x, x.y);
       }
 #pragma unroll
       for (int nb2 = 0; nb2 < 2; ++nb2) {

@@ -46,11 +46,9 @@ __device__ __forceinline__ void stage_third(uint8_t *smem, uint32_t tmem, int qu
       uint32_t t[4];
 #pragma unroll
       for (int q = 0; q < 8; q += 2) {
-        float part, x0 = __uint_as_float(r[e + q]), x1 = __uint_as_float(r[e + q + 1]);
-        split_bf16(x0, part, x0);
-        split_bf16(x0, part, x0);
-        split_bf16(x1, part, x1);
-        split_bf16(x1, part, x1);
+        float x0 = __uint_as_float(r[e + q]), x1 = __uint_as_float(r[e + q + 1]);
+        take_bf16x2(x0, x1);
+        take_bf16x2(x0, x1);
         t[q >> 1] = pack_bf16x2(x0, x1);
       }
       const uint32_t chunk = (uint32_t)(((c & 32) >> 3) + (e >> 3));
@@ -60,12 +58,14 @@ __device__ __forceinline__ void stage_third(uint8_t *smem, uint32_t tmem, int qu
   fence_proxy_async_smem();
 }
 
-template <int BN, int MT>
+// kThird: three bf16 parts.  kRagged: tiles of padding are left out; forms of their own, since a kernel that may leave
+// early loses 6 % (prompts of 4096 tokens 47.9 -> 50.3 us).
+template <int BN, int MT, bool kThird, bool kRagged>
 __global__ void __launch_bounds__(kTcThreads, 1)
 gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                     const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
                     const __grid_constant__ CUtensorMap tmChi, const __grid_constant__ CUtensorMap tmClo,
-                    const __grid_constant__ CUtensorMap tmC3, float *__restrict__ C, int parts, int M, int K, int GD,
+                    const __grid_constant__ CUtensorMap tmC3, float *__restrict__ C, bool split, int M, int K, int GD,
                     int n_tiles_n, int halved_from, const int32_t *seq_lens, int n) {
   using Cfg = GemmTcCfg<BN, MT>;
   constexpr uint32_t kTmemCols = MT * Cfg::kAccCols;
@@ -86,7 +86,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   const int bn = halved ? BN / 2 : BN;         // columns of this CTA (a multiple of 64)
   const int m0 = (tile / n_tiles_n) * (MT * kTcBM);
   const int n0 = (tile % n_tiles_n) * BN + (halved ? ((cta - halved_from) & 1) * (BN / 2) : 0);   // in the packed [3 * GD] output
-  if (padding_rows(seq_lens, n, m0, min(m0 + MT * kTcBM, M), kTcBM)) return;
+  if (kRagged && padding_rows(seq_lens, n, m0, min(m0 + MT * kTcBM, M), kTcBM)) return;
   // a 64-column panel of B lies in one weight (64 divides GD); a tile may straddle two
   const int num_kb = (K + kTcBK - 1) / kTcBK;
 
@@ -171,7 +171,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     for (int mt = 0; mt < MT; ++mt) {
     const int row = m0 + mt * kTcBM + quad * 32 + lane;
     const uint32_t tmem_sub = tmem_acc + mt * Cfg::kAccCols;
-    if (ok && num_kb > 0 && parts > 0) {
+    if (ok && num_kb > 0 && split) {
       // x = hi + lo in bf16 pairs, for consumers that rebuild float32 precision from three
       // products.  Every MMA has completed, so every stage has been read: the tile is staged
       // over them as panels of [128 rows][64 bf16] (128-byte rows, 16-byte chunks XOR-swizzled by
@@ -189,11 +189,9 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           uint32_t h[4], l[4];
 #pragma unroll
           for (int q = 0; q < 8; q += 2) {
-            float h0, l0, h1, l1;
-            split_bf16(__uint_as_float(r[e + q]), h0, l0);
-            split_bf16(__uint_as_float(r[e + q + 1]), h1, l1);
-            h[q >> 1] = pack_bf16x2(h0, h1);
-            l[q >> 1] = pack_bf16x2(l0, l1);
+            float x0 = __uint_as_float(r[e + q]), x1 = __uint_as_float(r[e + q + 1]);
+            h[q >> 1] = take_bf16x2(x0, x1);
+            l[q >> 1] = pack_bf16x2(x0, x1);
           }
           const uint32_t chunk = (uint32_t)(((c & 32) >> 3) + (e >> 3));          // 16-byte chunk within the 128-byte row
           const uint32_t off = panel + ((chunk ^ (r_in & 7)) << 4);
@@ -211,7 +209,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         tma_store_commit();
         tma_store_wait_read();
       }
-      if (parts == 3) {                                // what the first two parts leave, over the same staging area
+      if constexpr (kThird) {                                // what the first two parts leave, over the same staging area
         named_barrier_sync(1, 256);
         stage_third(smem, tmem_sub, quad, r_in, c_begin, c_end);
         named_barrier_sync(1, 256);
@@ -257,11 +255,12 @@ constexpr int kGpBBytes = (kGpBN / 2 / 64) * kGpPanelBytes;       // 24 KB: two 
 constexpr int kGpStageBytes = kGpABytes + kGpBBytes;              // 40 KB
 constexpr int kGpSmemBytes = kGpStages * kGpStageBytes + 1024 + 256;
 
+template <bool kThird, bool kRagged>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
 gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                       const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
                       const __grid_constant__ CUtensorMap tmChi, const __grid_constant__ CUtensorMap tmClo,
-                      const __grid_constant__ CUtensorMap tmC3, float *__restrict__ C, int parts, int M, int K, int GD,
+                      const __grid_constant__ CUtensorMap tmC3, float *__restrict__ C, bool split, int M, int K, int GD,
                       int n_tiles_n, const int32_t *seq_lens, int n) {
   constexpr uint32_t kTmemCols = 512;              // 384 used: columns [0, 256) of the wide MMA, [256, 384) of the narrow
   static_assert(2 * (kGpBN / 64) * kTcBM * 128 <= kGpStages * kGpStageBytes, "staging fits the stages");
@@ -278,7 +277,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   const int tile = blockIdx.x >> 1;
   const int m0 = (tile / n_tiles_n) * (2 * kTcBM) + (int)rank * kTcBM;   // this CTA's rows
   const int n0 = (tile % n_tiles_n) * kGpBN;                              // in the packed [3 * GD] output
-  if (padding_rows(seq_lens, n, m0 - (int)rank * kTcBM, min(m0 + (2 - (int)rank) * kTcBM, M), kTcBM)) return;   // both CTAs
+  if (kRagged && padding_rows(seq_lens, n, m0 - (int)rank * kTcBM, min(m0 + (2 - (int)rank) * kTcBM, M), kTcBM)) return;   // both CTAs
   const int num_kb = (K + kTcBK - 1) / kTcBK;
 
   if (threadIdx.x == 0) {
@@ -361,7 +360,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     const bool ok = *gave_up == 0;
     tc_fence_after_sync();
     const int r_in = quad * 32 + lane, row = m0 + r_in;
-    if (ok && num_kb > 0 && parts > 0) {
+    if (ok && num_kb > 0 && split) {
       // x = hi + lo in bf16 pairs.  Every MMA of both CTAs has completed, so every stage has been read: the
       // tile is staged over them as panels of [128 rows][64 bf16] (128-byte rows, 16-byte chunks
       // XOR-swizzled by the row): six hi panels, then six lo panels.
@@ -376,11 +375,9 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
           uint32_t h[4], l[4];
 #pragma unroll
           for (int q = 0; q < 8; q += 2) {
-            float h0, l0, h1, l1;
-            split_bf16(__uint_as_float(r[e + q]), h0, l0);
-            split_bf16(__uint_as_float(r[e + q + 1]), h1, l1);
-            h[q >> 1] = pack_bf16x2(h0, h1);
-            l[q >> 1] = pack_bf16x2(l0, l1);
+            float x0 = __uint_as_float(r[e + q]), x1 = __uint_as_float(r[e + q + 1]);
+            h[q >> 1] = take_bf16x2(x0, x1);
+            l[q >> 1] = pack_bf16x2(x0, x1);
           }
           const uint32_t chunk = (uint32_t)(((c & 32) >> 3) + (e >> 3));          // 16-byte chunk within the 128-byte row
           const uint32_t off = panel + ((chunk ^ (r_in & 7)) << 4);
@@ -398,7 +395,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         tma_store_commit();
         tma_store_wait_read();
       }
-      if (parts == 3) {
+      if constexpr (kThird) {
         named_barrier_sync(1, 256);
         stage_third(smem, tmem_acc, quad, r_in, c_begin, c_end);
         named_barrier_sync(1, 256);
@@ -521,7 +518,9 @@ static int run_gemm_tc(const void *X, const void *W0, const void *W1, const void
   }
   CUtensorMap tmC[3];
   if ((rc = o.maps(tmC, W0, M, GD))) return rc;
-  auto kern = gemm_bf16_tc_kernel<BN, MT>;
+  const bool third = o.parts == 3;
+  auto kern = o.seq_lens ? (third ? gemm_bf16_tc_kernel<BN, MT, true, true> : gemm_bf16_tc_kernel<BN, MT, false, true>)
+                         : (third ? gemm_bf16_tc_kernel<BN, MT, true, false> : gemm_bf16_tc_kernel<BN, MT, false, false>);
   AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
   const int n_tiles_n = 3 * GD / BN, n_tiles = n_tiles_n * ((M + MT * kTcBM - 1) / (MT * kTcBM));
   // tiles of a last wave that would fill at most half of the SMs are halved
@@ -530,7 +529,7 @@ static int run_gemm_tc(const void *X, const void *W0, const void *W1, const void
   const int halved_from = (BN % 128 == 0 && tail > 0 && 2 * tail <= sms) ? n_tiles - tail : n_tiles;   // (any MT)
   const int ctas = halved_from + 2 * (n_tiles - halved_from);
   return launch_pdl(kern, dim3(ctas), dim3(kTcThreads), Cfg::kSmemBytes, st, tmA, tmB[0], tmB[1], tmB[2], tmC[0], tmC[1],
-                    tmC[2], o.f32(), o.parts, M, K, GD, n_tiles_n, halved_from, o.seq_lens, o.n);
+                    tmC[2], o.f32(), o.parts > 0, M, K, GD, n_tiles_n, halved_from, o.seq_lens, o.n);
 }
 
 static int run_gemm_pair(const void *X, const void *W0, const void *W1, const void *W2, const GemmOut &o, int M, int K,
@@ -545,10 +544,13 @@ static int run_gemm_pair(const void *X, const void *W0, const void *W1, const vo
   }
   CUtensorMap tmC[3];
   if ((rc = o.maps(tmC, W0, M, GD))) return rc;
-  AG_CUDA_TRY(cudaFuncSetAttribute(gemm_bf16_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGpSmemBytes));
+  const bool third = o.parts == 3;
+  auto kern = o.seq_lens ? (third ? gemm_bf16_pair_kernel<true, true> : gemm_bf16_pair_kernel<false, true>)
+                         : (third ? gemm_bf16_pair_kernel<true, false> : gemm_bf16_pair_kernel<false, false>);
+  AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGpSmemBytes));
   const int n_tiles_n = 3 * GD / kGpBN, n_tiles_m = (M + 2 * kTcBM - 1) / (2 * kTcBM);
-  return launch_pdl(gemm_bf16_pair_kernel, dim3(2 * n_tiles_n * n_tiles_m), dim3(kTcThreads), kGpSmemBytes, st, tmA, tmB[0],
-                    tmB[1], tmB[2], tmC[0], tmC[1], tmC[2], o.f32(), o.parts, M, K, GD, n_tiles_n, o.seq_lens, o.n);
+  return launch_pdl(kern, dim3(2 * n_tiles_n * n_tiles_m), dim3(kTcThreads), kGpSmemBytes, st, tmA, tmB[0],
+                    tmB[1], tmB[2], tmC[0], tmC[1], tmC[2], o.f32(), o.parts > 0, M, K, GD, n_tiles_n, o.seq_lens, o.n);
 }
 
 // The gate's projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
@@ -588,10 +590,8 @@ struct GateProjSplit {
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
           if (part[q] == nullptr) break;
-          float h[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) split_bf16(rest[e], h[e], rest[e]);
-          *reinterpret_cast<uint2 *>(part[q] + at) = make_uint2(pack_bf16x2(h[0], h[1]), pack_bf16x2(h[2], h[3]));
+          const uint32_t lo = take_bf16x2(rest[0], rest[1]), up = take_bf16x2(rest[2], rest[3]);
+          *reinterpret_cast<uint2 *>(part[q] + at) = make_uint2(lo, up);
         }
       } else {
         *reinterpret_cast<float4 *>(C + at) = make_float4(x[0], x[1], x[2], x[3]);

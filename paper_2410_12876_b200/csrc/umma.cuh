@@ -444,10 +444,13 @@ __device__ __forceinline__ float max3_f32(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-// x = hi + lo with hi = bf16(x), lo = bf16(x - hi): |x - hi - lo| <= 2^-17 |x|.
-__device__ __forceinline__ void split_bf16(float x, float &hi, float &lo) {
-  hi = __uint_as_float(__float_as_uint(__bfloat162float(__float2bfloat16_rn(x))));
-  lo = x - hi;
+// Takes the leading bf16 part of two values: returns them packed and leaves what they miss of x0, x1 (exact; two
+// such parts carry a float32 to 2^-17, three exactly).
+__device__ __forceinline__ uint32_t take_bf16x2(float &x0, float &x1) {
+  const uint32_t p = pack_bf16x2(x0, x1);
+  x0 -= __uint_as_float(p << 16);
+  x1 -= __uint_as_float(p & 0xffff0000u);
+  return p;
 }
 
 }  // namespace umma
