@@ -79,7 +79,6 @@ gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   tc_fence_after_sync();
   const uint32_t tmem_acc = *tmem_slot;
   pdl_wait();                                        // set-up is done: what the kernel before wrote may be read
-  pdl_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {

@@ -462,12 +462,14 @@ static int run_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, 
   a.prefix = prefix; a.row_off = c.row_off; a.len = c.len;
   a.n = d.seq; a.n_qtiles = (d.seq + kPfBM - 1) / kPfBM; a.slabs = slabs;
   a.heads = d.heads; a.kv_heads = kv_heads_of(d);
-  // Cache rows of a band: at most 32 MB of keys and 32 MB of values if every token were kept (half of L2 with
-  // what else passes through it), but enough tiles for a full round of the chip at the lightest query tiles' end.
-  const long long slab_bytes = (long long)d.seq * kPfD * 2 / (d.heads / a.kv_heads);
-  a.band_slabs = (int)((32LL << 20) / (slab_bytes > 0 ? slab_bytes : 1));
-  if (a.band_slabs < 32) a.band_slabs = 32;
-  if (a.band_slabs > slabs) a.band_slabs = slabs;
+  // Bands of about 40 MB of keys (and as much of values) if every token were kept, of equal size; at least 32
+  // slabs, so that a band fills the chip.  8 x 32 heads of 4096 tokens: 660 us at 32 MB, 685 at 64, 875 in one band; a
+  // batch that is little more than a band stays whole (2 x 32 heads of 3001: 73 us whole, 80 in 43 + 21 slabs).
+  const double total = (double)kv_slabs * d.seq * kPfD * 2;
+  int bands = (int)(total / (40 << 20) + 0.5);
+  if (bands > slabs / 32) bands = slabs / 32;
+  if (bands < 1) bands = 1;
+  a.band_slabs = (slabs + bands - 1) / bands;
   a.scale_log2 = scale * 1.4426950408889634f;
   a.lse = lse;
   a.seq_lens = d.seq_lens;
