@@ -23,7 +23,7 @@ def test_bands(h, kv):
     O = T.gpu_prefill(shape, Q, K, V, flags, cache, prefix)
     one = shape.with_(batch=1)
     for b in range(3):
-        part = [t[b:b + 1].contiguous() for t in (Q, K, V, flags)]
+        part = [t[b:b + 1].clone() for t in (Q, K, V, flags)]
         c1, p1, _, _ = T.gpu_compact(one, part[1], part[2], part[3])
         assert torch.equal(T.gpu_prefill(one, *part, c1, p1), O[b:b + 1])
     g = h // shape.kvh
