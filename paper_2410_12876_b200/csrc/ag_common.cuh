@@ -125,17 +125,11 @@ int launch_prefill(const ag_layer_desc &d, const void *Q, const void *K, const v
                    const uint8_t *flags, const ag_cache &c, const int32_t *prefix, float scale,
                    void *O, void *ws, cudaStream_t st);
 
-// Tensor-core (tcgen05) prefill attention for bf16, head_dim 128.
+// Tensor-core (tcgen05) prefill attention for bf16, the recent-token window included.
 bool prefill_tc_supported(const ag_layer_desc &d, const ag_cache &c);
-// lse (NULL or [slabs, n]): log2 of each row's softmax denominator, in the units of the scaled
-// scores times log2(e); -inf where a whole query tile had no retained key (O = v_j there).
-int launch_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const ag_cache &c,
-                      const int32_t *prefix, float scale, void *O, float *lse, cudaStream_t st);
+int launch_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const uint8_t *flags,
+                      const ag_cache &c, const int32_t *prefix, float scale, void *O, cudaStream_t st);
 int prefill_tc_wait_timeouts();
-// Band pass of a recent-token window on the tensor cores (bf16, head_dim 128): extends every row of O
-// by the evicted tokens of its window, given the rows' log-sum-exp.
-int launch_prefill_band_mma(const ag_layer_desc &d, const void *Q, const void *K, const void *V,
-                            const uint8_t *flags, const float *lse, float scale, void *O, cudaStream_t st);
 
 // Output projection of Eq. 1 with the skip connection: Y = X_res + [H_1 .. H_h] Wo (tensor cores for
 // bf16, head_dim 128; CUDA cores otherwise).

@@ -18,6 +18,11 @@
 // The self term seeds the running softmax (m = s_jj, l = 1) and its value row
 // is added in the epilogue: O_j = (sum_r p_r v_r + w_self v_j) / l.  Every byte
 // that enters or leaves the CTA travels by TMA.
+//
+// With a recent-token window (kBand) query j also sees the EVICTED tokens among the R = w - 1 <= 16 before it.
+// They and the token itself lie in the dense rows [j0 - 16, j0 + 128): three more key tiles (64, 64 and 16
+// rows of the dense K, V) in front of the cache's, masked to the band, take the place of the self tile.  (As a
+// pass of its own over Q, O and the dense K, V the band took 38 us at 4096 tokens of 32 heads, 57 us at 4 x 1999.)
 #include "ag_common.cuh"
 #include "umma.cuh"
 
@@ -54,7 +59,8 @@ struct PrefillTcArgs {
   int band_slabs;                   // slabs per band of the tile order
   int heads, kv_heads;              // query heads share key/value heads in groups of heads / kv_heads
   float scale_log2;
-  float *lse;                       // NULL, or [slabs, n]: m + log2(l) of every row (see launch_prefill_tc)
+  const uint8_t *flags;             // kBand: [kv slabs, n]
+  int recent;                       // kBand: tokens before the current one that stay visible, 1..16
   const int32_t *seq_lens;          // NULL, or [batch]: a query tile that holds padding only is skipped
 };
 
@@ -74,7 +80,7 @@ __device__ __forceinline__ uint32_t tile_chunk_offset(int row, int chunk) {
 // CTA's own 128 rows, of which only the diagonal (q_j . k_j) is read.  Last,
 // the dense V tile is brought in for the self term of the output, and the O
 // tile leaves through shared memory with one TMA store.
-template <int kPfD>
+template <int kPfD, bool kBand>
 __global__ void __launch_bounds__(kPfThreads, kPfCtasPerSm)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKd,
                   const __grid_constant__ CUtensorMap tmVd, const __grid_constant__ CUtensorMap tmO,
@@ -132,7 +138,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   // keys any row of this tile may see; never past the slab's valid rows (a slab that overflowed at
   // compaction has len = 0 under full prefix counts: its queries see themselves only)
   const int max_bound = min(pre[j_last], a.len[kv_slab]);
-  const int n_kv = (max_bound + kPfBN - 1) / kPfBN;
+  constexpr int kBandTiles = kBand ? 3 : 0;         // key tiles of dense rows in front of the cache's
+  const int n_kv = (max_bound + kPfBN - 1) / kPfBN + kBandTiles;
+  // tokens of this slab's sequence (rows of the dense K, V past it are padding)
+  const int seq_len = a.seq_lens != nullptr ? min(a.seq_lens[slab / a.heads], a.n) : a.n;
   const int row0 = (int)a.row_off[kv_slab];
   static_assert(kPfKvBuf == kPfTile, "the self tile below spans exactly the two V stages");
   // uses of K stage 0 / 1 before the dense V tile: even / odd cache tiles
@@ -151,33 +160,44 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       bool ok = true;
-      if (n_kv > 0) {
+      if (kBand || n_kv > 0) {
         mbar_arrive_expect_tx(q_full, kPfTile);
 #pragma unroll
         for (int p = 0; p < C::kPanels; ++p) tma_load_3d(sQ + p * kPfPanel, &tmQ, q_full, p * 64, j0, slab);
         // self tile: dense K rows j0 .. j0 + 127 across both V stages, which no P V needs before
         // the first softmax is done; the first cache tiles of K load alongside it
-        mbar_arrive_expect_tx(&v_full[0], kPfTile);
+        if constexpr (!kBand) {
+          mbar_arrive_expect_tx(&v_full[0], kPfTile);
 #pragma unroll
-        for (int p = 0; p < C::kPanels; ++p) tma_load_3d(sV + p * kPfPanel, &tmKd, &v_full[0], p * 64, j0, kv_slab);
+          for (int p = 0; p < C::kPanels; ++p) tma_load_3d(sV + p * kPfPanel, &tmKd, &v_full[0], p * 64, j0, kv_slab);
+        }
         for (int i = 0; i < n_kv && ok; ++i) {
           const int st = i & 1;
-          const int y = row0 + i * kPfBN;
+          // band tiles: dense rows (outside [0, n): zeros); then the cache's
+          const bool dense = i < kBandTiles;
+          const int y = dense ? j0 - 16 + i * kPfBN : row0 + (i - kBandTiles) * kPfBN;
           ok = mbar_wait(&k_empty[st], ((i >> 1) & 1) ^ 1);     // earlier uses of the stage: i >> 1
           if (!ok) break;
           mbar_arrive_expect_tx(&k_full[st], kPfKvTile);
 #pragma unroll
-          for (int p = 0; p < C::kPanels; ++p)
-            tma_load_2d(sK + st * kPfKvTile + p * kPfKvPanel, &tmK, &k_full[st], p * 64, y);
-          ok = mbar_wait(&v_empty[st], (i >> 1) & 1);           // the self tile + i >> 1 earlier tiles
+          for (int p = 0; p < C::kPanels; ++p) {
+            uint8_t *dst = sK + st * kPfKvTile + p * kPfKvPanel;
+            if (kBand && dense) tma_load_3d(dst, &tmKd, &k_full[st], p * 64, y, kv_slab);
+            else tma_load_2d(dst, &tmK, &k_full[st], p * 64, y);
+          }
+          ok = mbar_wait(&v_empty[st], ((i >> 1) + (kBand ? 1 : 0)) & 1);   // (the self tile +) i >> 1 earlier tiles
           if (!ok) break;
           mbar_arrive_expect_tx(&v_full[st], kPfKvTile);
 #pragma unroll
-          for (int p = 0; p < C::kPanels; ++p)
-            tma_load_2d(sV + st * kPfKvTile + p * kPfKvPanel, &tmV, &v_full[st], p * 64, y);
+          for (int p = 0; p < C::kPanels; ++p) {
+            uint8_t *dst = sV + st * kPfKvTile + p * kPfKvPanel;
+            if (kBand && dense) tma_load_3d(dst, &tmVd, &v_full[st], p * 64, y, kv_slab);
+            else tma_load_2d(dst, &tmV, &v_full[st], p * 64, y);
+          }
         }
       }
       // dense V rows for the self term of the output, into the K buffer once both stages are free
+      if (kBand) ok = false;
       if (ok && k0_uses > 0) ok = mbar_wait(&k_empty[0], (k0_uses & 1) ^ 1);
       if (ok && k1_uses > 0) ok = mbar_wait(&k_empty[1], (k1_uses & 1) ^ 1);
       if (ok) {
@@ -190,7 +210,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     // -------------------------------------------------------------- MMA issuer
     // Every lane runs the control flow so that operands stay warp-uniform (the tensor-core
     // instructions take uniform registers); one elected lane issues.
-    if (n_kv > 0) {
+    if (kBand || n_kv > 0) {
       // descriptors as (low, high) words: the high words are fixed per operand kind, the low
       // words are a base plus a compile-time offset per K step
       const uint64_t dq = desc_kmajor_sw128(smem_u32(sQ)), dk = desc_kmajor_sw128(smem_u32(sK));
@@ -201,7 +221,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       const uint32_t v_lo = (uint32_t)dv, v_hi = (uint32_t)(dv >> 32);
       constexpr uint32_t idesc_pv = idesc_bf16_f32(kPfBM, kPfD, false, true);
       // keys of cache tile i any row can see, rounded up to the MMA's N / K granularity
-      auto tile_keys = [&](int i) { return min(kPfBN, (max_bound - i * kPfBN + 15) & ~15); };
+      auto tile_keys = [&](int i) {
+        if (kBand && i < kBandTiles) return i == 2 ? 16 : kPfBN;
+        return min(kPfBN, (max_bound - (i - kBandTiles) * kPfBN + 15) & ~15);
+      };
       auto issue_qk = [&](int i) -> bool {
         const int st = i & 1;
         if (!mbar_wait(&k_full[st], (i >> 1) & 1)) return false;
@@ -224,8 +247,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       // self tile: 128 dense K rows (in the V stages); its scores land in the columns of O,
       // which are free until the first P V - that one starts a fresh accumulation, and it cannot
       // be issued before the softmax threads, who read the diagonal first, are done with tile 0
-      ok = ok && mbar_wait(&v_full[0], 0);
-      if (ok) {
+      if constexpr (!kBand) ok = ok && mbar_wait(&v_full[0], 0);
+      if (!kBand && ok) {
         tc_fence_after_sync();
         constexpr uint32_t idesc_self = idesc_bf16_f32(kPfBM, 128, false, false);
         const uint32_t s_lo = (uint32_t)dself, s_hi = (uint32_t)(dself >> 32);
@@ -251,7 +274,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const int st = i & 1;
         if (!mbar_wait(&p_ready[st], (i >> 1) & 1)) { ok = false; break; }
         // V stage 0 has held the self tile before (stage 1 shared that load's barrier)
-        if (!mbar_wait(&v_full[st], ((i >> 1) + (st == 0 ? 1 : 0)) & 1)) { ok = false; break; }
+        if (!mbar_wait(&v_full[st], ((i >> 1) + (!kBand && st == 0 ? 1 : 0)) & 1)) { ok = false; break; }
         tc_fence_after_sync();
         const int ksteps = tile_keys(i) / 16;
         const uint32_t vb = v_lo + ((st * kPfKvTile) >> 4);
@@ -276,10 +299,18 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const int L = a.len[kv_slab];
     const int bound = valid ? min(pre[j], L) : 0;
     const uint32_t tm_lane = tmem + ((uint32_t)(quad * 32) << 16);
-    float m = 0.f, self2 = 0.f, l = 1.f;
+    float m = kBand ? -INFINITY : 0.f, self2 = 0.f, l = kBand ? 0.f : 1.f;
     bool ok = true;
+    // kBand: bit b set = token j - 16 + b is seen through the window (bit 16: the token itself)
+    uint32_t seen = 1u << 16;
+    if (kBand && valid) {
+      const uint8_t *f = a.flags + (size_t)kv_slab * a.n + j;
+#pragma unroll
+      for (int back = 1; back <= 16; ++back)
+        if (back <= a.recent && back <= j && f[-back] == 0) seen |= 1u << (16 - back);
+    }
 
-    if (n_kv > 0) {
+    if (!kBand && n_kv > 0) {
       // self tile: this thread's diagonal element S[row][row] = q_j . k_j
       ok = mbar_wait(self_full, 0);
       tc_fence_after_sync();
@@ -297,12 +328,22 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       ok = mbar_wait(&s_full[st], (i >> 1) & 1);
       if (!ok) break;
       tc_fence_after_sync();
-      const int nvalid = min(max(bound - i * kPfBN, 0), kPfBN);
+      const bool dense = kBand && i < kBandTiles;
+      const int nvalid = min(max(bound - (i - kBandTiles) * kPfBN, 0), kPfBN);
       const uint32_t tS = tm_lane + kColS + st * kPfBN;
 
       uint32_t r[kPfBN];
       tmem_ld_x64_sync(tS, r);
-      if (nvalid < kPfBN) {
+      if (dense) {
+        // column e is token j0 - 16 + 64 i + e, i.e. bit e - (row - 64 i) of `seen`; row = j - j0
+        const int shift = row - i * kPfBN;            // -128 .. 127
+        const unsigned long long vis = shift >= 64 || shift <= -32 ? 0ull
+                                       : shift >= 0 ? (unsigned long long)seen << shift : (unsigned long long)(seen >> -shift);
+        const uint32_t vis_lo = (uint32_t)vis, vis_hi = (uint32_t)(vis >> 32);
+#pragma unroll
+        for (int e = 0; e < kPfBN; ++e)
+          if (!(((e < 32 ? vis_lo : vis_hi) >> (e & 31)) & 1u)) r[e] = 0xff800000u;
+      } else if (nvalid < kPfBN) {
 #pragma unroll
         for (int e = 0; e < kPfBN; ++e)
           if (e >= nvalid) r[e] = 0xff800000u;        // -inf: weight 0 below
@@ -322,13 +363,15 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       float m_new;
       if (i == 0) m_new = fmaxf(m, tmax);
       else m_new = (tmax > m + kRescaleThreshold) ? tmax : m;
-      const bool rescale = (i > 0) && __any_sync(0xffffffffu, m_new != m);
-      const float alpha = fast_exp2(m - m_new);
+      // kBand: a row may have met no key yet (m = -inf, O = 0, l = 0): nothing of it to rescale
+      const bool moved = m_new != m && (!kBand || m != -INFINITY);
+      const bool rescale = (i > 0) && __any_sync(0xffffffffu, moved);
+      const float alpha = kBand && m == -INFINITY ? 0.f : fast_exp2(m - m_new);
 
       // p = 2^(s - m) as bf16 pairs, written over the columns S occupied; the scaling and the row
       // sums two elements per instruction
       float rs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      const float neg_m = -m_new;
+      const float neg_m = kBand && m_new == -INFINITY ? 0.f : -m_new;
 #pragma unroll
       for (int c = 0; c < kPfBN / 16; ++c) {
         uint32_t pk[8];
@@ -368,11 +411,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       // Rows of the V tile past the slab's valid length hold whatever the pool
       // holds (possibly NaN bit patterns): their weight is 0, but 0 * NaN is NaN
       // in the tensor core, so zero them in shared memory before P V reads them.
-      if ((i + 1) * kPfBN > L) {
-        ok = mbar_wait(&v_full[st], ((i >> 1) + (st == 0 ? 1 : 0)) & 1);
+      // (Dense rows past the sequence's end are padding: the same.)
+      const int first = dense ? j0 - 16 + i * kPfBN : (i - kBandTiles) * kPfBN, rows_end = dense ? seq_len : L;
+      if (first + kPfBN > rows_end) {
+        ok = mbar_wait(&v_full[st], ((i >> 1) + (!kBand && st == 0 ? 1 : 0)) & 1);
         if (!ok) break;
         const int vr = tid >> 1;                      // two threads per row, one half each
-        if (i * kPfBN + vr >= L) {
+        if (first + vr >= rows_end) {
           uint4 z = make_uint4(0, 0, 0, 0);
           uint8_t *v0 = sV + st * kPfKvTile + vr * 128 + (tid & 1) * (kPfD == 128 ? kPfKvPanel : 64);
 #pragma unroll
@@ -391,11 +436,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       ok = mbar_wait(&pv_done[(n_kv - 1) & 1], ((n_kv - 1) >> 1) & 1);
       tc_fence_after_sync();
     }
-    if (ok) ok = mbar_wait(&k_full[0], k0_uses & 1);          // dense V tile has landed in sK
+    if (!kBand && ok) ok = mbar_wait(&k_full[0], k0_uses & 1);          // dense V tile has landed in sK
     if (ok) {
-      const float w_self = fast_exp2(self2 - m);
+      const float w_self = kBand ? 0.f : fast_exp2(self2 - m);
       const float inv = 1.f / l;
-      if (a.lse != nullptr && valid) a.lse[(size_t)slab * a.n + j] = n_kv > 0 ? m + log2f(l) : -INFINITY;
 #pragma unroll 1
       for (int c = 0; c < kPfD / 32; ++c) {
         uint32_t r[32];
@@ -408,8 +452,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
           const uint32_t off = tile_chunk_offset(row, c * 4 + g);
-          float vf[8];
-          Elem<__nv_bfloat16>::unpack(*reinterpret_cast<const uint4 *>(sK + off), vf);
+          float vf[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+          if (!kBand) Elem<__nv_bfloat16>::unpack(*reinterpret_cast<const uint4 *>(sK + off), vf);
           uint32_t o[4];
 #pragma unroll
           for (int e = 0; e < 8; e += 2) {
@@ -441,16 +485,16 @@ bool prefill_tc_supported(const ag_layer_desc &d, const ag_cache &c) {
          (int64_t)d.batch * d.heads * ((d.seq + kPfBM - 1) / kPfBM) < ((int64_t)1 << 31);
 }
 
-template <int kPfD>
-static int run_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const ag_cache &c,
-                          const int32_t *prefix, float scale, void *O, float *lse, cudaStream_t st) {
+template <int kPfD, bool kBand>
+static int run_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const uint8_t *flags,
+                          const ag_cache &c, const int32_t *prefix, float scale, void *O, cudaStream_t st) {
   const int slabs = d.batch * d.heads;
   CUtensorMap tmQ, tmKd, tmVd, tmO, tmK, tmV;
   int rc;
   if ((rc = make_tmap_3d_bf16(&tmQ, Q, slabs, d.seq, kPfD, kPfBM, 64))) return rc;
   const int kv_slabs = d.batch * kv_heads_of(d);
-  if ((rc = make_tmap_3d_bf16(&tmKd, K, kv_slabs, d.seq, kPfD, kPfBM, 64))) return rc;
-  if ((rc = make_tmap_3d_bf16(&tmVd, V, kv_slabs, d.seq, kPfD, kPfBM, 64))) return rc;
+  if ((rc = make_tmap_3d_bf16(&tmKd, K, kv_slabs, d.seq, kPfD, kBand ? kPfBN : kPfBM, 64))) return rc;
+  if ((rc = make_tmap_3d_bf16(&tmVd, V, kv_slabs, d.seq, kPfD, kBand ? kPfBN : kPfBM, 64))) return rc;
   if ((rc = make_tmap_3d_bf16(&tmO, O, slabs, d.seq, kPfD, kPfBM, 64))) return rc;
   // an empty pool still needs a valid map: describe one row of the dense K / V instead (never read)
   const bool empty = c.pool_rows == 0;
@@ -471,18 +515,20 @@ static int run_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, 
   if (bands < 1) bands = 1;
   a.band_slabs = (slabs + bands - 1) / bands;
   a.scale_log2 = scale * 1.4426950408889634f;
-  a.lse = lse;
+  a.flags = flags;
+  a.recent = recent_rows(d);
   a.seq_lens = d.seq_lens;
   constexpr int smem = PfCfg<kPfD>::kSmemBytes;
-  AG_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel<kPfD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  return launch_pdl(prefill_tc_kernel<kPfD>, dim3(a.n_qtiles * slabs), dim3(kPfThreads), smem, st, tmQ, tmKd, tmVd, tmO, tmK,
+  AG_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel<kPfD, kBand>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  return launch_pdl(prefill_tc_kernel<kPfD, kBand>, dim3(a.n_qtiles * slabs), dim3(kPfThreads), smem, st, tmQ, tmKd, tmVd, tmO, tmK,
                     tmV, a);
 }
 
-int launch_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const ag_cache &c,
-                      const int32_t *prefix, float scale, void *O, float *lse, cudaStream_t st) {
-  return d.head_dim == 64 ? run_prefill_tc<64>(d, Q, K, V, c, prefix, scale, O, lse, st)
-                          : run_prefill_tc<128>(d, Q, K, V, c, prefix, scale, O, lse, st);
+int launch_prefill_tc(const ag_layer_desc &d, const void *Q, const void *K, const void *V, const uint8_t *flags,
+                      const ag_cache &c, const int32_t *prefix, float scale, void *O, cudaStream_t st) {
+  auto run = recent_rows(d) > 0 ? (d.head_dim == 64 ? run_prefill_tc<64, true> : run_prefill_tc<128, true>)
+                                : (d.head_dim == 64 ? run_prefill_tc<64, false> : run_prefill_tc<128, false>);
+  return run(d, Q, K, V, flags, c, prefix, scale, O, st);
 }
 
 int prefill_tc_wait_timeouts() {
