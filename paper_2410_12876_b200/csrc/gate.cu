@@ -182,10 +182,9 @@ static int run_gate(const ag_layer_desc &d, const void *X, const void *Wq, const
   const float logit_tau = (float)log((double)d.tau / (1.0 - (double)d.tau));
   if (sizeof(T) == 2 && gate_attn_tc_supported(d)) {
     // tensor-core path: projections as bf16 parts, MHA' on tcgen05 with a product per pair of parts that matters.
-    // Padding is projected only as far as MHA' reads it: the causal one stops at the query tile (128 tokens)
-    // that holds a sequence's end, the bidirectional one visits every key tile.
+    // Padding is projected only as far as MHA' reads it, to the end of the 128-token tile a sequence ends in.
     const int parts = gate_attn_parts(d);
-    int rc = launch_gate_proj_tc(X, Wq, Wk, Wv, ws, parts, M, d.hidden, GD, d.gate_causal ? d.seq_lens : nullptr, d.seq, st);
+    int rc = launch_gate_proj_tc(X, Wq, Wk, Wv, ws, parts, M, d.hidden, GD, d.seq_lens, d.seq, st);
     if (rc) return rc;
     void *partials = static_cast<char *>(ws) + align_up((size_t)M * 3 * GD * 2 * parts, 256);   // H' stays on chip
     // the merge of the split-K partials carries the output layer and the threshold with it

@@ -16,7 +16,8 @@
 // Work is the list of all (query tile, key tile) steps, query tiles in order
 // and each one's key tiles in order.  The list is cut into equal segments, one
 // CTA (one SM) each, so every SM gets the same number of steps whatever the
-// shape of the causal triangle.  A segment crosses query tiles: the CTA handles
+// shape of the causal triangle or the lengths of the sequences (a padded batch: the list holds the sequences' own
+// tiles only; it is laid out on the device, from the lengths).  A segment crosses query tiles: the CTA handles
 // its pieces one after the other, the loads of the next piece running under the
 // tail of the current one.  Every piece leaves an un-normalised partial
 // (O, m, l); gate_merge_out_kernel combines the pieces of a query tile and
@@ -59,69 +60,138 @@ constexpr uint32_t kGaColS = 0, kGaTmemCols = 512;
 constexpr float kGaRescaleThreshold = 8.f;
 
 constexpr int kGaMaxSeg = 256;       // segments at most (one per SM)
-constexpr int kGaPieceCost = 3;      // set-up + epilogue of a piece, in half tile steps
+constexpr int kGaOverhead = 2;       // set-up + epilogue of a query tile, in key tiles (even)
 
+// The list of work: for every sequence b, gate head g and query tile q of the sequence's own length, kGaOverhead places
+// that stand for the tile's set-up and epilogue and one place per key tile.  The list is cut into n_seg segments
+// of equal length; the key tiles of a query tile inside a segment are a piece.  All lengths are even, so a piece
+// starts on a 128-key boundary and its first tile holds a key every row of the query tile may see.
 struct GateAttnArgs {
   const int32_t *seq_lens;  // [B] or NULL: tokens past seq_lens[b] are padding
   float *part_o;            // [items, 128, D] un-normalised partial outputs
   float *part_ml;           // [items, 128, 2]   running max (log2 units) and sum per row
-  int n, n_qtiles, gate_heads, problems, GD, causal;
-  int steps_per_prob;       // (query tile, key tile) steps of one (sequence, head)
-  int total_steps;          // over all problems
+  int n, n_qtiles, batch, gate_heads, GD, causal;
   int n_seg;                // segments (= CTAs of the attention kernel)
-  // Segment s covers steps [seg_begin[s], seg_begin[s + 1]) of the list.  Every boundary is even: a
-  // piece starts on a 128-key boundary, so its first tile holds a key every row of the query tile
-  // may see.  Segments are cut to equal cost, a piece counting as much as kGaPieceCost / 2 steps.
-  int seg_begin[kGaMaxSeg + 1];
   float scale_log2;
 };
 
 // One map per part (all 3 encoded): boxes of a query tile's rows and of a key tile's.
 struct GateAttnMaps { CUtensorMap q[3], kv[3]; };
 
-// Key tiles query tile qt attends to, and the work items they are cut into.
-// (key tiles hold 64 keys, query tiles 128 queries)
-__host__ __device__ inline int ga_key_tiles(int qt, int n_qtiles, int causal) {
-  return (kGaBM / kGaBN) * (causal ? qt + 1 : n_qtiles);
+// Key tiles (64 keys) of query tile q (128 queries) of a sequence of nq query tiles, and list places: of the tile,
+// before the tile within its (sequence, gate head), and of a whole (sequence, gate head).
+__host__ __device__ inline int ga_key_tiles(int q, int nq, int causal) { return 2 * (causal ? q + 1 : nq); }
+__host__ __device__ inline int ga_tile_places(int q, int nq, int causal) { return ga_key_tiles(q, nq, causal) + kGaOverhead; }
+__host__ __device__ inline int ga_places_before(int q, int nq, int causal) {
+  return causal ? q * (q + 1) + kGaOverhead * q : q * (2 * nq + kGaOverhead);
 }
-// First step of query tile qt within its problem's list.
-__host__ __device__ inline int ga_first_step(int qt, int n_qtiles, int causal) {
-  return causal ? qt * (qt + 1) : qt * 2 * n_qtiles;
+__host__ __device__ inline int ga_head_places(int nq, int causal) { return ga_places_before(nq, nq, causal); }
+__device__ inline int ga_seq_tiles(const GateAttnArgs &a, int b) {
+  return a.seq_lens == nullptr ? a.n_qtiles : (min(max(a.seq_lens[b], 0), a.n) + kGaBM - 1) / kGaBM;
 }
-// The piece of a segment that starts at global step x (x < x_end, the segment's end).
-struct GaPiece {
-  int prob, qt, kv_begin, n_kv;
-};
-__device__ inline GaPiece ga_piece(const GateAttnArgs &a, int x, int x_end) {
-  GaPiece p;
-  p.prob = x / a.steps_per_prob;
-  const int y = x - p.prob * a.steps_per_prob;
-  if (a.causal) {
-    int qt = (int)((sqrtf(4.f * (float)y + 1.f) - 1.f) * 0.5f);
-    while (qt > 0 && qt * (qt + 1) > y) --qt;
-    while ((qt + 1) * (qt + 2) <= y) ++qt;
-    p.qt = qt;
+__device__ inline int ga_seg_len(const GateAttnArgs &a, int total) {
+  return max(2 * kGaOverhead, ((total + a.n_seg - 1) / a.n_seg + 1) & ~1);
+}
+// Whole-warp call: places of the list in all, and before sequence b_end.
+__device__ inline int ga_total(const GateAttnArgs &a, int b_end, int &before) {
+  if (a.seq_lens == nullptr) {
+    const int per = a.gate_heads * ga_head_places(a.n_qtiles, a.causal);
+    before = b_end * per;
+    return a.batch * per;
+  }
+  int total = 0, bef = 0;
+  for (int b = threadIdx.x & 31; b < a.batch; b += 32) {
+    const int v = a.gate_heads * ga_head_places(ga_seq_tiles(a, b), a.causal);
+    total += v;
+    if (b < b_end) bef += v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    total += __shfl_xor_sync(0xffffffffu, total, o);
+    bef += __shfl_xor_sync(0xffffffffu, bef, o);
+  }
+  before = bef;
+  return total;
+}
+
+// Where a CTA stands in the list: sequence, gate head, query tile of nq, place within the tile, places left.
+struct GaWalk { int b, g, q, nq, v, left; };
+struct GaPiece { int b, g, qt, kv_begin, n_kv; };
+// Whole-warp call: the start of segment seg.
+__device__ inline GaWalk ga_start(const GateAttnArgs &a, int seg) {
+  GaWalk w = {};
+  int before;
+  const int total = ga_total(a, 0, before), len = ga_seg_len(a, total);
+  int x = seg * len;
+  w.left = min(len, total - x);
+  if (w.left <= 0) return w;
+  if (a.seq_lens == nullptr) {
+    const int per = a.gate_heads * ga_head_places(a.n_qtiles, a.causal);
+    w.b = x / per;
+    x -= w.b * per;
   } else {
-    p.qt = y / (2 * a.n_qtiles);
+    const int lane = threadIdx.x & 31;
+    for (int b0 = 0;; b0 += 32) {                    // (x < total: some sequence holds it)
+      const int v = b0 + lane < a.batch ? a.gate_heads * ga_head_places(ga_seq_tiles(a, b0 + lane), a.causal) : 0;
+      int incl = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
+      }
+      const unsigned past = __ballot_sync(0xffffffffu, incl > x);
+      if (past != 0) {
+        const int l = __ffs(past) - 1;
+        w.b = b0 + l;
+        x -= __shfl_sync(0xffffffffu, incl - v, l);
+        break;
+      }
+      x -= __shfl_sync(0xffffffffu, incl, 31);
+      if (b0 + 32 >= a.batch) { w.left = 0; return w; }
+    }
   }
-  p.kv_begin = y - ga_first_step(p.qt, a.n_qtiles, a.causal);
-  const int tile_end = x - p.kv_begin + ga_key_tiles(p.qt, a.n_qtiles, a.causal);   // global end of the query tile
-  p.n_kv = min(x_end, tile_end) - x;
-  return p;
-}
-// A piece whose query tile lies wholly in its sequence's padding: nothing to compute (every role
-// skips it the same way; the softmax role leaves an empty partial for the merge).
-__device__ inline bool ga_padding_only(const GateAttnArgs &a, const GaPiece &p) {
-  return a.seq_lens != nullptr && p.qt * kGaBM >= a.seq_lens[p.prob / a.gate_heads];
-}
-// Segment that holds global step x.
-__device__ inline int ga_segment_of(const GateAttnArgs &a, int x) {
-  int lo = 0, hi = a.n_seg - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (a.seg_begin[mid] <= x) lo = mid; else hi = mid - 1;
+  w.nq = ga_seq_tiles(a, w.b);
+  const int head = ga_head_places(w.nq, a.causal);
+  w.g = x / head;
+  const int y = x - w.g * head;
+  if (a.causal) {
+    int q = (int)((sqrtf(4.f * (float)y + 9.f) - 3.f) * 0.5f);      // q (q + 1) + 2 q = y
+    while (q > 0 && ga_places_before(q, w.nq, 1) > y) --q;
+    while (ga_places_before(q + 1, w.nq, 1) <= y) ++q;
+    w.q = q;
+  } else {
+    w.q = y / ga_tile_places(0, w.nq, 0);
   }
-  return lo;
+  w.v = y - ga_places_before(w.q, w.nq, a.causal);
+  return w;
+}
+// The next piece of the segment; false at its end.
+__device__ inline bool ga_next(const GateAttnArgs &a, GaWalk &w, GaPiece &p) {
+  while (w.left > 0) {
+    const int tile = ga_tile_places(w.q, w.nq, a.causal), end = min(tile, w.v + w.left);
+    const int k0 = max(w.v - kGaOverhead, 0);
+    p.b = w.b; p.g = w.g; p.qt = w.q;
+    p.kv_begin = k0;
+    p.n_kv = end - kGaOverhead - k0;
+    w.left -= end - w.v;
+    w.v = end;
+    if (end == tile) {
+      w.v = 0;
+      if (++w.q == w.nq) {
+        w.q = 0;
+        if (++w.g == a.gate_heads) {
+          w.g = 0;
+          do {
+            ++w.b;
+            w.nq = w.b < a.batch ? ga_seq_tiles(a, w.b) : 0;
+          } while (w.nq == 0 && w.b < a.batch);
+          if (w.nq == 0) w.left = 0;
+        }
+      }
+    }
+    if (p.n_kv > 0) return true;
+  }
+  return false;
 }
 // Partial slot of the piece of query tile (prob, qt) that lies in segment seg: consecutive pieces
 // differ in the query tile, the segment or both, so the sum is unique and grows along the list.
@@ -150,11 +220,9 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 17);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // This CTA's segment of the step list.  Every role walks its pieces with the same arithmetic;
+  // Every role walks the pieces of this CTA's segment with the same arithmetic;
   // tiles are numbered t = 0, 1, ... across the pieces (stage and S buffer t & 1, in their use
   // number t >> 1; P and the P V barrier in their use number t), pieces pc = 0, 1, ...
-  const int x_begin = a.seg_begin[blockIdx.x];
-  const int x_end = a.seg_begin[blockIdx.x + 1];
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -181,15 +249,15 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
   const uint32_t tmem = *tmem_slot;
   pdl_wait();                                        // the projections are there
   pdl_launch_dependents();
+  GaWalk walk = ga_start(a, (int)blockIdx.x);
+  GaPiece pz;
 
   if (warp == 0) {
     if (lane == 0) {
       bool ok = true;
       int t = 0;
-      for (int x = x_begin, pc = 0; x < x_end && ok; ++pc) {      // pc counts the pieces that are computed
-        const GaPiece pz = ga_piece(a, x, x_end);
-        if (ga_padding_only(a, pz)) { x += pz.n_kv; --pc; continue; }
-        const int b = pz.prob / a.gate_heads, g = pz.prob % a.gate_heads, j0 = pz.qt * kGaBM;
+      for (int pc = 0; ok && ga_next(a, walk, pz); ++pc) {
+        const int b = pz.b, g = pz.g, j0 = pz.qt * kGaBM;
         const int xq = g * kGaD, xk = a.GD + g * kGaD, xv = 2 * a.GD + g * kGaD;   // columns in [Q' | K' | V']
         ok = mbar_wait(q_empty, (pc & 1) ^ 1);       // the previous piece's last Q K^T has read Q
         if (!ok) break;
@@ -216,7 +284,6 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
           if (!mbar_wait(&v_empty[st], ph ^ 1)) { ok = false; break; }
           load_kv(sV + st * kGaKvStage, &v_full[st], xv, y);
         }
-        x += pz.n_kv;
       }
     }
   } else if (warp == 1) {
@@ -252,10 +319,8 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
     };
     bool ok = true;
     int t0 = 0;                                      // tile number of the piece's first tile
-    for (int x = x_begin, pc = 0; x < x_end && ok; ++pc) {        // pc counts the pieces that are computed
-      const GaPiece pz = ga_piece(a, x, x_end);
+    for (int pc = 0; ok && ga_next(a, walk, pz); ++pc) {
       const int n_kv = pz.n_kv;
-      if (ga_padding_only(a, pz)) { x += n_kv; --pc; continue; }
       ok = mbar_wait(q_full, pc & 1);
       ok = ok && issue_qk(t0, n_kv == 1);
       for (int i = 0; i < n_kv && ok; ++i) {
@@ -284,7 +349,6 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
       __syncwarp();
       }
       t0 += n_kv;
-      x += n_kv;
     }
   } else {
     const int quad = warp & 3;
@@ -293,29 +357,15 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
     bool ok = true;
     int t0 = 0;                                      // tile number of the piece's first tile
 
-    for (int x = x_begin; x < x_end && ok;) {
-    const GaPiece pz = ga_piece(a, x, x_end);
+    while (ok && ga_next(a, walk, pz)) {
     const int n_kv = pz.n_kv, kv_begin = pz.kv_begin;
     const int j = pz.qt * kGaBM + row;
     const bool valid = j < a.n;
     const int jc = min(j, a.n - 1);
     // keys below bound are visible (bidirectional: the sequence's own tokens, not its padding)
-    const int seq_len = a.seq_lens ? a.seq_lens[pz.prob / a.gate_heads] : a.n;
+    const int seq_len = a.seq_lens ? a.seq_lens[pz.b] : a.n;
     const int bound = a.causal ? jc + 1 : seq_len;
     float m = -INFINITY, l = 0.f;
-    if (ga_padding_only(a, pz)) {
-      // padding only: an empty partial (weight 0 in the merge; the merge gives padding flag 0 anyway)
-      const size_t it = (size_t)ga_slot(pz.prob, pz.qt, a.n_qtiles, (int)blockIdx.x);
-      if (valid) {
-        float *op = a.part_o + (it * kGaBM + row) * kGaD;
-#pragma unroll 4
-        for (int e = 0; e < kGaD; e += 4) *reinterpret_cast<uint4 *>(op + e) = make_uint4(0, 0, 0, 0);
-        *reinterpret_cast<float2 *>(a.part_ml + (it * kGaBM + row) * 2) = make_float2(m, l);
-      }
-      x += n_kv;
-      continue;
-    }
-
     for (int i = 0; i < n_kv && ok; ++i) {
       const int t = t0 + i;
       ok = mbar_wait(&s_full[t & 1], (t >> 1) & 1);
@@ -406,7 +456,7 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
       tc_fence_after_sync();
     }
     if (ok) {
-      const size_t it = (size_t)ga_slot(pz.prob, pz.qt, a.n_qtiles, (int)blockIdx.x);
+      const size_t it = (size_t)ga_slot(pz.b * a.gate_heads + pz.g, pz.qt, a.n_qtiles, (int)blockIdx.x);
       float *op = a.part_o + (it * kGaBM + row) * kGaD;
 #pragma unroll 1
       for (int c = 0; c < kGaD / 32; ++c) {
@@ -425,7 +475,6 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
       if (valid) *reinterpret_cast<float2 *>(a.part_ml + (it * kGaBM + row) * 2) = make_float2(m, l);
     }
     t0 += n_kv;
-    x += n_kv;
     }
   }
   tc_fence_before_sync();
@@ -502,18 +551,17 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
       if (t0 + tok < a.n) flags[((size_t)b * h + i) * a.n + t0 + tok] = 0;
     return;
   }
-  // The CTA's 16 tokens lie in one query tile: which segments hold its pieces is looked up once per
-  // gate head (a binary search over the boundaries in constant memory), by one thread each.
-  {
-    const int qt = t0 / kGaBM;
-    const int y0 = ga_first_step(qt, a.n_qtiles, a.causal), y1 = y0 + ga_key_tiles(qt, a.n_qtiles, a.causal);
-    for (int g = threadIdx.x; g < a.gate_heads; g += kMoThreads) {
-      const int prob = b * a.gate_heads + g;
-      // the query tile's steps [x0, x1) of the list lie in segments seg0 .. seg1, one piece in each
-      const int x0 = prob * a.steps_per_prob + y0, x1 = prob * a.steps_per_prob + y1;
-      const int seg0 = ga_segment_of(a, x0);
-      seg_first[0][g] = seg0;
-      seg_first[1][g] = ga_segment_of(a, x1 - 1) - seg0 + 1;
+  // The CTA's 16 tokens lie in one query tile: which segments hold its pieces is looked up once per gate head.
+  if (warp == 0) {
+    const int qt = t0 / kGaBM, nq = ga_seq_tiles(a, b);
+    int before;
+    const int len = ga_seg_len(a, ga_total(a, b, before));
+    for (int g = lane; g < a.gate_heads; g += 32) {
+      // the query tile's key tiles [x0, x1) of the list lie in consecutive segments, one piece in each
+      const int x0 = before + g * ga_head_places(nq, a.causal) + ga_places_before(qt, nq, a.causal) + kGaOverhead;
+      const int x1 = x0 + ga_key_tiles(qt, nq, a.causal);
+      seg_first[0][g] = x0 / len;
+      seg_first[1][g] = (x1 - 1) / len - x0 / len + 1;
     }
   }
   __syncthreads();
@@ -635,41 +683,8 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
   }
 }
 
-// Cuts the step list into at most `n_target` segments of about equal cost (2 per tile step,
-// kGaPieceCost per piece) and writes their boundaries; returns the number of segments.
-static int cut_segments(int problems, int nq, int causal, int n_target, int target, int *seg_begin) {
-  int n = 0, cur = 0, x = 0;
-  seg_begin[n++] = 0;
-  for (int prob = 0; prob < problems; ++prob)
-    for (int qt = 0; qt < nq; ++qt) {
-      int r = ga_key_tiles(qt, nq, causal);
-      while (r > 0) {
-        if (cur > 0 && cur + kGaPieceCost + 4 > target) {      // not even a two-tile piece fits: new segment
-          if (n >= n_target) return n_target + 1;
-          seg_begin[n++] = x;
-          cur = 0;
-        }
-        cur += kGaPieceCost;
-        int fit = ((target - cur) / 2) & ~1;
-        if (fit < 2) fit = 2;
-        const int take = r < fit ? r : fit;
-        cur += 2 * take; x += take; r -= take;
-        if (r > 0) {                                           // segment full inside the query tile
-          if (n >= n_target) return n_target + 1;
-          seg_begin[n++] = x;
-          cur = 0;
-        }
-      }
-    }
-  seg_begin[n] = x;
-  return n;                                                    // seg_begin[0 .. n]
-}
-
-struct GateAttnPlan {
-  int steps_per_prob, total_steps, n_seg;
-  int seg_begin[kGaMaxSeg + 1];
-};
-static int gate_attn_plan(const ag_layer_desc &d, GateAttnPlan &p) {
+// Segments of the list: one per SM.
+static int gate_attn_segments(const ag_layer_desc &d, int *n_seg) {
   static int sm_count[64] = {0};                     // per device, read once
   int dev = 0;
   AG_CUDA_TRY(cudaGetDevice(&dev));
@@ -679,22 +694,10 @@ static int gate_attn_plan(const ag_layer_desc &d, GateAttnPlan &p) {
     AG_CUDA_TRY(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
     sm_count[dev] = v < 1 ? 1 : (v > kGaMaxSeg ? kGaMaxSeg : v);
   }
-  const int nq = (d.seq + kGaBM - 1) / kGaBM, problems = d.batch * d.gate_heads;
-  const long long per = d.gate_causal ? (long long)nq * (nq + 1) : 2LL * nq * nq;
-  const long long total = per * problems;
-  if (total >= (1LL << 28)) return AG_ERR_UNSUPPORTED;
-  p.steps_per_prob = (int)per;
-  p.total_steps = (int)total;
-  const int n_target = sm_count[dev];
-  // cost per segment: raised until the cuts fit into n_target segments
-  long long target = (2 * total + (long long)kGaPieceCost * ((long long)problems * nq + n_target) + n_target - 1) / n_target;
-  if (target < kGaPieceCost + 4) target = kGaPieceCost + 4;
-  for (;;) {
-    p.n_seg = cut_segments(problems, nq, d.gate_causal, n_target, (int)target, p.seg_begin);
-    if (p.n_seg <= n_target) break;
-    target += 1 + target / 64;
-  }
-  return AG_OK;
+  *n_seg = sm_count[dev];
+  const long long nq = (d.seq + kGaBM - 1) / kGaBM;
+  const long long head = d.gate_causal ? nq * (nq + 1 + kGaOverhead) : nq * (2 * nq + kGaOverhead);
+  return head * d.batch * d.gate_heads < (1LL << 28) ? AG_OK : AG_ERR_UNSUPPORTED;
 }
 
 size_t gate_attn_partial_bytes(const ag_layer_desc &d) {
@@ -721,18 +724,15 @@ static int run_gate_attn_tc(const ag_layer_desc &d, const void *qkv, void *parti
   GateAttnArgs a;
   a.seq_lens = d.seq_lens;
   a.n = d.seq; a.n_qtiles = (d.seq + kGaBM - 1) / kGaBM;
-  a.gate_heads = d.gate_heads; a.problems = d.batch * d.gate_heads; a.GD = GD; a.causal = d.gate_causal;
-  static thread_local GateAttnPlan plan;             // 1 KB of boundaries: not on the stack of every call
-  if ((rc = gate_attn_plan(d, plan))) return rc;
-  a.steps_per_prob = plan.steps_per_prob; a.total_steps = plan.total_steps; a.n_seg = plan.n_seg;
-  for (int i = 0; i <= plan.n_seg; ++i) a.seg_begin[i] = plan.seg_begin[i];
-  const size_t slots = (size_t)a.problems * a.n_qtiles + kGaMaxSeg;
+  a.batch = d.batch; a.gate_heads = d.gate_heads; a.GD = GD; a.causal = d.gate_causal;
+  if ((rc = gate_attn_segments(d, &a.n_seg))) return rc;
+  const size_t slots = (size_t)d.batch * d.gate_heads * a.n_qtiles + kGaMaxSeg;
   a.part_o = static_cast<float *>(partials);
   a.part_ml = reinterpret_cast<float *>(static_cast<char *>(partials) +
                                         align_up(slots * kGaBM * kGaD * sizeof(float), 256));
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)kGaD));
   AG_CUDA_TRY(cudaFuncSetAttribute(gate_attn_tc_kernel<kGaD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGaSmemBytes));
-  rc = launch_pdl(gate_attn_tc_kernel<kGaD>, dim3(plan.n_seg), dim3(kGaThreads), kGaSmemBytes, st, tm, a);
+  rc = launch_pdl(gate_attn_tc_kernel<kGaD>, dim3(a.n_seg), dim3(kGaThreads), kGaSmemBytes, st, tm, a);
   if (rc) return rc;
   auto mo = gate_merge_out_kernel<kGaD>;
   AG_CUDA_TRY(cudaFuncSetAttribute(mo, cudaFuncAttributeMaxDynamicSharedMemorySize, mo_smem_bytes(GD)));
