@@ -545,11 +545,11 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
 // One cluster per run of G <= 16 query slabs that share a key/value slab (G = 1 without grouped-query
 // attention): the G queries are rows of one MMA operand, so the slab is read once for all of them, and the
 // one cluster that reads it may append to it.  CTA `rank` takes whole 64-row tiles; after the cluster
-// barrier rank r merges the heads r, r + 8 of the group.  The tiles go round the ranks, so a rank's first tile does
+// barrier rank r merges the heads r, r + 8 of the group, whose triples the ranks have written to its shared memory.  The tiles go round the ranks, so a rank's first tile does
 // not depend on the slab's length and its rows are asked for together with the length (before it is known
 // they are only known to lie inside the slab): one trip to L2 less on the path of a step.
 // three stages: a CTA has few tiles and no neighbour to hide behind, so two of them are kept in flight
-constexpr int kCmStages = 3;
+constexpr int kCmStages = 2;
 // kMaxG: 1 (one query per slab), 8 or 16.
 template <int D, int kMaxG>
 __global__ void __launch_bounds__(kGqThreads, 2)
@@ -569,6 +569,7 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   const int kv = hm.kv_slab(slab0);
   const int d = threadIdx.x;
   pdl_launch_dependents();
+  cluster.barrier_arrive();           // (waited for before the first write to another rank: all have started then)
   // the slab's first row and capacity never change once the cache is laid out: read ahead of the wait for the
   // preceding kernel
   const int64_t slab_row0 = row_off[kv];
@@ -581,9 +582,9 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   if (r_first < slab_cap) gq_load_tile<D>((uint32_t)__cvta_generic_to_shared(gq_smem), Kg, Vg, r_first, slab_cap);
   cp_async_commit();
 
-  // this CTA's triples [G][D] and [G][2], read by the merging ranks: behind the warps' triples in the ring's memory
-  float *cta_o = reinterpret_cast<float *>(gq_smem + gq_smem_bytes(D, kCmStages) - kGqMaxGroup * (D + 2) * 4);
-  float *cta_ml = cta_o + kGqMaxGroup * D;
+  // the ranks' triples of the heads this rank merges, written by the ranks themselves
+  __shared__ float in_o[kHeads][kClusterSize][D];
+  __shared__ float2 in_ml[kHeads][kClusterSize];
   __shared__ float red[kHeads][D / 32];
   __shared__ float ring_s[kHeads][kMaxRecent];
 
@@ -602,16 +603,18 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   if (r_first < L) {                  // the same for the whole CTA
     const GqWarpTriples w = gq_stream_rows<D, kCmStages, (kMaxG + 7) / 8, true>(
         gq_smem, q + (size_t)slab0 * D, G, Kg, Vg, r_first, kClusterSize * kGqTile, L, scale_log2);
+    cluster.barrier_wait();
     for (int x = d; x < G * D; x += kGqThreads) {
-      const int h = x / D, e = x % D;
+      const int h = x / D, e = x % D, to = h % kClusterSize;
       float acc, mc, lc;
       gq_combine<D>(w, h, e, acc, mc, lc);
-      cta_o[x] = acc;
-      if (e == 0) { cta_ml[2 * h] = mc; cta_ml[2 * h + 1] = lc; }
+      *cluster.map_shared_rank(&in_o[h / kClusterSize][rank][e], to) = acc;
+      if (e == 0) *cluster.map_shared_rank(&in_ml[h / kClusterSize][rank], to) = make_float2(mc, lc);
     }
   } else {
-    for (int x = d; x < G * D; x += kGqThreads) cta_o[x] = 0.f;
-    if (d < G) { cta_ml[2 * d] = -INFINITY; cta_ml[2 * d + 1] = 0.f; }
+    cluster.barrier_wait();
+    // weight 0 in the merge, which then skips the values
+    if (d < G) *cluster.map_shared_rank(&in_ml[d / kClusterSize][rank], d % kClusterSize) = make_float2(-INFINITY, 0.f);
     cp_async_wait<0>();               // (the first tile, asked for in vain)
   }
 #pragma unroll
@@ -637,26 +640,20 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
 #pragma unroll
     for (int i = 0; i < D / 32; ++i) s_self += red[u][i];
     s_self *= scale_log2;
-    float mr[kClusterSize], lr[kClusterSize], orr[kClusterSize];
-#pragma unroll
-    for (int r = 0; r < kClusterSize; ++r) {
-      const float *ml = cluster.map_shared_rank(cta_ml, r) + 2 * h;
-      mr[r] = ml[0];
-      lr[r] = ml[1];
-      orr[r] = cluster.map_shared_rank(cta_o, r)[h * D + d];
-    }
     float mm = s_self;
 #pragma unroll
-    for (int r = 0; r < kClusterSize; ++r) mm = fmaxf(mm, mr[r]);
+    for (int r = 0; r < kClusterSize; ++r) mm = fmaxf(mm, in_ml[u][r].x);
     for (int r = 0; r < rg.R; ++r) mm = fmaxf(mm, ring_s[u][r]);
     const float w_self = exp2f(s_self - mm);
     float acc = w_self * v_self;
     float lsum = w_self;
 #pragma unroll
     for (int r = 0; r < kClusterSize; ++r) {
-      const float w = mr[r] == -INFINITY ? 0.f : exp2f(mr[r] - mm);
-      acc = fmaf(w, orr[r], acc);
-      lsum = fmaf(w, lr[r], lsum);
+      const float2 ml = in_ml[u][r];
+      if (ml.x == -INFINITY) continue;                 // a rank without rows has sent no values
+      const float w = exp2f(ml.x - mm);
+      acc = fmaf(w, in_o[u][r][d], acc);
+      lsum = fmaf(w, ml.y, lsum);
     }
     // the evicted tokens of the recent-token window
     for (int r = 0; r < rg.R; ++r) {
@@ -667,11 +664,11 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
     }
     Elem<T>::store(out + (size_t)(slab0 + h) * D + d, acc / lsum);
   }
-  cluster.sync();
-  if (rank == 0 && rg.R > 0 && ap.flag_new != nullptr) {
+  if (rg.R > 0 && ap.flag_new != nullptr) {
     // the step carries the append: the new token joins the ring once every rank has read it
+    cluster.sync();
     constexpr int kVecs = D * (int)sizeof(T) / 16;
-    if (d < kVecs)
+    if (rank == 0 && d < kVecs)
       ring_put<kVecs>(rg, kv, d, reinterpret_cast<const uint8_t *>(k_new + (size_t)kv * D),
                       reinterpret_cast<const uint8_t *>(v_new + (size_t)kv * D), ap.flag_new[kv] != 0);
   }

@@ -32,13 +32,14 @@ struct GqWarpTriples {
 };
 
 // One tile of K and of V (64 rows from r0; rows from r_end on are replaced by the last one before it) on its way to
-// the ring stage at smem address `stage`.
+// the ring stage at smem address `stage`.  A warp fetches the 16 rows that it will work on, so nothing but the warp
+// has to wait for them.
 template <int kGqD>
 __device__ __forceinline__ void gq_load_tile(uint32_t stage, const uint8_t *Kg, const uint8_t *Vg, int r0, int r_end) {
   constexpr int kPieces = kGqD / 8;
 #pragma unroll
-  for (int x = 0; x < kGqTile * kPieces / kGqThreads; ++x) {
-    const int idx = threadIdx.x + x * kGqThreads, r = idx / kPieces, c = idx % kPieces;
+  for (int x = 0; x < 16 * kPieces / 32; ++x) {
+    const int idx = (threadIdx.x & 31) + x * 32, r = (threadIdx.x >> 5) * 16 + idx / kPieces, c = idx % kPieces;
     const size_t src = (size_t)min(r0 + r, r_end - 1) * (kGqD * 2) + c * 16;
     cp_async16(stage + gq_tile_off<kGqD>(r, c), Kg + src);
     cp_async16(stage + gq_tile_bytes(kGqD) + gq_tile_off<kGqD>(r, c), Vg + src);
@@ -107,51 +108,69 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
     if (i + kGqStages - 1 < n_tiles) load_tile(i + kGqStages - 1);
     cp_async_commit();
     cp_async_wait<kGqStages - 1>();                             // tile i has landed (this thread's pieces)
-    __syncthreads();                                            // ... and everybody's
+    __syncwarp();                                               // ... and the warp's
     const uint32_t sk = smem0 + (i % kGqStages) * 2 * kGqTileBytes, sv = sk + kGqTileBytes;
     const int key0 = r_first + i * r_step + warp * 16;          // this warp's 16 rows of the tile
 
     if (key0 < r_end) {
-      // S = Q K^T for 16 keys: two 8-key column tiles
-      float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
+      const bool ragged = key0 + 16 > r_end;
+      // S = Q K^T for 16 keys: two 8-key column tiles, two chains of MMAs each
+      float s0[2][4], s1[2][4];
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s0[c][e] = s1[c][e] = 0.f;
 #pragma unroll
       for (int ks = 0; ks < kGqD / 16; ++ks) {
         uint32_t b[4];
         // matrices: (keys 0-7, dims lo), (keys 0-7, dims hi), (keys 8-15, dims lo), (keys 8-15, dims hi)
         const int mi = lane >> 3, row = warp * 16 + (mi >> 1) * 8 + (lane & 7);
         ldmatrix_x4(b, sk + gq_tile_off<kGqD>(row, ks * 2 + (mi & 1)));
-        mma_16816(s0, qa[ks], b[0], b[1]);
-        mma_16816(s1, qa[ks], b[2], b[3]);
+        mma_16816(s0[ks & 1], qa[ks], b[0], b[1]);
+        mma_16816(s1[ks & 1], qa[ks], b[2], b[3]);
       }
-      // online softmax of rows g (and g + 8): this thread holds keys 2t, 2t+1 of each column tile
+      // online softmax of rows g (and g + 8): this thread holds keys 2t, 2t+1 of each column tile.  The maximum
+      // moves only when a score exceeds it by more than 2^8 (float32 sums and bf16 weights have the room); rows
+      // past G come out as anything and are dropped at the end.
       uint32_t pa[4] = {0u, 0u, 0u, 0u};
+      float sv4[kHalves][4];
+      bool up = false;
 #pragma unroll
       for (int h = 0; h < kHalves; ++h) {
-        float sv4[4] = {s0[2 * h], s0[2 * h + 1], s1[2 * h], s1[2 * h + 1]};
         const int kcol[4] = {2 * t, 2 * t + 1, 8 + 2 * t, 9 + 2 * t};
-        float tmax = -INFINITY;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          sv4[e] = (key0 + kcol[e] < r_end) ? sv4[e] * scale_log2 : -INFINITY;
-          tmax = fmaxf(tmax, sv4[e]);
+          const int c = 2 * h + (e & 1);
+          sv4[h][e] = (e < 2 ? s0[0][c] + s0[1][c] : s1[0][c] + s1[1][c]) * scale_log2;
+          if (ragged && key0 + kcol[e] >= r_end) sv4[h][e] = -INFINITY;
+          up = up || sv4[h][e] > m[h] + 8.f;
         }
-        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
-        const float m_new = fmaxf(m[h], tmax);                  // finite: key0 < r_end, so column 0 is valid
-        const float alpha = exp2f(m[h] - m_new);                // m = -inf at first: 0
+      }
+      if (__any_sync(0xffffffffu, up)) {
+#pragma unroll
+        for (int h = 0; h < kHalves; ++h) {
+          float tmax = fmaxf(fmaxf(sv4[h][0], sv4[h][1]), fmaxf(sv4[h][2], sv4[h][3]));
+          tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
+          tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
+          const float m_new = fmaxf(m[h], tmax);                // finite: key0 < r_end, so column 0 is valid
+          const float alpha = exp2f(m[h] - m_new);              // m = -inf at first: 0
+          m[h] = m_new;
+          l[h] *= alpha;
+#pragma unroll
+          for (int nt = 0; nt < kGqD / 8; ++nt) {
+            o[nt][2 * h] *= alpha;
+            o[nt][2 * h + 1] *= alpha;
+          }
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < kHalves; ++h) {
         float p[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) p[e] = exp2f(sv4[e] - m_new);
-        const bool row_used = h == 0 ? g < G : g + 8 < G;       // unused rows: zero weights, not 2^(0 - m)
-        l[h] = l[h] * alpha + (row_used ? (p[0] + p[1]) + (p[2] + p[3]) : 0.f);
-        m[h] = m_new;
-        pa[h] = row_used ? pack2_bf16(p[0], p[1]) : 0u;
-        pa[2 + h] = row_used ? pack2_bf16(p[2], p[3]) : 0u;
-#pragma unroll
-        for (int nt = 0; nt < kGqD / 8; ++nt) {
-          o[nt][2 * h] *= alpha;
-          o[nt][2 * h + 1] *= alpha;
-        }
+        for (int e = 0; e < 4; ++e) p[e] = exp2f(sv4[h][e] - m[h]);
+        l[h] += (p[0] + p[1]) + (p[2] + p[3]);
+        pa[h] = pack2_bf16(p[0], p[1]);
+        pa[2 + h] = pack2_bf16(p[2], p[3]);
       }
       // O += P V: 16 keys x D dims, two 8-dim column tiles per ldmatrix
       uint32_t vmask[2];                                        // valid keys among 2t, 2t + 1 | 2t + 8, 2t + 9
@@ -174,9 +193,10 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
         mma_16816(o[2 * nt2 + 1], pa, b[2], b[3]);
       }
     }
-    __syncthreads();                                            // the stage may be refilled
+    __syncwarp();                                               // the warp's rows of the stage may be refilled
   }
   cp_async_wait<0>();
+  __syncthreads();
 
   // merge the four warps' triples through shared memory (the tiles are no longer needed)
 #pragma unroll

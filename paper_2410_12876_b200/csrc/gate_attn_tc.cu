@@ -90,7 +90,7 @@ __device__ inline int ga_seq_tiles(const GateAttnArgs &a, int b) {
   return a.seq_lens == nullptr ? a.n_qtiles : (min(max(a.seq_lens[b], 0), a.n) + kGaBM - 1) / kGaBM;
 }
 __device__ inline int ga_seg_len(const GateAttnArgs &a, int total) {
-  return max(2 * kGaOverhead, ((total + a.n_seg - 1) / a.n_seg + 1) & ~1);
+  return max(2, ((total + a.n_seg - 1) / a.n_seg + 1) & ~1);
 }
 // Whole-warp call: places of the list in all, and before sequence b_end.
 __device__ inline int ga_total(const GateAttnArgs &a, int b_end, int &before) {

@@ -1,0 +1,43 @@
+"""Decode of few slabs reads 16-row blocks straight into registers, the first of each warp before the slab's length is
+known: lengths at the edges of a block, of a warp's second block (512 rows later) and of its third, with every row that
+was never written holding NaN."""
+import numpy as np
+import pytest
+import torch
+
+import agtest as T
+from oracle import ag_oracle as orc
+from paper_2410_12876_b200 import binding as ag
+from paper_2410_12876_b200 import inputs
+from paper_2410_12876_b200.inputs import LayerShape
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    T.ensure_built()
+
+
+@pytest.mark.parametrize("D,h,hk", [(128, 8, 8), (64, 8, 8), (128, 64, 8), (64, 128, 8), (128, 72, 8)])
+def test_lengths_at_the_edges_of_blocks(D, h, hk):
+    lens = np.array([1, 15, 16, 17, 527, 528, 1025, 1551])
+    shape = LayerShape(1, 1600, 64, h, D, 1, 64, "bf16", kv_heads=hk)
+    cache = ag.RaggedCache.allocate(shape, lens + 20, DEV)
+    nan = float("nan")
+    cache.k_rows.fill_(nan)
+    cache.v_rows.fill_(nan)
+    off = cache.row_off.cpu().numpy()
+    for s, n in enumerate(lens):
+        cache.k_rows[off[s]:off[s] + n] = inputs.randn((int(n), D), 41 + s, DEV, torch.bfloat16)
+        cache.v_rows[off[s]:off[s] + n] = inputs.randn((int(n), D), 61 + s, DEV, torch.bfloat16)
+    cache.len.copy_(torch.from_numpy(lens.astype(np.int32)))
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    for step in range(2):
+        held = T.gpu_cache_as_lists(cache, shape)
+        q, kn, vn, fn = inputs.decode_inputs(shape, 50, step, DEV, keep_new=1.0)
+        o = T.gpu_decode_step(shape, q, kn, vn, fn, cache, status, fused=True)
+        T.check_close(T.f64(o), orc.decode_attention(T.f64(q), T.f64(kn), T.f64(vn), held), "bf16", f"step {step}")
+    assert np.array_equal(cache.len.cpu().numpy(), lens + 2)
+    assert int(status.item()) == 0 and ag.ag_device_wait_timeouts() == 0
