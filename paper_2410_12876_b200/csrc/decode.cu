@@ -48,27 +48,38 @@ struct AppendArgs {
   void *k_rows, *v_rows;
   int32_t *dev_status;
 };
-// Called by the threads [first, first + row vectors) of ONE CTA per slab (every thread may call, the
-// others return), after every read of len[slab] and of the slab's rows by this launch has
-// completed.  L = the length those reads saw.
+// What an append needs to know, asked for ahead of the work of the step: after the barrier that ends it nothing is left
+// but the stores (the flag, the capacity, then the row were three trips to L2 in a row at the end of every step).
+struct NewRow { uint4 k, v; size_t dst; int cap; bool on; };
+// The threads [first, first + row vectors) of ONE CTA per slab carry a row; the others get on = false.
 template <typename T, int D>
-__device__ __forceinline__ void append_new_row(const AppendArgs &ap, int slab, int L, int64_t row0,
-                                               const T *k_new, const T *v_new,
-                                               int first = 0) {
+__device__ __forceinline__ NewRow load_new_row(const AppendArgs &ap, int slab, int64_t row0, const T *k_new,
+                                               const T *v_new, int first = 0) {
   constexpr int kVecs = D * (int)sizeof(T) / 16;
   const int vec = (int)threadIdx.x - first;
-  if (ap.flag_new == nullptr || vec < 0 || vec >= kVecs || ap.flag_new[slab] == 0) return;
-  if (L >= ap.cap[slab]) {
-    if (vec == 0 && ap.dev_status) atomicOr(ap.dev_status, AG_DEV_OVERFLOW);
+  NewRow r;
+  r.on = false;
+  if (ap.flag_new == nullptr || vec < 0 || vec >= kVecs) return r;
+  r.k = ld128(k_new + (size_t)slab * D + vec * (16 / (int)sizeof(T)));
+  r.v = ld128(v_new + (size_t)slab * D + vec * (16 / (int)sizeof(T)));
+  r.cap = ap.cap[slab];
+  r.on = ap.flag_new[slab] != 0;
+  r.dst = (size_t)row0 * D * sizeof(T) + vec * 16;
+  return r;
+}
+// After every read of len[slab] and of the slab's rows by this launch has completed.  L = the length those reads saw.
+template <typename T, int D>
+__device__ __forceinline__ void append_new_row(const AppendArgs &ap, const NewRow &r, int slab, int L, int first = 0) {
+  if (!r.on) return;
+  const bool lead = (int)threadIdx.x == first;
+  if (L >= r.cap) {
+    if (lead && ap.dev_status) atomicOr(ap.dev_status, AG_DEV_OVERFLOW);
     return;
   }
-  const size_t dst = ((size_t)row0 + L) * D * sizeof(T) + vec * 16;
-  const size_t src = (size_t)slab * D * sizeof(T) + vec * 16;
-  *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ap.k_rows) + dst) =
-      *reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(k_new) + src);
-  *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ap.v_rows) + dst) =
-      *reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(v_new) + src);
-  if (vec == 0) ap.len[slab] = L + 1;
+  const size_t dst = r.dst + (size_t)L * D * sizeof(T);
+  *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ap.k_rows) + dst) = r.k;
+  *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ap.v_rows) + dst) = r.v;
+  if (lead) ap.len[slab] = L + 1;
 }
 
 // Recent-token window: scores of the query against the ring of its key/value slab, by warps 0 .. n_warps - 1
@@ -345,6 +356,9 @@ decode_combine_kernel(const T *q, const T *k_new,
   pdl_wait();
   const float kn = Elem<T>::load(k_new + (size_t)kv * D + d), vn = Elem<T>::load(v_new + (size_t)kv * D + d);
   const int L = len[kv];
+  NewRow row;
+  row.on = false;
+  if (y == 0) row = load_new_row<T, D>(ap, kv, row_off[kv], k_new, v_new);
   const int n_chunks = (L + chunk_rows - 1) / chunk_rows;
   for (int h0 = 0; h0 < G; h0 += blockDim.y) {
     const int h = h0 + y;
@@ -401,7 +415,7 @@ decode_combine_kernel(const T *q, const T *k_new,
   // Every thread of the CTA has read the slab's length, and the chunk pass, the only reader of the slab's
   // rows, has completed: the new row may go in and the length may move; the ring has been read too.
   if (y == 0) {
-    append_new_row<T, D>(ap, kv, L, row_off[kv], k_new, v_new);
+    append_new_row<T, D>(ap, row, kv, L);
     constexpr int kVecs = D * (int)sizeof(T) / 16;
     if (rg.R > 0 && ap.flag_new != nullptr && d < kVecs)
       ring_put<kVecs>(rg, kv, d, reinterpret_cast<const uint8_t *>(k_new + (size_t)kv * D),
@@ -453,9 +467,13 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
     k_raw = k_new[(size_t)kv * D + threadIdx.x];
     v_raw = v_new[(size_t)kv * D + threadIdx.x];
   }
+  const int64_t row0 = row_off[kv];
+  NewRow row;
+  row.on = false;
+  if (rank == 0) row = load_new_row<T, D>(ap, kv, row0, k_new, v_new, D);
 
   float m, l, o[kEpl];
-  decode_stream_rows<T, D, kThreads>(q, k_rows, v_rows, row_off[kv], slab, r_begin, r_end, scale_log2, m, l, o);
+  decode_stream_rows<T, D, kThreads>(q, k_rows, v_rows, row0, slab, r_begin, r_end, scale_log2, m, l, o);
 
   if (v == 0) { sm_m[g] = m; sm_l[g] = l; }
 #pragma unroll
@@ -491,7 +509,7 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
   // every CTA of the cluster has read the length and its rows: the new row may go in
   // (never asked for when query heads share a slab: another head's cluster may still be reading its length)
   // by threads that have no part in the merge below, so that the two run side by side
-  if (rank == 0) append_new_row<T, D>(ap, kv, L, row_off[kv], k_new, v_new, D);
+  if (rank == 0) append_new_row<T, D>(ap, row, kv, L, D);
   if (rank == 0 && threadIdx.x < D) {
     const int d = threadIdx.x;
     float s_self = 0.f;
@@ -599,6 +617,9 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
     k_raw = k_new[(size_t)kv * D + d];
     v_raw = v_new[(size_t)kv * D + d];
   }
+  NewRow row;
+  row.on = false;
+  if (rank == 0) row = load_new_row<T, D>(ap, kv, slab_row0, k_new, v_new);
 
   if (r_first < L) {                  // the same for the whole CTA
     const GqWarpTriples w = gq_stream_rows<D, kCmStages, (kMaxG + 7) / 8, true>(
@@ -631,7 +652,7 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   cluster.sync();
   // every CTA of the cluster has read the length and its rows: the new row may go in
   // (never asked for when a query slab outside this cluster shares the slab)
-  if (rank == 0) append_new_row<T, D>(ap, kv, L, slab_row0, k_new, v_new);
+  if (rank == 0) append_new_row<T, D>(ap, row, kv, L);
 #pragma unroll
   for (int u = 0; u < kHeads; ++u) {
     const int h = rank + u * kClusterSize;

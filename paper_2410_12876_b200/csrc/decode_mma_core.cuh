@@ -53,13 +53,14 @@ __device__ __forceinline__ void gq_load_tile(uint32_t stage, const uint8_t *Kg, 
 // kGqStages - 1 tiles are in flight while one is worked on).
 // kFirstLoaded: the caller has issued tile 0 into stage 0 and committed it, perhaps before it knew r_end: its rows
 // past r_end may then hold anything.  Their scores are masked; their values are masked too (0 * NaN is NaN).
-// kHalves: 1 for G <= 8 (rows 8..15 of the operand are zero and their softmax is left out), 2 for G <= 16.
-template <int kGqD, int kGqStages, int kHalves, bool kFirstLoaded>
+// kN: groups of 8 heads (G <= 8 kN).
+template <int kGqD, int kGqStages, int kN, bool kFirstLoaded>
 __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const __nv_bfloat16 *q, int G,
                                                         const uint8_t *Kg, const uint8_t *Vg, int r_first, int r_step,
                                                         int r_end, float scale_log2) {
   static_assert(kGqD == 64 || kGqD == 128, "head_dim");
   constexpr int kGqTileBytes = gq_tile_bytes(kGqD);
+  constexpr int kChains = 2;        // chains of MMAs that the scores of a block are summed in
   const int n_tiles = (r_end - r_first + r_step - 1) / r_step;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;                                       // fragment row, column pair
@@ -69,23 +70,16 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
   };
 
   // (Q is asked for first: these loads cannot move ahead of the asynchronous copies by themselves)
-  // A fragments of Q: row g = query head g of the group (rows >= G are zero), 8 steps of 16 dims
-  uint32_t qa[kGqD / 16][4];
+  // Second operand of the scores: head 8 n + g (zeros past G), 16 dims per step
+  uint32_t qb[kN][kGqD / 16][2];
 #pragma unroll
-  for (int ks = 0; ks < kGqD / 16; ++ks) {
-    const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + (size_t)min(g, G - 1) * kGqD);
-    const uint32_t lo = qrow[ks * 8 + t], hi = qrow[ks * 8 + 4 + t];
-    qa[ks][0] = g < G ? lo : 0u;
-    qa[ks][1] = 0u;
-    qa[ks][2] = g < G ? hi : 0u;
-    qa[ks][3] = 0u;
-  }
-  if (kHalves == 2) {
+  for (int n = 0; n < kN; ++n) {
+    const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + (size_t)min(8 * n + g, G - 1) * kGqD);
 #pragma unroll
     for (int ks = 0; ks < kGqD / 16; ++ks) {
-      const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + (size_t)min(g + 8, G - 1) * kGqD);
-      qa[ks][1] = g + 8 < G ? qrow[ks * 8 + t] : 0u;
-      qa[ks][3] = g + 8 < G ? qrow[ks * 8 + 4 + t] : 0u;
+      const uint32_t lo = qrow[ks * 8 + t], hi = qrow[ks * 8 + 4 + t];
+      qb[n][ks][0] = 8 * n + g < G ? lo : 0u;
+      qb[n][ks][1] = 8 * n + g < G ? hi : 0u;
     }
   }
 
@@ -95,14 +89,17 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
     cp_async_commit();
   }
 
-  float o[kGqD / 8][4];
+  // o[n][j]: dims 16 j + g (and + 8) of heads 8 n + 2t, 2t + 1; m, l: those heads (l: this thread's keys)
+  float o[kN][kGqD / 16][4], m[kN][2], l[kN][2];
 #pragma unroll
-  for (int nt = 0; nt < kGqD / 8; ++nt)
+  for (int n = 0; n < kN; ++n) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) o[nt][e] = 0.f;
-  float m[kHalves], l[kHalves];                                 // rows g (and g + 8)
+    for (int j = 0; j < kGqD / 16; ++j)
 #pragma unroll
-  for (int h = 0; h < kHalves; ++h) { m[h] = -INFINITY; l[h] = 0.f; }
+      for (int e = 0; e < 4; ++e) o[n][j][e] = 0.f;
+    m[n][0] = m[n][1] = -INFINITY;
+    l[n][0] = l[n][1] = 0.f;
+  }
 
   for (int i = 0; i < n_tiles; ++i) {
     if (i + kGqStages - 1 < n_tiles) load_tile(i + kGqStages - 1);
@@ -114,65 +111,69 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
 
     if (key0 < r_end) {
       const bool ragged = key0 + 16 > r_end;
-      // S = Q K^T for 16 keys: two 8-key column tiles, two chains of MMAs each
-      float s0[2][4], s1[2][4];
+      const int mi = lane >> 3;
+      // S^T = K Q^T: 16 keys x 8 heads per MMA
+      float s[kN][kChains][4];
 #pragma unroll
-      for (int c = 0; c < 2; ++c)
+      for (int n = 0; n < kN; ++n)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s0[c][e] = s1[c][e] = 0.f;
+        for (int c = 0; c < kChains; ++c)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) s[n][c][e] = 0.f;
 #pragma unroll
       for (int ks = 0; ks < kGqD / 16; ++ks) {
-        uint32_t b[4];
-        // matrices: (keys 0-7, dims lo), (keys 0-7, dims hi), (keys 8-15, dims lo), (keys 8-15, dims hi)
-        const int mi = lane >> 3, row = warp * 16 + (mi >> 1) * 8 + (lane & 7);
-        ldmatrix_x4(b, sk + gq_tile_off<kGqD>(row, ks * 2 + (mi & 1)));
-        mma_16816(s0[ks & 1], qa[ks], b[0], b[1]);
-        mma_16816(s1[ks & 1], qa[ks], b[2], b[3]);
+        uint32_t a[4];
+        // matrices: (keys 0-7, dims lo), (keys 8-15, dims lo), (keys 0-7, dims hi), (keys 8-15, dims hi)
+        ldmatrix_x4(a, sk + gq_tile_off<kGqD>(warp * 16 + (mi & 1) * 8 + (lane & 7), ks * 2 + (mi >> 1)));
+#pragma unroll
+        for (int n = 0; n < kN; ++n) mma_16816(s[n][ks % kChains], a, qb[n][ks][0], qb[n][ks][1]);
       }
-      // online softmax of rows g (and g + 8): this thread holds keys 2t, 2t+1 of each column tile.  The maximum
-      // moves only when a score exceeds it by more than 2^8 (float32 sums and bf16 weights have the room); rows
-      // past G come out as anything and are dropped at the end.
-      uint32_t pa[4] = {0u, 0u, 0u, 0u};
-      float sv4[kHalves][4];
+      // Online softmax of heads 2t, 2t + 1: this thread holds keys g, g + 8.  The maximum moves only when a score
+      // exceeds it by more than 2^8 (float32 sums and bf16 weights have the room).
       bool up = false;
 #pragma unroll
-      for (int h = 0; h < kHalves; ++h) {
-        const int kcol[4] = {2 * t, 2 * t + 1, 8 + 2 * t, 9 + 2 * t};
+      for (int n = 0; n < kN; ++n)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const int c = 2 * h + (e & 1);
-          sv4[h][e] = (e < 2 ? s0[0][c] + s0[1][c] : s1[0][c] + s1[1][c]) * scale_log2;
-          if (ragged && key0 + kcol[e] >= r_end) sv4[h][e] = -INFINITY;
-          up = up || sv4[h][e] > m[h] + 8.f;
+          float x = s[n][0][e];
+#pragma unroll
+          for (int c = 1; c < kChains; ++c) x += s[n][c][e];
+          x *= scale_log2;
+          if (ragged && key0 + g + 8 * (e >> 1) >= r_end) x = -INFINITY;
+          s[n][0][e] = x;
+          up = up || x > m[n][e & 1] + 8.f;
         }
-      }
       if (__any_sync(0xffffffffu, up)) {
 #pragma unroll
-        for (int h = 0; h < kHalves; ++h) {
-          float tmax = fmaxf(fmaxf(sv4[h][0], sv4[h][1]), fmaxf(sv4[h][2], sv4[h][3]));
-          tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-          tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
-          const float m_new = fmaxf(m[h], tmax);                // finite: key0 < r_end, so column 0 is valid
-          const float alpha = exp2f(m[h] - m_new);              // m = -inf at first: 0
-          m[h] = m_new;
-          l[h] *= alpha;
+        for (int n = 0; n < kN; ++n)
 #pragma unroll
-          for (int nt = 0; nt < kGqD / 8; ++nt) {
-            o[nt][2 * h] *= alpha;
-            o[nt][2 * h + 1] *= alpha;
+          for (int e = 0; e < 2; ++e) {
+            float mx = fmaxf(s[n][0][e], s[n][0][e + 2]);
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            const float m_new = fmaxf(m[n][e], mx);             // finite: key0 < r_end, so key 0 is valid
+            const float alpha = exp2f(m[n][e] - m_new);         // m = -inf at first: 0
+            m[n][e] = m_new;
+            l[n][e] *= alpha;
+#pragma unroll
+            for (int j = 0; j < kGqD / 16; ++j) {
+              o[n][j][e] *= alpha;
+              o[n][j][e + 2] *= alpha;
+            }
           }
-        }
       }
+      uint32_t pb[kN][2];                                       // P^T: keys 2t, 2t + 1 (| + 8) of head 8 n + g
 #pragma unroll
-      for (int h = 0; h < kHalves; ++h) {
+      for (int n = 0; n < kN; ++n) {
         float p[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) p[e] = exp2f(sv4[h][e] - m[h]);
-        l[h] += (p[0] + p[1]) + (p[2] + p[3]);
-        pa[h] = pack2_bf16(p[0], p[1]);
-        pa[2 + h] = pack2_bf16(p[2], p[3]);
+        for (int e = 0; e < 4; ++e) p[e] = exp2f(s[n][0][e] - m[n][e & 1]);
+        l[n][0] += p[0] + p[2];
+        l[n][1] += p[1] + p[3];
+        pb[n][0] = movmatrix_trans(pack2_bf16(p[0], p[1]));
+        pb[n][1] = movmatrix_trans(pack2_bf16(p[2], p[3]));
       }
-      // O += P V: 16 keys x D dims, two 8-dim column tiles per ldmatrix
+      // O^T += V^T P^T: 16 dims x 16 keys per ldmatrix
       uint32_t vmask[2];                                        // valid keys among 2t, 2t + 1 | 2t + 8, 2t + 9
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
@@ -180,17 +181,16 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
         vmask[e] = k + 1 < r_end ? 0xffffffffu : (k < r_end ? 0xffffu : 0u);
       }
 #pragma unroll
-      for (int nt2 = 0; nt2 < kGqD / 16; ++nt2) {
-        uint32_t b[4];
-        // matrices: (keys 0-7, dims lo), (keys 8-15, dims lo), (keys 0-7, dims hi), (keys 8-15, dims hi)
-        const int mi = lane >> 3, row = warp * 16 + (mi & 1) * 8 + (lane & 7);
-        ldmatrix_x4_trans(b, sv + gq_tile_off<kGqD>(row, nt2 * 2 + (mi >> 1)));
+      for (int j = 0; j < kGqD / 16; ++j) {
+        uint32_t a[4];
+        // matrices: (dims lo, keys 0-7), (dims hi, keys 0-7), (dims lo, keys 8-15), (dims hi, keys 8-15)
+        ldmatrix_x4_trans(a, sv + gq_tile_off<kGqD>(warp * 16 + (mi >> 1) * 8 + (lane & 7), j * 2 + (mi & 1)));
         if (kFirstLoaded && i == 0) {
 #pragma unroll
-          for (int e = 0; e < 4; ++e) b[e] &= vmask[e & 1];
+          for (int e = 0; e < 4; ++e) a[e] &= vmask[e >> 1];
         }
-        mma_16816(o[2 * nt2], pa, b[0], b[1]);
-        mma_16816(o[2 * nt2 + 1], pa, b[2], b[3]);
+#pragma unroll
+        for (int n = 0; n < kN; ++n) mma_16816(o[n][j], a, pb[n][0], pb[n][1]);
       }
     }
     __syncwarp();                                               // the warp's rows of the stage may be refilled
@@ -199,30 +199,29 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
   __syncthreads();
 
   // merge the four warps' triples through shared memory (the tiles are no longer needed)
-#pragma unroll
-  for (int h = 0; h < kHalves; ++h) {
-    l[h] += __shfl_xor_sync(0xffffffffu, l[h], 1);
-    l[h] += __shfl_xor_sync(0xffffffffu, l[h], 2);
-  }
   float *sm_o = reinterpret_cast<float *>(gq_smem);             // [warps][16][D]
   float *sm_m = sm_o + kGqWarps * kGqMaxGroup * kGqD;           // [warps][16]
   float *sm_l = sm_m + kGqWarps * kGqMaxGroup;
 #pragma unroll
-  for (int h = 0; h < kHalves; ++h) {
-    const int row = g + 8 * h;
-    if (row < G) {
+  for (int n = 0; n < kN; ++n)
 #pragma unroll
-      for (int nt = 0; nt < kGqD / 8; ++nt) {
-        float *dst = sm_o + ((size_t)(warp * kGqMaxGroup + row)) * kGqD + nt * 8 + 2 * t;
-        dst[0] = o[nt][2 * h];
-        dst[1] = o[nt][2 * h + 1];
-      }
-      if (t == 0) {
-        sm_m[warp * kGqMaxGroup + row] = m[h];
-        sm_l[warp * kGqMaxGroup + row] = l[h];
+    for (int e = 0; e < 2; ++e) {
+      const int head = 8 * n + 2 * t + e;
+#pragma unroll
+      for (int off = 4; off < 32; off <<= 1) l[n][e] += __shfl_xor_sync(0xffffffffu, l[n][e], off);
+      if (head < G) {
+        float *dst = sm_o + ((size_t)(warp * kGqMaxGroup + head)) * kGqD + g;
+#pragma unroll
+        for (int j = 0; j < kGqD / 16; ++j) {
+          dst[16 * j] = o[n][j][e];
+          dst[16 * j + 8] = o[n][j][e + 2];
+        }
+        if (g == 0) {
+          sm_m[warp * kGqMaxGroup + head] = m[n][e];
+          sm_l[warp * kGqMaxGroup + head] = l[n][e];
+        }
       }
     }
-  }
   __syncthreads();
   return GqWarpTriples{sm_o, sm_m, sm_l};
 }
