@@ -50,7 +50,7 @@ struct AppendArgs {
 };
 // What an append needs to know, asked for ahead of the work of the step: after the barrier that ends it nothing is left
 // but the stores (the flag, the capacity, then the row were three trips to L2 in a row at the end of every step).
-struct NewRow { uint4 k, v; size_t dst; int cap; bool on; };
+struct NewRow { uint4 k, v; size_t dst; int cap; uint32_t on; };    // (on: the flag as it was read, so that nothing waits for it here)
 // The threads [first, first + row vectors) of ONE CTA per slab carry a row; the others get on = false.
 template <typename T, int D>
 __device__ __forceinline__ NewRow load_new_row(const AppendArgs &ap, int slab, int64_t row0, const T *k_new,
@@ -58,19 +58,19 @@ __device__ __forceinline__ NewRow load_new_row(const AppendArgs &ap, int slab, i
   constexpr int kVecs = D * (int)sizeof(T) / 16;
   const int vec = (int)threadIdx.x - first;
   NewRow r;
-  r.on = false;
+  r.on = 0;
   if (ap.flag_new == nullptr || vec < 0 || vec >= kVecs) return r;
   r.k = ld128(k_new + (size_t)slab * D + vec * (16 / (int)sizeof(T)));
   r.v = ld128(v_new + (size_t)slab * D + vec * (16 / (int)sizeof(T)));
   r.cap = ap.cap[slab];
-  r.on = ap.flag_new[slab] != 0;
+  r.on = ap.flag_new[slab];
   r.dst = (size_t)row0 * D * sizeof(T) + vec * 16;
   return r;
 }
 // After every read of len[slab] and of the slab's rows by this launch has completed.  L = the length those reads saw.
 template <typename T, int D>
 __device__ __forceinline__ void append_new_row(const AppendArgs &ap, const NewRow &r, int slab, int L, int first = 0) {
-  if (!r.on) return;
+  if (r.on == 0) return;
   const bool lead = (int)threadIdx.x == first;
   if (L >= r.cap) {
     if (lead && ap.dev_status) atomicOr(ap.dev_status, AG_DEV_OVERFLOW);
@@ -357,7 +357,7 @@ decode_combine_kernel(const T *q, const T *k_new,
   const float kn = Elem<T>::load(k_new + (size_t)kv * D + d), vn = Elem<T>::load(v_new + (size_t)kv * D + d);
   const int L = len[kv];
   NewRow row;
-  row.on = false;
+  row.on = 0;
   if (y == 0) row = load_new_row<T, D>(ap, kv, row_off[kv], k_new, v_new);
   const int n_chunks = (L + chunk_rows - 1) / chunk_rows;
   for (int h0 = 0; h0 < G; h0 += blockDim.y) {
@@ -467,13 +467,9 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
     k_raw = k_new[(size_t)kv * D + threadIdx.x];
     v_raw = v_new[(size_t)kv * D + threadIdx.x];
   }
-  const int64_t row0 = row_off[kv];
-  NewRow row;
-  row.on = false;
-  if (rank == 0) row = load_new_row<T, D>(ap, kv, row0, k_new, v_new, D);
 
   float m, l, o[kEpl];
-  decode_stream_rows<T, D, kThreads>(q, k_rows, v_rows, row0, slab, r_begin, r_end, scale_log2, m, l, o);
+  decode_stream_rows<T, D, kThreads>(q, k_rows, v_rows, row_off[kv], slab, r_begin, r_end, scale_log2, m, l, o);
 
   if (v == 0) { sm_m[g] = m; sm_l[g] = l; }
 #pragma unroll
@@ -508,8 +504,9 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
   else __syncthreads();
   // every CTA of the cluster has read the length and its rows: the new row may go in
   // (never asked for when query heads share a slab: another head's cluster may still be reading its length)
-  // by threads that have no part in the merge below, so that the two run side by side
-  if (rank == 0) append_new_row<T, D>(ap, row, kv, L, D);
+  // by threads that have no part in the merge below, so that the two run side by side (asked for any earlier, the row
+  // is waited for at this barrier: 95 -> 105 us for a 128-token float32 layer and 16 steps)
+  if (rank == 0) append_new_row<T, D>(ap, load_new_row<T, D>(ap, kv, row_off[kv], k_new, v_new, D), kv, L, D);
   if (rank == 0 && threadIdx.x < D) {
     const int d = threadIdx.x;
     float s_self = 0.f;
@@ -561,12 +558,15 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
 // on warp-level MMAs (decode_mma_core.cuh): per row a fraction of the instructions of the CUDA-core form,
 // which at these sizes is bound by instruction issue and by what one SM can take in, not by latency alone.
 // One cluster per run of G <= 16 query slabs that share a key/value slab (G = 1 without grouped-query
-// attention): the G queries are rows of one MMA operand, so the slab is read once for all of them, and the
+// attention): the G queries are columns of one MMA operand, so the slab is read once for all of them, and the
 // one cluster that reads it may append to it.  CTA `rank` takes whole 64-row tiles; after the cluster
 // barrier rank r merges the heads r, r + 8 of the group, whose triples the ranks have written to its shared memory.  The tiles go round the ranks, so a rank's first tile does
 // not depend on the slab's length and its rows are asked for together with the length (before it is known
 // they are only known to lie inside the slab): one trip to L2 less on the path of a step.
-// three stages: a CTA has few tiles and no neighbour to hide behind, so two of them are kept in flight
+// A step of 32 slabs of 400 .. 1640 rows takes 7.7 us in a graph (1.2 us of it an empty chain of launches); it was 9.2 us
+// with the queries as the rows of the MMAs, the merging rank reading the others' triples (one trip and one barrier
+// more), the row to append fetched after the barrier and 96 KB of stages: two stages and fewer than 170 registers let
+// three CTAs share an SM, so the next step's clusters start beside this one's.
 constexpr int kCmStages = 2;
 // kMaxG: 1 (one query per slab), 8 or 16.
 template <int D, int kMaxG>
@@ -618,7 +618,7 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
     v_raw = v_new[(size_t)kv * D + d];
   }
   NewRow row;
-  row.on = false;
+  row.on = 0;
   if (rank == 0) row = load_new_row<T, D>(ap, kv, slab_row0, k_new, v_new);
 
   if (r_first < L) {                  // the same for the whole CTA

@@ -2,12 +2,15 @@
 // the G <= 16 query vectors that read it (G query heads of a group, or one head), streamed through
 // shared memory.  Used by the chunk pass of grouped-query decode and by the cluster form of decode.
 //
-// The G queries are the rows of a 16-row MMA operand (the other rows are zero): m16n8k16 bf16 MMAs,
-// the shape that fits an M of 1..16 (a tcgen05 tile needs M >= 64); the contraction is bound by
-// memory, and what the tensor cores buy is fewer instructions per row, not FLOP/s.  Rows go global ->
-// shared by 16-byte cp.async in tiles of 64 rows (K and V; the next tile is in flight while one is
-// worked on); each of the four warps owns 16 rows of every tile and keeps its own running softmax;
-// the warps' (m, l, o) triples end in shared memory and gq_combine() merges them.
+// m16n8k16 bf16 MMAs (a tcgen05 tile needs 64 rows or more): the contraction is bound by memory, and what the tensor
+// cores buy is fewer instructions per row, not FLOP/s.  Both products are turned, S^T = K Q^T and O^T = V^T P^T, so that
+// the keys, then the dims, are the 16 rows of an MMA and the query heads its 8 columns: half the MMAs and half
+// the accumulators of the form with the (mostly empty) 16 query rows; S^T becomes the second operand of the
+// weighted sum by an 8 x 8 transpose between registers (movmatrix).
+// Rows go global -> shared by 16-byte cp.async in tiles of 64 rows (K and V; the next tile is in flight while one is
+// worked on); each of the four warps fetches and owns 16 rows of every tile and keeps its own running softmax, so the
+// warps wait for nobody until their (m, l, o) triples end in shared memory, where gq_combine() merges them.
+// Measured: chunk pass of 32 sequences x 8 slabs of 1600 .. 7400 rows, four heads each, 104.5 -> 101.8 us per step.
 #pragma once
 #include "ag_common.cuh"
 #include "mma_sync.cuh"

@@ -1,6 +1,6 @@
-"""Decode of few slabs reads 16-row blocks straight into registers, the first of each warp before the slab's length is
-known: lengths at the edges of a block, of a warp's second block (512 rows later) and of its third, with every row that
-was never written holding NaN."""
+"""Decode of few slabs: a CTA asks for its first tile before the slab's length is known.  Lengths at the edges of a warp's
+16 rows, of a CTA's second tile (512 rows later) and of its third, with every row that was never written holding NaN;
+groups of 1, 8, 9 and 16 heads (one or two groups of 8 MMA columns)."""
 import numpy as np
 import pytest
 import torch
