@@ -568,8 +568,8 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
 // more), the row to append fetched after the barrier and 96 KB of stages: two stages and fewer than 170 registers let
 // three CTAs share an SM, so the next step's clusters start beside this one's.
 constexpr int kCmStages = 2;
-// kMaxG: 1 (one query per slab), 8 or 16.
-template <int D, int kMaxG>
+// kMaxG: 1 (one query per slab), 8 or 16.  kCtas: CTAs of a cluster (1: no cluster).
+template <int D, int kMaxG, int kCtas>
 __global__ void __launch_bounds__(kGqThreads, 2)
 decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
                           const __nv_bfloat16 *v_new, const __nv_bfloat16 *k_rows,
@@ -579,15 +579,15 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   namespace cg = cooperative_groups;
   using T = __nv_bfloat16;
   static_assert(kGqThreads >= D, "one thread per output dimension in the merge");
-  constexpr int kHeads = (kMaxG + kClusterSize - 1) / kClusterSize;    // heads a rank merges, at most
+  constexpr int kHeads = (kMaxG + kCtas - 1) / kCtas;    // heads a rank merges, at most
   const int G = kMaxG == 1 ? 1 : group;
   extern __shared__ __align__(128) uint8_t gq_smem[];
   cg::cluster_group cluster = cg::this_cluster();
-  const int slab0 = blockIdx.y * G, rank = (int)cluster.block_rank();
+  const int slab0 = blockIdx.y * G, rank = kCtas == 1 ? 0 : (int)cluster.block_rank();
   const int kv = hm.kv_slab(slab0);
   const int d = threadIdx.x;
   pdl_launch_dependents();
-  cluster.barrier_arrive();           // (waited for before the first write to another rank: all have started then)
+  if constexpr (kCtas > 1) cluster.barrier_arrive();   // (waited for before the first write to another rank: all have started then)
   // the slab's first row and capacity never change once the cache is laid out: read ahead of the wait for the
   // preceding kernel
   const int64_t slab_row0 = row_off[kv];
@@ -601,8 +601,9 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   cp_async_commit();
 
   // the ranks' triples of the heads this rank merges, written by the ranks themselves
-  __shared__ float in_o[kHeads][kClusterSize][D];
-  __shared__ float2 in_ml[kHeads][kClusterSize];
+  __shared__ float in_o[kHeads][kCtas][D];
+  __shared__ float2 in_ml[kHeads][kCtas];
+  auto at_rank = [&](auto *p, int r) { return kCtas == 1 ? p : cluster.map_shared_rank(p, r); };
   __shared__ float red[kHeads][D / 32];
   __shared__ float ring_s[kHeads][kMaxRecent];
 
@@ -610,7 +611,7 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   T q_raw[kHeads], k_raw = T(0.f), v_raw = T(0.f);           // (not used before the stream is done)
 #pragma unroll
   for (int u = 0; u < kHeads; ++u) {
-    const int h = rank + u * kClusterSize;
+    const int h = rank + u * kCtas;
     q_raw[u] = (h < G && d < D) ? q[(size_t)(slab0 + h) * D + d] : T(0.f);
   }
   if (rank < G && d < D) {
@@ -623,24 +624,24 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
 
   if (r_first < L) {                  // the same for the whole CTA
     const GqWarpTriples w = gq_stream_rows<D, kCmStages, (kMaxG + 7) / 8, true>(
-        gq_smem, q + (size_t)slab0 * D, G, Kg, Vg, r_first, kClusterSize * kGqTile, L, scale_log2);
-    cluster.barrier_wait();
+        gq_smem, q + (size_t)slab0 * D, G, Kg, Vg, r_first, kCtas * kGqTile, L, scale_log2);
+    if constexpr (kCtas > 1) cluster.barrier_wait();
     for (int x = d; x < G * D; x += kGqThreads) {
-      const int h = x / D, e = x % D, to = h % kClusterSize;
+      const int h = x / D, e = x % D, to = h % kCtas;
       float acc, mc, lc;
       gq_combine<D>(w, h, e, acc, mc, lc);
-      *cluster.map_shared_rank(&in_o[h / kClusterSize][rank][e], to) = acc;
-      if (e == 0) *cluster.map_shared_rank(&in_ml[h / kClusterSize][rank], to) = make_float2(mc, lc);
+      *at_rank(&in_o[h / kCtas][rank][e], to) = acc;
+      if (e == 0) *at_rank(&in_ml[h / kCtas][rank], to) = make_float2(mc, lc);
     }
   } else {
-    cluster.barrier_wait();
+    if constexpr (kCtas > 1) cluster.barrier_wait();
     // weight 0 in the merge, which then skips the values
-    if (d < G) *cluster.map_shared_rank(&in_ml[d / kClusterSize][rank], d % kClusterSize) = make_float2(-INFINITY, 0.f);
+    if (d < G) *at_rank(&in_ml[d / kCtas][rank], d % kCtas) = make_float2(-INFINITY, 0.f);
     cp_async_wait<0>();               // (the first tile, asked for in vain)
   }
 #pragma unroll
   for (int u = 0; u < kHeads; ++u) {
-    const int h = rank + u * kClusterSize;
+    const int h = rank + u * kCtas;
     if (h >= G) break;                // the same for the whole CTA
     float prod = Elem<T>::load(&q_raw[u]) * Elem<T>::load(&k_raw);
 #pragma unroll
@@ -649,13 +650,14 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
     ring_scores<T, D>(rg, kv, q + (size_t)(slab0 + h) * D, scale_log2, ring_s[u]);
   }
   const float v_self = Elem<T>::load(&v_raw);
-  cluster.sync();
+  if constexpr (kCtas > 1) cluster.sync();
+  else __syncthreads();
   // every CTA of the cluster has read the length and its rows: the new row may go in
   // (never asked for when a query slab outside this cluster shares the slab)
   if (rank == 0) append_new_row<T, D>(ap, row, kv, L);
 #pragma unroll
   for (int u = 0; u < kHeads; ++u) {
-    const int h = rank + u * kClusterSize;
+    const int h = rank + u * kCtas;
     if (h >= G || d >= D) break;
     float s_self = 0.f;
 #pragma unroll
@@ -663,13 +665,13 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
     s_self *= scale_log2;
     float mm = s_self;
 #pragma unroll
-    for (int r = 0; r < kClusterSize; ++r) mm = fmaxf(mm, in_ml[u][r].x);
+    for (int r = 0; r < kCtas; ++r) mm = fmaxf(mm, in_ml[u][r].x);
     for (int r = 0; r < rg.R; ++r) mm = fmaxf(mm, ring_s[u][r]);
     const float w_self = exp2f(s_self - mm);
     float acc = w_self * v_self;
     float lsum = w_self;
 #pragma unroll
-    for (int r = 0; r < kClusterSize; ++r) {
+    for (int r = 0; r < kCtas; ++r) {
       const float2 ml = in_ml[u][r];
       if (ml.x == -INFINITY) continue;                 // a rank without rows has sent no values
       const float w = exp2f(ml.x - mm);
@@ -687,7 +689,8 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   }
   if (rg.R > 0 && ap.flag_new != nullptr) {
     // the step carries the append: the new token joins the ring once every rank has read it
-    cluster.sync();
+    if constexpr (kCtas > 1) cluster.sync();
+    else __syncthreads();
     constexpr int kVecs = D * (int)sizeof(T) / 16;
     if (rank == 0 && d < kVecs)
       ring_put<kVecs>(rg, kv, d, reinterpret_cast<const uint8_t *>(k_new + (size_t)kv * D),
@@ -696,25 +699,25 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
 }
 
 // groups: clusters (runs of G query slabs on one key/value slab each)
-template <int D, int kMaxG>
+template <int D, int kMaxG, int kCtas>
 static int launch_decode_cluster_mma(int groups, int G, const void *q, const void *k_new, const void *v_new,
                                      const ag_cache &c, float scale_log2, void *o, const AppendArgs &ap,
                                      const HeadMap &hm, const RecentRing &rg, cudaStream_t st) {
   using T = __nv_bfloat16;
   constexpr int smem = gq_smem_bytes(D, kCmStages);
-  AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kClusterSize, groups);
+  cfg.gridDim = dim3(kCtas, groups);
   cfg.blockDim = dim3(kGqThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kClusterSize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[0].val.clusterDim.x = kCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1] = pdl_attribute();
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_mma_kernel<D, kMaxG>, static_cast<const T *>(q),
+  cfg.attrs = kCtas == 1 ? attr + 1 : attr;
+  cfg.numAttrs = kCtas == 1 ? 1 : 2;
+  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_mma_kernel<D, kMaxG, kCtas>, static_cast<const T *>(q),
                                  static_cast<const T *>(k_new), static_cast<const T *>(v_new),
                                  static_cast<const T *>(c.k_rows), static_cast<const T *>(c.v_rows),
                                  c.row_off, c.cap, c.len, scale_log2, static_cast<T *>(o), G, ap, hm, rg));
@@ -755,6 +758,11 @@ static bool decode_carries_append(const ag_layer_desc &d) {
   return d.dtype == AG_BF16 && d.heads / kv_heads_of(d) <= kGqMaxGroup;
 }
 
+// CTAs per slab of the cluster form; 0: the split form.
+static int decode_ctas(int slabs, int max_cap) {
+  return slabs <= kClusterMaxSlabs ? kClusterSize : 0;
+}
+
 template <typename T, int D>
 static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, const void *v_new,
                       const ag_cache &c, float scale, void *o, void *ws, const AppendArgs &ap, cudaStream_t st) {
@@ -765,11 +773,19 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
   const float scale_log2 = scale * 1.4426950408889634f;
   if constexpr (std::is_same_v<T, __nv_bfloat16>) {
     // grouped-query attention: one cluster per key/value slab reads it for all its query heads
-    if (group <= kGqMaxGroup && kv_slabs <= kClusterMaxSlabs)
-      return (group == 1 ? launch_decode_cluster_mma<D, 1> : group <= 8 ? launch_decode_cluster_mma<D, 8> :
-              launch_decode_cluster_mma<D, 16>)(kv_slabs, group, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
-    if (slabs <= kClusterMaxSlabs)
-      return launch_decode_cluster_mma<D, 1>(slabs, 1, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
+    auto cluster = [&](auto ctas, int groups, int G) {
+      constexpr int kCtas = decltype(ctas)::value;
+      return (G == 1 ? launch_decode_cluster_mma<D, 1, kCtas> : G <= 8 ? launch_decode_cluster_mma<D, 8, kCtas> :
+              launch_decode_cluster_mma<D, 16, kCtas>)(groups, G, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
+    };
+    const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
+    // (clusters of one query head each never carry the append: see decode_carries_append)
+    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas(n, c.max_cap) : 0) {
+      case 1: return cluster(std::integral_constant<int, 1>{}, n, G);
+      case 2: return cluster(std::integral_constant<int, 2>{}, n, G);
+      case 4: return cluster(std::integral_constant<int, 4>{}, n, G);
+      case 8: return cluster(std::integral_constant<int, 8>{}, n, G);
+    }
   } else {
     // caches of at most two rounds of one CTA's rows (host-known bound): no cluster
     constexpr int kRound = kUnroll * kClusterThreads / (D / Elem<T>::kPerVec);
