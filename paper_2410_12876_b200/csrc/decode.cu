@@ -758,9 +758,24 @@ static bool decode_carries_append(const ag_layer_desc &d) {
   return d.dtype == AG_BF16 && d.heads / kv_heads_of(d) <= kGqMaxGroup;
 }
 
-// CTAs per slab of the cluster form; 0: the split form.
+// CTAs per slab of the bf16 cluster form; 0: the split form.  From a sweep over 8 .. 1024 slabs of 100 .. 13,000 rows, head_dim
+// 64 and 128, one and four heads per slab (us per step, CTAs per slab 1 | 2 | 4 | 8, split form last):
+//   32 slabs, cap 102      3.1 | 3.6 | 3.7 | 3.9,  5.9     64 slabs, cap 819   7.9 | 6.4 | 5.9 | 8.2,  7.7
+//   128 slabs, cap 1638    15.4 | 12.3 | 13.5 | 15.7,  15.2    384 slabs, cap 409   7.8 | 11.4 | 17.4 | -,  13.3
+//   640 slabs, cap 3276    113 | 108 | 107 | -,  115      1024 slabs, cap 7372   342 | 329 | 323 | 323,  342
+//   8 slabs, cap 13107     79 | 42 | 23 | 13.4,  11.5
+// While a step waits for latency: as many CTAs per slab as one wave holds (3 per SM at 128, 5 at 64), unless the slab
+// has too few rows for them.  Where it waits for HBM: 1024 rows per CTA or fewer, so that long slabs do not end alone.
+// Only few slabs of very many rows need more CTAs than a cluster has.
+template <int D>
 static int decode_ctas(int slabs, int max_cap) {
-  return slabs <= kClusterMaxSlabs ? kClusterSize : 0;
+  constexpr int kSms = 148, kWave = kSms * (D == 128 ? 3 : 5);
+  if (slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
+  int wave = max_cap <= 128 ? 1 : max_cap <= 512 ? 4 : kClusterSize;
+  while (wave > 1 && (int64_t)slabs * wave > kWave) wave /= 2;
+  if (wave == 2 && max_cap <= 512) wave = 1;
+  const int rows = max_cap <= 2048 ? 1 : max_cap <= 4096 ? 4 : kClusterSize;
+  return wave > rows ? wave : rows;
 }
 
 template <typename T, int D>
@@ -780,7 +795,7 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     };
     const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
     // (clusters of one query head each never carry the append: see decode_carries_append)
-    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas(n, c.max_cap) : 0) {
+    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas<D>(n, c.max_cap) : 0) {
       case 1: return cluster(std::integral_constant<int, 1>{}, n, G);
       case 2: return cluster(std::integral_constant<int, 2>{}, n, G);
       case 4: return cluster(std::integral_constant<int, 4>{}, n, G);
@@ -804,11 +819,12 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
   if (n_chunks > 0 && decode_gqa_mma_supported(d)) {
     // grouped-query attention, bf16: the group's heads are the rows of a tensor-core tile
     rc = launch_decode_partial_gqa_mma(d, q, c, scale_log2, chunk_rows, n_chunks, part_o, part_ml, kMaxSplits, st);
-  } else if (n_chunks > 0 && (group == 2 || group == 4)) {
+  } else if (std::is_same_v<T, float> && n_chunks > 0 && (group == 2 || group == 4)) {
     // grouped-query attention: the rows of a key/value slab are read once for its query heads
-    rc = launch_pdl(group == 2 ? decode_partial_gqa_kernel<T, D, 2> : decode_partial_gqa_kernel<T, D, 4>,
-                    dim3(n_chunks, kv_slabs), dim3(kPartThreads), 0, st, qp, kr, vr, c.row_off, c.len, scale_log2,
-                    chunk_rows, part_o, part_ml, hm.kv_heads);
+    if constexpr (std::is_same_v<T, float>)
+      rc = launch_pdl(group == 2 ? decode_partial_gqa_kernel<T, D, 2> : decode_partial_gqa_kernel<T, D, 4>,
+                      dim3(n_chunks, kv_slabs), dim3(kPartThreads), 0, st, qp, kr, vr, c.row_off, c.len, scale_log2,
+                      chunk_rows, part_o, part_ml, hm.kv_heads);
   } else if (n_chunks > 0) {
     rc = launch_pdl(decode_partial_kernel<T, D>, dim3(n_chunks, slabs), dim3(kPartThreads), 0, st, qp, kr, vr, c.row_off,
                     c.len, scale_log2, chunk_rows, part_o, part_ml, hm);

@@ -41,3 +41,36 @@ def test_lengths_at_the_edges_of_blocks(D, h, hk):
         T.check_close(T.f64(o), orc.decode_attention(T.f64(q), T.f64(kn), T.f64(vn), held), "bf16", f"step {step}")
     assert np.array_equal(cache.len.cpu().numpy(), lens + 2)
     assert int(status.item()) == 0 and ag.ag_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("B,h,hk,D,longest", [
+    (28, 8, 8, 128, 120), (3, 64, 4, 64, 120),           # one CTA per slab, 1 and 16 heads
+    (24, 32, 8, 64, 300), (20, 32, 8, 128, 700),         # one and two: what one wave holds
+    (12, 16, 8, 128, 400), (60, 8, 8, 128, 2100),        # four: by the wave, by the rows per CTA
+    (9, 18, 9, 64, 4200),                                # eight, by the rows per CTA
+    (1, 8, 8, 128, 8300), (1, 32, 2, 64, 8300),          # few slabs of very many rows: the split form
+])
+def test_ctas_per_slab(B, h, hk, D, longest):
+    """Each choice of CTAs per slab, over empty, one-row and full slabs among ragged ones, with the append."""
+    rng = np.random.default_rng(longest)
+    lens = rng.integers(0, longest // 4, size=B * hk)
+    lens[:3] = 0, 1, longest
+    shape = LayerShape(B, longest + 8, 64, h, D, 1, 64, "bf16", kv_heads=hk)
+    cap = lens + 2
+    cap[1] = 1                                           # full: the append is refused
+    cache = ag.RaggedCache.allocate(shape, cap, DEV)
+    cache.k_rows.copy_(inputs.randn(tuple(cache.k_rows.shape), 41, DEV, torch.bfloat16))
+    cache.v_rows.copy_(inputs.randn(tuple(cache.v_rows.shape), 42, DEV, torch.bfloat16))
+    cache.len.copy_(torch.from_numpy(lens.astype(np.int32)))
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    for step in range(2):
+        held = T.gpu_cache_as_lists(cache, shape)
+        q, kn, vn, fn = inputs.decode_inputs(shape, 50, step, DEV, keep_new=1.0)
+        o = T.gpu_decode_step(shape, q, kn, vn, fn, cache, status, fused=True)
+        T.check_close(T.f64(o), orc.decode_attention(T.f64(q), T.f64(kn), T.f64(vn), held), "bf16", f"step {step}")
+    assert np.array_equal(cache.len.cpu().numpy(), np.minimum(lens + 2, cap))
+    rows, off = T.f64(cache.k_rows), cache.row_off.cpu().numpy()
+    for s in range(0, B * hk, 5):
+        if s != 1:
+            assert np.array_equal(rows[off[s] + lens[s] + 1], T.f64(kn).reshape(-1, D)[s])
+    assert int(status.item()) == ag.AG_DEV_OVERFLOW and ag.ag_device_wait_timeouts() == 0
