@@ -8,11 +8,10 @@
 // HBM-bound: every cache row is read exactly once with 16-byte vector loads,
 // one row per group of kLanes consecutive lanes, several rows in flight per lane.
 //
-// Two forms.  Few slabs (a launch is latency-bound): one thread-block cluster
-// per slab, one chunk per CTA, the triples merged through distributed shared
-// memory by the cluster's first CTA - one kernel, no scratch.  Many slabs:
-// decode_partial_kernel writes the triples of up to kMaxSplits chunks per slab
-// to the workspace and decode_combine_kernel merges them.
+// Two forms.  One thread-block cluster (or one CTA) per slab, the triples merged through distributed shared
+// memory - one kernel, no scratch: bf16 nearly always (decode_ctas), float32 up to kClusterMaxSlabs slabs.
+// Otherwise decode_partial_kernel writes the triples of up to kMaxSplits chunks per slab to the workspace and
+// decode_combine_kernel merges them.
 #include <cooperative_groups.h>
 #include <math.h>
 #include <nvtx3/nvToolsExt.h>
@@ -27,7 +26,7 @@ namespace ag {
 constexpr int kMaxSplits = 32;     // chunks per slab the workspace is sized for
 constexpr int kPartThreads = 256;
 constexpr int kUnroll = 8;         // rows in flight per lane group (x2: K and V)
-constexpr int kClusterMaxSlabs = 64;    // up to here one cluster per slab; beyond, split-K through the workspace
+constexpr int kClusterMaxSlabs = 64;    // float32, and groups of more than 16 heads: up to here one cluster per slab
 constexpr int kClusterThreads = 512;    // 256 rows in flight per CTA of a cluster (bf16, D = 128)
 
 // Grouped-query attention: slab s = (sequence, query head) of q and o reads the cache slab, k_new

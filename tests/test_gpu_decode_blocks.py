@@ -48,7 +48,7 @@ def test_lengths_at_the_edges_of_blocks(D, h, hk):
     (24, 32, 8, 64, 300), (20, 32, 8, 128, 700),         # one and two: what one wave holds
     (12, 16, 8, 128, 400), (60, 8, 8, 128, 2100),        # four: by the wave, by the rows per CTA
     (9, 18, 9, 64, 4200),                                # eight, by the rows per CTA
-    (1, 8, 8, 128, 8300), (1, 32, 2, 64, 8300),          # few slabs of very many rows: the split form
+    (1, 8, 8, 128, 8300), (1, 64, 4, 64, 8300),          # few slabs of very many rows: the split form
 ])
 def test_ctas_per_slab(B, h, hk, D, longest):
     """Each choice of CTAs per slab, over empty, one-row and full slabs among ragged ones, with the append."""
