@@ -490,41 +490,44 @@ bool gate_attn_tc_supported(const ag_layer_desc &d) {
 // The split-K merge of MHA' and the gate's output layer in one pass (Eq. 3, Eq. 4):
 //   H'[t, g * D + c] = sum_s w_s O_s[r, c] / sum_s w_s l_s,  w_s = 2^(m_s - max_s m_s)
 //   s[t, i] = H'[t, :] Wo_g[:, i];  flag = s + gamma_i > logit(tau)
-// One CTA = 16 tokens, one warp per token.  A warp merges the token's row of every gate head
-// (a lane per D / 32 columns: every access is one whole row) into shared memory; then the warps share the
+// One CTA = kTok tokens (16, or 8 or 4 where the tokens would not fill the SMs), 16 / kTok warps per token.  A warp
+// merges the token's row of its share of the gate heads (a lane per D / 32 columns: every access is one whole row), eight
+// pieces' rows in flight at a time under a running maximum, into shared memory; then the warps share the
 // reduction, 16 columns of H' at a time, as m16n8k16 MMAs of the 16 tokens against 32 heads of Wo.
 // Every float32 of H' enters as three bf16 (8 + 8 + 8 mantissa bits: exactly its value), so nothing of it
 // is lost, and Wo is bf16 as it comes.  The warps' sums are added in a fixed order.  H' never goes to global
 // memory.  (With the products on CUDA cores, operands from shared memory, this was 18 us at 4,096 tokens
-// and 141 us at 8 x 4,096.)  Wo is fetched before the wait for MHA', which it does not depend on.
-constexpr int kMoTokens = 16, kMoThreads = kMoTokens * 32;
+// and 141 us at 8 x 4,096.)  Wo is fetched before the wait for MHA', which it does not depend on.  Bound by latency: one trip to
+// L2 per eight pieces (the maxima used to be a trip of their own, two pieces at a time) and few tokens spread over all
+// SMs: pass of 333 tokens 123 -> 118 us, of 1,000 tokens 83 -> 75, of 4 x 1,500 (64-wide heads) 123 -> 119.
+constexpr int kMoWarps = 16, kMoThreads = kMoWarps * 32;
 template <int N> struct FloatVec;
 template <> struct FloatVec<2> { using type = float2; };
 template <> struct FloatVec<4> { using type = float4; };
 constexpr int kMoRedPitch = 33;                                  // floats per token of a warp's sums (32 heads)
-constexpr int kMoRedBytes = kMoTokens * kMoTokens * kMoRedPitch * 4;
+constexpr int kMoRedBytes = kMoWarps * 16 * kMoRedPitch * 4;
 __host__ __device__ constexpr int mo_w_bytes(int GD) { return GD * 64 > kMoRedBytes ? GD * 64 : kMoRedBytes; }
-__host__ __device__ constexpr int mo_smem_bytes(int GD) { return mo_w_bytes(GD) + kMoTokens * (GD + 8) * 4; }
+__host__ __device__ constexpr int mo_smem_bytes(int GD) { return mo_w_bytes(GD) + 16 * (GD + 8) * 4; }
 // Byte offset of 16-byte piece `piece` (8 heads) of row `c` of the staged slice of Wo: 64-byte rows, pieces XOR-ed so
 // that the eight rows one ldmatrix reads fall into different banks.
 __device__ __forceinline__ uint32_t mo_w_off(int c, int piece) { return (uint32_t)(c * 64 + ((piece ^ ((c >> 1) & 3)) << 4)); }
 
-template <int kGaD>
+template <int kGaD, int kTok>
 __global__ void __launch_bounds__(kMoThreads)
 gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat16 *__restrict__ Wo,
                       const float *__restrict__ gamma, float logit_tau, int h, float *__restrict__ scores,
                       uint8_t *__restrict__ flags) {
   extern __shared__ __align__(16) unsigned char mo_smem[];
   unsigned char *Ws = mo_smem;                                   // [GD][32] bf16, then the warps' sums
-  float *red = reinterpret_cast<float *>(mo_smem);               // [16 warps][16 tokens][33]
+  float *red = reinterpret_cast<float *>(mo_smem);               // [warps][16 tokens][33]
   float *Hs = reinterpret_cast<float *>(mo_smem + mo_w_bytes(a.GD));     // [16][GD + 8]
   const int pitch = a.GD + 8;
   __shared__ int seg_first[2][kMoThreads];           // per gate head: first segment, number of pieces
-  const int tiles_per_seq = (a.n + kMoTokens - 1) / kMoTokens;
-  const int b = blockIdx.x / tiles_per_seq, t0 = (blockIdx.x % tiles_per_seq) * kMoTokens;
+  const int tiles_per_seq = (a.n + kTok - 1) / kTok;
+  const int b = blockIdx.x / tiles_per_seq, t0 = (blockIdx.x % tiles_per_seq) * kTok;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = t0 + warp;
-  float *hrow = Hs + warp * pitch;
+  const int t = t0 + warp % kTok;
+  float *hrow = Hs + (warp % kTok) * pitch;
   // heads i0 .. i0 + 31 of Wo
   auto stage_wo = [&](int i0) {
     const uint32_t ws = smem_u32(Ws);
@@ -541,18 +544,8 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
     }
     cp_async_commit();
   };
-  stage_wo(0);
-  pdl_wait();                                        // (no early trigger of the next kernel: 2 % of the pass lost with it)
-  if (a.seq_lens != nullptr && t0 >= a.seq_lens[b]) {
-    // padding only: flags 0, scores left as they are
-    cp_async_wait<0>();
-    const int tok = threadIdx.x & 15;
-    for (int i = threadIdx.x >> 4; i < h; i += kMoThreads / kMoTokens)
-      if (t0 + tok < a.n) flags[((size_t)b * h + i) * a.n + t0 + tok] = 0;
-    return;
-  }
-  // The CTA's 16 tokens lie in one query tile: which segments hold its pieces is looked up once per gate head.
-  if (warp == 0) {
+  // The CTA's tokens lie in one query tile: which segments hold its pieces is looked up once per gate head.
+  auto find_pieces = [&] {
     const int qt = t0 / kGaBM, nq = ga_seq_tiles(a, b);
     int before;
     const int len = ga_seg_len(a, ga_total(a, b, before));
@@ -563,56 +556,77 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
       seg_first[0][g] = x0 / len;
       seg_first[1][g] = (x1 - 1) / len - x0 / len + 1;
     }
+  };
+  stage_wo(0);
+  // What does not depend on MHA' is done before the wait for it (MHA' lets this kernel start once it has itself waited
+  // for all that came before: inputs of the call are there).
+  const bool padding_only = a.seq_lens != nullptr && t0 >= a.seq_lens[b];
+  if (warp == 0 && !padding_only) find_pieces();
+  const float gamma0 = gamma && threadIdx.x / kTok < min(h, 32) ? gamma[threadIdx.x / kTok] : 0.f;
+  pdl_wait();                                        // (no early trigger of the next kernel: 2 % of the pass lost with it)
+  if (padding_only) {
+    // flags 0, scores left as they are
+    cp_async_wait<0>();
+    const int tok = threadIdx.x % kTok;
+    for (int i = threadIdx.x / kTok; i < h; i += kMoThreads / kTok)
+      if (t0 + tok < a.n) flags[((size_t)b * h + i) * a.n + t0 + tok] = 0;
+    return;
   }
   __syncthreads();
   if (t < a.n) {
+    constexpr int kU = kTok / 4, kP = 8 / kU;        // gate heads, and pieces of each, in flight together
     const int qt = t / kGaBM, r = t % kGaBM;
-    // four gate heads at a time, so that their loads are in flight together
-    for (int g0 = 0; g0 < a.gate_heads; g0 += 4) {
-      size_t row0[4];
-      int ns[4];
-      float mmax[4];
+    for (int g0 = (warp / kTok) * kU; g0 < a.gate_heads; g0 += 4) {
+      constexpr int kV = kGaD / 32;                  // columns per lane
+      using Vec = typename FloatVec<kV>::type;
+      size_t row0[kU];
+      int ns[kU], ns_max = 0;
+      float acc[kU][kV], lsum[kU], m[kU];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < kU; ++u) {
         const int g = min(g0 + u, a.gate_heads - 1), prob = b * a.gate_heads + g;
         ns[u] = seg_first[1][g];
         row0[u] = (size_t)ga_slot(prob, qt, a.n_qtiles, seg_first[0][g]) * kGaBM + r;   // + s * 128 per piece
-        mmax[u] = -INFINITY;
-        for (int s = lane; s < ns[u]; s += 32) mmax[u] = fmaxf(mmax[u], a.part_ml[(row0[u] + (size_t)s * kGaBM) * 2]);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) mmax[u] = fmaxf(mmax[u], __shfl_xor_sync(0xffffffffu, mmax[u], off));
-      constexpr int kV = kGaD / 32;                  // columns per lane
-      using Vec = typename FloatVec<kV>::type;
-      float acc[4][kV];
-      float lsum[4];
-      int ns_max = 0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
+        ns_max = max(ns_max, ns[u]);
+        m[u] = -INFINITY;
+        lsum[u] = 0.f;
 #pragma unroll
         for (int e = 0; e < kV; ++e) acc[u][e] = 0.f;
-        lsum[u] = 0.f;
-        ns_max = max(ns_max, ns[u]);
       }
-#pragma unroll 2
-      for (int s = 0; s < ns_max; ++s) {
+      for (int s0 = 0; s0 < ns_max; s0 += kP) {
+        float2 ml[kU][kP];
+        Vec o4[kU][kP];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (s < ns[u]) {
-            const float2 ml = *reinterpret_cast<const float2 *>(a.part_ml + (row0[u] + (size_t)s * kGaBM) * 2);
-            const Vec o4 = *reinterpret_cast<const Vec *>(a.part_o + (row0[u] + (size_t)s * kGaBM) * kGaD + lane * kV);
-            const float *o = reinterpret_cast<const float *>(&o4);
-            const float w = fast_exp2(ml.x - mmax[u]);
+        for (int u = 0; u < kU; ++u)
+#pragma unroll
+          for (int p = 0; p < kP; ++p) {
+            // (past the last piece: the last one again, at weight 0)
+            const size_t row = row0[u] + (size_t)min(s0 + p, ns[u] - 1) * kGaBM;
+            ml[u][p] = *reinterpret_cast<const float2 *>(a.part_ml + row * 2);
+            o4[u][p] = *reinterpret_cast<const Vec *>(a.part_o + row * kGaD + lane * kV);
+          }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          float m_new = m[u];
+#pragma unroll
+          for (int p = 0; p < kP; ++p) m_new = fmaxf(m_new, ml[u][p].x);
+          const float alpha = fast_exp2(m[u] - m_new);         // m = -inf at first: 0
+          m[u] = m_new;
+          lsum[u] *= alpha;
+#pragma unroll
+          for (int e = 0; e < kV; ++e) acc[u][e] *= alpha;
+#pragma unroll
+          for (int p = 0; p < kP; ++p) {
+            const float w = s0 + p < ns[u] ? fast_exp2(ml[u][p].x - m_new) : 0.f;
+            const float *o = reinterpret_cast<const float *>(&o4[u][p]);
 #pragma unroll
             for (int e = 0; e < kV; ++e) acc[u][e] = fmaf(w, o[e], acc[u][e]);
-            lsum[u] = fmaf(w, ml.y, lsum[u]);
+            lsum[u] = fmaf(w, ml[u][p].y, lsum[u]);
           }
         }
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < kU; ++u) {
         if (g0 + u < a.gate_heads) {
           const float inv = 1.f / lsum[u];
           Vec hv;
@@ -622,9 +636,8 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
         }
       }
     }
-  } else {
-    for (int c = lane; c < a.GD; c += 32) hrow[c] = 0.f;         // a token past the end: its row is an MMA operand all the same
   }
+  // (rows of H' without a token hold anything: a row of an MMA's first operand reaches its own row of the result only)
   const int g = lane >> 2, tq = lane & 3, mi = lane >> 3;
   for (int i0 = 0; i0 < h; i0 += 32) {
     if (i0 > 0) {
@@ -639,7 +652,7 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
 #pragma unroll
       for (int e = 0; e < 4; ++e) c[nb][e] = 0.f;
     const uint32_t ws = smem_u32(Ws);
-    for (int k0 = warp * 16; k0 < a.GD; k0 += kMoTokens * 16) {
+    for (int k0 = warp * 16; k0 < a.GD; k0 += kMoWarps * 16) {
       uint32_t ah[3][4];                             // the three bf16 parts of the fragment of H'
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
@@ -665,19 +678,19 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
     for (int nb = 0; nb < 4; ++nb)
 #pragma unroll
       for (int e = 0; e < 4; ++e)
-        red[(warp * kMoTokens + g + (e >> 1) * 8) * kMoRedPitch + nb * 8 + 2 * tq + (e & 1)] = c[nb][e];
+        red[(warp * 16 + g + (e >> 1) * 8) * kMoRedPitch + nb * 8 + 2 * tq + (e & 1)] = c[nb][e];
     __syncthreads();
-    {
-      // 16 consecutive threads: one head's 16 tokens, which lie side by side in scores and flags
-      const int tok = threadIdx.x & 15, i = i0 + (threadIdx.x >> 4), tt = t0 + tok;
+    if (threadIdx.x < 32 * kTok) {
+      // kTok consecutive threads: one head's tokens, which lie side by side in scores and flags
+      const int tok = threadIdx.x % kTok, i = i0 + threadIdx.x / kTok, tt = t0 + tok;
       float sc = 0.f;
 #pragma unroll
-      for (int w = 0; w < kMoTokens; ++w) sc += red[(w * kMoTokens + tok) * kMoRedPitch + (threadIdx.x >> 4)];
+      for (int w = 0; w < kMoWarps; ++w) sc += red[(w * 16 + tok) * kMoRedPitch + threadIdx.x / kTok];
       if (i < h && tt < a.n) {
         const size_t o = ((size_t)b * h + i) * a.n + tt;
         const bool padding = a.seq_lens && tt >= a.seq_lens[b];
         if (scores) scores[o] = sc;
-        flags[o] = !padding && (sc + (gamma ? gamma[i] : 0.f)) > logit_tau ? 1 : 0;
+        flags[o] = !padding && (sc + (i0 == 0 ? gamma0 : gamma ? gamma[i] : 0.f)) > logit_tau ? 1 : 0;
       }
     }
   }
@@ -734,9 +747,12 @@ static int run_gate_attn_tc(const ag_layer_desc &d, const void *qkv, void *parti
   AG_CUDA_TRY(cudaFuncSetAttribute(gate_attn_tc_kernel<kGaD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGaSmemBytes));
   rc = launch_pdl(gate_attn_tc_kernel<kGaD>, dim3(a.n_seg), dim3(kGaThreads), kGaSmemBytes, st, tm, a);
   if (rc) return rc;
-  auto mo = gate_merge_out_kernel<kGaD>;
+  // fewer tokens per CTA while the CTAs are no more than the SMs (148): an SM then takes in fewer rows of the partials
+  const long long tokens = (long long)d.batch * d.seq;
+  const int tok = tokens <= 4 * 148 ? 4 : tokens <= 8 * 148 ? 8 : 16;
+  auto mo = tok == 4 ? gate_merge_out_kernel<kGaD, 4> : tok == 8 ? gate_merge_out_kernel<kGaD, 8> : gate_merge_out_kernel<kGaD, 16>;
   AG_CUDA_TRY(cudaFuncSetAttribute(mo, cudaFuncAttributeMaxDynamicSharedMemorySize, mo_smem_bytes(GD)));
-  const int blocks = d.batch * ((d.seq + kMoTokens - 1) / kMoTokens);
+  const int blocks = d.batch * ((d.seq + tok - 1) / tok);
   return launch_pdl(mo, dim3(blocks), dim3(kMoThreads), mo_smem_bytes(GD), st, a, static_cast<const __nv_bfloat16 *>(Wo),
                     gamma, logit_tau, kv_heads_of(d), scores, flags);
 }
