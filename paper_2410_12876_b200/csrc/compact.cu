@@ -7,7 +7,8 @@
 //                    before its chunk and in the slab, ranks its own tokens by warp ballot +
 //                    popc, writes prefix and idx for them, and moves the retained rows of its
 //                    chunk: 16-byte-vector row moves, only retained rows are read, every access
-//                    is a full row.  One launch; no pass over the flags on its own.
+//                    is a full row.  One launch; no pass over the flags on its own.  A slab's last CTA also fills the
+//                    ring of a recent-token window (a launch of its own cost ~5 us).
 #include "ag_common.cuh"
 
 namespace ag {
@@ -17,6 +18,37 @@ constexpr int kCompactThreads = 256;   // = tokens per CTA
 // Bytes of a 32-bit word that are not zero.
 __device__ __forceinline__ int nonzero_bytes(uint32_t w) { return __popc(__vcmpne4(w, 0u) & 0x01010101u); }
 
+// Recent-token window: after the prompt, the ring of a slab holds its last R tokens (token t in
+// slot t % R), the evicted ones marked live; a prompt shorter than R leaves the other slots dead.
+// With per-sequence lengths the prompt of a slab is the first seq_lens[b] of its n positions.
+// The threads of one CTA per slab: (slot, 16-byte piece) pairs in turn.
+struct RecentFill {
+  RecentRing ring;
+  const int32_t *seq_lens;
+  int kv_heads;
+};
+template <int kRowBytes>
+__device__ __forceinline__ void recent_fill(const uint8_t *K, const uint8_t *V, const uint8_t *flags, int n,
+                                            const RecentFill &rf, int slab) {
+  constexpr int kVecs = kRowBytes / 16;
+  const RecentRing &ring = rf.ring;
+  const int len = rf.seq_lens ? min(max(rf.seq_lens[slab / rf.kv_heads], 0), n) : n;   // tokens of this slab's prompt
+  for (int x = threadIdx.x; x < ring.R * kVecs; x += blockDim.x) {
+    const int slot = x / kVecs, v = x % kVecs;
+    // the last token whose number is slot modulo R, if the prompt has one
+    const bool have = slot <= len - 1;
+    const int t = have ? slot + (len - 1 - slot) / ring.R * ring.R : 0;
+    if (have) {
+      const size_t src = ((size_t)slab * n + t) * kRowBytes + v * 16;
+      const size_t dst = ((size_t)slab * ring.R + slot) * kRowBytes + v * 16;
+      *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ring.k) + dst) = *reinterpret_cast<const uint4 *>(K + src);
+      *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ring.v) + dst) = *reinterpret_cast<const uint4 *>(V + src);
+    }
+    if (v == 0) ring.live[(size_t)slab * ring.R + slot] = (have && flags[(size_t)slab * n + t] == 0) ? 1 : 0;
+  }
+  if (threadIdx.x == 0) ring.pos[slab] = len;
+}
+
 // One row = D * sizeof(T) bytes = kVecs 16-byte vectors; a group of kVecs consecutive lanes moves
 // one row of K and one row of V.  kRowBytes = 0: count pass, no rows move.
 template <int kRowBytes>
@@ -25,7 +57,7 @@ compact_kernel(const uint8_t *flags, int n, const int32_t *cap,
                int32_t *len, int32_t *prefix, int32_t *idx,
                int32_t *dev_status, const uint8_t *K,
                const uint8_t *V, const int64_t *row_off,
-               uint8_t *k_rows, uint8_t *v_rows) {
+               uint8_t *k_rows, uint8_t *v_rows, const RecentFill rf) {
   const int slab = blockIdx.y, t0 = blockIdx.x * kCompactThreads;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint8_t *f = flags + (size_t)slab * n;
@@ -37,20 +69,29 @@ compact_kernel(const uint8_t *flags, int n, const int32_t *cap,
   pdl_launch_dependents();
   // retained tokens before this chunk, and in the slab
   int before = 0, total = 0;
-  if ((n & 15) == 0) {                       // rows of the flag array start on 16-byte boundaries
-    const uint4 *fv = reinterpret_cast<const uint4 *>(f);
-    for (int x = threadIdx.x; x < n / 16; x += kCompactThreads) {
-      const uint4 w = ld128(fv + x);
-      const int c = nonzero_bytes(w.x) + nonzero_bytes(w.y) + nonzero_bytes(w.z) + nonzero_bytes(w.w);
-      total += c;
-      if (x * 16 < t0) before += c;          // t0 is a multiple of 16: a vector lies on one side
+  // 16-byte vectors from the first 16-byte boundary of the row, single flags before it and after the last vector
+  const int head = min((int)(-reinterpret_cast<intptr_t>(f) & 15), n), n_vec = (n - head) / 16, tail0 = head + n_vec * 16;
+  for (int x = threadIdx.x; x < n_vec; x += kCompactThreads) {
+    const uint4 w = ld128(f + head + x * 16);
+    const int c = nonzero_bytes(w.x) + nonzero_bytes(w.y) + nonzero_bytes(w.z) + nonzero_bytes(w.w);
+    total += c;
+    const int below = t0 - (head + x * 16);  // the vector's tokens before this chunk
+    if (below >= 16) {
+      before += c;
+    } else if (below > 0) {
+      const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int b = below - 4 * e;
+        before += nonzero_bytes(b >= 4 ? ws[e] : b > 0 ? ws[e] & ((1u << (8 * b)) - 1u) : 0u);
+      }
     }
-  } else {
-    for (int x = threadIdx.x; x < n; x += kCompactThreads) {
-      const int c = f[x] != 0;
-      total += c;
-      if (x < t0) before += c;
-    }
+  }
+  if (threadIdx.x < 32) {
+    const int x = lane < 16 ? (lane < head ? lane : n) : tail0 + lane - 16;      // (at most 15 of either)
+    const int c = x < n && f[x] != 0;
+    total += c;
+    if (x < t0) before += c;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -88,6 +129,10 @@ compact_kernel(const uint8_t *flags, int n, const int32_t *cap,
     pre[n] = total;
     len[slab] = overflow ? 0 : total;
     if (overflow && dev_status) atomicOr(dev_status, AG_DEV_OVERFLOW);
+  }
+  if constexpr (kRowBytes != 0) {
+    // (a slab's last CTA has the fewest rows to move)
+    if (rf.ring.R > 0 && blockIdx.x == gridDim.x - 1) recent_fill<kRowBytes>(K, V, flags, n, rf, slab);
   }
   if (kRowBytes == 0 || overflow) return;    // count pass, or a slab that does not fit: nothing moves
   __syncthreads();
@@ -150,29 +195,12 @@ append_rows_kernel(const uint8_t *k_new, const uint8_t *v_new,
     ring_put<kVecs>(ring, slab, v, k_new + (size_t)slab * kRowBytes, v_new + (size_t)slab * kRowBytes, want);
 }
 
-// Recent-token window: after the prompt, the ring of a slab holds its last R tokens (token t in
-// slot t % R), the evicted ones marked live; a prompt shorter than R leaves the other slots dead.
-// With per-sequence lengths the prompt of a slab is the first seq_lens[b] of its n positions.
-// One CTA per slab, thread (slot, 16-byte piece).
+// The same as a launch of its own, one CTA per slab: for a projection that moves the rows itself.
 template <int kRowBytes>
-__global__ void recent_fill_kernel(const uint8_t *K, const uint8_t *V,
-                                   const uint8_t *flags, int n, const int32_t *seq_lens,
-                                   int kv_heads, const RecentRing ring) {
-  constexpr int kVecs = kRowBytes / 16;
-  const int slab = blockIdx.x, slot = threadIdx.x / kVecs, v = threadIdx.x % kVecs;
-  if (slot >= ring.R) return;
-  const int len = seq_lens ? min(max(seq_lens[slab / kv_heads], 0), n) : n;   // tokens of this slab's prompt
-  // the last token whose number is slot modulo R, if the prompt has one
-  const bool have = slot <= len - 1;
-  const int t = have ? slot + (len - 1 - slot) / ring.R * ring.R : 0;
-  if (have) {
-    const size_t src = ((size_t)slab * n + t) * kRowBytes + v * 16;
-    const size_t dst = ((size_t)slab * ring.R + slot) * kRowBytes + v * 16;
-    *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ring.k) + dst) = *reinterpret_cast<const uint4 *>(K + src);
-    *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ring.v) + dst) = *reinterpret_cast<const uint4 *>(V + src);
-  }
-  if (v == 0) ring.live[(size_t)slab * ring.R + slot] = (have && flags[(size_t)slab * n + t] == 0) ? 1 : 0;
-  if (threadIdx.x == 0) ring.pos[slab] = len;
+__global__ void recent_fill_kernel(const uint8_t *K, const uint8_t *V, const uint8_t *flags, int n, const RecentFill rf) {
+  pdl_launch_dependents();
+  pdl_wait();
+  recent_fill<kRowBytes>(K, V, flags, n, rf, blockIdx.x);
 }
 
 static int row_bytes(const ag_layer_desc &d) {
@@ -202,12 +230,8 @@ int launch_compact(const ag_layer_desc &d, const void *K, const void *V, const u
     case 512: kern = compact_kernel<512>; break;
     default: return AG_ERR_UNSUPPORTED;
   }
-  const int rc = launch_pdl(kern, grid, dim3(kCompactThreads), 0, st, flags, d.seq, c.cap, c.len, prefix, ix, dev_status, Kb,
-                            Vb, c.row_off, kr, vr);
-  if (rc) return rc;
-  const RecentRing ring = ring_of(d, c);
-  if (K && ring.R > 0) return launch_recent_fill(d, K, V, flags, c, st);
-  return AG_OK;
+  return launch_pdl(kern, grid, dim3(kCompactThreads), 0, st, flags, d.seq, c.cap, c.len, prefix, ix, dev_status, Kb,
+                            Vb, c.row_off, kr, vr, RecentFill{ring_of(d, c), d.seq_lens, kv_heads_of(d)});
 }
 
 // Ring of a recent-token window from the dense K, V of the prompt (one more small launch).
@@ -218,14 +242,9 @@ int launch_recent_fill(const ag_layer_desc &d, const void *K, const void *V, con
   const int slabs = d.batch * kv_heads_of(d);
   auto Kb = static_cast<const uint8_t *>(K);
   auto Vb = static_cast<const uint8_t *>(V);
-  const int threads = ring.R * (row_bytes(d) / 16);
-  switch (row_bytes(d)) {
-    case 128: recent_fill_kernel<128><<<slabs, threads, 0, st>>>(Kb, Vb, flags, d.seq, d.seq_lens, kv_heads_of(d), ring); break;
-    case 256: recent_fill_kernel<256><<<slabs, threads, 0, st>>>(Kb, Vb, flags, d.seq, d.seq_lens, kv_heads_of(d), ring); break;
-    default: recent_fill_kernel<512><<<slabs, threads, 0, st>>>(Kb, Vb, flags, d.seq, d.seq_lens, kv_heads_of(d), ring); break;
-  }
-  AG_LAUNCH_CHECK();
-  return AG_OK;
+  auto kern = row_bytes(d) == 128 ? recent_fill_kernel<128> : row_bytes(d) == 256 ? recent_fill_kernel<256> : recent_fill_kernel<512>;
+  return launch_pdl(kern, dim3(slabs), dim3(ring.R * (row_bytes(d) / 16)), 0, st, Kb, Vb, flags, d.seq,
+                    RecentFill{ring, d.seq_lens, kv_heads_of(d)});
 }
 
 int launch_append(const ag_layer_desc &d, const void *k_new, const void *v_new,
