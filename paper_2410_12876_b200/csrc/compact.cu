@@ -51,7 +51,8 @@ __device__ __forceinline__ void recent_fill(const uint8_t *K, const uint8_t *V, 
 
 // One row = D * sizeof(T) bytes = kVecs 16-byte vectors; a group of kVecs consecutive lanes moves
 // one row of K and one row of V.  kRowBytes = 0: count pass, no rows move.
-template <int kRowBytes>
+// kRing: the layer has a recent-token window (without one, its code costs the copy 1 us in 13).
+template <int kRowBytes, bool kRing>
 __global__ void __launch_bounds__(kCompactThreads)
 compact_kernel(const uint8_t *flags, int n, const int32_t *cap,
                int32_t *len, int32_t *prefix, int32_t *idx,
@@ -75,16 +76,17 @@ compact_kernel(const uint8_t *flags, int n, const int32_t *cap,
     const uint4 w = ld128(f + head + x * 16);
     const int c = nonzero_bytes(w.x) + nonzero_bytes(w.y) + nonzero_bytes(w.z) + nonzero_bytes(w.w);
     total += c;
-    const int below = t0 - (head + x * 16);  // the vector's tokens before this chunk
-    if (below >= 16) {
-      before += c;
-    } else if (below > 0) {
-      const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+    if (head + x * 16 + 16 <= t0) before += c;
+  }
+  // the one vector that t0 may fall into: its tokens before this chunk (a warp of its own: nothing in the loop above waits)
+  const int cut = (t0 - head) & 15, x_cut = (t0 - head) / 16;
+  if (threadIdx.x == 32 && t0 > head && cut != 0 && x_cut < n_vec) {
+    const uint4 w = ld128(f + head + x_cut * 16);
+    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int b = below - 4 * e;
-        before += nonzero_bytes(b >= 4 ? ws[e] : b > 0 ? ws[e] & ((1u << (8 * b)) - 1u) : 0u);
-      }
+    for (int e = 0; e < 4; ++e) {
+      const int b = cut - 4 * e;
+      before += nonzero_bytes(b >= 4 ? ws[e] : b > 0 ? ws[e] & ((1u << (8 * b)) - 1u) : 0u);
     }
   }
   if (threadIdx.x < 32) {
@@ -130,9 +132,9 @@ compact_kernel(const uint8_t *flags, int n, const int32_t *cap,
     len[slab] = overflow ? 0 : total;
     if (overflow && dev_status) atomicOr(dev_status, AG_DEV_OVERFLOW);
   }
-  if constexpr (kRowBytes != 0) {
+  if constexpr (kRing) {
     // (a slab's last CTA has the fewest rows to move)
-    if (rf.ring.R > 0 && blockIdx.x == gridDim.x - 1) recent_fill<kRowBytes>(K, V, flags, n, rf, slab);
+    if (blockIdx.x == gridDim.x - 1) recent_fill<kRowBytes>(K, V, flags, n, rf, slab);
   }
   if (kRowBytes == 0 || overflow) return;    // count pass, or a slab that does not fit: nothing moves
   __syncthreads();
@@ -222,16 +224,18 @@ int launch_compact(const ag_layer_desc &d, const void *K, const void *V, const u
   auto Vb = static_cast<const uint8_t *>(V);
   auto kr = static_cast<uint8_t *>(c.k_rows);
   auto vr = static_cast<uint8_t *>(c.v_rows);
-  decltype(&compact_kernel<0>) kern;
+  const RecentRing ring = ring_of(d, c);
+  const bool r = ring.R > 0;
+  decltype(&compact_kernel<0, false>) kern;
   switch (K ? row_bytes(d) : 0) {
-    case 0: kern = compact_kernel<0>; break;
-    case 128: kern = compact_kernel<128>; break;
-    case 256: kern = compact_kernel<256>; break;
-    case 512: kern = compact_kernel<512>; break;
+    case 0: kern = compact_kernel<0, false>; break;
+    case 128: kern = r ? compact_kernel<128, true> : compact_kernel<128, false>; break;
+    case 256: kern = r ? compact_kernel<256, true> : compact_kernel<256, false>; break;
+    case 512: kern = r ? compact_kernel<512, true> : compact_kernel<512, false>; break;
     default: return AG_ERR_UNSUPPORTED;
   }
   return launch_pdl(kern, grid, dim3(kCompactThreads), 0, st, flags, d.seq, c.cap, c.len, prefix, ix, dev_status, Kb,
-                            Vb, c.row_off, kr, vr, RecentFill{ring_of(d, c), d.seq_lens, kv_heads_of(d)});
+                            Vb, c.row_off, kr, vr, RecentFill{ring, d.seq_lens, kv_heads_of(d)});
 }
 
 // Ring of a recent-token window from the dense K, V of the prompt (one more small launch).
