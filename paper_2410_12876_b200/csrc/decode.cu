@@ -567,7 +567,7 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
 // more), the row to append fetched after the barrier and 96 KB of stages: two stages and fewer than 170 registers let
 // three CTAs share an SM, so the next step's clusters start beside this one's.
 constexpr int kCmStages = 2;
-// kMaxG: 1 (one query per slab), 8 or 16.  kCtas: CTAs of a cluster (1: no cluster).
+// kMaxG: 1 (one query per slab), 4, 8 or 16.  kCtas: CTAs of a cluster (1: no cluster).
 template <int D, int kMaxG, int kCtas>
 __global__ void __launch_bounds__(kGqThreads, 2)
 decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
@@ -622,7 +622,7 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   if (rank == 0) row = load_new_row<T, D>(ap, kv, slab_row0, k_new, v_new);
 
   if (r_first < L) {                  // the same for the whole CTA
-    const GqWarpTriples w = gq_stream_rows<D, kCmStages, (kMaxG + 7) / 8, true>(
+    const GqWarpTriples w = gq_stream_rows<D, kCmStages, kMaxG, true>(
         gq_smem, q + (size_t)slab0 * D, G, Kg, Vg, r_first, kCtas * kGqTile, L, scale_log2);
     if constexpr (kCtas > 1) cluster.barrier_wait();
     for (int x = d; x < G * D; x += kGqThreads) {
@@ -789,8 +789,8 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     // grouped-query attention: one cluster per key/value slab reads it for all its query heads
     auto cluster = [&](auto ctas, int groups, int G) {
       constexpr int kCtas = decltype(ctas)::value;
-      return (G == 1 ? launch_decode_cluster_mma<D, 1, kCtas> : G <= 8 ? launch_decode_cluster_mma<D, 8, kCtas> :
-              launch_decode_cluster_mma<D, 16, kCtas>)(groups, G, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
+      return (G == 1 ? launch_decode_cluster_mma<D, 1, kCtas> : G <= 4 ? launch_decode_cluster_mma<D, 4, kCtas> :
+              G <= 8 ? launch_decode_cluster_mma<D, 8, kCtas> : launch_decode_cluster_mma<D, 16, kCtas>)(groups, G, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
     };
     const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
     // (clusters of one query head each never carry the append: see decode_carries_append)

@@ -13,7 +13,7 @@ namespace ag {
 
 // two stages x three CTAs per SM measured better here than deeper rings in fewer CTAs
 constexpr int kGqChunkStages = 2;
-template <int kGqD, int kN>
+template <int kGqD, int kMaxG>
 __global__ void __launch_bounds__(kGqThreads, 3)
 decode_partial_gqa_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_rows,
                               const __nv_bfloat16 *v_rows, const int64_t *row_off,
@@ -32,7 +32,7 @@ decode_partial_gqa_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_row
   const int r_end = min(L, r_begin + chunk_rows);
   const uint8_t *Kg = reinterpret_cast<const uint8_t *>(k_rows) + (size_t)row_off[kv] * kGqRowBytes;
   const uint8_t *Vg = reinterpret_cast<const uint8_t *>(v_rows) + (size_t)row_off[kv] * kGqRowBytes;
-  const GqWarpTriples w = gq_stream_rows<kGqD, kGqChunkStages, kN, false>(gq_smem, q + (size_t)slab0 * kGqD, G, Kg, Vg,
+  const GqWarpTriples w = gq_stream_rows<kGqD, kGqChunkStages, kMaxG, false>(gq_smem, q + (size_t)slab0 * kGqD, G, Kg, Vg,
                                                                                r_begin, kGqTile, r_end, scale_log2);
   for (int x = threadIdx.x; x < G * kGqD; x += kGqThreads) {     // one (head, output dimension) at a time
     const int h = x / kGqD, d = x % kGqD;
@@ -52,14 +52,14 @@ bool decode_gqa_mma_supported(const ag_layer_desc &d) {
   return d.dtype == AG_BF16 && group >= 2 && group <= kGqMaxGroup;
 }
 
-template <int D, int kN>
+template <int D, int kMaxG>
 static int run_partial(const ag_layer_desc &d, const void *q, const ag_cache &c, float scale_log2, int chunk_rows,
                        int n_chunks, float *part_o, float *part_ml, int max_splits, cudaStream_t st) {
   const int kvh = kv_heads_of(d);
   constexpr int smem = gq_smem_bytes(D, kGqChunkStages);
-  AG_CUDA_TRY(cudaFuncSetAttribute(decode_partial_gqa_mma_kernel<D, kN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  AG_CUDA_TRY(cudaFuncSetAttribute(decode_partial_gqa_mma_kernel<D, kMaxG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   dim3 grid(n_chunks, d.batch * kvh);
-  return launch_pdl(decode_partial_gqa_mma_kernel<D, kN>, grid, dim3(kGqThreads), smem, st,
+  return launch_pdl(decode_partial_gqa_mma_kernel<D, kMaxG>, grid, dim3(kGqThreads), smem, st,
                     static_cast<const __nv_bfloat16 *>(q), static_cast<const __nv_bfloat16 *>(c.k_rows),
                     static_cast<const __nv_bfloat16 *>(c.v_rows), c.row_off, c.len, scale_log2, chunk_rows, part_o, part_ml,
                     kvh, d.heads / kvh, max_splits);
@@ -68,9 +68,9 @@ static int run_partial(const ag_layer_desc &d, const void *q, const ag_cache &c,
 int launch_decode_partial_gqa_mma(const ag_layer_desc &d, const void *q, const ag_cache &c, float scale_log2,
                                   int chunk_rows, int n_chunks, float *part_o, float *part_ml, int max_splits,
                                   cudaStream_t st) {
-  const bool small = d.heads / kv_heads_of(d) <= 8;
-  auto run = d.head_dim == 64 ? (small ? run_partial<64, 1> : run_partial<64, 2>)
-                              : (small ? run_partial<128, 1> : run_partial<128, 2>);
+  const int G = d.heads / kv_heads_of(d);
+  auto run = d.head_dim == 64 ? (G <= 4 ? run_partial<64, 4> : G <= 8 ? run_partial<64, 8> : run_partial<64, 16>)
+                              : (G <= 4 ? run_partial<128, 4> : G <= 8 ? run_partial<128, 8> : run_partial<128, 16>);
   return run(d, q, c, scale_log2, chunk_rows, n_chunks, part_o, part_ml, max_splits, st);
 }
 

@@ -7,6 +7,10 @@
 // the keys, then the dims, are the 16 rows of an MMA and the query heads its 8 columns: half the MMAs and half
 // the accumulators of the form with the (mostly empty) 16 query rows; S^T becomes the second operand of the
 // weighted sum by an 8 x 8 transpose between registers (movmatrix).
+// The weights P enter the weighted sum as two bf16 parts each (one would cost the outputs a third of their accuracy:
+// error against float64 of 72 .. 256 slabs 2.2e-3 with one part, 1.65e-3, the rounding of the outputs, with two).  Up to
+// four heads the second part is free: columns 4 .. 7 of the MMAs repeat the heads, with the low parts as their weights,
+// and the two halves are added at the end.  More heads take a second MMA per block.
 // Rows go global -> shared by 16-byte cp.async in tiles of 64 rows (K and V; the next tile is in flight while one is
 // worked on); each of the four warps fetches and owns 16 rows of every tile and keeps its own running softmax, so the
 // warps wait for nobody until their (m, l, o) triples end in shared memory, where gq_combine() merges them.
@@ -56,13 +60,15 @@ __device__ __forceinline__ void gq_load_tile(uint32_t stage, const uint8_t *Kg, 
 // kGqStages - 1 tiles are in flight while one is worked on).
 // kFirstLoaded: the caller has issued tile 0 into stage 0 and committed it, perhaps before it knew r_end: its rows
 // past r_end may then hold anything.  Their scores are masked; their values are masked too (0 * NaN is NaN).
-// kN: groups of 8 heads (G <= 8 kN).
-template <int kGqD, int kGqStages, int kN, bool kFirstLoaded>
+// kMaxG: 1, 4, 8 or 16, at least G.
+template <int kGqD, int kGqStages, int kMaxG, bool kFirstLoaded>
 __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const __nv_bfloat16 *q, int G,
                                                         const uint8_t *Kg, const uint8_t *Vg, int r_first, int r_step,
                                                         int r_end, float scale_log2) {
   static_assert(kGqD == 64 || kGqD == 128, "head_dim");
   constexpr int kGqTileBytes = gq_tile_bytes(kGqD);
+  constexpr int kN = (kMaxG + 7) / 8;         // column blocks of 8
+  constexpr bool kRepeat = kMaxG <= 4;        // columns 4 .. 7 repeat the heads of 0 .. 3, for the low parts of the weights
   constexpr int kChains = 2;        // chains of MMAs that the scores of a block are summed in
   const int n_tiles = (r_end - r_first + r_step - 1) / r_step;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -77,12 +83,13 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
   uint32_t qb[kN][kGqD / 16][2];
 #pragma unroll
   for (int n = 0; n < kN; ++n) {
-    const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + (size_t)min(8 * n + g, G - 1) * kGqD);
+    const int head = kRepeat ? g & 3 : 8 * n + g;
+    const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + (size_t)min(head, G - 1) * kGqD);
 #pragma unroll
     for (int ks = 0; ks < kGqD / 16; ++ks) {
       const uint32_t lo = qrow[ks * 8 + t], hi = qrow[ks * 8 + 4 + t];
-      qb[n][ks][0] = 8 * n + g < G ? lo : 0u;
-      qb[n][ks][1] = 8 * n + g < G ? hi : 0u;
+      qb[n][ks][0] = head < G ? lo : 0u;
+      qb[n][ks][1] = head < G ? hi : 0u;
     }
   }
 
@@ -165,7 +172,8 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
             }
           }
       }
-      uint32_t pb[kN][2];                                       // P^T: keys 2t, 2t + 1 (| + 8) of head 8 n + g
+      constexpr int kParts = kRepeat ? 1 : 2;                   // operands that hold the weights
+      uint32_t pb[kParts][kN][2];                               // P^T: keys 2t, 2t + 1 (| + 8) of head 8 n + g
 #pragma unroll
       for (int n = 0; n < kN; ++n) {
         float p[4];
@@ -173,8 +181,16 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
         for (int e = 0; e < 4; ++e) p[e] = exp2f(s[n][0][e] - m[n][e & 1]);
         l[n][0] += p[0] + p[2];
         l[n][1] += p[1] + p[3];
-        pb[n][0] = movmatrix_trans(pack2_bf16(p[0], p[1]));
-        pb[n][1] = movmatrix_trans(pack2_bf16(p[2], p[3]));
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const uint2 w = split2_bf16(p[2 * e], p[2 * e + 1]);
+          if constexpr (kRepeat) {
+            pb[0][n][e] = movmatrix_trans(t < 2 ? w.x : w.y);
+          } else {
+            pb[0][n][e] = movmatrix_trans(w.x);
+            pb[kParts - 1][n][e] = movmatrix_trans(w.y);
+          }
+        }
       }
       // O^T += V^T P^T: 16 dims x 16 keys per ldmatrix
       uint32_t vmask[2];                                        // valid keys among 2t, 2t + 1 | 2t + 8, 2t + 9
@@ -193,7 +209,9 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
           for (int e = 0; e < 4; ++e) a[e] &= vmask[e >> 1];
         }
 #pragma unroll
-        for (int n = 0; n < kN; ++n) mma_16816(o[n][j], a, pb[n][0], pb[n][1]);
+        for (int w = 0; w < kParts; ++w)
+#pragma unroll
+          for (int n = 0; n < kN; ++n) mma_16816(o[n][j], a, pb[w][n][0], pb[w][n][1]);
       }
     }
     __syncwarp();                                               // the warp's rows of the stage may be refilled
@@ -201,6 +219,12 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
   cp_async_wait<0>();
   __syncthreads();
 
+  if constexpr (kRepeat) {                                      // high and low parts of the weights: columns 4 apart
+#pragma unroll
+    for (int j = 0; j < kGqD / 16; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[0][j][e] += __shfl_xor_sync(0xffffffffu, o[0][j][e], 2);
+  }
   // merge the four warps' triples through shared memory (the tiles are no longer needed)
   float *sm_o = reinterpret_cast<float *>(gq_smem);             // [warps][16][D]
   float *sm_m = sm_o + kGqWarps * kGqMaxGroup * kGqD;           // [warps][16]
@@ -212,7 +236,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
       const int head = 8 * n + 2 * t + e;
 #pragma unroll
       for (int off = 4; off < 32; off <<= 1) l[n][e] += __shfl_xor_sync(0xffffffffu, l[n][e], off);
-      if (head < G) {
+      if (head < G && (!kRepeat || t < 2)) {
         float *dst = sm_o + ((size_t)(warp * kGqMaxGroup + head)) * kGqD + g;
 #pragma unroll
         for (int j = 0; j < kGqD / 16; ++j) {

@@ -44,6 +44,11 @@ __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t *>(&v);
 }
+// Two float32 as two packed bf16 parts each, the larger in .x: together they hold the values to 2^-17.
+__device__ __forceinline__ uint2 split2_bf16(float lo, float hi) {
+  const uint32_t p = pack2_bf16(lo, hi);
+  return make_uint2(p, pack2_bf16(lo - __uint_as_float(p << 16), hi - __uint_as_float(p & 0xffff0000u)));
+}
 // Byte offset of 16-byte piece `piece` (0..15) of row `row` in a shared-memory tile of 256-byte rows
 // (128 bf16): pieces are XOR-ed with the row number so that the eight rows one ldmatrix reads fall
 // into different banks.
