@@ -14,7 +14,11 @@
 //               P written back to TMEM as bf16, O rescaled only when the running
 //               maximum grows by more than 2^8, final normalisation and store
 //
-// TMEM columns: S0 [0,64) S1 [64,128), each overwritten in place by its P (bf16 pairs); O [128,128 + D).
+// TMEM columns: S0 [0,64) S1 [64,128), each overwritten in place by its P (bf16 pairs, 32 columns; where the weights
+// are held in two bf16 parts, the low parts take the other 32); O [128,128 + D).
+// Weights in two parts (P V takes twice the MMAs): heads of 64, whose weights were float32 on CUDA cores (error against
+// float64 at 1500 tokens 1.61e-3 there, 2.03e-3 with one part), and the dense tiles of a window, which
+// hold the token's own weight, float32 elsewhere.
 // The self term seeds the running softmax (m = s_jj, l = 1) and its value row
 // is added in the epilogue: O_j = (sum_r p_r v_r + w_self v_j) / l.  Every byte
 // that enters or leaves the CTA travels by TMA.
@@ -23,6 +27,8 @@
 // They and the token itself lie in the dense rows [j0 - 16, j0 + 128): three more key tiles (64, 64 and 16
 // rows of the dense K, V) in front of the cache's, masked to the band, take the place of the self tile.  (As a
 // pass of its own over Q, O and the dense K, V the band took 38 us at 4096 tokens of 32 heads, 57 us at 4 x 1999.)
+#include <type_traits>
+
 #include "ag_common.cuh"
 #include "umma.cuh"
 
@@ -281,8 +287,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const uint32_t pa = tmem + kColS + st * kPfBN;
         if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < kPfBN / 16; ++k)
-            if (k < ksteps) mma_ts_lohi(tmem + kColO, pa + k * 8, vb + ((k * 2048) >> 4), v_hi, idesc_pv, (i | k) != 0);
+          for (int w = 0; w < (kPfD == 64 || kBand ? 2 : 1); ++w) {
+            if (w == 1 && kPfD != 64 && i >= kBandTiles) break;        // one part
+#pragma unroll
+            for (int k = 0; k < kPfBN / 16; ++k)
+              if (k < ksteps)
+                mma_ts_lohi(tmem + kColO, pa + w * (kPfBN / 2) + k * 8, vb + ((k * 2048) >> 4), v_hi, idesc_pv, (i | w | k) != 0);
+          }
           mma_commit(&v_empty[st]);
           mma_commit(&pv_done[st]);
         }
@@ -372,21 +383,32 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       // sums two elements per instruction
       float rs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       const float neg_m = kBand && m_new == -INFINITY ? 0.f : -m_new;
+      auto weights = [&](auto n_parts, int keys) {   // of the tile's first `keys` keys
+        constexpr int parts = decltype(n_parts)::value;
 #pragma unroll
-      for (int c = 0; c < kPfBN / 16; ++c) {
-        uint32_t pk[8];
+        for (int c = 0; c < kPfBN / 16; ++c) {
+          if (c * 16 >= keys) break;
+          uint32_t pk[parts][8];
 #pragma unroll
-        for (int e = 0; e < 16; e += 2) {
-          float t0, t1;
-          fma_f32x2(t0, t1, __uint_as_float(r[c * 16 + e]), __uint_as_float(r[c * 16 + e + 1]), a.scale_log2,
-                    a.scale_log2, neg_m, neg_m);
-          const float p0 = fast_exp2(t0), p1 = fast_exp2(t1);
-          const int k = ((e >> 1) & 3) * 2;
-          add_f32x2(rs[k], rs[k + 1], rs[k], rs[k + 1], p0, p1);
-          pk[e >> 1] = pack_bf16x2(p0, p1);
+          for (int e = 0; e < 16; e += 2) {
+            float t0, t1;
+            fma_f32x2(t0, t1, __uint_as_float(r[c * 16 + e]), __uint_as_float(r[c * 16 + e + 1]), a.scale_log2,
+                      a.scale_log2, neg_m, neg_m);
+            float p0 = fast_exp2(t0), p1 = fast_exp2(t1);
+            const int k = ((e >> 1) & 3) * 2;
+            add_f32x2(rs[k], rs[k + 1], rs[k], rs[k + 1], p0, p1);
+            if constexpr (parts == 2) pk[0][e >> 1] = take_bf16x2(p0, p1);
+            pk[parts - 1][e >> 1] = pack_bf16x2(p0, p1);
+          }
+#pragma unroll
+          for (int w = 0; w < parts; ++w) tmem_st_x8(tS + w * (kPfBN / 2) + c * 8, pk[w]);
         }
-        tmem_st_x8(tS + c * 8, pk);
-      }
+      };
+      using One = std::integral_constant<int, 1>;
+      using Two = std::integral_constant<int, 2>;
+      if constexpr (kPfD == 64 && !kBand) weights(Two{}, kPfBN);
+      else if (dense) weights(Two{}, i == 2 ? 16 : kPfBN);
+      else weights(std::conditional_t<kPfD == 64, Two, One>{}, kPfBN);
       l = l * alpha + (((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7])));
       m = m_new;
 

@@ -50,3 +50,18 @@ def test_decode(B, h, hk, D, longest):
     ag.ag_decode_attn(desc, q, kn, vn, cache, 0.0, o, ag.workspace(desc, ag.AG_CALL_DECODE))
     want = orc.decode_attention(T.f64(q), T.f64(kn), T.f64(vn), T.gpu_cache_as_lists(cache, shape))
     check_rounding(o, want, max(np.abs(T.f64(cache.v_rows)).max(), np.abs(T.f64(vn)).max()))
+
+
+@pytest.mark.parametrize("B,n,h,hk,D,window,keep", [
+    (1, 1, 4, 4, 64, 0, 0.5), (2, 40, 4, 4, 64, 0, 0.5), (1, 129, 4, 2, 64, 0, 0.3), (1, 300, 2, 2, 64, 0, 0.9),
+    (1, 64, 4, 4, 64, 10, 0.2), (2, 145, 4, 2, 64, 17, 0.1),
+    (1, 40, 4, 4, 128, 5, 0.0), (1, 257, 4, 2, 128, 17, 0.0),     # nothing but the window: its dense tiles
+])
+def test_prefill(B, n, h, hk, D, window, keep):
+    shape = LayerShape(B, n, 64, h, D, 1, 64, "bf16", kv_heads=hk, recent_window=window)
+    Q, K, V = inputs.qkv_gaussian(shape, 70 + n, DEV)
+    flags = torch.from_numpy((np.random.default_rng(n).random((B, hk, n)) < keep).astype(np.uint8)).to(DEV)
+    cache, prefix, _, _ = T.gpu_compact(shape, K, V, flags)
+    O = T.gpu_prefill(shape, Q, K, V, flags, cache, prefix)
+    want = orc.prefill_attention(T.f64(Q), T.f64(K), T.f64(V), flags.cpu().numpy(), window=max(window, 1))
+    check_rounding(O, want, np.abs(T.f64(V)).max())
