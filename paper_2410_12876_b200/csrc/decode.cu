@@ -49,7 +49,7 @@ struct AppendArgs {
 };
 // What an append needs to know, asked for ahead of the work of the step: after the barrier that ends it nothing is left
 // but the stores (the flag, the capacity, then the row were three trips to L2 in a row at the end of every step).
-struct NewRow { uint4 k, v; size_t dst; int cap; uint32_t on; };    // (on: the flag as it was read, so that nothing waits for it here)
+struct NewRow { uint4 k, v; int64_t row0; int cap; uint32_t on; };    // (as they were read: nothing waits for them here)
 // The threads [first, first + row vectors) of ONE CTA per slab carry a row; the others get on = false.
 template <typename T, int D>
 __device__ __forceinline__ NewRow load_new_row(const AppendArgs &ap, int slab, int64_t row0, const T *k_new,
@@ -63,7 +63,7 @@ __device__ __forceinline__ NewRow load_new_row(const AppendArgs &ap, int slab, i
   r.v = ld128(v_new + (size_t)slab * D + vec * (16 / (int)sizeof(T)));
   r.cap = ap.cap[slab];
   r.on = ap.flag_new[slab];
-  r.dst = (size_t)row0 * D * sizeof(T) + vec * 16;
+  r.row0 = row0;
   return r;
 }
 // After every read of len[slab] and of the slab's rows by this launch has completed.  L = the length those reads saw.
@@ -75,7 +75,7 @@ __device__ __forceinline__ void append_new_row(const AppendArgs &ap, const NewRo
     if (lead && ap.dev_status) atomicOr(ap.dev_status, AG_DEV_OVERFLOW);
     return;
   }
-  const size_t dst = r.dst + (size_t)L * D * sizeof(T);
+  const size_t dst = (size_t)(r.row0 + L) * D * sizeof(T) + ((int)threadIdx.x - first) * 16;
   *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ap.k_rows) + dst) = r.k;
   *reinterpret_cast<uint4 *>(static_cast<uint8_t *>(ap.v_rows) + dst) = r.v;
   if (lead) ap.len[slab] = L + 1;
@@ -559,10 +559,11 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
 // One cluster per run of G <= 16 query slabs that share a key/value slab (G = 1 without grouped-query
 // attention): the G queries are columns of one MMA operand, so the slab is read once for all of them, and the
 // one cluster that reads it may append to it.  CTA `rank` takes whole 64-row tiles; after the cluster
-// barrier rank r merges the heads r, r + 8 of the group, whose triples the ranks have written to its shared memory.  The tiles go round the ranks, so a rank's first tile does
-// not depend on the slab's length and its rows are asked for together with the length (before it is known
-// they are only known to lie inside the slab): one trip to L2 less on the path of a step.
-// A step of 32 slabs of 400 .. 1640 rows takes 7.7 us in a graph (1.2 us of it an empty chain of launches); it was 9.2 us
+// barrier rank r merges the heads r, r + 8 of the group, whose triples the ranks have written to its shared memory.
+// Nothing of the cache is read ahead of the wait for the preceding kernel, which may be one that lays it out: where a
+// slab begins arrives with its length, the queries in the same trip (the queries behind the length: 127.5 -> 133.6 us for
+// 16 steps; the first tile asked for from where the slab seemed to lie before the wait, checked after it: 131.3).
+// A step of 32 slabs of 400 .. 1640 rows takes 7.8 us in a graph (1.2 us of it an empty chain of launches); it was 9.2 us
 // with the queries as the rows of the MMAs, the merging rank reading the others' triples (one trip and one barrier
 // more), the row to append fetched after the barrier and 96 KB of stages: two stages and fewer than 170 registers let
 // three CTAs share an SM, so the next step's clusters start beside this one's.
@@ -572,7 +573,7 @@ template <int D, int kMaxG, int kCtas>
 __global__ void __launch_bounds__(kGqThreads, 2)
 decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
                           const __nv_bfloat16 *v_new, const __nv_bfloat16 *k_rows,
-                          const __nv_bfloat16 *v_rows, const int64_t *row_off, const int32_t *cap,
+                          const __nv_bfloat16 *v_rows, const int64_t *row_off,
                           const int32_t *len, float scale_log2, __nv_bfloat16 *out, int group,
                           const AppendArgs ap, const HeadMap hm, const RecentRing rg) {
   namespace cg = cooperative_groups;
@@ -587,17 +588,11 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   const int d = threadIdx.x;
   pdl_launch_dependents();
   if constexpr (kCtas > 1) cluster.barrier_arrive();   // (waited for before the first write to another rank: all have started then)
-  // the slab's first row and capacity never change once the cache is laid out: read ahead of the wait for the
-  // preceding kernel
-  const int64_t slab_row0 = row_off[kv];
-  const int slab_cap = cap[kv];
   pdl_wait();
   const int L = len[kv];
+  const int64_t slab_row0 = row_off[kv];
   const int r_first = rank * kGqTile;
-  const uint8_t *Kg = reinterpret_cast<const uint8_t *>(k_rows) + (size_t)slab_row0 * (D * 2);
-  const uint8_t *Vg = reinterpret_cast<const uint8_t *>(v_rows) + (size_t)slab_row0 * (D * 2);
-  if (r_first < slab_cap) gq_load_tile<D>((uint32_t)__cvta_generic_to_shared(gq_smem), Kg, Vg, r_first, slab_cap);
-  cp_async_commit();
+  const GqQuery<D, kMaxG> qf = gq_load_query<D, kMaxG>(q + (size_t)slab0 * D, G);
 
   // the ranks' triples of the heads this rank merges, written by the ranks themselves
   __shared__ float in_o[kHeads][kCtas][D];
@@ -621,9 +616,11 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   row.on = 0;
   if (rank == 0) row = load_new_row<T, D>(ap, kv, slab_row0, k_new, v_new);
 
+  const uint8_t *Kg = reinterpret_cast<const uint8_t *>(k_rows) + (size_t)slab_row0 * (D * 2);
+  const uint8_t *Vg = reinterpret_cast<const uint8_t *>(v_rows) + (size_t)slab_row0 * (D * 2);
   if (r_first < L) {                  // the same for the whole CTA
-    const GqWarpTriples w = gq_stream_rows<D, kCmStages, kMaxG, true>(
-        gq_smem, q + (size_t)slab0 * D, G, Kg, Vg, r_first, kCtas * kGqTile, L, scale_log2);
+    const GqWarpTriples w = gq_stream_rows<D, kCmStages, kMaxG>(gq_smem, qf, G, Kg, Vg, r_first, kCtas * kGqTile, L,
+                                                                scale_log2);
     if constexpr (kCtas > 1) cluster.barrier_wait();
     for (int x = d; x < G * D; x += kGqThreads) {
       const int h = x / D, e = x % D, to = h % kCtas;
@@ -636,7 +633,6 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
     if constexpr (kCtas > 1) cluster.barrier_wait();
     // weight 0 in the merge, which then skips the values
     if (d < G) *at_rank(&in_ml[d / kCtas][rank], d % kCtas) = make_float2(-INFINITY, 0.f);
-    cp_async_wait<0>();               // (the first tile, asked for in vain)
   }
 #pragma unroll
   for (int u = 0; u < kHeads; ++u) {
@@ -719,7 +715,7 @@ static int launch_decode_cluster_mma(int groups, int G, const void *q, const voi
   AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_mma_kernel<D, kMaxG, kCtas>, static_cast<const T *>(q),
                                  static_cast<const T *>(k_new), static_cast<const T *>(v_new),
                                  static_cast<const T *>(c.k_rows), static_cast<const T *>(c.v_rows),
-                                 c.row_off, c.cap, c.len, scale_log2, static_cast<T *>(o), G, ap, hm, rg));
+                                 c.row_off, c.len, scale_log2, static_cast<T *>(o), G, ap, hm, rg));
   return AG_OK;
 }
 

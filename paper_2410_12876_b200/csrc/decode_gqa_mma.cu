@@ -32,8 +32,9 @@ decode_partial_gqa_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_row
   const int r_end = min(L, r_begin + chunk_rows);
   const uint8_t *Kg = reinterpret_cast<const uint8_t *>(k_rows) + (size_t)row_off[kv] * kGqRowBytes;
   const uint8_t *Vg = reinterpret_cast<const uint8_t *>(v_rows) + (size_t)row_off[kv] * kGqRowBytes;
-  const GqWarpTriples w = gq_stream_rows<kGqD, kGqChunkStages, kMaxG, false>(gq_smem, q + (size_t)slab0 * kGqD, G, Kg, Vg,
-                                                                               r_begin, kGqTile, r_end, scale_log2);
+  const GqQuery<kGqD, kMaxG> qf = gq_load_query<kGqD, kMaxG>(q + (size_t)slab0 * kGqD, G);
+  const GqWarpTriples w = gq_stream_rows<kGqD, kGqChunkStages, kMaxG>(gq_smem, qf, G, Kg, Vg, r_begin, kGqTile, r_end,
+                                                                      scale_log2);
   for (int x = threadIdx.x; x < G * kGqD; x += kGqThreads) {     // one (head, output dimension) at a time
     const int h = x / kGqD, d = x % kGqD;
     float acc, mc, lc;

@@ -53,22 +53,44 @@ __device__ __forceinline__ void gq_load_tile(uint32_t stage, const uint8_t *Kg, 
   }
 }
 
+// The query vectors as the second operand of the scores: thread (g, t) of a warp holds head 8 n + g (head g % 4 where
+// columns 4 .. 7 repeat the heads; zeros past G), 16 dims per step.  kMaxG: 1, 4, 8 or 16, at least G.
+__host__ __device__ constexpr int gq_blocks(int max_g) { return (max_g + 7) / 8; }     // blocks of 8 columns
+__host__ __device__ constexpr bool gq_repeats(int max_g) { return max_g <= 4; }        // columns 4 .. 7 repeat the heads of 0 .. 3
+template <int kGqD, int kMaxG>
+struct GqQuery { uint32_t b[gq_blocks(kMaxG)][kGqD / 16][2]; };
+// q: G consecutive query vectors [G][D].  (To be asked for as early as may be: these loads cannot move ahead of
+// asynchronous copies, or of a branch, by themselves.)
+template <int kGqD, int kMaxG>
+__device__ __forceinline__ GqQuery<kGqD, kMaxG> gq_load_query(const __nv_bfloat16 *q, int G) {
+  const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+  GqQuery<kGqD, kMaxG> r;
+#pragma unroll
+  for (int n = 0; n < gq_blocks(kMaxG); ++n) {
+    const int head = gq_repeats(kMaxG) ? g & 3 : 8 * n + g;
+    const uint32_t *row = reinterpret_cast<const uint32_t *>(q + (size_t)head * kGqD);
+#pragma unroll
+    for (int ks = 0; ks < kGqD / 16; ++ks) {
+      r.b[n][ks][0] = head < G ? row[ks * 8 + t] : 0u;
+      r.b[n][ks][1] = head < G ? row[ks * 8 + 4 + t] : 0u;
+    }
+  }
+  return r;
+}
+
 // Every thread of the CTA (kGqThreads of them) calls this with the same arguments.  The CTA's tiles are the 64
 // rows from r_first + i * r_step for i = 0, 1, ... while that is below r_end (at least one).
-// q: G consecutive query vectors [G][D]; Kg, Vg: first row of the slab.  Returns after a CTA barrier
+// q: the G query vectors; Kg, Vg: first row of the slab.  Returns after a CTA barrier
 // with the warps' triples in shared memory (gq_smem: gq_smem_bytes(D, kGqStages) of dynamic shared memory;
 // kGqStages - 1 tiles are in flight while one is worked on).
-// kFirstLoaded: the caller has issued tile 0 into stage 0 and committed it, perhaps before it knew r_end: its rows
-// past r_end may then hold anything.  Their scores are masked; their values are masked too (0 * NaN is NaN).
-// kMaxG: 1, 4, 8 or 16, at least G.
-template <int kGqD, int kGqStages, int kMaxG, bool kFirstLoaded>
-__device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const __nv_bfloat16 *q, int G,
+template <int kGqD, int kGqStages, int kMaxG>
+__device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const GqQuery<kGqD, kMaxG> &q, int G,
                                                         const uint8_t *Kg, const uint8_t *Vg, int r_first, int r_step,
                                                         int r_end, float scale_log2) {
   static_assert(kGqD == 64 || kGqD == 128, "head_dim");
   constexpr int kGqTileBytes = gq_tile_bytes(kGqD);
-  constexpr int kN = (kMaxG + 7) / 8;         // column blocks of 8
-  constexpr bool kRepeat = kMaxG <= 4;        // columns 4 .. 7 repeat the heads of 0 .. 3, for the low parts of the weights
+  constexpr int kN = gq_blocks(kMaxG);
+  constexpr bool kRepeat = gq_repeats(kMaxG); // for the low parts of the weights
   constexpr int kChains = 2;        // chains of MMAs that the scores of a block are summed in
   const int n_tiles = (r_end - r_first + r_step - 1) / r_step;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -78,23 +100,8 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
     gq_load_tile<kGqD>(smem0 + (i % kGqStages) * 2 * kGqTileBytes, Kg, Vg, r_first + i * r_step, r_end);
   };
 
-  // (Q is asked for first: these loads cannot move ahead of the asynchronous copies by themselves)
-  // Second operand of the scores: head 8 n + g (zeros past G), 16 dims per step
-  uint32_t qb[kN][kGqD / 16][2];
 #pragma unroll
-  for (int n = 0; n < kN; ++n) {
-    const int head = kRepeat ? g & 3 : 8 * n + g;
-    const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + (size_t)min(head, G - 1) * kGqD);
-#pragma unroll
-    for (int ks = 0; ks < kGqD / 16; ++ks) {
-      const uint32_t lo = qrow[ks * 8 + t], hi = qrow[ks * 8 + 4 + t];
-      qb[n][ks][0] = head < G ? lo : 0u;
-      qb[n][ks][1] = head < G ? hi : 0u;
-    }
-  }
-
-#pragma unroll
-  for (int i = kFirstLoaded ? 1 : 0; i < kGqStages - 1; ++i) {
+  for (int i = 0; i < kGqStages - 1; ++i) {
     if (i < n_tiles) load_tile(i);
     cp_async_commit();
   }
@@ -136,7 +143,7 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
         // matrices: (keys 0-7, dims lo), (keys 8-15, dims lo), (keys 0-7, dims hi), (keys 8-15, dims hi)
         ldmatrix_x4(a, sk + gq_tile_off<kGqD>(warp * 16 + (mi & 1) * 8 + (lane & 7), ks * 2 + (mi >> 1)));
 #pragma unroll
-        for (int n = 0; n < kN; ++n) mma_16816(s[n][ks % kChains], a, qb[n][ks][0], qb[n][ks][1]);
+        for (int n = 0; n < kN; ++n) mma_16816(s[n][ks % kChains], a, q.b[n][ks][0], q.b[n][ks][1]);
       }
       // Online softmax of heads 2t, 2t + 1: this thread holds keys g, g + 8.  The maximum moves only when a score
       // exceeds it by more than 2^8 (float32 sums and bf16 weights have the room).
@@ -193,21 +200,11 @@ __device__ __forceinline__ GqWarpTriples gq_stream_rows(uint8_t *gq_smem, const 
         }
       }
       // O^T += V^T P^T: 16 dims x 16 keys per ldmatrix
-      uint32_t vmask[2];                                        // valid keys among 2t, 2t + 1 | 2t + 8, 2t + 9
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int k = key0 + e * 8 + 2 * t;
-        vmask[e] = k + 1 < r_end ? 0xffffffffu : (k < r_end ? 0xffffu : 0u);
-      }
 #pragma unroll
       for (int j = 0; j < kGqD / 16; ++j) {
         uint32_t a[4];
         // matrices: (dims lo, keys 0-7), (dims hi, keys 0-7), (dims lo, keys 8-15), (dims hi, keys 8-15)
         ldmatrix_x4_trans(a, sv + gq_tile_off<kGqD>(warp * 16 + (mi >> 1) * 8 + (lane & 7), j * 2 + (mi & 1)));
-        if (kFirstLoaded && i == 0) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) a[e] &= vmask[e >> 1];
-        }
 #pragma unroll
         for (int w = 0; w < kParts; ++w)
 #pragma unroll
