@@ -482,11 +482,6 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
   if (warp == 1) tmem_dealloc(tmem, kGaTmemCols);
 }
 
-bool gate_attn_tc_supported(const ag_layer_desc &d) {
-  const int GD = d.gate_heads * d.gate_head_dim;
-  return d.dtype == AG_BF16 && (d.gate_head_dim == 128 || d.gate_head_dim == 64) && gate_proj_tc_supported(d.hidden, GD);
-}
-
 // The split-K merge of MHA' and the gate's output layer in one pass (Eq. 3, Eq. 4):
 //   H'[t, g * D + c] = sum_s w_s O_s[r, c] / sum_s w_s l_s,  w_s = 2^(m_s - max_s m_s)
 //   s[t, i] = H'[t, :] Wo_g[:, i];  flag = s + gamma_i > logit(tau)
@@ -508,6 +503,8 @@ constexpr int kMoRedPitch = 33;                                  // floats per t
 constexpr int kMoRedBytes = kMoWarps * 16 * kMoRedPitch * 4;
 __host__ __device__ constexpr int mo_w_bytes(int GD) { return GD * 64 > kMoRedBytes ? GD * 64 : kMoRedBytes; }
 __host__ __device__ constexpr int mo_smem_bytes(int GD) { return mo_w_bytes(GD) + 16 * (GD + 8) * 4; }
+constexpr int kMoPieceBytes = 2 * kMoThreads * 4;                // static: where the pieces of each gate head lie
+constexpr int kMaxSmemBytes = 227 * 1024;                        // of one CTA
 // Byte offset of 16-byte piece `piece` (8 heads) of row `c` of the staged slice of Wo: 64-byte rows, pieces XOR-ed so
 // that the eight rows one ldmatrix reads fall into different banks.
 __device__ __forceinline__ uint32_t mo_w_off(int c, int piece) { return (uint32_t)(c * 64 + ((piece ^ ((c >> 1) & 3)) << 4)); }
@@ -523,6 +520,7 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
   float *Hs = reinterpret_cast<float *>(mo_smem + mo_w_bytes(a.GD));     // [16][GD + 8]
   const int pitch = a.GD + 8;
   __shared__ int seg_first[2][kMoThreads];           // per gate head: first segment, number of pieces
+  static_assert(sizeof(seg_first) == kMoPieceBytes, "gate_attn_tc_supported");
   const int tiles_per_seq = (a.n + kTok - 1) / kTok;
   const int b = blockIdx.x / tiles_per_seq, t0 = (blockIdx.x % tiles_per_seq) * kTok;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -696,6 +694,21 @@ gate_merge_out_kernel(const __grid_constant__ GateAttnArgs a, const __nv_bfloat1
   }
 }
 
+// Steps of (query tile, key tile) of the whole batch: the list's 32-bit places hold twice this many.
+static bool gate_attn_list_fits(const ag_layer_desc &d) {
+  const long long nq = (d.seq + kGaBM - 1) / kGaBM;
+  return (d.gate_causal ? nq * (nq + 1) : 2 * nq * nq) * d.batch * d.gate_heads < (1LL << 28);
+}
+
+bool gate_attn_tc_supported(const ag_layer_desc &d) {
+  const int GD = d.gate_heads * d.gate_head_dim;
+  if (d.dtype != AG_BF16 || !gate_proj_tc_supported(d.hidden, GD)) return false;
+  // Gate heads of 64 have the CUDA-core form for what goes beyond this one: 28 heads, where the output layer alone
+  // fits an SM's shared memory and the merge's does not, and prompts of about a million tokens.  (128-wide heads end there.)
+  return d.gate_head_dim == 128 ||
+         (mo_smem_bytes(GD) + kMoPieceBytes <= kMaxSmemBytes && gate_attn_list_fits(d));
+}
+
 // Segments of the list: one per SM.
 static int gate_attn_segments(const ag_layer_desc &d, int *n_seg) {
   static int sm_count[64] = {0};                     // per device, read once
@@ -708,9 +721,7 @@ static int gate_attn_segments(const ag_layer_desc &d, int *n_seg) {
     sm_count[dev] = v < 1 ? 1 : (v > kGaMaxSeg ? kGaMaxSeg : v);
   }
   *n_seg = sm_count[dev];
-  const long long nq = (d.seq + kGaBM - 1) / kGaBM;
-  const long long head = d.gate_causal ? nq * (nq + 1 + kGaOverhead) : nq * (2 * nq + kGaOverhead);
-  return head * d.batch * d.gate_heads < (1LL << 28) ? AG_OK : AG_ERR_UNSUPPORTED;
+  return gate_attn_list_fits(d) ? AG_OK : AG_ERR_UNSUPPORTED;
 }
 
 size_t gate_attn_partial_bytes(const ag_layer_desc &d) {

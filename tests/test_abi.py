@@ -50,6 +50,23 @@ def test_workspace_sizes(lib):
     assert ag.ag_workspace_bytes(bad, ag.AG_CALL_DECODE) == 0
 
 
+def test_gate_workspace_names_the_form(lib):
+    """Gate heads of 64 beyond the tensor-core form keep the CUDA-core form and its workspace: Q', K', V' and H' in float32."""
+    def cuda_core(s):
+        rows, GD = s.batch * s.seq, s.gate_heads * s.gate_head_dim
+        return -(-rows * 3 * GD * 4 // 256) * 256 + -(-rows * GD * 4 // 256) * 256
+
+    s = inputs.LayerShape(1, 70, 128, 32, 64, 28, 64, "bf16")
+    assert ag.ag_workspace_bytes(ag.make_desc(s), ag.AG_CALL_GATE) == cuda_core(s)
+    s = s.with_(gate_heads=26)
+    assert ag.ag_workspace_bytes(ag.make_desc(s), ag.AG_CALL_GATE) > cuda_core(s)
+    # 4 heads: query tiles of 128, nq (nq + 1) / 2 pairs of tiles per head
+    s = s.with_(gate_heads=4, seq=8191 * 128)
+    assert ag.ag_workspace_bytes(ag.make_desc(s), ag.AG_CALL_GATE) > cuda_core(s)
+    s = s.with_(seq=8191 * 128 + 1)
+    assert ag.ag_workspace_bytes(ag.make_desc(s), ag.AG_CALL_GATE) == cuda_core(s)
+
+
 def test_status_strings(lib):
     assert ag.ag_status_string(0) == "ok"
     for s in (-1, -2, -3, -4, -5, -99):

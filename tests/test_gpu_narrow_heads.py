@@ -83,3 +83,17 @@ def test_decode_step_of_shared_slabs(D, h, hk, B):
         for s in np.nonzero(after > before)[0]:
             assert np.array_equal(rows[off[s] + before[s]], T.f64(kn).reshape(-1, D)[s])
     assert int(status.item()) == ag.AG_DEV_OVERFLOW and ag.ag_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("n,causal,gh", [(70, 1, 28), (70, 0, 26), (2400, 1, 28)])
+def test_gate_of_many_64_wide_heads(n, causal, gh):
+    """The widest gates of 64-wide heads: 26 are the last the tensor-core form takes, 28 go to the CUDA cores (4 tokens per
+    CTA of its output layer, and 16 beyond 2,368 tokens)."""
+    shape = LayerShape(1, n, 128, 32, 64, gh, 64, "bf16", gate_causal=causal)
+    X, W = inputs.hidden_states(shape, 900, DEV), inputs.layer_weights(shape, 901, DEV)
+    W["Wo_g"] = inputs.randn(tuple(W["Wo_g"].shape), 902, DEV, shape.torch_dtype, 0.1)
+    scores, flags = T.gpu_gate(shape, X, W, None)
+    s_ref, f_ref = T.oracle_gate(shape, X, W, None)
+    assert np.max(np.abs(T.f64(scores) - s_ref)) < 1e-4                # the bound every gate path is held to
+    T.check_flags(shape, flags, s_ref, f_ref, None)
+    assert ag.ag_device_wait_timeouts() == 0
