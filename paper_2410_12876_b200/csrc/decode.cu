@@ -761,11 +761,12 @@ static bool decode_carries_append(const ag_layer_desc &d) {
 //   8 slabs, cap 13107     79 | 42 | 23 | 13.4,  11.5
 // While a step waits for latency: as many CTAs per slab as one wave holds (3 per SM at 128, 5 at 64), unless the slab
 // has too few rows for them.  Where it waits for HBM: 1024 rows per CTA or fewer, so that long slabs do not end alone.
-// Only few slabs of very many rows need more CTAs than a cluster has.
+// Only few slabs of very many rows need more CTAs than a cluster has, and only with more than kClusterMaxSlabs query slabs
+// (query_slabs) may they have them: up to there the scratch stays untouched, which callers without scratch of their own count on.
 template <int D>
-static int decode_ctas(int slabs, int max_cap) {
+static int decode_ctas(int slabs, int query_slabs, int max_cap) {
   constexpr int kSms = 148, kWave = kSms * (D == 128 ? 3 : 5);
-  if (slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
+  if (query_slabs > kClusterMaxSlabs && slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
   int wave = max_cap <= 128 ? 1 : max_cap <= 512 ? 4 : kClusterSize;
   while (wave > 1 && (int64_t)slabs * wave > kWave) wave /= 2;
   if (wave == 2 && max_cap <= 512) wave = 1;
@@ -790,7 +791,7 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     };
     const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
     // (clusters of one query head each never carry the append: see decode_carries_append)
-    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas<D>(n, c.max_cap) : 0) {
+    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas<D>(n, slabs, c.max_cap) : 0) {
       case 1: return cluster(std::integral_constant<int, 1>{}, n, G);
       case 2: return cluster(std::integral_constant<int, 2>{}, n, G);
       case 4: return cluster(std::integral_constant<int, 4>{}, n, G);

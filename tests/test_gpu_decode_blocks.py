@@ -48,7 +48,8 @@ def test_lengths_at_the_edges_of_blocks(D, h, hk):
     (24, 32, 8, 64, 300), (20, 32, 8, 128, 700),         # one and two: what one wave holds
     (12, 16, 8, 128, 400), (60, 8, 8, 128, 2100),        # four: by the wave, by the rows per CTA
     (9, 18, 9, 64, 4200),                                # eight, by the rows per CTA
-    (1, 8, 8, 128, 8300), (1, 64, 4, 64, 8300),          # few slabs of very many rows: the split form
+    (1, 8, 8, 128, 8300), (1, 64, 4, 64, 8300),          # eight, few slabs of very many rows
+    (2, 40, 8, 128, 8300), (1, 128, 8, 64, 8300),        # the same with more than 64 query heads: the split form
 ])
 def test_ctas_per_slab(B, h, hk, D, longest):
     """Each choice of CTAs per slab, over empty, one-row and full slabs among ragged ones, with the append."""
@@ -74,3 +75,23 @@ def test_ctas_per_slab(B, h, hk, D, longest):
         if s != 1:
             assert np.array_equal(rows[off[s] + lens[s] + 1], T.f64(kn).reshape(-1, D)[s])
     assert int(status.item()) == ag.AG_DEV_OVERFLOW and ag.ag_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("B,h,hk,D,dtype,longest,untouched", [
+    (1, 8, 8, 128, "bf16", 8300, True), (2, 32, 8, 128, "bf16", 8300, True), (1, 64, 4, 64, "bf16", 8300, True),
+    (2, 32, 1, 64, "bf16", 300, True), (16, 4, 4, 64, "f32", 300, True),
+    (2, 40, 8, 128, "bf16", 8300, False), (17, 4, 4, 64, "f32", 300, False),
+])
+def test_up_to_64_slabs_leave_the_scratch_alone(B, h, hk, D, dtype, longest, untouched):
+    """Callers of ag_decode_attn_noalloc may count on it: calls of so few slabs share no array."""
+    shape = LayerShape(B, longest + 8, 64, h, D, 1, 64, dtype, kv_heads=hk)
+    lens = np.random.default_rng(1).integers(1, 40, size=B * hk)
+    lens[0] = longest
+    cache = ag.RaggedCache.allocate(shape, lens, DEV)
+    cache.len.copy_(torch.from_numpy(lens.astype(np.int32)))
+    desc = ag.make_desc(shape)
+    ws = ag.workspace(desc, ag.AG_CALL_DECODE)
+    ws.fill_(77)
+    q, kn, vn, _ = inputs.decode_inputs(shape, 50, 0, DEV)
+    ag.ag_decode_attn(desc, q, kn, vn, cache, 0.0, torch.empty_like(q), ws)
+    assert bool((ws == 77).all()) == untouched
