@@ -42,6 +42,12 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
   return v;
 }
 
+__device__ __forceinline__ int ld_cluster_s32(uint32_t addr) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+
 template <int BN, int splits, class P>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
@@ -52,7 +58,7 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
   uint64_t *empty = full + C::kStages;
   uint64_t *acc_full = empty + C::kStages;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_full + 1);
-  int *gave_up = reinterpret_cast<int *>(tmem_slot + 1);       // an epilogue thread's wait for the accumulator expired
+  int *gave_up = reinterpret_cast<int *>(tmem_slot + 1);       // a wait of this CTA expired: its share of the sums is not there
   __shared__ typename P::Shared psh;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -99,7 +105,10 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
     const uint32_t b_lo0 = (uint32_t)db0, b_hi = (uint32_t)(db0 >> 32);
     for (int kb = kb_begin; kb < kb_end; ++kb) {
       const int i = kb - kb_begin, s = i % C::kStages;
-      if (!mbar_wait(&full[s], (i / C::kStages) & 1)) break;
+      if (!mbar_wait(&full[s], (i / C::kStages) & 1)) {
+        *gave_up = 1;
+        break;
+      }
       tc_fence_after_sync();
       const uint32_t a_lo = a_lo0 + ((s * C::kStageBytes) >> 4), b_lo = b_lo0 + ((s * C::kStageBytes) >> 4);
       if (elect_one()) {
@@ -136,6 +145,8 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
   __syncwarp();
   cluster_arrive_wait();                             // every CTA's accumulator lies in its shared memory
   if (warp >= 2 && *gave_up == 0) {
+    // (A CTA that gave up holds operands where its sums should be: its tile is left unwritten by every rank.  Looked at
+    // with the sums, so that nothing waits for it.)
     // Distributed shared memory answers late: kRows rows per warp in flight (up to 16 loads of 16 bytes per lane).
     constexpr int kChunks = BN / 128;                // 16-byte chunks (four columns) per lane
     constexpr int kRows = 16 / ((splits - 1) * kChunks);
@@ -148,9 +159,12 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
       // The CTA's own share comes from its shared memory, the others' in the order rank + 1, rank + 2, ...: no
       // CTA is asked by all at once, and a row's sum has a fixed order.
       float4 sum[kRows][kChunks], v[splits - 1][kRows][kChunks];
+      int lost = 0;
 #pragma unroll
       for (int i = 1; i < splits; ++i) {
-        const uint32_t peer = mapa_shared(base, rank + i < splits ? rank + i : rank + i - splits);
+        const int from = rank + i < splits ? rank + i : rank + i - splits;
+        const uint32_t peer = mapa_shared(base, from);
+        lost |= ld_cluster_s32(mapa_shared(smem_u32(gave_up), from));
 #pragma unroll
         for (int u = 0; u < kRows; ++u)
 #pragma unroll
@@ -168,6 +182,7 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
           }
           sum[u][c] = t;
         }
+      if (lost != 0) break;
 #pragma unroll
       for (int u = 0; u < kRows; ++u)
         if (row0 + u < row_end)
