@@ -132,6 +132,11 @@ def _marshal():
     """The extension module that unpacks the arguments and makes the C call (csrc/py_binding.cpp)."""
     global _m
     lib()
+    from . import build
+    # (looked at before it is imported: a module for another torch would read tensors by the wrong layout)
+    if os.path.exists(build.MARSHAL) and not build.marshal_matches(build.MARSHAL):
+        raise RuntimeError(f"{build.MARSHAL} was built for another torch or Python (this is {build.marshal_tag()!r}): "
+                           "build it again with `python -m paper_2410_12876_b200.build`")
     m = importlib.import_module("._marshal", __package__)
     _m = m
     return m

@@ -21,11 +21,24 @@ def _newest_source_mtime():
     return max(os.path.getmtime(p) for p in paths)
 
 
+def marshal_tag():
+    """What _marshal.so depends on beside its sources: it reads torch's tensors and Python's objects by their layout."""
+    import sysconfig
+    import torch
+    return f"AG_MARSHAL_FOR torch {torch.__version__} python {sysconfig.get_config_var('SOABI')}"
+
+
+def marshal_matches(path):
+    """Whether the module at `path` was built for this torch and this Python; its tag lies in it as text."""
+    with open(path, "rb") as f:
+        return marshal_tag().encode() + b"\0" in f.read()
+
+
 def build_marshal(force=False):
     """Compile csrc/py_binding.cpp into _marshal.so, linked against libag.so and torch."""
     src = os.path.join(CSRC, "py_binding.cpp")
     newest = max(os.path.getmtime(p) for p in (src, os.path.join(HERE, "..", "include", "ag.h"), os.path.abspath(__file__)))
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= newest:
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= newest and marshal_matches(MARSHAL):
         return MARSHAL
     import sysconfig
     import torch
@@ -35,7 +48,7 @@ def build_marshal(force=False):
            os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
     # torch's own libraries are in the process already when the module is imported; libag.so lies beside it
     subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-                    f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                    f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DAG_MARSHAL_TAG="{marshal_tag()}"',
                     *[f"-I{p}" for p in inc], src, "-o", MARSHAL, f"-L{HERE}", "-lag", "-Wl,-rpath,$ORIGIN",
                     "-L" + os.path.join(T, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"], check=True)
     return MARSHAL

@@ -261,5 +261,7 @@ PyMODINIT_FUNC PyInit__marshal(void) {
       method<decode_attn_noalloc>("decode_attn_noalloc"), method<decode_step>("decode_step"),
       method<cache_append>("cache_append"), {nullptr, nullptr, 0, nullptr}};
   static PyModuleDef def = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
-  return PyModule_Create(&def);
+  PyObject *m = PyModule_Create(&def);
+  if (m && PyModule_AddStringConstant(m, "tag", AG_MARSHAL_TAG) != 0) Py_CLEAR(m);
+  return m;
 }
