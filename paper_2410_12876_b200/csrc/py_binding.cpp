@@ -15,11 +15,18 @@
 namespace {
 
 // Reads the positional arguments of one call in order.  The first failure sets the Python error and
-// makes every later read return zero; the caller looks at ok() once.
+// makes every later read return zero; the caller looks at done() once.
 class Args {
  public:
   Args(PyObject *const *args, Py_ssize_t n) : a_(args), n_(n) {}
-  bool ok() const { return ok_; }
+  // After the last argument: whether all were read and none is left over.
+  bool done() {
+    if (ok_ && i_ < n_) {
+      PyErr_SetString(PyExc_TypeError, "too many arguments");
+      ok_ = false;
+    }
+    return ok_;
+  }
 
   const ag_layer_desc *desc() {
     PyObject *o = next();
@@ -112,8 +119,8 @@ class Args {
 
 // Runs the C call without the interpreter lock (a launch may block on a full queue).
 template <typename F>
-PyObject *finish(const Args &a, F &&call) {
-  if (!a.ok()) return nullptr;
+PyObject *finish(Args &a, F &&call) {
+  if (!a.done()) return nullptr;
   int st;
   Py_BEGIN_ALLOW_THREADS
   st = call();

@@ -136,3 +136,13 @@ def test_binding_raises_with_status(lib):
     with pytest.raises(ag.AgError) as e:
         ag.ag_gate_forward(d, 4096, 4096, 4096, 4096, 4096, None, None, 4096, None, stream=0)
     assert e.value.status == ag.AG_ERR_INVALID_ARG
+
+
+def test_marshalling_takes_no_argument_too_many(lib):
+    m = ag._marshal()
+    d = ag.make_desc(inputs.TINY.with_(seq=0))                         # refused by the call itself
+    assert m.out_project(d, 4096, 4096, None, 4096, 0) == ag.AG_ERR_INVALID_ARG
+    with pytest.raises(TypeError, match="too few"):
+        m.out_project(d, 4096, 4096, None, 4096)
+    with pytest.raises(TypeError, match="too many"):
+        m.out_project(d, 4096, 4096, None, 4096, 0, 0)
