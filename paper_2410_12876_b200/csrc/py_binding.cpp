@@ -82,8 +82,7 @@ class Args {
     PyObject *o = next();
     if (!o) return nullptr;
     if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-    if (PyLong_Check(o)) return PyLong_AsVoidPtr(o);
-    PyObject *s = PyObject_GetAttrString(o, "cuda_stream");
+    PyObject *s = PyLong_Check(o) ? Py_NewRef(o) : PyObject_GetAttrString(o, "cuda_stream");
     if (!s) return fail<void *>();
     void *p = PyLong_AsVoidPtr(s);
     Py_DECREF(s);

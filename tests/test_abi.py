@@ -146,3 +146,13 @@ def test_marshalling_takes_no_argument_too_many(lib):
         m.out_project(d, 4096, 4096, None, 4096)
     with pytest.raises(TypeError, match="too many"):
         m.out_project(d, 4096, 4096, None, 4096, 0, 0)
+
+
+def test_marshalling_refuses_a_stream_handle_out_of_range(lib):
+    """... before the call is made: not as an error after it has run on another stream."""
+    d = ag.make_desc(inputs.TINY.with_(seq=0))
+    for bad in (1 << 80, -(1 << 80)):
+        with pytest.raises(OverflowError):
+            ag.ag_out_project(d, 4096, 4096, None, 4096, bad)
+    with pytest.raises(AttributeError):
+        ag.ag_out_project(d, 4096, 4096, None, 4096, "stream")
