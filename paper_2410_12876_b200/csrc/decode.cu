@@ -332,11 +332,13 @@ decode_partial_gqa_kernel(const T *q, const T *k_rows,
   }
 }
 
-// Merges the chunks' triples of every query slab with the self term.  One CTA per key/value slab: D threads
-// (thread d owns output dimension d) for each of blockDim.y query heads of the group, in rounds, so that the
-// CTA that appends to the slab is the only one that reads its length.  The chunks' weights are computed
+// Merges the chunks' triples of every query slab with the self term.  CTA (slab, y): D threads
+// (thread d owns output dimension d) for each of blockDim.y query heads of the key/value slab's group.  One CTA per slab
+// where it appends, which then is the only one that reads the slab's length; else as many as the group fills (in one CTA, eight
+// rounds for 32 heads, a step of 4 such slabs took 35 us, 23 with an append of its own).  The chunks' weights are computed
 // side by side, a chunk per lane, and the partial outputs are loaded eight at a time: one chunk after the
 // other, each load waiting for its turn, took 11.5 us for 1024 query slabs of 17 chunks.
+__host__ __device__ constexpr int combine_heads(int D) { return 512 / D; }     // query heads at once
 template <typename T, int D>
 __global__ void __launch_bounds__(512)
 decode_combine_kernel(const T *q, const T *k_new,
@@ -346,7 +348,7 @@ decode_combine_kernel(const T *q, const T *k_new,
                       const int64_t *row_off, int G, const AppendArgs ap, const RecentRing rg) {
   static_assert(kMaxSplits == 32, "a lane per chunk");
   const int kv = blockIdx.x, d = threadIdx.x, y = threadIdx.y, lane = d & 31;
-  constexpr int kMaxHeads = 512 / D;
+  constexpr int kMaxHeads = combine_heads(D);
   __shared__ float red[kMaxHeads][D / 32];
   __shared__ float ring_s[kMaxHeads][kMaxRecent];
   __shared__ float wgt[kMaxHeads][kMaxSplits];       // weight of every chunk
@@ -359,7 +361,7 @@ decode_combine_kernel(const T *q, const T *k_new,
   row.on = 0;
   if (y == 0) row = load_new_row<T, D>(ap, kv, row_off[kv], k_new, v_new);
   const int n_chunks = (L + chunk_rows - 1) / chunk_rows;
-  for (int h0 = 0; h0 < G; h0 += blockDim.y) {
+  for (int h0 = blockIdx.y * blockDim.y; h0 < G; h0 += gridDim.y * blockDim.y) {
     const int h = h0 + y;
     const bool on = h < G;                           // whole warps: D is a multiple of 32
     const int slab = kv * G + min(h, G - 1);
@@ -745,14 +747,6 @@ size_t decode_workspace_bytes(const ag_layer_desc &d) {
   return align_up(slabs * kMaxSplits * (d.head_dim + 2) * sizeof(float), 256);
 }
 
-// Whether the kernels a decode step of this layer takes can carry the append: whichever CTA or cluster
-// appends to a slab has to be the only one that reads it.  Not so where query heads that share a slab go to
-// clusters of their own.
-static bool decode_carries_append(const ag_layer_desc &d) {
-  if (kv_heads_of(d) == d.heads || d.batch * d.heads > kClusterMaxSlabs) return true;
-  return d.dtype == AG_BF16 && d.heads / kv_heads_of(d) <= kGqMaxGroup;
-}
-
 // CTAs per slab of the bf16 cluster form; 0: the split form.  From a sweep over 8 .. 1024 slabs of 100 .. 13,000 rows, head_dim
 // 64 and 128, one and four heads per slab (us per step, CTAs per slab 1 | 2 | 4 | 8, split form last):
 //   32 slabs, cap 102      3.1 | 3.6 | 3.7 | 3.9,  5.9     64 slabs, cap 819   7.9 | 6.4 | 5.9 | 8.2,  7.7
@@ -772,6 +766,19 @@ static int decode_ctas(int slabs, int query_slabs, int max_cap) {
   if (wave == 2 && max_cap <= 512) wave = 1;
   const int rows = max_cap <= 2048 ? 1 : max_cap <= 4096 ? 4 : kClusterSize;
   return wave > rows ? wave : rows;
+}
+
+// Whether the kernels a decode step takes can carry the append: whichever CTA or cluster appends to a slab has to be the
+// only one that reads it.  Not so where query heads that share a slab go to clusters of their own, or are more than a CTA
+// of the merge takes at once.
+static bool decode_carries_append(const ag_layer_desc &d, const ag_cache &c) {
+  const int slabs = d.batch * d.heads, group = d.heads / kv_heads_of(d);
+  if (group == 1) return true;
+  const bool grouped = d.dtype == AG_BF16 && group <= kGqMaxGroup;        // one cluster per key/value slab
+  if (slabs <= kClusterMaxSlabs) return grouped;
+  const int ctas = !grouped ? 0 : d.head_dim == 64 ? decode_ctas<64>(slabs / group, slabs, c.max_cap)
+                                                   : decode_ctas<128>(slabs / group, slabs, c.max_cap);
+  return ctas > 0 || group <= combine_heads(d.head_dim);
 }
 
 template <typename T, int D>
@@ -826,7 +833,8 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
                     c.len, scale_log2, chunk_rows, part_o, part_ml, hm);
   }
   if (rc) return rc;
-  return launch_pdl(decode_combine_kernel<T, D>, dim3(kv_slabs), dim3(D, group < 512 / D ? group : 512 / D), 0, st, qp, kn,
+  const int heads = group < combine_heads(D) ? group : combine_heads(D);
+  return launch_pdl(decode_combine_kernel<T, D>, dim3(kv_slabs, ap.flag_new ? 1 : (group + heads - 1) / heads), dim3(D, heads), 0, st, qp, kn,
                     vn, c.len, scale_log2, chunk_rows, part_o, part_ml, static_cast<T *>(o), c.row_off, group, ap, rg);
 }
 
@@ -850,7 +858,7 @@ int launch_decode(const ag_layer_desc &d, const void *q, const void *k_new, cons
 int launch_decode_step(const ag_layer_desc &d, const void *q, const void *k_new, const void *v_new,
                        const uint8_t *flag_new, const ag_cache &c, float scale, void *o,
                        int32_t *dev_status, void *ws, cudaStream_t st) {
-  if (!decode_carries_append(d)) {
+  if (!decode_carries_append(d, c)) {
     // query heads share a slab: the append waits for all of them, in a launch of its own
     int rc = dispatch_decode(d, q, k_new, v_new, c, scale, o, ws, AppendArgs{}, st);
     if (rc) return rc;

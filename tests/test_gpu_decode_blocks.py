@@ -50,6 +50,7 @@ def test_lengths_at_the_edges_of_blocks(D, h, hk):
     (9, 18, 9, 64, 4200),                                # eight, by the rows per CTA
     (1, 8, 8, 128, 8300), (1, 64, 4, 64, 8300),          # eight, few slabs of very many rows
     (2, 40, 8, 128, 8300), (1, 128, 8, 64, 8300),        # the same with more than 64 query heads: the split form
+    (5, 18, 1, 128, 300), (3, 34, 1, 64, 300),           # more than 16 heads per slab, more than 64 in all: the split form
 ])
 def test_ctas_per_slab(B, h, hk, D, longest):
     """Each choice of CTAs per slab, over empty, one-row and full slabs among ragged ones, with the append."""
