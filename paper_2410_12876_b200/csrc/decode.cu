@@ -747,24 +747,29 @@ size_t decode_workspace_bytes(const ag_layer_desc &d) {
   return align_up(slabs * kMaxSplits * (d.head_dim + 2) * sizeof(float), 256);
 }
 
-// CTAs per slab of the bf16 cluster form; 0: the split form.  From a sweep over 8 .. 1024 slabs of 100 .. 13,000 rows, head_dim
-// 64 and 128, one and four heads per slab (us per step, CTAs per slab 1 | 2 | 4 | 8, split form last):
-//   32 slabs, cap 102      3.1 | 3.6 | 3.7 | 3.9,  5.9     64 slabs, cap 819   7.9 | 6.4 | 5.9 | 8.2,  7.7
-//   128 slabs, cap 1638    15.4 | 12.3 | 13.5 | 15.7,  15.2    384 slabs, cap 409   7.8 | 11.4 | 17.4 | -,  13.3
-//   640 slabs, cap 3276    113 | 108 | 107 | -,  115      1024 slabs, cap 7372   342 | 329 | 323 | 323,  342
-//   8 slabs, cap 13107     79 | 42 | 23 | 13.4,  11.5
-// While a step waits for latency: as many CTAs per slab as one wave holds (3 per SM at 128, 5 at 64), unless the slab
-// has too few rows for them.  Where it waits for HBM: 1024 rows per CTA or fewer, so that long slabs do not end alone.
+// CTAs per slab of the bf16 cluster form for groups of G heads; 0: the split form.  From a sweep over 8 .. 1024 slabs of 100 ..
+// 16,000 rows, head_dim 64 and 128 (us per step, CTAs per slab 1 | 2 | 4 | 8, split form last; "of" a capacity: 1 - 3 % full):
+//   32 slabs, cap 130      2.9 | 3.4 | 3.5 | 3.7,  5.3     64 slabs, cap 800   7.2 | 6.1 | 5.5 | 7.7,  7.5
+//   128 slabs, cap 1600    14.5 | 11.4 | 12.1 | 14.2,  13.7    384 slabs, cap 400   7.5 | 10.7 | 16.0 | 28,  12.3
+//   640 slabs, cap 3200    109 | 105 | 104 | 110,  113      1024 slabs, cap 6550   336 | 326 | 321 | 321,  343
+//   512 slabs, cap 12,800  351 | 328 | 318 | 314,  334      512 of 8000  7.8 | 12.4 | 18.8 | 35.9,  30.1
+//   320 slabs of 64, cap 560   7.4 | 9.1 | 11.0 | 16.7,  14.3    1024 of 64, cap 4800   132 | 126 | 124 | 132,  155
+//   64 slabs, 16 heads, cap 1600   22.4 | 16.7 | 12.3 | 20.1,  24.1    192, 16 heads, cap 6400   92 | 86 | 79 | 93,  106
+//   256 slabs, 4 heads, cap 6550   97 | 97 | 89 | 87,  95     8 slabs, cap 13,107 (without the low weights)   79 | 42 | 23 | 13.4,  11.5
+// While a step waits for latency: as many CTAs per slab as one wave holds (the registers allow 3 per SM at 128, 2 with more
+// than 8 heads; 4 and 3 at 64), unless the slab has too few rows for them.  Where it waits for HBM: 1024 rows per CTA or fewer,
+// so that long slabs do not end alone, but of eight CTAs no more than five waves: slabs may hold far less than their capacity.
 // Only few slabs of very many rows need more CTAs than a cluster has, and only with more than kClusterMaxSlabs query slabs
 // (query_slabs) may they have them: up to there the scratch stays untouched, which callers without scratch of their own count on.
 template <int D>
-static int decode_ctas(int slabs, int query_slabs, int max_cap) {
-  constexpr int kSms = 148, kWave = kSms * (D == 128 ? 3 : 5);
+static int decode_ctas(int slabs, int query_slabs, int G, int max_cap) {
+  constexpr int kSms = 148;
+  const int wave_ctas = kSms * (D == 128 ? (G <= 8 ? 3 : 2) : (G <= 8 ? 4 : 3));
   if (query_slabs > kClusterMaxSlabs && slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
   int wave = max_cap <= 128 ? 1 : max_cap <= 512 ? 4 : kClusterSize;
-  while (wave > 1 && (int64_t)slabs * wave > kWave) wave /= 2;
+  while (wave > 1 && (int64_t)slabs * wave > wave_ctas) wave /= 2;
   if (wave == 2 && max_cap <= 512) wave = 1;
-  const int rows = max_cap <= 2048 ? 1 : max_cap <= 4096 ? 4 : kClusterSize;
+  const int rows = max_cap <= 2048 ? 1 : max_cap <= 4096 || (int64_t)slabs * kClusterSize > 5 * wave_ctas ? 4 : kClusterSize;
   return wave > rows ? wave : rows;
 }
 
@@ -776,8 +781,8 @@ static bool decode_carries_append(const ag_layer_desc &d, const ag_cache &c) {
   if (group == 1) return true;
   const bool grouped = d.dtype == AG_BF16 && group <= kGqMaxGroup;        // one cluster per key/value slab
   if (slabs <= kClusterMaxSlabs) return grouped;
-  const int ctas = !grouped ? 0 : d.head_dim == 64 ? decode_ctas<64>(slabs / group, slabs, c.max_cap)
-                                                   : decode_ctas<128>(slabs / group, slabs, c.max_cap);
+  const int ctas = !grouped ? 0 : d.head_dim == 64 ? decode_ctas<64>(slabs / group, slabs, group, c.max_cap)
+                                                   : decode_ctas<128>(slabs / group, slabs, group, c.max_cap);
   return ctas > 0 || group <= combine_heads(d.head_dim);
 }
 
@@ -798,7 +803,7 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     };
     const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
     // (clusters of one query head each never carry the append: see decode_carries_append)
-    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas<D>(n, slabs, c.max_cap) : 0) {
+    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas<D>(n, slabs, G, c.max_cap) : 0) {
       case 1: return cluster(std::integral_constant<int, 1>{}, n, G);
       case 2: return cluster(std::integral_constant<int, 2>{}, n, G);
       case 4: return cluster(std::integral_constant<int, 4>{}, n, G);
