@@ -35,7 +35,8 @@ gate_proj_kernel(const T *A, const T *W0, const T *W1, const T *W2, float *C, in
   const int n0 = blockIdx.x * BT;                // column in the packed [3*GD] output
   const int which = n0 / GD, nw = n0 % GD;       // GD is a multiple of 64: a tile never straddles
   const T *W = which == 0 ? W0 : (which == 1 ? W1 : W2);
-  pdl_launch_dependents();
+  // (No early trigger of MHA': its CTAs, set up beside this kernel's, crowded onto few SMs; 95 -> 40 us for the pass of 500
+  // tokens of two 64-wide gate heads, 224 -> 135 for 1,000 of three with bf16 inputs.)
   // k-block kb -> buffer kb & 1; rows past M are clamped (never stored), k past Kd is zero (Kd is a multiple of 8)
   auto load_block = [&](int kb) {
     const int k0 = kb * kGemmBK, buf = kb & 1;
@@ -195,8 +196,9 @@ static int run_gate(const ag_layer_desc &d, const void *X, const void *Wq, const
       if (rc) return rc;
     } else {
       auto p = [](const void *x) { return static_cast<const T *>(x); };
-      // 64 x 64 outputs per CTA, or 32 x 32 where that leaves SMs without a CTA
-      if ((long long)(3 * GD / 64) * ((M + 63) / 64) >= 148)
+      // 64 x 64 outputs per CTA, or 32 x 32 where that leaves half of the SMs without a CTA (pass of 48 tiles of 64: 41.4 us,
+      // 39.7 at 32; of 120: 58.7, 68.6; of 144: 109, 135)
+      if ((long long)(3 * GD / 64) * ((M + 63) / 64) >= 148 / 2)
         gate_proj_kernel<T, 64><<<dim3(3 * GD / 64, (M + 63) / 64), 256, 0, st>>>(p(X), p(Wq), p(Wk), p(Wv), qkv, M, d.hidden, GD);
       else
         gate_proj_kernel<T, 32><<<dim3(3 * GD / 32, (M + 31) / 32), 256, 0, st>>>(p(X), p(Wq), p(Wk), p(Wv), qkv, M, d.hidden, GD);
