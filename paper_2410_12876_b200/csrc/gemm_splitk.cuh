@@ -8,7 +8,7 @@
 // r adds up rows [r 128 / S, (r + 1) 128 / S) of the tile through distributed shared memory
 // and hands them to the projection's epilogue, a warp per row.
 //
-// P (the projection) supplies: args; skip (a tile nobody wants); load_a / load_b (the TMA boxes of a k-block); prepare (work of the
+// P (the projection) supplies: kExchangeUs (see choose_split); skip (a tile nobody wants); load_a / load_b (the TMA boxes of a k-block); prepare (work of the
 // epilogue warps while the MMAs run); load_row (what the row's epilogue reads from memory, asked for together
 // with the sums) and row (one finished row of BN columns: lane l has columns 4 l .. 4 l + 3 of every group of 128).
 #pragma once
@@ -194,18 +194,22 @@ gemm_splitk_kernel(const __grid_constant__ P p, int num_kb) {
   if (warp == 1) tmem_dealloc(tmem_acc, BN);
 }
 
-// Host side: how many CTAs to split the reduction of `tiles` tiles over (1: not at all).
-// A round of tiles takes as long as its k-blocks (~0.5 us each) plus, in k-blocks' worth, ~6 for set-up and drain and,
-// when split, ~10 for the two cluster barriers and the exchange (measured on the 7B-shaped gate and output
-// projection at 333 tokens); cap[s] is how many clusters of s CTAs the device holds at once.
-inline int choose_split(long long tiles, int num_kb, const int *cap) {
+// Host side: how many CTAs to split the reduction of `tiles` tiles over (1: not at all); cap[s] is how many clusters of s CTAs
+// the device holds at once.  A round of tiles takes (us, fitted to the three projections at 100 .. 1500 tokens, hidden 512 ..
+// 4096, 4 .. 32 heads, every number of CTAs) 0.33 per k-block of 256 columns (0.25 of 128) and 5 beside them; split, 0.45
+// (0.34) per k-block, and exchange_us for set-up, the two cluster barriers and the exchange.  Split in 1 | 2 | 3 | 4 | 5:
+//   output projection of 100 tokens, 64 k-blocks   26.2 | 21.9 | 18.2 | 15.0 | 14.8     300 tokens, 16   10.4 | 12.1 | 11.8 | 9.9 | 10.3
+//   key/value projection of 100 tokens, 64   26.4 | 26.3 | 22.0 | 18.0 | 31.1     500 tokens, 9 heads, 32   13.9 | 17.7 | 26.0 | 31.5 | 30.3
+template <int BN>
+int choose_split(long long tiles, int num_kb, const int *cap, double exchange_us) {
+  constexpr double kKbUs = BN == 256 ? 0.33 : 0.25;
   int best = 1;
   double best_t = 1e30;
   for (int s = 1; s <= kMaxSplit; ++s) {
     if (cap[s] <= 0 || (s > 1 && num_kb / s < 2)) continue;
     const double rounds = (double)((tiles + cap[s] - 1) / cap[s]);
-    const double t = rounds * ((num_kb + s - 1) / s + (s > 1 ? 16 : 6));
-    if (t < 0.95 * best_t) { best_t = t; best = s; }
+    const double t = rounds * (s == 1 ? kKbUs * num_kb + 5 : 1.36 * kKbUs * ((num_kb + s - 1) / s) + exchange_us);
+    if (t < 0.97 * best_t) { best_t = t; best = s; }
   }
   return best;
 }

@@ -556,6 +556,7 @@ static int run_gemm_pair(const void *X, const void *W0, const void *W1, const vo
 // The gate's projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
 template <int BN>
 struct GateProjSplit {
+  static constexpr double kExchangeUs = 8;
   CUtensorMap tmA, tmB[3];
   float *C;
   __nv_bfloat16 *part[3];
@@ -609,7 +610,7 @@ static int try_gemm_split(const void *X, const void *W0, const void *W1, const v
   if (rc) return rc;
   const int n_tiles_n = 3 * GD / BN, num_kb = (K + kTcBK - 1) / kTcBK;
   const long long tiles = (long long)n_tiles_n * ((M + kTcBM - 1) / kTcBM);
-  const int splits = splitk::choose_split(tiles, num_kb, cap);
+  const int splits = splitk::choose_split<BN>(tiles, num_kb, cap, GateProjSplit<BN>::kExchangeUs);
   *done = splits > 1;
   if (splits == 1) return AG_OK;
   GateProjSplit<BN> p;

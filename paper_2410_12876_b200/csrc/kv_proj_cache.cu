@@ -463,6 +463,7 @@ int sm_count() {
 // The same projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
 template <int BN>
 struct KvProjSplit {
+  static constexpr double kExchangeUs = 10.5;
   CUtensorMap tmA, tmB[3];                        // weights of keys, values, queries
   KvEpilogue e;
   __nv_bfloat16 *out[3];                          // dense K, V, Q
@@ -525,7 +526,7 @@ int try_split(const ag_layer_desc &d, const void *X, const void *Wq, const void 
   p.e.tps = (d.seq + kBM - 1) / kBM;
   p.e.n_sub = d.batch * p.e.tps;
   const long long tiles = (long long)p.n_tiles_n * p.e.n_sub;
-  const int splits = splitk::choose_split(tiles, num_kb, cap);
+  const int splits = splitk::choose_split<BN>(tiles, num_kb, cap, KvProjSplit<BN>::kExchangeUs);
   *done = splits > 1;
   if (splits == 1) return AG_OK;
   if ((rc = make_tmap_3d_bf16(&p.tmA, X, d.batch, d.seq, d.hidden, kBM, kBK))) return rc;

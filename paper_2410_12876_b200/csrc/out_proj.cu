@@ -487,6 +487,7 @@ int run_pair(const ag_layer_desc &dsc, const void *O, const void *Wo, const void
 // The same projection with its reduction split over clusters (few tokens; gemm_splitk.cuh).
 template <int BN>
 struct OutProjSplit {
+  static constexpr double kExchangeUs = 8;
   CUtensorMap tmO, tmW;
   const __nv_bfloat16 *X_res;
   __nv_bfloat16 *Y;
@@ -547,7 +548,7 @@ int try_split(const ag_layer_desc &dsc, const void *O, const void *Wo, const voi
   if (rc) return rc;
   const int d = dsc.hidden, num_kb = dsc.heads * (kD / kBK), tps = (dsc.seq + kBM - 1) / kBM;
   const long long tiles = (long long)(d / BN) * dsc.batch * tps;
-  const int splits = splitk::choose_split(tiles, num_kb, cap);
+  const int splits = splitk::choose_split<BN>(tiles, num_kb, cap, OutProjSplit<BN>::kExchangeUs);
   *done = splits > 1;
   if (splits == 1) return AG_OK;
   OutProjSplit<BN> p;
