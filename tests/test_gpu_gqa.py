@@ -23,7 +23,7 @@ SHAPES = {
     "bf16_tc_8over2": LayerShape(2, 333, 512, 8, 128, 2, 128, "bf16", kv_heads=2),
     "bf16_d64_4over1": LayerShape(1, 200, 256, 4, 64, 2, 64, "bf16", kv_heads=1),
     "f32_6over3": LayerShape(1, 150, 128, 6, 128, 1, 128, "f32", kv_heads=3),
-    "bf16_many_slabs": LayerShape(5, 140, 256, 16, 128, 2, 128, "bf16", kv_heads=4),   # 80 query slabs: workspace form
+    "bf16_many_slabs": LayerShape(5, 140, 256, 16, 128, 2, 128, "bf16", kv_heads=4),   # 80 query slabs
 }
 
 
@@ -78,8 +78,8 @@ def test_gqa_rejects_heads_that_do_not_divide():
 @pytest.mark.parametrize("heads,kv_heads", [(16, 8), (24, 8), (16, 4), (16, 2), (16, 1)],
                          ids=["group2", "group3", "group4", "group8", "group16"])
 @pytest.mark.parametrize("n", [700, 65, 1])
-def test_gqa_decode_chunk_pass_on_tensor_cores(heads, kv_heads, n):
-    """bf16, head_dim 128, more than 64 query slabs: the group's heads are the rows of one MMA tile.
+def test_gqa_decode_of_many_slabs_on_tensor_cores(heads, kv_heads, n):
+    """bf16, head_dim 128, more than 64 query slabs, a cluster per slab: the group's heads are the columns of the MMAs.
     Slabs of every length from empty to full, several tiles and a ragged tail, caches that grow."""
     shape = LayerShape(5, n, 256, heads, 128, 2, 128, "bf16", kv_heads=kv_heads)
     B, hk = shape.batch, shape.kvh

@@ -279,20 +279,24 @@ def test_decode_long_slabs_many_chunks():
 
 
 @pytest.mark.parametrize("shape", [LayerShape(9, 300, 256, 8, 128, 2, 128, "bf16"),
-                                   LayerShape(17, 150, 128, 4, 64, 1, 64, "f32")],
-                         ids=["bf16_72slabs", "f32_d64_68slabs"])
+                                   LayerShape(17, 150, 128, 4, 64, 1, 64, "f32"),
+                                   LayerShape(9, 150, 128, 16, 64, 1, 64, "f32", kv_heads=4),
+                                   LayerShape(9, 150, 128, 18, 128, 1, 64, "f32", kv_heads=9),
+                                   LayerShape(3, 300, 256, 51, 128, 2, 128, "bf16", kv_heads=3)],
+                         ids=["bf16_72slabs_cluster", "f32_d64_68slabs", "f32_d64_group4", "f32_group2", "bf16_group17"])
 @pytest.mark.parametrize("fused", [False, True], ids=["two_calls", "one_call"])
-def test_decode_many_slabs_takes_the_workspace_form(shape, fused):
-    """More slabs than the one-cluster-per-slab form serves: chunk pass + merge through the
-    workspace, at a size the oracle checks in full; ragged and empty slabs included."""
+def test_decode_of_many_slabs(shape, fused):
+    """More than 64 slabs, at sizes the oracle checks in full; ragged and empty slabs included.  bf16 stays with a cluster per
+    slab; float32, and more than 16 heads per slab, go through the workspace: chunk pass (float32 groups of 2 and 4 in
+    one pass per slab) and merge."""
     Q, K, V = inputs.qkv_gaussian(shape, 470, DEV)
-    f = inputs.bernoulli_flags((shape.batch, shape.heads, shape.seq), 0.6, 471).numpy()
+    f = inputs.bernoulli_flags((shape.batch, shape.kvh, shape.seq), 0.6, 471).numpy()
     f[0, 0] = 1
     f[1, 1] = 0
     f[2, 2, 5:] = 0
     flags = torch.from_numpy(f).to(DEV)
     steps = 3
-    cap = [shape.seq + steps] * (shape.batch * shape.heads)
+    cap = [shape.seq + steps] * (shape.batch * shape.kvh)
     cache, prefix, idx, status = T.gpu_compact(shape, K, V, flags, cap=cap)
     ocache = orc.compact_kv(T.f64(K), T.f64(V), f)
     for step in range(steps):

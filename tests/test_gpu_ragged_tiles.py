@@ -1,7 +1,7 @@
 """Padding that whole tiles of the gate's kernels consist of: the projection GEMMs (single tiles, CTA pairs, reduction split
 over a cluster) leave such tiles out, so their part of the workspace keeps what it held - here NaN, which must reach no
-valid token.  Lengths at the edges of the 128-token tiles; gate heads of 64 (three bf16 parts) and 128; the window's
-band pass and the local gate on the same batches."""
+valid token.  Lengths at the edges of the 128-token tiles; gate heads of 64 (three bf16 parts) and 128; prefill attention
+under a window and the local gate on the same batches."""
 import numpy as np
 import pytest
 import torch

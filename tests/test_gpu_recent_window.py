@@ -20,7 +20,11 @@ SHAPES = {
     "bf16_d64": LayerShape(1, 200, 256, 4, 64, 2, 64, "bf16"),
     "f32_d128": LayerShape(1, 150, 128, 3, 128, 1, 128, "f32"),
     "bf16_gqa": LayerShape(2, 300, 512, 8, 128, 2, 128, "bf16", kv_heads=2),
-    "bf16_many_slabs": LayerShape(9, 140, 256, 8, 128, 2, 128, "bf16"),      # decode through the workspace
+    "bf16_many_slabs": LayerShape(9, 140, 256, 8, 128, 2, 128, "bf16"),
+    # decode through the workspace: the merge reads the ring, and fills it where it carries the append (float32)
+    "f32_many_slabs": LayerShape(17, 60, 128, 4, 64, 1, 64, "f32"),
+    "f32_many_slabs_gqa": LayerShape(9, 60, 128, 16, 64, 2, 64, "f32", kv_heads=4),
+    "bf16_group17": LayerShape(2, 140, 256, 34, 128, 2, 128, "bf16", kv_heads=2),
 }
 
 

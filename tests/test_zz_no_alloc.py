@@ -65,14 +65,15 @@ def _oracle_cache(shape, K, V, f):
     return orc, orc.compact_kv(T.f64(K), T.f64(V), f)
 
 
-# Up to 64 slabs the decode call keeps its partial results on chip and touches no scratch at all; above,
-# it goes through the scratch (the caller's workspace, or here the array inside the library).  Both
-# sizes are run: the first shows the entry point itself, the other two make the kernels write and
-# read the shared array.
+# Up to 64 slabs the decode call keeps its partial results on chip and touches no scratch at all, and bf16 beyond that
+# nearly always; float32, more than 16 heads per slab and few long slabs go through the scratch (the caller's workspace,
+# or here the array inside the library).  The first two show the entry point itself, the others make the kernels
+# write and read the shared array.
 CASES = {
     "16_slabs_no_scratch": LayerShape(2, 900, 512, 8, 128, 2, 128, "bf16"),
     "72_slabs_bf16": LayerShape(9, 900, 256, 8, 128, 2, 128, "bf16"),
     "68_slabs_f32_d64": LayerShape(17, 300, 128, 4, 64, 1, 64, "f32"),
+    "136_slabs_bf16_17_heads_per_slab": LayerShape(2, 300, 256, 68, 128, 2, 128, "bf16", kv_heads=4),
 }
 
 
@@ -83,12 +84,12 @@ def test_matches_the_workspace_call_twice_in_a_row(case):
     shape = CASES[case]
     desc = ag.make_desc(shape)
     Q, K, V = inputs.qkv_gaussian(shape, 700, dev)
-    f = inputs.bernoulli_flags((shape.batch, shape.heads, shape.seq), 0.6, 701).numpy()
+    f = inputs.bernoulli_flags((shape.batch, shape.kvh, shape.seq), 0.6, 701).numpy()
     f[0, 1] = 0                                     # an empty slab: only the self term
     f[1, 2] = 1                                     # a full one: several split-K chunks
     f[1, 3, 7:] = 0                                 # a short one: one partly filled chunk
     flags = torch.from_numpy(f).to(dev)
-    cap = (f.reshape(shape.batch * shape.heads, -1).sum(axis=1) + 2).tolist()
+    cap = (f.reshape(shape.batch * shape.kvh, -1).sum(axis=1) + 2).tolist()
     cache, prefix, idx, status = T.gpu_compact(shape, K, V, flags, cap=cap)
     orc, ocache = _oracle_cache(shape, K, V, f)
     ws = ag.workspace(desc, ag.AG_CALL_DECODE)
