@@ -27,7 +27,7 @@ constexpr int kMaxSplits = 32;     // chunks per slab the workspace is sized for
 constexpr int kPartThreads = 256;
 constexpr int kUnroll = 8;         // rows in flight per lane group (x2: K and V)
 constexpr int kClusterMaxSlabs = 64;    // float32, and groups of more than 16 heads: up to here one cluster per slab
-constexpr int kClusterThreads = 512;    // 256 rows in flight per CTA of a cluster (bf16, D = 128)
+constexpr int kClusterThreads = 512;    // float32 cluster form: 128 rows in flight per CTA (D = 128)
 
 // Grouped-query attention: slab s = (sequence, query head) of q and o reads the cache slab, k_new
 // and v_new of its key/value head.
@@ -825,7 +825,7 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
   auto kr = static_cast<const T *>(c.k_rows), vr = static_cast<const T *>(c.v_rows);
   int rc = AG_OK;
   if (n_chunks > 0 && decode_gqa_mma_supported(d)) {
-    // grouped-query attention, bf16: the group's heads are the rows of a tensor-core tile
+    // grouped-query attention, bf16: the group's heads are the columns of the MMAs
     rc = launch_decode_partial_gqa_mma(d, q, c, scale_log2, chunk_rows, n_chunks, part_o, part_ml, kMaxSplits, st);
   } else if (std::is_same_v<T, float> && n_chunks > 0 && (group == 2 || group == 4)) {
     // grouped-query attention: the rows of a key/value slab are read once for its query heads

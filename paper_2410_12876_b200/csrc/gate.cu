@@ -2,8 +2,8 @@
 // with the optional constant gamma inside the Sigmoid (Sec. 3.5).
 //
 //   1. projection   [Q' | K' | V'] = X [Wq_g | Wk_g | Wv_g]   (tcgen05 GEMM for bf16, else CUDA cores)
-//   2. MHA'         H'_g = Softmax(Q'_g K'_g^T / sqrt(d'_k)) V'_g  (tcgen05 on bf16 hi/lo pairs for
-//                   bf16 layers with d'_k = 128, else float32 on CUDA cores)
+//   2. MHA'         H'_g = Softmax(Q'_g K'_g^T / sqrt(d'_k)) V'_g  (tcgen05 on two or three bf16
+//                   parts per value for bf16 layers with h' d'_k a multiple of 128, else float32 on CUDA cores)
 //   3. output layer    s = [H'_1 .. H'_h'] Wo_g;  flag = s + gamma > logit(tau)
 //                   (gate_out_kernel; on the tensor-core path fused into the merge of MHA's split-K partials)
 //

@@ -393,9 +393,8 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
                          fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
       tmax *= a.scale_log2;
       // The first tile of a piece holds a key visible to every row (key 0, or a tile wholly before
-      // the query tile) - unless the sequence is shorter than its padded length and the bidirectional
-      // MHA' has no key in this piece at all: m then stays -inf, every weight is 0, and the piece's
-      // partial (m = -inf, l = 0, O = 0) drops out of the merge.
+      // the query tile; the list has no tiles of padding).  m = -inf after it takes scores of -inf, out of
+      // inputs that overflow: every weight is 0 then.
       float m_new;
       if (i == 0) m_new = tmax;
       else m_new = (tmax > m + kGaRescaleThreshold) ? tmax : m;

@@ -10,7 +10,8 @@
 namespace ag {
 
 // With a recent-token window the CUDA-core attention leaves each row's log-sum-exp in the workspace
-// for the band pass below.
+// for the band pass below.  (bf16 layers go there with a pool of 2^31 rows or 2^31 query tiles only, where the coordinates of
+// the tensor-core kernel end; which pool it will be is not known when the size is asked for.)
 size_t prefill_workspace_bytes(const ag_layer_desc &d) {
   if (recent_rows(d) == 0) return 0;
   return align_up((size_t)d.batch * d.heads * d.seq * sizeof(float), 256);
@@ -71,22 +72,7 @@ prefill_band_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *_
   }
   if (smax == -INFINITY || !valid) return;           // no shuffles below: lanes may leave
 
-  float row_lse = lse[(size_t)slab * n + j];
-  if (row_lse == -INFINITY) {
-    // the attention kernel skipped the scores of this tile (no retained key): O_j = v_j, weight 2^(q_j . k_j)
-    float kf[kEpl];
-    Elem<T>::unpack(ldg128(Kd + (size_t)j * D), kf);
-    float a = 0.f;
-#pragma unroll
-    for (int e = 0; e < kEpl; ++e) a = fmaf(qf[e], kf[e], a);
-    // the lanes of a group are still together here (the early return above is uniform per group),
-    // but other groups of the warp may have left: reduce through the group's own lanes only
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned group_mask = kLanes == 32 ? 0xffffffffu : (((1u << kLanes) - 1u) << (lane / kLanes * kLanes));
-#pragma unroll
-    for (int off = kLanes / 2; off > 0; off >>= 1) a += __shfl_xor_sync(group_mask, a, off);
-    row_lse = a;
-  }
+  const float row_lse = lse[(size_t)slab * n + j];
   const float M = fmaxf(row_lse, smax);
   const float w0 = exp2f(row_lse - M);
   float of[kEpl];
