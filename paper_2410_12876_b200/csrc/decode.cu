@@ -335,7 +335,7 @@ decode_partial_gqa_kernel(const T *q, const T *k_rows,
 // Merges the chunks' triples of every query slab with the self term.  CTA (slab, y): D threads
 // (thread d owns output dimension d) for each of blockDim.y query heads of the key/value slab's group.  One CTA per slab
 // where it appends, which then is the only one that reads the slab's length; else as many as the group fills (in one CTA, eight
-// rounds for 32 heads, a step of 4 such slabs took 35 us, 23 with an append of its own).  The chunks' weights are computed
+// rounds for 32 heads, a step of 4 such slabs took 35 us, 21 with an append of its own).  The chunks' weights are computed
 // side by side, a chunk per lane, and the partial outputs are loaded eight at a time: one chunk after the
 // other, each load waiting for its turn, took 11.5 us for 1024 query slabs of 17 chunks.
 __host__ __device__ constexpr int combine_heads(int D) { return 512 / D; }     // query heads at once
