@@ -52,24 +52,23 @@ WORKLOADS = {
 # captures summarised under profiles/ (None for workloads that were not captured).  To be reset to
 # None whenever the kernel changes after the capture.
 TRAFFIC = {
-    ("prefill7b", "prefill"): 155.20e6 + 17.45e6,        # prefill_tc_kernel
-    ("prefill7b", "decode"): 41.22e6 + 0.003e6,          # decode_cluster_mma_kernel
-    ("prefill7b", "compact"): 41.26e6 + 2.46e6,          # compact_kernel<256> (written rows still in L2 at kernel end)
+    ("prefill7b", "prefill"): 153.60e6 + 14.66e6,        # prefill_tc_kernel
+    ("prefill7b", "decode"): 41.17e6,          # decode_cluster_mma_kernel
+    ("prefill7b", "compact"): 41.26e6 + 2.43e6,          # compact_kernel<256> (written rows still in L2 at kernel end)
     ("prefill7b", "kv_project_cache"): 182.23e6 + 82.20e6,   # kv_proj_cache_pair_kernel
-    ("prefill7b_proj", "prefill"): 155.20e6 + 17.45e6,
-    ("prefill7b_proj", "decode"): 41.22e6 + 0.003e6,
+    ("prefill7b_proj", "prefill"): 153.60e6 + 14.66e6,
+    ("prefill7b_proj", "decode"): 41.17e6,
     ("prefill7b_proj", "project"): 251.70e6 + 121.58e6,  # kv_proj_cache_pair_kernel with the query projection
-    ("prefill7b_out", "prefill"): 155.20e6 + 17.45e6,
+    ("prefill7b_out", "prefill"): 153.60e6 + 14.66e6,
     ("prefill7b_out", "project"): 251.70e6 + 121.58e6,
     ("prefill7b_out", "out_project"): 132.63e6 + 16.75e6,    # out_proj_pair_kernel
     ("deep_layer", "prefill"): 364.64e6 + 106.70e6,      # prefill_tc_kernel
     ("deep_layer", "compact"): 20.48e6 + 0.34e6,         # compact_kernel<256>
-    ("decode_ragged", "decode"): 2.3530e9 + 7.1e6,       # decode_partial_kernel<bf16,128>
 }
 # kernels launched per call of the library
-# (decode step, attention + append: one cluster kernel up to DECODE_CLUSTER_MAX_SLABS slabs, else chunk pass + merge)
-LAUNCHES = {"gate": 3, "compact": 1, "prefill": 1, "decode": 2}
-DECODE_CLUSTER_MAX_SLABS = 64
+# (decode step, attention + append: one cluster kernel on every workload; the split form, chunk pass + merge, takes float32 of
+# more than 64 slabs, more than 16 heads per slab, and few slabs of more than 8192 rows)
+LAUNCHES = {"gate": 3, "compact": 1, "prefill": 1, "decode": 1}
 L2_BYTES = 126e6
 MIN_TIMED_S = 0.6     # a run's timed region lasts at least about this long
 
@@ -477,14 +476,9 @@ class LayerRun:
 
     def launches_per_step(self):
         gates = (self.layers - self.first_gated) if self.has_gate else 0      # the last guided layer's gate has no consumer
-        window = 2 if self.shape.recent_window > 1 else 0      # the ring fill after compaction, the band pass after prefill
         return gates * LAUNCHES["gate"] + self.layers * (
-            (LAUNCHES["compact"] + LAUNCHES["prefill"] + window + (1 if self.chain else 0) if self.has_prefill else 0)
-            + self.decode_steps * self.decode_launches())
-
-    def decode_launches(self):
-        slabs = self.shape.batch * self.shape.heads
-        return 1 if slabs <= DECODE_CLUSTER_MAX_SLABS else LAUNCHES["decode"]
+            (LAUNCHES["compact"] + LAUNCHES["prefill"] + (1 if self.chain else 0) if self.has_prefill else 0)
+            + self.decode_steps * LAUNCHES["decode"])
 
     def work_per_call(self):
         """Algorithmic work of one call, averaged over the layers of a pass (untimed extra pass):
