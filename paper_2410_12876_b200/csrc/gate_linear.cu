@@ -7,9 +7,16 @@
 // kernel is bound by reading X once.  bf16 layers run on the tensor cores
 // (products of bf16 inputs are exact in the float32 accumulator): one CTA owns
 // 128 tokens and a slice of d; the CTAs of a thread-block cluster split d among
-// them so that enough CTAs stream X, and the cluster's first CTA adds the
+// them so that enough CTAs stream X, and then the heads: each adds its heads'
 // partial accumulators in rank order through distributed shared memory (a fixed
 // order: results do not vary from run to run), thresholds and writes.
+//
+// A CTA alone takes 16 KB of X and 8 KB of W per trip; three CTAs of three stages share an SM, so that one's set-up, first
+// trip and exchange lie under the others' streams.  us for 100 | 2000 | 4096 | 2 x 3001 | 11,000 | 20,000 tokens of 4096, 32 heads:
+//   one CTA of six stages, all heads added up by one rank      11.1 | 21.7 | 14.7 | 16.4 | 24.8 | 49.6
+//   the heads shared among the ranks, one CTA of eight stages  6.5 | 12.2 | 11.7 | 16.2 | 25.9 | 53.0
+//   two of four stages                                         6.5 | 7.9 | 10.9 | 14.8 | 23.6 | 38.7
+//   three of three                                             6.4 | 7.9 | 11.2 | 13.6 | 21.7 | 34.6   (4.7 TB/s)
 //   A = X      [B n, d]  row-major -> K-major operand, 128-byte swizzled rows
 //   B = W_lin  [d, h]    row-major -> MN-major operand: one panel of [64 k][64 n],
 //                                     columns past h filled with zeros by TMA
@@ -25,13 +32,15 @@ namespace ag {
 using namespace umma;
 namespace cg = cooperative_groups;
 
-constexpr int kGlBM = 128, kGlBK = 64, kGlThreads = 192, kGlStages = 6;
+constexpr int kGlBM = 128, kGlBK = 64, kGlThreads = 192, kGlStages = 3;
+constexpr int kGlCtasPerSm = 3, kGlMaxSplit = 8;
 constexpr int kGlABytes = kGlBM * kGlBK * 2;              // 16 KB
 constexpr int kGlBBytes = kGlBK * 64 * 2;                 // one panel [64 k][64 n] = 8 KB
 constexpr int kGlStageBytes = kGlABytes + kGlBBytes;
 constexpr int kGlMaxN = 64;                               // heads the tensor-core kernel serves
-constexpr int kGlPartBytes = kGlBM * kGlMaxN * 4;         // a CTA's partial accumulator, [col][row]
-constexpr int kGlSmemBytes = kGlStages * kGlStageBytes + kGlPartBytes + 1024 /*align*/ + 256 /*barriers*/;
+// The partial accumulator of a CTA, [col][row], lies over the stages once every MMA has read them.
+static_assert(kGlBM * kGlMaxN * 4 <= kGlStages * kGlStageBytes, "partial sums");
+constexpr int kGlSmemBytes = kGlStages * kGlStageBytes + 1024 /*align*/ + 256 /*barriers*/;
 constexpr uint32_t kGlTmemCols = 64;
 
 struct GateLinearArgs {
@@ -44,13 +53,13 @@ struct GateLinearArgs {
 };
 
 template <int N>   // MMA width: heads rounded up to 32
-__global__ void __launch_bounds__(kGlThreads, 1)
+__global__ void __launch_bounds__(kGlThreads, kGlCtasPerSm)
 gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                       const GateLinearArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  float *part = reinterpret_cast<float *>(smem + kGlStages * kGlStageBytes);          // [N][128]
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + kGlStages * kGlStageBytes + kGlPartBytes);
+  float *part = reinterpret_cast<float *>(smem);          // [N][128]
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + kGlStages * kGlStageBytes);
   uint64_t *empty = full + kGlStages;
   uint64_t *acc_full = empty + kGlStages;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_full + 1);
@@ -136,27 +145,26 @@ gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     }
   }
   cluster.sync();                       // every CTA's partial sums are in its shared memory
-  if (rank == 0 && warp >= 2) {
+  if (warp >= 2) {
+    // each CTA adds up, thresholds and writes its share of the heads: rank, rank + nranks, ...
     const int quad = warp & 3, r_in = quad * 32 + lane;
     const int tok = m0 + r_in;
     if (tok < a.M) {
       const int b = tok / a.n, t = tok % a.n;
       const bool padding = a.seq_lens && t >= a.seq_lens[b];
-      float s[N];
+      const float *p[kGlMaxSplit];
 #pragma unroll
-      for (int i = 0; i < N; ++i) s[i] = 0.f;
-      for (int rk = 0; rk < nranks; ++rk) {          // rank order: the sum does not depend on timing
-        const float *p = cluster.map_shared_rank(part, rk) + r_in;
+      for (int rk = 0; rk < kGlMaxSplit; ++rk) p[rk] = cluster.map_shared_rank(part, rk < nranks ? rk : rank) + r_in;
+#pragma unroll 4
+      for (int i = rank; i < a.h; i += nranks) {
+        float x[kGlMaxSplit], s = 0.f;
 #pragma unroll
-        for (int i = 0; i < N; ++i) s[i] += p[i * kGlBM];   // independent loads, all in flight
-      }
+        for (int rk = 0; rk < kGlMaxSplit; ++rk) x[rk] = rk < nranks ? p[rk][i * kGlBM] : 0.f;
 #pragma unroll
-      for (int i = 0; i < N; ++i) {
-        if (i < a.h) {
-          const size_t o = ((size_t)b * a.h + i) * a.n + t;   // lanes = consecutive tokens: coalesced
-          if (a.scores) a.scores[o] = s[i];
-          a.flags[o] = !padding && (s[i] + (a.gamma ? a.gamma[i] : 0.f)) > a.logit_tau ? 1 : 0;
-        }
+        for (int rk = 0; rk < kGlMaxSplit; ++rk) s += x[rk];   // rank order: the sum does not depend on timing
+        const size_t o = ((size_t)b * a.h + i) * a.n + t;      // lanes = consecutive tokens: coalesced
+        if (a.scores) a.scores[o] = s;
+        a.flags[o] = !padding && (s + (a.gamma ? a.gamma[i] : 0.f)) > a.logit_tau ? 1 : 0;
       }
     }
   }
@@ -215,10 +223,11 @@ static int run_gate_linear_tc(const ag_layer_desc &d, const void *X, const void 
   if (rc) return rc;
   rc = make_tmap_2d_bf16(&tmW, W, d.hidden, kv_heads_of(d), (uint64_t)kv_heads_of(d) * 2, kGlBK, 64);
   if (rc) return rc;
-  // split d over a cluster until about one CTA per SM streams X (at least four k blocks each)
+  // Split d over a cluster while one wave holds all its CTAs and each has at least four k blocks.  Powers of two only: clusters
+  // of six of two CTAs per SM left a second wave at 47 tiles (20.2 us against 14.8 in four).
   const int m_tiles = (a.M + kGlBM - 1) / kGlBM;
   int split = 1;
-  while (split < 8 && m_tiles * split * 2 <= 160 && a.kb_total / (split * 2) >= 4) split *= 2;
+  while (split < kGlMaxSplit && m_tiles * split * 2 <= kGlCtasPerSm * 148 && a.kb_total / (split * 2) >= 4) split *= 2;
   a.kb_per_cta = (a.kb_total + split - 1) / split;
   auto kern = gate_linear_tc_kernel<N>;
   AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGlSmemBytes));

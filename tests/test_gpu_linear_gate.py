@@ -86,3 +86,14 @@ def test_linear_gate_rejects_bad_arguments():
         ag.ag_gate_linear_forward(ag.make_desc(shape), X, None, None, None, flags)
     with pytest.raises(ag.AgError):
         ag.ag_gate_linear_forward(ag.make_desc(shape.with_(tau=1.5)), X, W, None, None, flags)
+
+
+@pytest.mark.parametrize("batch,seq,hidden,heads", [
+    (1, 7040, 2048, 40), (1, 7041, 2048, 24),            # eight CTAs to a tile, four: what one wave holds
+    (2, 7111, 1032, 8), (1, 28417, 512, 16),             # two, one
+    (1, 129, 2048 + 8, 64),                              # the last k block alone with one rank
+])
+def test_linear_gate_shares_of_a_cluster(batch, seq, hidden, heads):
+    """Every number of CTAs a tile is shared by, heads that do not divide among them, a ragged last tile."""
+    _run(LayerShape(batch, seq, hidden, heads, 128, 1, 64, "bf16"), 730)
+    assert ag.ag_device_wait_timeouts() == 0
