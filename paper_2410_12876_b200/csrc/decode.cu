@@ -430,6 +430,7 @@ decode_combine_kernel(const T *q, const T *k_new,
 // second barrier keeps every CTA's shared memory alive until it has been read.  No CTA leaves
 // early: the cluster barriers need all of them.
 constexpr int kClusterSize = 8;
+constexpr int kWideCluster = 16, kWideMaxSlabs = 16;    // bf16, few slabs of many rows (see decode_ctas)
 //
 // kCtas = 1: a cluster of one, for caches that one CTA streams in a round or two (its barriers are the CTA's own).
 template <typename T, int D, int kThreads, int kCtas>
@@ -561,7 +562,7 @@ decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
 // One cluster per run of G <= 16 query slabs that share a key/value slab (G = 1 without grouped-query
 // attention): the G queries are columns of one MMA operand, so the slab is read once for all of them, and the
 // one cluster that reads it may append to it.  CTA `rank` takes whole 64-row tiles; after the cluster
-// barrier rank r merges the heads r, r + 8 of the group, whose triples the ranks have written to its shared memory.
+// barrier rank r merges the heads r, r + kCtas, ... of the group, whose triples the ranks have written to its shared memory.
 // Nothing of the cache is read ahead of the wait for the preceding kernel, which may be one that lays it out: where a
 // slab begins arrives with its length, the queries in the same trip (the queries behind the length: 127.5 -> 133.6 us for
 // 16 steps; the first tile asked for from where the slab seemed to lie before the wait, checked after it: 131.3).
@@ -702,6 +703,8 @@ static int launch_decode_cluster_mma(int groups, int G, const void *q, const voi
                                      const HeadMap &hm, const RecentRing &rg, cudaStream_t st) {
   using T = __nv_bfloat16;
   constexpr int smem = gq_smem_bytes(D, kCmStages);
+  if constexpr (kCtas > kClusterSize)
+    AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG, kCtas>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kCtas, groups);
@@ -766,6 +769,12 @@ static int decode_ctas(int slabs, int query_slabs, int G, int max_cap) {
   constexpr int kSms = 148;
   const int wave_ctas = kSms * (D == 128 ? (G <= 8 ? 3 : 2) : (G <= 8 ? 4 : 3));
   if (query_slabs > kClusterMaxSlabs && slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
+  // A cluster of sixteen takes its place later and merges more triples, but streams a long slab in half the time.  Up to
+  // sixteen of them run at once (24 and more wait for one another: 8.0 -> 10.1 us).  us per step, 8 | 16 CTAs per slab:
+  //   4 slabs   cap 2200 4.35 | 3.88, 6400 7.54 | 5.40     8 slabs, 4 heads   1200 4.74 | 4.90, 2200 5.30 | 5.28, 3300 6.04 | 5.75, 6400 8.24 | 7.07
+  //   16 slabs   2200 5.07 | 4.90, 6400 8.61 | 7.29     16 slabs, 4 heads   2200 5.65 | 5.90, 3300 6.56 | 6.56, 6400 9.12 | 8.31
+  //   2 slabs, 16 heads   480 7.34 | 5.66, 2200 7.61 | 6.16, 6400 11.8 | 8.37
+  if (slabs <= kWideMaxSlabs && max_cap > (G > 8 ? 512 : slabs * 2 <= kWideMaxSlabs ? 2048 : 4096)) return kWideCluster;
   int wave = max_cap <= 128 ? 1 : max_cap <= 512 ? 4 : kClusterSize;
   while (wave > 1 && (int64_t)slabs * wave > wave_ctas) wave /= 2;
   if (wave == 2 && max_cap <= 512) wave = 1;
@@ -808,6 +817,7 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
       case 2: return cluster(std::integral_constant<int, 2>{}, n, G);
       case 4: return cluster(std::integral_constant<int, 4>{}, n, G);
       case 8: return cluster(std::integral_constant<int, 8>{}, n, G);
+      case kWideCluster: return cluster(std::integral_constant<int, kWideCluster>{}, n, G);
     }
   } else {
     // caches of at most two rounds of one CTA's rows (host-known bound): no cluster

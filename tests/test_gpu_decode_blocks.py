@@ -78,6 +78,15 @@ def test_ctas_per_slab(B, h, hk, D, longest):
     assert int(status.item()) == ag.AG_DEV_OVERFLOW and ag.ag_device_wait_timeouts() == 0
 
 
+@pytest.mark.parametrize("B,h,hk,D,longest", [
+    (1, 4, 4, 128, 2060), (2, 20, 4, 64, 2060),          # up to eight slabs, from 2048 rows
+    (4, 4, 4, 128, 4100), (2, 64, 8, 64, 4100),          # up to sixteen, from 4096
+    (1, 64, 4, 128, 520), (1, 48, 3, 64, 1040),          # 16 heads per slab, from 512; a second tile for one rank
+])
+def test_sixteen_ctas_per_slab(B, h, hk, D, longest):
+    test_ctas_per_slab(B, h, hk, D, longest)
+
+
 @pytest.mark.parametrize("B,h,hk,D,dtype,longest,untouched", [
     (1, 8, 8, 128, "bf16", 8300, True), (2, 32, 8, 128, "bf16", 8300, True), (1, 64, 4, 64, "bf16", 8300, True),
     (2, 32, 1, 64, "bf16", 300, True), (16, 4, 4, 64, "f32", 300, True),
