@@ -10,8 +10,14 @@
 //
 // Structure as in the prefill kernel: warp 0 TMA, warp 1 tcgen05.mma issue,
 // warps 2..5 softmax with one row per thread.  A query tile is 128 queries of
-// one (sequence, gate head); key tiles hold 64 keys (32 KB per K or V stage with
-// the hi and lo halves), two stages each, so loads run a tile ahead of the MMAs.
+// one (sequence, gate head).  Scores are computed for pairs of key tiles (N = 128: an MMA of N = 64 waits for the 6 KB of
+// operands it fetches, 52 cycles for 32 of arithmetic), weights and P V for tiles of 64 keys, whose V has two
+// stages.  There is room for one pair's K only: it is taken in slices, each released as soon as its own MMAs have read it
+// (a panel of 64 columns of both parts, or one part of 64-wide heads, the part with the fewest products
+// first), so that the next pair's arrive while the rest of the scores and two P V run.
+// Gate call, scores of one tile at a time | of pairs, us: 4 heads of 128, 333 tokens 31.0 | 31.0, 1500 50.1 | 48.6, 4096 102.3 |
+// 95.7, 8192 265 | 247, 4 x 1999 155 | 149; 4 heads of 64, 4 x 1500 65.0 | 60.1, 8192 205 | 175.  Bound by the tensor cores,
+// 3,072 cycles per pair.  (The first tile's scores on their own, as a branch of the issuing warp: 8192 of 64 175 -> 213.)
 //
 // Work is the list of all (query tile, key tile) steps, query tiles in order
 // and each one's key tiles in order.  The list is cut into equal segments, one
@@ -23,8 +29,8 @@
 // (O, m, l); gate_merge_out_kernel combines the pieces of a query tile and
 // applies the gate's output layer and threshold.
 //
-// TMEM columns: S0 [0,64) S1 [128,192) O [256,256 + D) then 64 columns per part of P, each holding two
-// tiles' weights (32 columns per tile).
+// TMEM columns: scores of an even pair [0,128), of an odd one [128,256), O [256,256 + D) then 64 columns per part of P,
+// each holding two tiles' weights (32 columns per tile).
 #include "ag_common.cuh"
 #include "mma_sync.cuh"
 #include "umma.cuh"
@@ -46,6 +52,11 @@ struct GaCfg {
   static constexpr int kTile = kPanels * kGaPanel;        // one part of Q
   static constexpr int kKvTile = kPanels * kGaKvPanel;    // one part of K or V
   static constexpr int kKvStage = kParts * kKvTile;
+  // K of a pair of key tiles: panels of [128 keys][64 columns], in slices
+  static constexpr int kSlices = D == 64 ? kParts : kPanels;
+  static constexpr int kSliceParts = D == 64 ? 1 : kParts;
+  static constexpr int kSliceBytes = kSliceParts * kGaPanel;
+  static_assert(kSlices * kSliceBytes == 2 * kKvStage, "K of a pair takes two stages");
   static constexpr int kUsedBytes = kParts * kTile + 4 * kKvStage + 1024 + 256;   // Q + 2 K stages + 2 V stages
   static constexpr uint32_t kColO = 256, kColP = kColO + D;
   static_assert(kColP + 64 * kParts <= 512, "tensor memory");
@@ -210,27 +221,27 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
   uint8_t *sK = sQ + C::kParts * kGaTile;      // [stage][part]
   uint8_t *sV = sK + 2 * kGaKvStage;
   uint64_t *bars = reinterpret_cast<uint64_t *>(sV + 2 * kGaKvStage);
-  uint64_t *q_full = bars, *k_full = bars + 1, *k_empty = bars + 3, *v_full = bars + 5, *v_empty = bars + 7;  // [2]
-  uint64_t *s_full = bars + 9;           // [2]
+  uint64_t *q_empty = bars, *o_free = bars + 1;
+  uint64_t *k_full = bars + 2, *k_empty = bars + 5;                          // [slice]
+  uint64_t *v_full = bars + 8, *v_empty = bars + 10, *s_full = bars + 12;    // [2]
   // p_ready[2], pv_done[2]: even / odd tiles.  P is double-buffered (32 of each half's 64 columns per tile), so
   // the weights of tile t are written while the P V of tile t - 1 runs; a softmax warp may be a tile ahead
-  // of a slower one, never two (the scores of tile t + 2 exist only after every thread arrived for tile t).
-  uint64_t *p_ready = bars + 11, *pv_done = bars + 13;
-  uint64_t *q_empty = bars + 15, *o_free = bars + 16;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 17);
+  // of a slower one, never two (the weights of tile t + 2 wait for the P V of tile t).
+  uint64_t *p_ready = bars + 14, *pv_done = bars + 16;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 18);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // Every role walks the pieces of this CTA's segment with the same arithmetic;
-  // tiles are numbered t = 0, 1, ... across the pieces (stage and S buffer t & 1, in their use
-  // number t >> 1; P and the P V barrier in their use number t), pieces pc = 0, 1, ...
+  // tiles are numbered t = 0, 1, ... across the pieces (stage of V, P and the P V barrier t & 1, in their use
+  // number t >> 1), pairs of tiles u = t >> 1 (K slices in their use number u, scores u & 1 in their use
+  // number u >> 1), pieces pc = 0, 1, ...
 
   if (threadIdx.x == 0) {
-    mbar_init(q_full, 1);
     for (int s = 0; s < 2; ++s) {
-      mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], 1);
       mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1);
       mbar_init(&s_full[s], 1);
     }
+    for (int s = 0; s < C::kSlices; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], 1); }
     mbar_init(&p_ready[0], 128); mbar_init(&p_ready[1], 128);
     mbar_init(&pv_done[0], 1); mbar_init(&pv_done[1], 1);
     mbar_init(q_empty, 1);
@@ -250,88 +261,99 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
   pdl_wait();                                        // the projections are there
   pdl_launch_dependents();
   GaWalk walk = ga_start(a, (int)blockIdx.x);
-  GaPiece pz;
+  GaPiece pz = {};
 
   if (warp == 0) {
     if (lane == 0) {
-      bool ok = true;
       int t = 0;
-      for (int pc = 0; ok && ga_next(a, walk, pz); ++pc) {
-        const int b = pz.b, g = pz.g, j0 = pz.qt * kGaBM;
-        const int xq = g * kGaD, xk = a.GD + g * kGaD, xv = 2 * a.GD + g * kGaD;   // columns in [Q' | K' | V']
-        ok = mbar_wait(q_empty, (pc & 1) ^ 1);       // the previous piece's last Q K^T has read Q
-        if (!ok) break;
-        mbar_arrive_expect_tx(q_full, C::kParts * kGaTile);
+      // Pair i of the piece, pair u of the segment; columns of [Q' | K' | V']: g D, GD + g D, 2 GD + g D.  With the first pair
+      // of a piece comes its Q, in slices of the same shape: slice s of the scores needs no more of Q than slices 0 .. s.
+      auto load_k = [&](int u, int i, int pc) -> bool {
+        const int y = (pz.kv_begin + 2 * i) * kGaBN;
+        if (i == 0 && !mbar_wait(q_empty, (pc & 1) ^ 1)) return false;      // the previous piece's last Q K^T has read Q
+#pragma unroll
+        for (int s = 0; s < C::kSlices; ++s) {
+          if (!mbar_wait(&k_empty[s], (u & 1) ^ 1)) return false;
+          mbar_arrive_expect_tx(&k_full[s], i == 0 ? 2 * C::kSliceBytes : C::kSliceBytes);
+          const int col = pz.g * kGaD + (kGaD == 64 ? 0 : s * 64);
+#pragma unroll
+          for (int x = 0; x < C::kSliceParts; ++x) {
+            if (i == 0)
+              tma_load_3d(kGaD == 64 ? sQ + s * kGaTile : sQ + x * kGaTile + s * kGaPanel, &tm.q[kGaD == 64 ? s : x], &k_full[s], col,
+                          pz.qt * kGaBM, pz.b);
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+              tma_load_3d(sK + s * C::kSliceBytes + x * kGaPanel + r * kGaKvPanel, &tm.kv[kGaD == 64 ? C::kParts - 1 - s : x],
+                          &k_full[s], a.GD + col, y + r * kGaBN, pz.b);
+          }
+        }
+        return true;
+      };
+      auto load_v = [&](int t, int b, int x, int y) -> bool {
+        const int st = t & 1;
+        if (!mbar_wait(&v_empty[st], ((t >> 1) & 1) ^ 1)) return false;
+        mbar_arrive_expect_tx(&v_full[st], kGaKvStage);
 #pragma unroll
         for (int i = 0; i < C::kParts; ++i)
 #pragma unroll
           for (int p = 0; p < C::kPanels; ++p)
-            tma_load_3d(sQ + i * kGaTile + p * kGaPanel, &tm.q[i], q_full, xq + p * 64, j0, b);
-        auto load_kv = [&](uint8_t *dst, uint64_t *bar, int xc, int y) {
-          mbar_arrive_expect_tx(bar, kGaKvStage);
-#pragma unroll
-          for (int i = 0; i < C::kParts; ++i)
-#pragma unroll
-            for (int p = 0; p < C::kPanels; ++p)
-              tma_load_3d(dst + i * kGaKvTile + p * kGaKvPanel, &tm.kv[i], bar, xc + p * 64, y, b);
-        };
-        for (int i = 0; i < pz.n_kv; ++i, ++t) {
-          const int st = t & 1;
-          const uint32_t ph = (t >> 1) & 1;
-          const int y = (pz.kv_begin + i) * kGaBN;
-          if (!mbar_wait(&k_empty[st], ph ^ 1)) { ok = false; break; }
-          load_kv(sK + st * kGaKvStage, &k_full[st], xk, y);
-          if (!mbar_wait(&v_empty[st], ph ^ 1)) { ok = false; break; }
-          load_kv(sV + st * kGaKvStage, &v_full[st], xv, y);
+            tma_load_3d(sV + st * kGaKvStage + i * kGaKvTile + p * kGaKvPanel, &tm.kv[i], &v_full[st], x + p * 64, y, b);
+        return true;
+      };
+      // in the order in which the buffers become free: K of pair u + 1 (with Q where a piece begins), then the V tiles of pair u
+      // (those of the first pair at once)
+      bool more = ga_next(a, walk, pz), ok = more && load_k(0, 0, 0);
+      for (int pc = 1; ok && more; ++pc) {
+        const int pairs = pz.n_kv / 2, b = pz.b, xv = 2 * a.GD + pz.g * kGaD, kv_begin = pz.kv_begin;
+        for (int i = 0; i < pairs && ok; ++i, t += 2) {
+          const int y = (kv_begin + 2 * i) * kGaBN;
+          if (t == 0) ok = load_v(0, b, xv, y) && load_v(1, b, xv, y + kGaBN);
+          if (i + 1 < pairs) ok = ok && load_k((t >> 1) + 1, i + 1, pc);
+          else if ((more = ga_next(a, walk, pz))) ok = ok && load_k((t >> 1) + 1, 0, pc);
+          if (t != 0) ok = ok && load_v(t, b, xv, y) && load_v(t + 1, b, xv, y + kGaBN);
         }
       }
     }
   } else if (warp == 1) {
     // every lane runs the control flow (operands stay warp-uniform); one elected lane issues
-    constexpr uint32_t idesc_qk = idesc_bf16_f32(kGaBM, kGaBN, false, false);
+    constexpr uint32_t idesc_qk = idesc_bf16_f32(kGaBM, 2 * kGaBN, false, false);
     constexpr uint32_t idesc_pv = idesc_bf16_f32(kGaBM, kGaD, false, true);
     const uint64_t dq = desc_kmajor_sw128(smem_u32(sQ)), dk = desc_kmajor_sw128(smem_u32(sK));
     const uint64_t dv = desc_mnmajor_sw128(smem_u32(sV), kGaKvPanel);
     const uint32_t q_lo = (uint32_t)dq, q_hi = (uint32_t)(dq >> 32);
     const uint32_t k_lo = (uint32_t)dk, k_hi = (uint32_t)(dk >> 32);
     const uint32_t v_lo = (uint32_t)dv, v_hi = (uint32_t)(dv >> 32);
-    auto issue_qk = [&](int t, bool last) -> bool {   // t: tile number across the pieces
-      const int st = t & 1;
-      if (!mbar_wait(&k_full[st], (t >> 1) & 1)) return false;
-      tc_fence_after_sync();
-      const uint32_t d = tmem + kGaColS + st * 128;
-      const uint32_t kb = k_lo + ((st * kGaKvStage) >> 4);
-      if (elect_one()) {
+    auto issue_qk = [&](int u, bool last) -> bool {   // u: pair number across the pieces
+      const uint32_t d = tmem + kGaColS + (u & 1) * 128;
 #pragma unroll
-        for (int t = 0; t < C::kProducts; ++t) {
-          const uint32_t qa = q_lo + ((C::first(t) * kGaTile) >> 4), ka = kb + ((C::second(t) * kGaKvTile) >> 4);
+      for (int s = 0; s < C::kSlices; ++s) {
+        if (!mbar_wait(&k_full[s], u & 1)) return false;
+        tc_fence_after_sync();
+        if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < kGaD / 16; ++k)
-            mma_ss_lohi(d, qa + (((k >> 2) * kGaPanel + (k & 3) * 32) >> 4), q_hi,
-                        ka + (((k >> 2) * kGaKvPanel + (k & 3) * 32) >> 4), k_hi, idesc_qk, (t | k) != 0);
+          for (int t = 0; t < C::kProducts; ++t) {
+            if (kGaD == 64 && C::second(t) != C::kParts - 1 - s) continue;
+            const uint32_t qa = q_lo + ((C::first(t) * kGaTile + (kGaD == 64 ? 0 : s * kGaPanel)) >> 4);
+            const uint32_t ka = k_lo + ((s * C::kSliceBytes + (kGaD == 64 ? 0 : C::second(t) * kGaPanel)) >> 4);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)               // a panel is 64 columns
+              mma_ss_lohi(d, qa + ((k * 32) >> 4), q_hi, ka + ((k * 32) >> 4), k_hi, idesc_qk,
+                          s != 0 || k != 0 || (kGaD != 64 && t != 0));
+          }
+          mma_commit(&k_empty[s]);
+          if (s + 1 == C::kSlices) {
+            mma_commit(&s_full[u & 1]);
+            if (last) mma_commit(q_empty);            // Q may be replaced by the next piece's
+          }
         }
-        mma_commit(&k_empty[st]);
-        mma_commit(&s_full[st]);
-        if (last) mma_commit(q_empty);               // Q may be replaced by the next piece's
+        __syncwarp();
       }
-      __syncwarp();
       return true;
     };
-    bool ok = true;
-    int t0 = 0;                                      // tile number of the piece's first tile
-    for (int pc = 0; ok && ga_next(a, walk, pz); ++pc) {
-      const int n_kv = pz.n_kv;
-      ok = mbar_wait(q_full, pc & 1);
-      ok = ok && issue_qk(t0, n_kv == 1);
-      for (int i = 0; i < n_kv && ok; ++i) {
-      const int t = t0 + i;
-      if (i + 1 < n_kv) ok = issue_qk(t + 1, i + 2 == n_kv);
-      if (!ok) break;
+    auto issue_pv = [&](int t, bool first) -> bool {  // first: of its piece
       const int st = t & 1;
-      if (!mbar_wait(&p_ready[t & 1], (t >> 1) & 1)) { ok = false; break; }
-      if (!mbar_wait(&v_full[st], (t >> 1) & 1)) { ok = false; break; }
-      // the first P V of a piece overwrites O: the previous piece's epilogue must have read it
-      if (i == 0 && pc > 0 && !mbar_wait(o_free, (pc - 1) & 1)) { ok = false; break; }
+      if (!mbar_wait(&p_ready[st], (t >> 1) & 1)) return false;
+      if (!mbar_wait(&v_full[st], (t >> 1) & 1)) return false;
       tc_fence_after_sync();
       const uint32_t vb = v_lo + ((st * kGaKvStage) >> 4);
       if (elect_one()) {
@@ -341,14 +363,31 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
           const uint32_t va = vb + ((C::second(t) * kGaKvTile) >> 4);
 #pragma unroll
           for (int k = 0; k < kGaBN / 16; ++k)
-            mma_ts_lohi(tmem + C::kColO, pa + k * 8, va + ((k * 2048) >> 4), v_hi, idesc_pv, (i | t | k) != 0);
+            mma_ts_lohi(tmem + C::kColO, pa + k * 8, va + ((k * 2048) >> 4), v_hi, idesc_pv, !first || (t | k) != 0);
         }
         mma_commit(&v_empty[st]);
         mma_commit(&pv_done[st]);
       }
       __syncwarp();
+      return true;
+    };
+    // The scores of a pair ahead of the two P V of the pair before; those of a piece's first pair behind the piece before
+    // (between its last two P V, its Q is awaited too early: 4096 tokens 99.3 us against 96.6).  One place in the code for
+    // each: the loops stay small beside the softmax warps' code.
+    bool ok = true;
+    int u0 = 0;                                      // number of the piece's first pair
+    for (int pc = 0; ok && ga_next(a, walk, pz); ++pc) {
+      const int pairs = pz.n_kv / 2;
+#pragma unroll 1
+      for (int i = -1; i < pairs && ok; ++i) {
+        if (i + 1 < pairs) ok = issue_qk(u0 + i + 1, i + 2 == pairs);
+        if (i < 0) continue;
+        // the first P V of a piece overwrites O: the previous piece's epilogue must have read it
+        if (i == 0 && pc > 0) ok = ok && mbar_wait(o_free, (pc - 1) & 1);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) ok = ok && issue_pv(2 * (u0 + i) + h, i == 0 && h == 0);
       }
-      t0 += n_kv;
+      u0 += pairs;
     }
   } else {
     const int quad = warp & 3;
@@ -368,10 +407,10 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
     float m = -INFINITY, l = 0.f;
     for (int i = 0; i < n_kv && ok; ++i) {
       const int t = t0 + i;
-      ok = mbar_wait(&s_full[t & 1], (t >> 1) & 1);
+      ok = mbar_wait(&s_full[(t >> 1) & 1], (t >> 2) & 1);
       if (!ok) break;
       tc_fence_after_sync();
-      const uint32_t tS = tm_lane + kGaColS + (t & 1) * 128;
+      const uint32_t tS = tm_lane + kGaColS + ((t >> 1) & 1) * 128 + (t & 1) * kGaBN;
       const int nvalid = min(max(bound - (kv_begin + i) * kGaBN, 0), kGaBN);
       const bool full = nvalid >= kGaBN;
 
@@ -382,15 +421,17 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
         for (int e = 0; e < kGaBN; ++e)
           if (e >= nvalid) r[e] = 0xff800000u;        // -inf: weight 0 below
       }
+      // eight independent chains, two elements per instruction
       float mx[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) mx[q] = __uint_as_float(r[q]);
+      for (int q = 0; q < 8; ++q) mx[q] = max3_f32(__uint_as_float(r[q]), __uint_as_float(r[q + 8]), __uint_as_float(r[q + 16]));
 #pragma unroll
-      for (int e = 8; e < kGaBN; e += 8)
+      for (int e = 24; e + 8 < kGaBN; e += 16)
 #pragma unroll
-        for (int q = 0; q < 8; ++q) mx[q] = fmaxf(mx[q], __uint_as_float(r[e + q]));
-      float tmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
-                         fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
+        for (int q = 0; q < 8; ++q) mx[q] = max3_f32(mx[q], __uint_as_float(r[e + q]), __uint_as_float(r[e + q + 8]));
+#pragma unroll
+      for (int q = 0; q < 8; ++q) mx[q] = fmaxf(mx[q], __uint_as_float(r[kGaBN - 8 + q]));
+      float tmax = max3_f32(max3_f32(mx[0], mx[1], mx[2]), max3_f32(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
       tmax *= a.scale_log2;
       // The first tile of a piece holds a key visible to every row (key 0, or a tile wholly before
       // the query tile; the list has no tiles of padding).  m = -inf after it takes scores of -inf, out of
@@ -425,15 +466,18 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
         tc_fence_after_sync();
       }
 
-      float rs[4] = {0.f, 0.f, 0.f, 0.f};
+      float rs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int c = 0; c < kGaBN / 16; ++c) {
         uint32_t pk[C::kParts][8];
 #pragma unroll
         for (int e = 0; e < 16; e += 2) {
-          float p0 = fast_exp2(fmaf(__uint_as_float(r[c * 16 + e]), a.scale_log2, -m_exp));
-          float p1 = fast_exp2(fmaf(__uint_as_float(r[c * 16 + e + 1]), a.scale_log2, -m_exp));
-          rs[(e >> 1) & 3] += p0 + p1;
+          float x0, x1;
+          fma_f32x2(x0, x1, __uint_as_float(r[c * 16 + e]), __uint_as_float(r[c * 16 + e + 1]), a.scale_log2,
+                    a.scale_log2, -m_exp, -m_exp);
+          float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+          const int k = ((e >> 1) & 3) * 2;
+          add_f32x2(rs[k], rs[k + 1], rs[k], rs[k + 1], p0, p1);
 #pragma unroll
           for (int i = 0; i + 1 < C::kParts; ++i) pk[i][e >> 1] = take_bf16x2(p0, p1);
           pk[C::kParts - 1][e >> 1] = pack_bf16x2(p0, p1);
@@ -442,8 +486,7 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
         for (int i = 0; i < C::kParts; ++i)
           tmem_st_x8(tm_lane + C::kColP + i * 64 + (t & 1) * (kGaBN / 2) + c * 8, pk[i]);
       }
-      const float rowsum = (rs[0] + rs[1]) + (rs[2] + rs[3]);
-      l += rowsum;
+      l += ((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7]));
       m = m_new;
       tmem_st_wait();
       tc_fence_before_sync();
