@@ -48,7 +48,7 @@ def test_lengths_at_the_edges_of_blocks(D, h, hk):
     (24, 32, 8, 64, 300), (20, 32, 8, 128, 700),         # one and two: what one wave holds
     (12, 16, 8, 128, 400), (60, 8, 8, 128, 2100),        # four: by the wave, by the rows per CTA
     (9, 18, 9, 64, 4200),                                # eight, by the rows per CTA
-    (1, 8, 8, 128, 8300), (1, 64, 4, 64, 8300),          # eight, few slabs of very many rows
+    (1, 8, 8, 128, 8300), (1, 64, 4, 64, 8300),          # sixteen, few slabs of very many rows
     (2, 40, 8, 128, 8300), (1, 128, 8, 64, 8300),        # the same with more than 64 query heads: the split form
     (5, 18, 1, 128, 300), (3, 34, 1, 64, 300),           # more than 16 heads per slab, more than 64 in all: the split form
 ])
