@@ -17,7 +17,8 @@
 // first), so that the next pair's arrive while the rest of the scores and two P V run.
 // Gate call, scores of one tile at a time | of pairs, us: 4 heads of 128, 333 tokens 31.0 | 31.0, 1500 50.1 | 48.6, 4096 102.3 |
 // 95.7, 8192 265 | 247, 4 x 1999 155 | 149; 4 heads of 64, 4 x 1500 65.0 | 60.1, 8192 205 | 175.  A pair takes 3,072
-// cycles of the tensor cores, which were busy 51 % of the time at 4096 tokens and are 60 %.  (The first tile's scores on their own, as a branch of the issuing warp: 8192 of 64 175 -> 213.)
+// cycles of the tensor cores, which were busy 51 % of the time at 4096 tokens and are 60 %.  (The first tile's
+// scores on their own, as a branch of the issuing warp: 8192 tokens of 64-wide heads 175 -> 213.)
 //
 // Work is the list of all (query tile, key tile) steps, query tiles in order
 // and each one's key tiles in order.  The list is cut into equal segments, one
