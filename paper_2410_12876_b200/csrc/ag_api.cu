@@ -1,5 +1,6 @@
 // C boundary of the AG-gated attention layer: argument checks and dispatch.
 // Every check that can be made on the host is made here, before any launch.
+#include <cuda.h>
 #include <math.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -8,6 +9,18 @@
 namespace ag {
 static thread_local int g_last_cuda_error = 0;
 void set_last_cuda_error(int e) { g_last_cuda_error = e; }
+
+unsigned long long current_context() {
+  using GetId = CUresult (*)(CUcontext, unsigned long long *);
+  static const GetId get_id = [] {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const cudaError_t e = cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q);
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<GetId>(p) : nullptr;
+  }();
+  unsigned long long id = 0;
+  return get_id && get_id(nullptr, &id) == CUDA_SUCCESS ? id : 0;      // (NULL: the current one)
+}
 
 static bool dim_ok(int d) { return d == 64 || d == 128; }
 

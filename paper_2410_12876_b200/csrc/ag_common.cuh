@@ -10,6 +10,8 @@ namespace ag {
 
 // ---------------------------------------------------------------- host side
 void set_last_cuda_error(int e);
+// The calling thread's CUDA context by its number, which no other context of the process ever has; 0: none yet, or not known.
+unsigned long long current_context();
 
 #define AG_CUDA_TRY(expr)                                 \
   do {                                                    \

@@ -20,13 +20,13 @@
 
 #include "ag_common.cuh"
 #include "decode_mma_core.cuh"
+#include "launch_rules.cuh"
 
 namespace ag {
 
 constexpr int kMaxSplits = 32;     // chunks per slab the workspace is sized for
 constexpr int kPartThreads = 256;
 constexpr int kUnroll = 8;         // rows in flight per lane group (x2: K and V)
-constexpr int kClusterMaxSlabs = 64;    // float32, and groups of more than 16 heads: up to here one cluster per slab
 constexpr int kClusterThreads = 512;    // float32 cluster form: 128 rows in flight per CTA (D = 128)
 
 // Grouped-query attention: slab s = (sequence, query head) of q and o reads the cache slab, k_new
@@ -439,8 +439,6 @@ decode_combine_kernel(const T *q, const T *k_new,
 // triples through distributed shared memory, adds the self term and writes the output.  The
 // second barrier keeps every CTA's shared memory alive until it has been read.  No CTA leaves
 // early: the cluster barriers need all of them.
-constexpr int kClusterSize = 8;
-constexpr int kWideCluster = 16, kWideMaxSlabs = 16;    // bf16, few slabs of many rows (see decode_ctas)
 //
 // kCtas = 1: a cluster of one, for caches that one CTA streams in a round or two (its barriers are the CTA's own).
 template <typename T, int D, int kThreads, int kCtas>
@@ -706,27 +704,55 @@ decode_cluster_mma_kernel(const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
   }
 }
 
+template <int D, int kMaxG, int kCtas>
+static cudaLaunchConfig_t cluster_mma_config(int groups, cudaStream_t st, cudaLaunchAttribute *attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCtas, groups);
+  cfg.blockDim = dim3(kGqThreads);
+  cfg.dynamicSmemBytes = gq_smem_bytes(D, kCmStages);
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1] = pdl_attribute();
+  cfg.attrs = kCtas == 1 ? attr + 1 : attr;
+  cfg.numAttrs = kCtas == 1 ? 1 : 2;
+  return cfg;
+}
+
+// Clusters of kWideCluster CTAs that the device holds at once, 0 where it cannot place one (the size is not portable: part of
+// a device, or a context with few SMs).  Asked for once per thread and context, and the kernel's attributes are set then.
+template <int D, int kMaxG>
+static int wide_clusters_at_once() {
+  struct Answer { unsigned long long context; int clusters; };
+  static thread_local Answer known[8] = {};
+  const unsigned long long context = current_context();
+  Answer &a = known[context % 8];
+  if (context == 0 || a.context != context) {
+    auto kern = decode_cluster_mma_kernel<D, kMaxG, kWideCluster>;
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_mma_config<D, kMaxG, kWideCluster>(1, nullptr, attr);
+    a.clusters = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&a.clusters, kern, &cfg) != cudaSuccess) {
+      a.clusters = 0;
+      (void)cudaGetLastError();
+    }
+    a.context = context;
+  }
+  return a.clusters;
+}
+
 // groups: clusters (runs of G query slabs on one key/value slab each)
 template <int D, int kMaxG, int kCtas>
 static int launch_decode_cluster_mma(int groups, int G, const void *q, const void *k_new, const void *v_new,
                                      const ag_cache &c, float scale_log2, void *o, const AppendArgs &ap,
                                      const HeadMap &hm, const RecentRing &rg, cudaStream_t st) {
   using T = __nv_bfloat16;
-  constexpr int smem = gq_smem_bytes(D, kCmStages);
-  if constexpr (kCtas > kClusterSize)
-    AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG, kCtas>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kCtas, groups);
-  cfg.blockDim = dim3(kGqThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
+  if constexpr (kCtas <= kClusterSize)               // (the wide ones': wide_clusters_at_once)
+    AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq_smem_bytes(D, kCmStages)));
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  attr[1] = pdl_attribute();
-  cfg.attrs = kCtas == 1 ? attr + 1 : attr;
-  cfg.numAttrs = kCtas == 1 ? 1 : 2;
+  const cudaLaunchConfig_t cfg = cluster_mma_config<D, kMaxG, kCtas>(groups, st, attr);
   AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_cluster_mma_kernel<D, kMaxG, kCtas>, static_cast<const T *>(q),
                                  static_cast<const T *>(k_new), static_cast<const T *>(v_new),
                                  static_cast<const T *>(c.k_rows), static_cast<const T *>(c.v_rows),
@@ -760,38 +786,6 @@ size_t decode_workspace_bytes(const ag_layer_desc &d) {
   return align_up(slabs * kMaxSplits * (d.head_dim + 2) * sizeof(float), 256);
 }
 
-// CTAs per slab of the bf16 cluster form for groups of G heads; 0: the split form.  From a sweep over 8 .. 1024 slabs of 100 ..
-// 16,000 rows, head_dim 64 and 128 (us per step, CTAs per slab 1 | 2 | 4 | 8, split form last; "of" a capacity: 1 - 3 % full):
-//   32 slabs, cap 130      2.9 | 3.4 | 3.5 | 3.7,  5.3     64 slabs, cap 800   7.2 | 6.1 | 5.5 | 7.7,  7.5
-//   128 slabs, cap 1600    14.5 | 11.4 | 12.1 | 14.2,  13.7    384 slabs, cap 400   7.5 | 10.7 | 16.0 | 28,  12.3
-//   640 slabs, cap 3200    109 | 105 | 104 | 110,  113      1024 slabs, cap 6550   336 | 326 | 321 | 321,  343
-//   512 slabs, cap 12,800  351 | 328 | 318 | 314,  334      512 of 8000  7.8 | 12.4 | 18.8 | 35.9,  30.1
-//   320 slabs of 64, cap 560   7.4 | 9.1 | 11.0 | 16.7,  14.3    1024 of 64, cap 4800   132 | 126 | 124 | 132,  155
-//   64 slabs, 16 heads, cap 1600   22.4 | 16.7 | 12.3 | 20.1,  24.1    192, 16 heads, cap 6400   92 | 86 | 79 | 93,  106
-//   256 slabs, 4 heads, cap 6550   97 | 97 | 89 | 87,  95     8 slabs, cap 13,107 (without the low weights)   79 | 42 | 23 | 13.4,  11.5
-// While a step waits for latency: as many CTAs per slab as one wave holds (the registers allow 3 per SM at 128, 2 with more
-// than 8 heads; 4 and 3 at 64), unless the slab has too few rows for them.  Where it waits for HBM: 1024 rows per CTA or fewer,
-// so that long slabs do not end alone, but of eight CTAs no more than five waves: slabs may hold far less than their capacity.
-// Only few slabs of very many rows need more CTAs than a cluster has, and only with more than kClusterMaxSlabs query slabs
-// (query_slabs) may they have them: up to there the scratch stays untouched, which callers without scratch of their own count on.
-template <int D>
-static int decode_ctas(int slabs, int query_slabs, int G, int max_cap) {
-  constexpr int kSms = 148;
-  const int wave_ctas = kSms * (D == 128 ? (G <= 8 ? 3 : 2) : (G <= 8 ? 4 : 3));
-  if (query_slabs > kClusterMaxSlabs && slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
-  // A cluster of sixteen takes its place later and merges more triples, but streams a long slab in half the time.  Up to
-  // sixteen of them run at once (24 and more wait for one another: 8.0 -> 10.1 us).  us per step, 8 | 16 CTAs per slab:
-  //   4 slabs   cap 2200 4.35 | 3.88, 6400 7.54 | 5.40     8 slabs, 4 heads   1200 4.74 | 4.90, 2200 5.30 | 5.28, 3300 6.04 | 5.75, 6400 8.24 | 7.07
-  //   16 slabs   2200 5.07 | 4.90, 6400 8.61 | 7.29     16 slabs, 4 heads   2200 5.65 | 5.90, 3300 6.56 | 6.56, 6400 9.12 | 8.31
-  //   2 slabs, 16 heads   480 7.34 | 5.66, 2200 7.61 | 6.16, 6400 11.8 | 8.37
-  if (slabs <= kWideMaxSlabs && max_cap > (G > 8 ? 512 : slabs * 2 <= kWideMaxSlabs ? 2048 : 4096)) return kWideCluster;
-  int wave = max_cap <= 128 ? 1 : max_cap <= 512 ? 4 : kClusterSize;
-  while (wave > 1 && (int64_t)slabs * wave > wave_ctas) wave /= 2;
-  if (wave == 2 && max_cap <= 512) wave = 1;
-  const int rows = max_cap <= 2048 ? 1 : max_cap <= 4096 || (int64_t)slabs * kClusterSize > 5 * wave_ctas ? 4 : kClusterSize;
-  return wave > rows ? wave : rows;
-}
-
 // Whether the kernels a decode step takes can carry the append: whichever CTA or cluster appends to a slab has to be the
 // only one that reads it.  Not so where query heads that share a slab go to clusters of their own, or are more than a CTA
 // of the merge takes at once.
@@ -800,8 +794,7 @@ static bool decode_carries_append(const ag_layer_desc &d, const ag_cache &c) {
   if (group == 1) return true;
   const bool grouped = d.dtype == AG_BF16 && group <= kGqMaxGroup;        // one cluster per key/value slab
   if (slabs <= kClusterMaxSlabs) return grouped;
-  const int ctas = !grouped ? 0 : d.head_dim == 64 ? decode_ctas<64>(slabs / group, slabs, group, c.max_cap)
-                                                   : decode_ctas<128>(slabs / group, slabs, group, c.max_cap);
+  const int ctas = !grouped ? 0 : decode_ctas(d.head_dim, slabs / group, slabs, group, c.max_cap, 0);
   return ctas > 0 || group <= combine_heads(d.head_dim);
 }
 
@@ -822,7 +815,9 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     };
     const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
     // (clusters of one query head each never carry the append: see decode_carries_append)
-    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas<D>(n, slabs, G, c.max_cap) : 0) {
+    const int wide = n > kWideMaxSlabs ? 0 : G == 1 ? wide_clusters_at_once<D, 1>() : G <= 4 ? wide_clusters_at_once<D, 4>() :
+                     G <= 8 ? wide_clusters_at_once<D, 8>() : wide_clusters_at_once<D, 16>();
+    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas(D, n, slabs, G, c.max_cap, wide) : 0) {
       case 1: return cluster(std::integral_constant<int, 1>{}, n, G);
       case 2: return cluster(std::integral_constant<int, 2>{}, n, G);
       case 4: return cluster(std::integral_constant<int, 4>{}, n, G);
