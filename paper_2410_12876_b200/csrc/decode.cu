@@ -719,11 +719,13 @@ static cudaLaunchConfig_t cluster_mma_config(int groups, cudaStream_t st, cudaLa
   return cfg;
 }
 
-// Clusters of kWideCluster CTAs that the device holds at once, 0 where it cannot place one (the size is not portable: part of
-// a device, or a context with few SMs).  Asked for once per thread and context, and the kernel's attributes are set then.
+// Clusters of kWideCluster CTAs that the device holds at once, and of those without a shared SM; 0 where it cannot place one (the
+// size is not portable: part of a device, or a context with few SMs).  Asked for once per thread and context, and the
+// kernel's attributes are set then.
+struct WideClusters { int at_once, apart; };
 template <int D, int kMaxG>
-static int wide_clusters_at_once() {
-  struct Answer { unsigned long long context; int clusters; };
+static WideClusters wide_clusters() {
+  struct Answer { unsigned long long context; WideClusters wide; };
   static thread_local Answer known[8] = {};
   const unsigned long long context = current_context();
   Answer &a = known[context % 8];
@@ -731,16 +733,18 @@ static int wide_clusters_at_once() {
     auto kern = decode_cluster_mma_kernel<D, kMaxG, kWideCluster>;
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = cluster_mma_config<D, kMaxG, kWideCluster>(1, nullptr, attr);
-    a.clusters = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&a.clusters, kern, &cfg) != cudaSuccess) {
-      a.clusters = 0;
+    a.wide = {};
+    int n = 0, per_sm = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGqThreads, cfg.dynamicSmemBytes) == cudaSuccess && per_sm > 0)
+      a.wide = {n, n / per_sm};
+    else
       (void)cudaGetLastError();
-    }
     a.context = context;
   }
-  return a.clusters;
+  return a.wide;
 }
 
 // groups: clusters (runs of G query slabs on one key/value slab each)
@@ -749,7 +753,7 @@ static int launch_decode_cluster_mma(int groups, int G, const void *q, const voi
                                      const ag_cache &c, float scale_log2, void *o, const AppendArgs &ap,
                                      const HeadMap &hm, const RecentRing &rg, cudaStream_t st) {
   using T = __nv_bfloat16;
-  if constexpr (kCtas <= kClusterSize)               // (the wide ones': wide_clusters_at_once)
+  if constexpr (kCtas <= kClusterSize)               // (the wide ones': wide_clusters)
     AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq_smem_bytes(D, kCmStages)));
   cudaLaunchAttribute attr[2];
   const cudaLaunchConfig_t cfg = cluster_mma_config<D, kMaxG, kCtas>(groups, st, attr);
@@ -794,7 +798,7 @@ static bool decode_carries_append(const ag_layer_desc &d, const ag_cache &c) {
   if (group == 1) return true;
   const bool grouped = d.dtype == AG_BF16 && group <= kGqMaxGroup;        // one cluster per key/value slab
   if (slabs <= kClusterMaxSlabs) return grouped;
-  const int ctas = !grouped ? 0 : decode_ctas(d.head_dim, slabs / group, slabs, group, c.max_cap, 0);
+  const int ctas = !grouped ? 0 : decode_ctas(d.head_dim, slabs / group, slabs, group, c.max_cap, 0, 0);
   return ctas > 0 || group <= combine_heads(d.head_dim);
 }
 
@@ -815,9 +819,9 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     };
     const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
     // (clusters of one query head each never carry the append: see decode_carries_append)
-    const int wide = n > kWideMaxSlabs ? 0 : G == 1 ? wide_clusters_at_once<D, 1>() : G <= 4 ? wide_clusters_at_once<D, 4>() :
-                     G <= 8 ? wide_clusters_at_once<D, 8>() : wide_clusters_at_once<D, 16>();
-    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas(D, n, slabs, G, c.max_cap, wide) : 0) {
+    const WideClusters wide = n > kWideMaxSlabs ? WideClusters{} : G == 1 ? wide_clusters<D, 1>() : G <= 4 ? wide_clusters<D, 4>() :
+                              G <= 8 ? wide_clusters<D, 8>() : wide_clusters<D, 16>();
+    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas(D, n, slabs, G, c.max_cap, wide.at_once, wide.apart) : 0) {
       case 1: return cluster(std::integral_constant<int, 1>{}, n, G);
       case 2: return cluster(std::integral_constant<int, 2>{}, n, G);
       case 4: return cluster(std::integral_constant<int, 4>{}, n, G);

@@ -22,17 +22,27 @@ constexpr int kWideCluster = 16, kWideMaxSlabs = 16;    // bf16, few slabs of ma
 // so that long slabs do not end alone, but of eight CTAs no more than five waves: slabs may hold far less than their capacity.
 // Only few slabs of very many rows need more CTAs than a cluster has, and only with more than kClusterMaxSlabs query slabs
 // (query_slabs) may they have them: up to there the scratch stays untouched, which callers without scratch of their own count on.
-// wide_at_once: clusters of sixteen CTAs that the device holds at the same time (0: none; eight is the portable size).
-inline int decode_ctas(int D, int slabs, int query_slabs, int G, int max_cap, int wide_at_once) {
+// wide_at_once: clusters of sixteen CTAs that the device holds at the same time (0: none; eight is the portable size),
+// wide_apart: as many with no more than one CTA on any SM (7 on a B200, whatever the kernel).
+inline int decode_ctas(int D, int slabs, int query_slabs, int G, int max_cap, int wide_at_once, int wide_apart) {
   constexpr int kSms = 148;
   const int wave_ctas = kSms * (D == 128 ? (G <= 8 ? 3 : 2) : (G <= 8 ? 4 : 3));
   if (query_slabs > kClusterMaxSlabs && slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
-  // A cluster of sixteen takes its place later and merges more triples, but streams a long slab in half the time.  Never
-  // more of them than run at once (24 and more waited for one another: 8.0 -> 10.1 us).  us per step, 8 | 16 CTAs per slab:
-  //   4 slabs   cap 2200 4.35 | 3.88, 6400 7.54 | 5.40     8 slabs, 4 heads   1200 4.74 | 4.90, 2200 5.30 | 5.28, 3300 6.04 | 5.75, 6400 8.24 | 7.07
-  //   16 slabs   2200 5.07 | 4.90, 6400 8.61 | 7.29     16 slabs, 4 heads   2200 5.65 | 5.90, 3300 6.56 | 6.56, 6400 9.12 | 8.31
-  //   2 slabs, 16 heads   480 7.34 | 5.66, 2200 7.61 | 6.16, 6400 11.8 | 8.37
-  if (slabs <= wide_at_once && slabs <= kWideMaxSlabs && max_cap > (G > 8 ? 512 : slabs * 2 <= kWideMaxSlabs ? 2048 : 4096)) return kWideCluster;
+  // A cluster of sixteen takes its place later and merges more triples, but streams a long slab in half the time.  How full
+  // the cache is, is not known here.  What it costs beside a short cache depends on whether every cluster has sixteen SMs to
+  // itself (wide_apart of them do: one per GPC of 16 SMs or more).  us per step, 8 | 16 CTAs per slab, lengths 2 - 5 %, 15 - 30 %
+  // and 38 - 100 % of the capacity; steps with another kernel between them:
+  //   7 slabs   cap 2200 3.48 | 3.58 (2 - 5 %), 4400 4.26 | 3.90, 6.26 | 5.11      of 64   3.24 | 3.28, 3.74 | 3.53, 5.22 | 4.33
+  //   7 slabs, 8 heads   4.37 | 4.49, 5.21 | 4.89, 7.60 | 5.92      16 heads   6.13 | 5.84, 7.27 | 6.46, 10.4 | 7.95
+  //   8 slabs   3.40 | 3.71, 4.11 | 4.28, 6.44 | 5.28      4 heads   3.91 | 4.40, 4.73 | 4.96, 6.75 | 6.13      8 heads   4.42 | 5.04, 5.22 | 5.75, 7.57 | 6.99
+  //   16 slabs   3.59 | 4.21, 4.63 | 4.83, 6.75 | 6.36      4 heads   4.30 | 5.13, 5.29 | 5.93, 7.49 | 7.61      16 heads   7.49 | 13.6, 9.01 | 14.4, 12.2 | 17.4
+  // and back to back: 2 slabs, cap 600 3.02 | 3.12, 3.04 | 3.16, 3.36 | 3.10; 16 heads 5.72 | 5.32, 5.82 | 5.39, 6.23 | 5.46.
+  // Up to there, from 2048 rows of capacity (512 for more than 8 heads), they are taken: at most 3 % lost, up to 30 % gained.  Beyond
+  // it short caches lose 10 - 20 %, so only where a long one has far more to gain, with few heads (back to back, cap 13,000):
+  //   8 slabs   3.57 | 3.73, 5.96 | 5.41, 12.4 | 9.55      4 heads   4.07 | 4.56, 6.48 | 6.33, 12.9 | 10.4      8 heads   4.50 | 5.62, 7.06 | 7.68, 13.7 | 12.3
+  //   16 slabs   3.65 | 3.99, 6.46 | 6.01, 14.8 | 11.0      4 heads   4.40 | 5.00, 7.25 | 7.02, 15.3 | 12.0      of 64, 4 heads   3.65 | 3.98, 5.63 | 5.33, 11.1 | 8.81
+  if (slabs <= wide_apart ? max_cap > (G > 8 ? 512 : 2048) : slabs <= wide_at_once && slabs <= kWideMaxSlabs && G <= 4 && max_cap > 8192)
+    return kWideCluster;
   int wave = max_cap <= 128 ? 1 : max_cap <= 512 ? 4 : kClusterSize;
   while (wave > 1 && (int64_t)slabs * wave > wave_ctas) wave /= 2;
   if (wave == 2 && max_cap <= 512) wave = 1;
