@@ -1,6 +1,6 @@
-"""Decode of few slabs: a CTA asks for its first tile before the slab's length is known.  Lengths at the edges of a warp's
-16 rows, of a CTA's second tile (512 rows later) and of its third, with every row that was never written holding NaN;
-groups of 1, 8, 9 and 16 heads (one or two groups of 8 MMA columns)."""
+"""Decode of few slabs.  Lengths at the edges of a warp's 16 rows, of a CTA's second tile (512 rows later, or 1024 where
+sixteen CTAs share a slab) and of its third, with every row that was never written holding NaN; groups of 1, 4, 8, 9 and 16
+heads (one or two groups of 8 MMA columns)."""
 import numpy as np
 import pytest
 import torch
@@ -21,9 +21,9 @@ def _lib():
 
 
 @pytest.mark.parametrize("D,h,hk", [(128, 8, 8), (64, 8, 8), (128, 64, 8), (64, 128, 8), (128, 72, 8)])
-def test_lengths_at_the_edges_of_blocks(D, h, hk):
-    lens = np.array([1, 15, 16, 17, 527, 528, 1025, 1551])
-    shape = LayerShape(1, 1600, 64, h, D, 1, 64, "bf16", kv_heads=hk)
+def test_lengths_at_the_edges_of_blocks(D, h, hk, lens=(1, 15, 16, 17, 527, 528, 1025, 1551)):
+    lens = np.array(lens)
+    shape = LayerShape(1, int(lens.max()) + 49, 64, h, D, 1, 64, "bf16", kv_heads=hk)
     cache = ag.RaggedCache.allocate(shape, lens + 20, DEV)
     nan = float("nan")
     cache.k_rows.fill_(nan)
@@ -41,6 +41,11 @@ def test_lengths_at_the_edges_of_blocks(D, h, hk):
         T.check_close(T.f64(o), orc.decode_attention(T.f64(q), T.f64(kn), T.f64(vn), held), "bf16", f"step {step}")
     assert np.array_equal(cache.len.cpu().numpy(), lens + 2)
     assert int(status.item()) == 0 and ag.ag_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("D,h,hk", [(128, 7, 7), (64, 7, 7), (128, 28, 7), (64, 56, 7), (128, 63, 7), (64, 112, 7)])
+def test_lengths_at_the_edges_of_sixteen_blocks(D, h, hk):
+    test_lengths_at_the_edges_of_blocks(D, h, hk, lens=(16, 17, 1024, 1039, 1040, 1041, 2063))
 
 
 @pytest.mark.parametrize("B,h,hk,D,longest", [
@@ -79,11 +84,21 @@ def test_ctas_per_slab(B, h, hk, D, longest):
 
 
 @pytest.mark.parametrize("B,h,hk,D,longest", [
-    (1, 4, 4, 128, 2060), (2, 20, 4, 64, 2060),          # up to eight slabs, from 2048 rows
-    (4, 4, 4, 128, 4100), (2, 64, 8, 64, 4100),          # up to sixteen, from 4096
+    (1, 4, 4, 128, 2060), (2, 20, 4, 64, 2060),          # up to seven slabs, from 2048 rows; eight of five heads: eight CTAs
+    (4, 4, 4, 128, 4100), (2, 64, 8, 64, 4100),          # sixteen slabs, too few rows for it
     (1, 64, 4, 128, 520), (1, 48, 3, 64, 1040),          # 16 heads per slab, from 512; a second tile for one rank
 ])
 def test_sixteen_ctas_per_slab(B, h, hk, D, longest):
+    test_ctas_per_slab(B, h, hk, D, longest)
+
+
+@pytest.mark.parametrize("B,h,hk,D,longest", [
+    (4, 4, 4, 128, 8300), (4, 16, 4, 64, 8300), (1, 28, 7, 128, 2060),    # sixteen CTAs: up to 16 slabs beyond 8192 rows, seven
+    (20, 16, 1, 128, 1100), (9, 18, 2, 64, 1100),        # 16 and 9 heads, eight CTAs: two heads for a rank
+    (20, 16, 1, 128, 400), (17, 12, 1, 64, 500),         # four CTAs, four and three heads for a rank
+    (80, 16, 1, 128, 700), (120, 10, 1, 64, 700),        # two CTAs, eight and five
+])
+def test_heads_shared_among_ranks(B, h, hk, D, longest):
     test_ctas_per_slab(B, h, hk, D, longest)
 
 

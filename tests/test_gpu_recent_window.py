@@ -24,6 +24,9 @@ SHAPES = {
     # decode through the workspace: the merge reads the ring, and fills it where it carries the append (float32)
     "f32_many_slabs": LayerShape(17, 60, 128, 4, 64, 1, 64, "f32"),
     "f32_many_slabs_gqa": LayerShape(9, 60, 128, 16, 64, 2, 64, "f32", kv_heads=4),
+    # 16 heads per slab: two heads for a rank of eight CTAs, one for each of sixteen
+    "bf16_eight_ctas": LayerShape(4, 530, 128, 32, 64, 2, 64, "bf16", kv_heads=2),
+    "bf16_sixteen_ctas": LayerShape(1, 530, 128, 32, 128, 2, 64, "bf16", kv_heads=2),
     "bf16_group17": LayerShape(2, 140, 256, 34, 128, 2, 128, "bf16", kv_heads=2),
 }
 
