@@ -172,16 +172,22 @@ __device__ __forceinline__ void decode_stream_rows(const T *q, const T *k_rows,
     }
     m = m_new;
   };
-  // The trip count is the same for every thread of the CTA (the shuffles need whole warps).  A last round of few rows
+  // The trip counts are the same for every thread of the CTA (the shuffles need whole warps).  A last round of few rows
   // goes in a half or a quarter of a round's registers: the clamped rows' arithmetic was most of a short step.
-  // us per step, all rounds whole | so: 4 slabs of 64, 64 rows 3.49 | 2.69, 128 rows 3.52 | 2.93, 256 3.58 | 3.59, 500 4.75 | 4.84;
-  // 8 slabs of 128, 64 rows 3.29 | 2.64, 256 rows in clusters of eight 4.71 | 3.29; 128 tokens of a float32 layer with 16 steps 94.0 | 82.6.
-  // (Skipped row by row instead, full rounds lost: 256 rows of a 512-thread CTA 3.5 -> 3.9 us, 2 x 8 slabs of 500 5.3 -> 7.0.)
-  for (int r0 = r_begin; r0 < r_end; r0 += kUnroll * kGroups) {
-    if (r_end - r0 > kUnroll / 2 * kGroups) rows(std::integral_constant<int, kUnroll>{}, r0);
-    else if (r_end - r0 > kUnroll / 4 * kGroups) rows(std::integral_constant<int, kUnroll / 2>{}, r0);
-    else rows(std::integral_constant<int, kUnroll / 4>{}, r0);
+  // us per step, all rounds whole | so: 4 slabs of 64, 64 rows 3.49 | 2.57, 128 rows 3.50 | 2.87, 256 3.52 | 3.45, 500 4.70 | 4.55, 2000 4.55 | 4.35;
+  // 8 slabs of 128, 64 rows 3.28 | 2.66, 256 rows in clusters of eight 4.52 | 3.18, 2000 5.55 | 5.45, 16 of them 4000 11.9 | 11.9.
+  // (Skipped row by row instead, full rounds lost: 256 rows of a 512-thread CTA 3.5 -> 3.9 us, 2 x 8 slabs of 500 5.3 -> 7.0.
+  // The choice inside the loop of the full rounds cost those 1 - 5 %, and a chunk of the split form - whole rounds, but for a
+  // slab's last chunk - pays for any code behind its loop: 512 slabs of 128 with 4000 rows 315 -> 321.)
+  constexpr int kRound = kUnroll * kGroups;
+  int r0 = r_begin;
+  if (kThreads == kPartThreads && (r_end - r_begin) % kRound == 0) {
+    for (; r0 < r_end; r0 += kRound) rows(std::integral_constant<int, kUnroll>{}, r0);
+    return;
   }
+  for (; r_end - r0 > kRound / 2; r0 += kRound) rows(std::integral_constant<int, kUnroll>{}, r0);
+  if (r_end - r0 > kRound / 4) rows(std::integral_constant<int, kUnroll / 2>{}, r0);
+  else if (r0 < r_end) rows(std::integral_constant<int, kUnroll / 4>{}, r0);
 }
 
 template <typename T, int D>
@@ -442,7 +448,7 @@ decode_combine_kernel(const T *q, const T *k_new,
 //
 // kCtas = 1: a cluster of one, for caches that one CTA streams in a round or two (its barriers are the CTA's own).
 template <typename T, int D, int kThreads, int kCtas>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 decode_cluster_kernel(const T *q, const T *k_new, const T *v_new,
                       const T *k_rows, const T *v_rows,
                       const int64_t *row_off, const int32_t *len,

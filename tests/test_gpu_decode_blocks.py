@@ -103,12 +103,13 @@ def test_heads_shared_among_ranks(B, h, hk, D, longest):
 
 
 @pytest.mark.parametrize("D,extra", [(64, 2), (64, 400), (128, 2), (128, 400)])
-def test_float32_rounds(D, extra):
+def test_float32_rounds(D, extra, batch=1, threads=512):
     """The float32 form's last round of rows in a quarter, a half or all of its registers: 512 threads take 32 rows of 64 or 16
     of 128 at a time, eight times a round; one CTA per slab, and eight where the capacity asks for them."""
-    step = 512 * 4 // D
+    step = threads * 4 // D
     lens = np.array([0, 1, 2 * step - 1, 2 * step, 2 * step + 1, 4 * step, 4 * step + 1, 8 * step, 8 * step + 1, 10 * step + 1])
-    shape = LayerShape(1, 16 * step + 400, 64, lens.size, D, 1, 64, "f32")
+    shape = LayerShape(batch, 16 * step + 400, 64, lens.size, D, 1, 64, "f32")
+    lens = np.tile(lens, batch)
     cache = ag.RaggedCache.allocate(shape, lens + extra, DEV)
     cache.k_rows.copy_(inputs.randn(tuple(cache.k_rows.shape), 41, DEV, torch.float32))
     cache.v_rows.copy_(inputs.randn(tuple(cache.v_rows.shape), 42, DEV, torch.float32))
@@ -120,6 +121,12 @@ def test_float32_rounds(D, extra):
         o = T.gpu_decode_step(shape, q, kn, vn, fn, cache, status, fused=True)
         T.check_close(T.f64(o), orc.decode_attention(T.f64(q), T.f64(kn), T.f64(vn), held), "f32", f"step {t}")
     assert np.array_equal(cache.len.cpu().numpy(), lens + 2) and int(status.item()) == 0
+
+
+@pytest.mark.parametrize("D,extra", [(64, 2), (64, 400), (128, 2), (128, 400)])
+def test_float32_rounds_of_chunks(D, extra):
+    """The split form's chunks of 128 rows: 256 threads, whole rounds but for a slab's last chunk."""
+    test_float32_rounds(D, extra, batch=7, threads=256)
 
 
 @pytest.mark.parametrize("B,h,hk,D,dtype,longest,untouched", [
