@@ -16,7 +16,7 @@
 //   one CTA of six stages, all heads added up by one rank      11.1 | 21.7 | 14.7 | 16.4 | 24.8 | 49.6
 //   the heads shared among the ranks, one CTA of eight stages  6.5 | 12.2 | 11.7 | 16.2 | 25.9 | 53.0
 //   two of four stages                                         6.5 | 7.9 | 10.9 | 14.8 | 23.6 | 38.7
-//   three of three                                             6.4 | 7.9 | 11.2 | 13.6 | 21.7 | 34.6   (4.7 TB/s)
+//   three of three                                             6.4 | 7.9 | 11.2 | 13.6 | 21.7 | 34.6
 //   A = X      [B n, d]  row-major -> K-major operand, 128-byte swizzled rows
 //   B = W_lin  [d, h]    row-major -> MN-major operand: one panel of [64 k][64 n],
 //                                     columns past h filled with zeros by TMA
@@ -33,7 +33,7 @@ using namespace umma;
 namespace cg = cooperative_groups;
 
 constexpr int kGlBM = 128, kGlBK = 64, kGlThreads = 192, kGlStages = 3;
-constexpr int kGlCtasPerSm = 3, kGlMaxSplit = 8;
+constexpr int kGlCtasPerSm = 3;
 constexpr int kGlABytes = kGlBM * kGlBK * 2;              // 16 KB
 constexpr int kGlBBytes = kGlBK * 64 * 2;                 // one panel [64 k][64 n] = 8 KB
 constexpr int kGlStageBytes = kGlABytes + kGlBBytes;
@@ -48,11 +48,12 @@ struct GateLinearArgs {
   const float *gamma;
   float *scores;
   uint8_t *flags;
-  int M, n, h, kb_total, kb_per_cta;   // tokens, sequence length, heads, 64-wide k blocks in all / per CTA
+  int M, n, h, kb_total;               // tokens, sequence length, heads, 64-wide k blocks
   float logit_tau;
 };
 
-template <int N>   // MMA width: heads rounded up to 32
+// N: MMA width, heads rounded up to 32.  kRanks: CTAs of a tile's cluster.
+template <int N, int kRanks>
 __global__ void __launch_bounds__(kGlThreads, kGlCtasPerSm)
 gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                       const GateLinearArgs a) {
@@ -65,12 +66,12 @@ gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_full + 1);
 
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank(), nranks = (int)cluster.num_blocks();
+  const int rank = kRanks == 1 ? 0 : (int)cluster.block_rank();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * kGlBM;
-  const int kb_begin = rank * a.kb_per_cta;
+  const int kb_begin = rank * a.kb_total / kRanks, kb_end = (rank + 1) * a.kb_total / kRanks;
   // a tile that holds padding only: no scores to compute, flags 0
-  const int num_kb = padding_rows(a.seq_lens, a.n, m0, min(m0 + kGlBM, a.M), 1) ? 0 : max(0, min(a.kb_total, kb_begin + a.kb_per_cta) - kb_begin);
+  const int num_kb = padding_rows(a.seq_lens, a.n, m0, min(m0 + kGlBM, a.M), 1) ? 0 : kb_end - kb_begin;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kGlStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -127,8 +128,17 @@ gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     if (elect_one()) mma_commit(acc_full);   // accumulator complete (or unwinding)
     __syncwarp();
   } else {
-    // this CTA's partial sums: thread = token row, into shared memory as [col][row]
+    // thread = token row
     const int quad = warp & 3, r_in = quad * 32 + lane;
+    const int tok = m0 + r_in;
+    const int b = tok / a.n, t = tok % a.n;
+    const bool valid = tok < a.M;
+    const bool padding = valid && a.seq_lens && t >= a.seq_lens[b];
+    auto write = [&](int i, float s) {
+      const size_t o = ((size_t)b * a.h + i) * a.n + t;        // lanes = consecutive tokens: coalesced
+      if (a.scores) a.scores[o] = s;
+      a.flags[o] = !padding && (s + (a.gamma ? a.gamma[i] : 0.f)) > a.logit_tau ? 1 : 0;
+    };
     const bool ok = mbar_wait(acc_full, 0);
     tc_fence_after_sync();
 #pragma unroll
@@ -141,34 +151,41 @@ gate_linear_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         for (int e = 0; e < 32; ++e) r[e] = 0u;
       }
 #pragma unroll
-      for (int e = 0; e < 32; ++e) part[(c + e) * kGlBM + r_in] = __uint_as_float(r[e]);
+      for (int e = 0; e < 32; ++e) {
+        if constexpr (kRanks > 1) part[(c + e) * kGlBM + r_in] = __uint_as_float(r[e]);     // the CTA's partial sums, [col][row]
+        else if (valid && c + e < a.h) write(c + e, __uint_as_float(r[e]));
+      }
     }
-  }
-  cluster.sync();                       // every CTA's partial sums are in its shared memory
-  if (warp >= 2) {
-    // each CTA adds up, thresholds and writes its share of the heads: rank, rank + nranks, ...
-    const int quad = warp & 3, r_in = quad * 32 + lane;
-    const int tok = m0 + r_in;
-    if (tok < a.M) {
-      const int b = tok / a.n, t = tok % a.n;
-      const bool padding = a.seq_lens && t >= a.seq_lens[b];
-      const float *p[kGlMaxSplit];
+    if constexpr (kRanks > 1) {
+      cluster.sync();                   // every CTA's partial sums are in its shared memory
+      // Each CTA adds up, thresholds and writes its share of the heads: rank, rank + kRanks, ...
+      // (All eight ranks' places gone over whatever kRanks: 2 us of a call with one or two CTAs to a tile.)
+      constexpr int kAtOnce = kRanks == 2 ? 8 : 4;             // heads: 16 or 32 values per thread in flight
+      const float *p[kRanks];
 #pragma unroll
-      for (int rk = 0; rk < kGlMaxSplit; ++rk) p[rk] = cluster.map_shared_rank(part, rk < nranks ? rk : rank) + r_in;
-#pragma unroll 4
-      for (int i = rank; i < a.h; i += nranks) {
-        float x[kGlMaxSplit], s = 0.f;
+      for (int rk = 0; rk < kRanks; ++rk) p[rk] = cluster.map_shared_rank(part, rk) + r_in;
+#pragma unroll 1
+      for (int i0 = rank; valid && i0 < a.h; i0 += kAtOnce * kRanks) {
+        float x[kAtOnce][kRanks];
 #pragma unroll
-        for (int rk = 0; rk < kGlMaxSplit; ++rk) x[rk] = rk < nranks ? p[rk][i * kGlBM] : 0.f;
+        for (int u = 0; u < kAtOnce; ++u)
 #pragma unroll
-        for (int rk = 0; rk < kGlMaxSplit; ++rk) s += x[rk];   // rank order: the sum does not depend on timing
-        const size_t o = ((size_t)b * a.h + i) * a.n + t;      // lanes = consecutive tokens: coalesced
-        if (a.scores) a.scores[o] = s;
-        a.flags[o] = !padding && (s + (a.gamma ? a.gamma[i] : 0.f)) > a.logit_tau ? 1 : 0;
+          for (int rk = 0; rk < kRanks; ++rk) x[u][rk] = i0 + u * kRanks < a.h ? p[rk][(i0 + u * kRanks) * kGlBM] : 0.f;
+#pragma unroll
+        for (int u = 0; u < kAtOnce; ++u) {
+          float s = 0.f;
+#pragma unroll
+          for (int rk = 0; rk < kRanks; ++rk) s += x[u][rk];   // rank order: the sum does not depend on timing
+          if (i0 + u * kRanks < a.h) write(i0 + u * kRanks, s);
+        }
       }
     }
   }
-  cluster.sync();                       // partial sums stay alive until the first CTA has read them
+  if constexpr (kRanks > 1) {
+    __syncwarp();
+    if (warp < 2) cluster.sync();       // (the one above)
+    cluster.sync();                     // partial sums stay alive until every CTA has read them
+  }
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem_acc, kGlTmemCols);
@@ -214,10 +231,32 @@ gate_linear_simt_kernel(const T *__restrict__ X, const T *__restrict__ W, const 
   }
 }
 
+static cudaLaunchConfig_t gate_linear_config(int ranks, int m_tiles, cudaStream_t st, cudaLaunchAttribute *attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ranks, m_tiles);
+  cfg.blockDim = dim3(kGlThreads);
+  cfg.dynamicSmemBytes = kGlSmemBytes;
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ranks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1] = pdl_attribute();
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cfg;
+}
+
+template <int N, int kRanks>
+static int launch_gate_linear_tc(const CUtensorMap &tmX, const CUtensorMap &tmW, const GateLinearArgs &a, int m_tiles, cudaStream_t st) {
+  auto kern = gate_linear_tc_kernel<N, kRanks>;
+  AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGlSmemBytes));
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = gate_linear_config(kRanks, m_tiles, st, attr);
+  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tmX, tmW, a));
+  return AG_OK;
+}
+
 template <int N>
-static int run_gate_linear_tc(const ag_layer_desc &d, const void *X, const void *W, const GateLinearArgs &a0,
-                              cudaStream_t st) {
-  GateLinearArgs a = a0;
+static int run_gate_linear_tc(const ag_layer_desc &d, const void *X, const void *W, const GateLinearArgs &a, cudaStream_t st) {
   CUtensorMap tmX, tmW;
   int rc = make_tmap_2d_bf16(&tmX, X, a.M, d.hidden, (uint64_t)d.hidden * 2, kGlBM, kGlBK);
   if (rc) return rc;
@@ -227,23 +266,13 @@ static int run_gate_linear_tc(const ag_layer_desc &d, const void *X, const void 
   // of six of two CTAs per SM left a second wave at 47 tiles (20.2 us against 14.8 in four).
   const int m_tiles = (a.M + kGlBM - 1) / kGlBM;
   int split = 1;
-  while (split < kGlMaxSplit && m_tiles * split * 2 <= kGlCtasPerSm * 148 && a.kb_total / (split * 2) >= 4) split *= 2;
-  a.kb_per_cta = (a.kb_total + split - 1) / split;
-  auto kern = gate_linear_tc_kernel<N>;
-  AG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGlSmemBytes));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(split, m_tiles);
-  cfg.blockDim = dim3(kGlThreads);
-  cfg.dynamicSmemBytes = kGlSmemBytes;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  attr[1] = pdl_attribute();
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  AG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tmX, tmW, a));
-  return AG_OK;
+  while (split < 8 && m_tiles * split * 2 <= kGlCtasPerSm * 148 && a.kb_total / (split * 2) >= 4) split *= 2;
+  switch (split) {
+    case 1: return launch_gate_linear_tc<N, 1>(tmX, tmW, a, m_tiles, st);
+    case 2: return launch_gate_linear_tc<N, 2>(tmX, tmW, a, m_tiles, st);
+    case 4: return launch_gate_linear_tc<N, 4>(tmX, tmW, a, m_tiles, st);
+    default: return launch_gate_linear_tc<N, 8>(tmX, tmW, a, m_tiles, st);
+  }
 }
 
 int launch_gate_linear(const ag_layer_desc &d, const void *X, const void *W, const float *gamma,
@@ -251,7 +280,7 @@ int launch_gate_linear(const ag_layer_desc &d, const void *X, const void *W, con
   GateLinearArgs a;
   a.seq_lens = d.seq_lens; a.gamma = gamma; a.scores = scores; a.flags = flags;
   a.M = d.batch * d.seq; a.n = d.seq; a.h = kv_heads_of(d);
-  a.kb_total = (d.hidden + kGlBK - 1) / kGlBK; a.kb_per_cta = a.kb_total;
+  a.kb_total = (d.hidden + kGlBK - 1) / kGlBK;
   a.logit_tau = (float)log((double)d.tau / (1.0 - (double)d.tau));
   const bool tc = d.dtype == AG_BF16 && kv_heads_of(d) <= kGlMaxN && kv_heads_of(d) % 8 == 0 && d.hidden % 8 == 0 &&
                   (int64_t)d.batch * d.seq < ((int64_t)1 << 31) - kGlBM && (a.M + kGlBM - 1) / kGlBM <= 65535;

@@ -89,11 +89,38 @@ def test_linear_gate_rejects_bad_arguments():
 
 
 @pytest.mark.parametrize("batch,seq,hidden,heads", [
-    (1, 7040, 2048, 40), (1, 7041, 2048, 24),            # eight CTAs to a tile, four: what one wave holds
-    (2, 7111, 1032, 8), (1, 28417, 512, 16),             # two, one
-    (1, 129, 2048 + 8, 64),                              # the last k block alone with one rank
+    (1, 7040, 2048, 40), (1, 7041, 2048, 24),
+    (2, 7111, 1032, 8), (1, 28417, 512, 16),
+    (1, 129, 2048 + 8, 64),                              # 33 k blocks for eight CTAs
 ])
 def test_linear_gate_shares_of_a_cluster(batch, seq, hidden, heads):
     """Every number of CTAs a tile is shared by, heads that do not divide among them, a ragged last tile."""
     _run(LayerShape(batch, seq, hidden, heads, 128, 1, 64, "bf16"), 730)
+    assert ag.ag_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("batch,seq,hidden,heads,ctas", [
+    (1, 129, 520, 24, 8), (1, 7000, 512, 16, 4), (1, 20000, 512, 32, 2), (1, 30000, 256, 24, 1),      # up to 32 heads
+    (2, 129, 520, 40, 8), (1, 7000, 512, 56, 4), (1, 20000, 512, 64, 2), (1, 30000, 256, 40, 1),      # up to 64
+])
+def test_linear_gate_ctas_of_a_tile(batch, seq, hidden, heads, ctas):
+    """Each number of CTAs, in both widths of the MMA, heads that no CTA's trip divides."""
+    _run(LayerShape(batch, seq, hidden, heads, 128, 1, 64, "bf16"), 740 + ctas)
+    assert ag.ag_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("seq,ctas", [(300, 8), (3500, 4), (12000, 2), (25000, 1)])
+def test_linear_gate_of_a_padded_batch(seq, ctas):
+    """Tiles of padding among the others, whatever shares a tile: their flags are 0, the tokens' those of each sequence alone."""
+    shape = LayerShape(3, seq, 256 if ctas == 1 else 512, 16, 128, 1, 64, "bf16")
+    X, W = inputs.hidden_states(shape, 750, DEV), inputs.linear_gate_weight(shape, 751, DEV)
+    lens = [seq, 130, seq // 2]
+    flags = torch.full((3, 16, seq), 7, dtype=torch.uint8, device=DEV)
+    scores = torch.zeros(3, 16, seq, device=DEV)
+    ag.ag_gate_linear_forward(ag.make_desc(shape, torch.tensor(lens, dtype=torch.int32, device=DEV)), X, W, None, scores, flags)
+    for b, n in enumerate(lens):
+        s_ref, f_ref = orc.linear_gate(T.f64(X[b:b + 1, :n]), T.f64(W), None, float(np.float32(shape.tau)))
+        assert np.max(np.abs(T.f64(scores[b:b + 1, :, :n]) - s_ref)) < 1e-4
+        T.check_flags(shape.with_(batch=1, seq=n), flags[b:b + 1, :, :n].contiguous(), s_ref, np.ascontiguousarray(f_ref), None)
+        assert int(flags[b, :, n:].max().item() if n < seq else 0) == 0
     assert ag.ag_device_wait_timeouts() == 0
