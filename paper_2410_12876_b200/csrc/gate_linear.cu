@@ -17,6 +17,8 @@
 //   the heads shared among the ranks, one CTA of eight stages  6.5 | 12.2 | 11.7 | 16.2 | 25.9 | 53.0
 //   two of four stages                                         6.5 | 7.9 | 10.9 | 14.8 | 23.6 | 38.7
 //   three of three                                             6.4 | 7.9 | 11.2 | 13.6 | 21.7 | 34.6
+// and calls back to back, X in L2 where it fits: three of three 6.6 | 7.9 | 9.7 | 10.9 | 17.0 | 34.0; heads added up by loops of as many
+// ranks as there are, CTAs to a tile by gate_linear_split  5.8 | 7.3 | 9.4 | 10.5 | 15.5 | 31.0   (5.3 TB/s)
 //   A = X      [B n, d]  row-major -> K-major operand, 128-byte swizzled rows
 //   B = W_lin  [d, h]    row-major -> MN-major operand: one panel of [64 k][64 n],
 //                                     columns past h filled with zeros by TMA
@@ -25,6 +27,7 @@
 #include <math.h>
 
 #include "ag_common.cuh"
+#include "launch_rules.cuh"
 #include "umma.cuh"
 
 namespace ag {
@@ -231,6 +234,10 @@ gate_linear_simt_kernel(const T *__restrict__ X, const T *__restrict__ W, const 
   }
 }
 
+// How many clusters of a size the device holds at once is asked of a kernel of the same threads and shared memory: one that
+// allocates tensor memory is answered for as if a CTA took all of an SM's.
+__global__ void __launch_bounds__(kGlThreads, kGlCtasPerSm) gate_linear_place_kernel() {}
+
 static cudaLaunchConfig_t gate_linear_config(int ranks, int m_tiles, cudaStream_t st, cudaLaunchAttribute *attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ranks, m_tiles);
@@ -243,6 +250,25 @@ static cudaLaunchConfig_t gate_linear_config(int ranks, int m_tiles, cudaStream_
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   return cfg;
+}
+
+// Asked for once per thread and context.
+static int gate_linear_places(GateLinearPlaces *out) {
+  struct Answer { unsigned long long context; GateLinearPlaces places; };
+  static thread_local Answer known[8] = {};
+  const unsigned long long context = current_context();
+  Answer &a = known[context % 8];
+  if (context == 0 || a.context != context) {
+    AG_CUDA_TRY(cudaFuncSetAttribute(gate_linear_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGlSmemBytes));
+    for (int i = 0; i < kGlSplits; ++i) {
+      cudaLaunchAttribute attr[2];
+      const cudaLaunchConfig_t cfg = gate_linear_config(1 << i, 1, nullptr, attr);
+      AG_CUDA_TRY(cudaOccupancyMaxActiveClusters(&a.places.clusters[i], gate_linear_place_kernel, &cfg));
+    }
+    a.context = context;
+  }
+  *out = a.places;
+  return AG_OK;
 }
 
 template <int N, int kRanks>
@@ -262,12 +288,10 @@ static int run_gate_linear_tc(const ag_layer_desc &d, const void *X, const void 
   if (rc) return rc;
   rc = make_tmap_2d_bf16(&tmW, W, d.hidden, kv_heads_of(d), (uint64_t)kv_heads_of(d) * 2, kGlBK, 64);
   if (rc) return rc;
-  // Split d over a cluster while one wave holds all its CTAs and each has at least four k blocks.  Powers of two only: clusters
-  // of six of two CTAs per SM left a second wave at 47 tiles (20.2 us against 14.8 in four).
+  GateLinearPlaces places;
+  if ((rc = gate_linear_places(&places))) return rc;
   const int m_tiles = (a.M + kGlBM - 1) / kGlBM;
-  int split = 1;
-  while (split < 8 && m_tiles * split * 2 <= kGlCtasPerSm * 148 && a.kb_total / (split * 2) >= 4) split *= 2;
-  switch (split) {
+  switch (gate_linear_split(m_tiles, a.kb_total, a.h, places)) {
     case 1: return launch_gate_linear_tc<N, 1>(tmX, tmW, a, m_tiles, st);
     case 2: return launch_gate_linear_tc<N, 2>(tmX, tmW, a, m_tiles, st);
     case 4: return launch_gate_linear_tc<N, 4>(tmX, tmW, a, m_tiles, st);

@@ -50,4 +50,28 @@ inline int decode_ctas(int D, int slabs, int query_slabs, int G, int max_cap, in
   return wave > rows ? wave : rows;
 }
 
+// CTAs that share a tile of the local gate (128 tokens): 1, 2, 4 or 8, a cluster each.  `tiles` tiles of kb k-blocks of 64.
+// A wave of clusters takes as long as its CTAs' k-blocks, and their set-up and exchange as long as four to six more; every CTA costs the
+// device its turn; and rows of W of 16 bytes (8 heads) all lie in the few lines that every CTA of a rank asks for at the same time.
+// In units of a k-block (0.25 us), fitted to 340 sizes of 256 .. 4104 hidden, 8 .. 64 heads, 1 .. 1000 tiles: 1.5 % behind the best
+// number of CTAs on average, 23 % at most.  us for 1 | 2 | 4 | 8 CTAs, hidden 4096, 32 heads:
+//   8 tiles 18.0 | 11.1 | 7.6 | 5.9     49 18.6 | 12.1 | 10.4 | 13.2     105 29.3 | 23.1 | 28.0 | 29.7     250 49.6 | 55.2 | 54.0 | 61.7     480 100 | 91.9 | 93.9 | 108
+//   8 heads: 105 tiles 37.5 | 30.4 | 25.6 | 28.6     250 73.5 | 65.0 | 53.5 | 59.1     hidden 512, 8 heads: 400 32.0 | 24.5 | 28.9 | 40.1
+// (A device of 148 SMs holds 444, 222, 104 and 48 such clusters.  As many CTAs as places, whatever their clusters: 49 tiles took a
+// second wave of clusters of eight, 12.1 -> 15.2 us, 105 one of four, 23.1 -> 31.)
+constexpr int kGlSplits = 4;
+struct GateLinearPlaces { int clusters[kGlSplits]; };    // of 1, 2, 4, 8 CTAs that the device holds at once
+inline int gate_linear_split(int tiles, int kb, int heads, const GateLinearPlaces &places) {
+  int best = 1;
+  double best_cost = 0.;
+  for (int i = 0; i < kGlSplits; ++i) {
+    const int s = 1 << i, at_once = places.clusters[i];
+    if (i > 0 && (at_once <= 0 || kb < s)) break;
+    const int waves = at_once > 0 ? (tiles + at_once - 1) / at_once : 1;
+    const double cost = waves * ((kb + s - 1) / s + 4 + 0.5 * i) + 0.01 * tiles * s + (heads <= 8 ? 0.01 * tiles * kb / s : 0.);
+    if (i == 0 || cost < best_cost) { best = s; best_cost = cost; }
+  }
+  return best;
+}
+
 }  // namespace ag

@@ -12,6 +12,9 @@ SHIM = """#include "launch_rules.cuh"
 extern "C" int decode_ctas(int D, int slabs, int query_slabs, int G, int cap, int at_once, int apart) {
   return ag::decode_ctas(D, slabs, query_slabs, G, cap, at_once, apart);
 }
+extern "C" int gate_linear_split(int tiles, int kb, int heads, int c1, int c2, int c4, int c8) {
+  return ag::gate_linear_split(tiles, kb, heads, ag::GateLinearPlaces{{c1, c2, c4, c8}});
+}
 """
 
 
@@ -49,3 +52,25 @@ def test_clusters_of_sixteen_only_where_the_device_places_them(rules, D, slabs, 
 def test_clusters_of_sixteen_by_room_and_rows(rules, D, slabs, G, cap, at_once, want):
     # (query_slabs: few enough that the split form is not asked for)
     assert (rules.decode_ctas(D, slabs, 64, G, cap, at_once, 7) == 16) == want
+
+
+B200 = (444, 222, 104, 48)
+
+
+@pytest.mark.parametrize("tiles,kb,heads,want", [
+    (1, 64, 32, 8), (48, 64, 32, 8), (49, 64, 32, 4), (55, 64, 32, 4), (104, 64, 32, 4), (105, 64, 32, 2), (111, 64, 32, 2), (222, 64, 32, 2),
+    (250, 64, 32, 1), (480, 64, 32, 2),                  # a second wave of single CTAs is longer than a third of pairs
+    (250, 64, 8, (4, 8)), (400, 8, 8, 2),                # 8 heads: not one CTA to a tile
+    (5, 1, 8, 1), (5, 2, 8, 2),                          # no more CTAs than k-blocks
+])
+def test_ctas_of_a_local_gate_tile(rules, tiles, kb, heads, want):
+    got = rules.gate_linear_split(tiles, kb, heads, *B200)
+    assert got in (want if isinstance(want, tuple) else (want,))
+
+
+def test_local_gate_clusters_only_where_the_device_places_them(rules):
+    for tiles in (1, 7, 50, 1000, 65535):
+        for kb in (1, 3, 33, 64, 4096):
+            assert rules.gate_linear_split(tiles, kb, 32, *B200) <= kb
+            assert rules.gate_linear_split(tiles, kb, 32, 12, 5, 0, 0) <= 2
+            assert rules.gate_linear_split(tiles, kb, 8, 0, 0, 0, 0) == 1
