@@ -725,32 +725,45 @@ static cudaLaunchConfig_t cluster_mma_config(int groups, cudaStream_t st, cudaLa
   return cfg;
 }
 
-// Clusters of kWideCluster CTAs that the device holds at once, and of those without a shared SM; 0 where it cannot place one (the
-// size is not portable: part of a device, or a context with few SMs).  Asked for once per thread and context, and the
-// kernel's attributes are set then.
-struct WideClusters { int at_once, apart; };
+// A kernel that leaves no room for another CTA on its SM, to ask how many clusters have an SM for each of their CTAs.
+constexpr int kAloneSmem = 120 * 1024;
+__global__ void __launch_bounds__(kGqThreads) decode_alone_kernel() {}
+
+// Clusters of `ctas` CTAs of `kern` that the device holds at once, 0 where it cannot place one (more than eight are not portable:
+// part of a device, or a context with few SMs).  Sets the kernel's attributes.
+static int clusters_at_once(const void *kern, cudaLaunchConfig_t cfg, cudaLaunchAttribute *attr, int ctas, size_t smem) {
+  cfg.gridDim.x = attr[0].val.clusterDim.x = ctas;
+  cfg.dynamicSmemBytes = smem;
+  int n = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess)
+    return n;
+  (void)cudaGetLastError();
+  return 0;
+}
+
+// Asked for once per thread and context; the attributes of the kernels of more than eight CTAs are set then.
 template <int D, int kMaxG>
-static WideClusters wide_clusters() {
-  struct Answer { unsigned long long context; WideClusters wide; };
+static DecodePlaces decode_places() {
+  struct Answer { unsigned long long context; DecodePlaces places; };
   static thread_local Answer known[8] = {};
   const unsigned long long context = current_context();
   Answer &a = known[context % 8];
   if (context == 0 || a.context != context) {
-    auto kern = decode_cluster_mma_kernel<D, kMaxG, kWideCluster>;
+    const void *alone = reinterpret_cast<const void *>(&decode_alone_kernel);
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = cluster_mma_config<D, kMaxG, kWideCluster>(1, nullptr, attr);
-    a.wide = {};
-    int n = 0, per_sm = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGqThreads, cfg.dynamicSmemBytes) == cudaSuccess && per_sm > 0)
-      a.wide = {n, n / per_sm};
-    else
-      (void)cudaGetLastError();
+    const size_t smem = cfg.dynamicSmemBytes;
+    a.places.wide = clusters_at_once(reinterpret_cast<const void *>(&decode_cluster_mma_kernel<D, kMaxG, kWideCluster>), cfg, attr, kWideCluster, smem);
+    a.places.wide_apart = a.places.wide > 0 ? clusters_at_once(alone, cfg, attr, kWideCluster, kAloneSmem) : 0;
+    a.places.ten_apart = 0;
+    if constexpr (kMaxG <= 8)
+      if (clusters_at_once(reinterpret_cast<const void *>(&decode_cluster_mma_kernel<D, kMaxG, kTenCluster>), cfg, attr, kTenCluster, smem) > 0)
+        a.places.ten_apart = clusters_at_once(alone, cfg, attr, kTenCluster, kAloneSmem);
     a.context = context;
   }
-  return a.wide;
+  return a.places;
 }
 
 // groups: clusters (runs of G query slabs on one key/value slab each)
@@ -759,7 +772,7 @@ static int launch_decode_cluster_mma(int groups, int G, const void *q, const voi
                                      const ag_cache &c, float scale_log2, void *o, const AppendArgs &ap,
                                      const HeadMap &hm, const RecentRing &rg, cudaStream_t st) {
   using T = __nv_bfloat16;
-  if constexpr (kCtas <= kClusterSize)               // (the wide ones': wide_clusters)
+  if constexpr (kCtas <= kClusterSize)               // (the larger ones': decode_places)
     AG_CUDA_TRY(cudaFuncSetAttribute(decode_cluster_mma_kernel<D, kMaxG, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq_smem_bytes(D, kCmStages)));
   cudaLaunchAttribute attr[2];
   const cudaLaunchConfig_t cfg = cluster_mma_config<D, kMaxG, kCtas>(groups, st, attr);
@@ -804,7 +817,7 @@ static bool decode_carries_append(const ag_layer_desc &d, const ag_cache &c) {
   if (group == 1) return true;
   const bool grouped = d.dtype == AG_BF16 && group <= kGqMaxGroup;        // one cluster per key/value slab
   if (slabs <= kClusterMaxSlabs) return grouped;
-  const int ctas = !grouped ? 0 : decode_ctas(d.head_dim, slabs / group, slabs, group, c.max_cap, 0, 0);
+  const int ctas = !grouped ? 0 : decode_ctas(d.head_dim, slabs / group, slabs, group, c.max_cap, DecodePlaces{});
   return ctas > 0 || group <= combine_heads(d.head_dim);
 }
 
@@ -820,18 +833,20 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     // grouped-query attention: one cluster per key/value slab reads it for all its query heads
     auto cluster = [&](auto ctas, int groups, int G) {
       constexpr int kCtas = decltype(ctas)::value;
+      constexpr int kMost = kCtas == kTenCluster ? 8 : 16;             // heads
       return (G == 1 ? launch_decode_cluster_mma<D, 1, kCtas> : G <= 4 ? launch_decode_cluster_mma<D, 4, kCtas> :
-              G <= 8 ? launch_decode_cluster_mma<D, 8, kCtas> : launch_decode_cluster_mma<D, 16, kCtas>)(groups, G, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
+              G <= 8 ? launch_decode_cluster_mma<D, 8, kCtas> : launch_decode_cluster_mma<D, kMost, kCtas>)(groups, G, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
     };
     const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
     // (clusters of one query head each never carry the append: see decode_carries_append)
-    const WideClusters wide = n > kWideMaxSlabs ? WideClusters{} : G == 1 ? wide_clusters<D, 1>() : G <= 4 ? wide_clusters<D, 4>() :
-                              G <= 8 ? wide_clusters<D, 8>() : wide_clusters<D, 16>();
-    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas(D, n, slabs, G, c.max_cap, wide.at_once, wide.apart) : 0) {
+    const DecodePlaces places = n > kWideMaxSlabs ? DecodePlaces{} : G == 1 ? decode_places<D, 1>() : G <= 4 ? decode_places<D, 4>() :
+                                G <= 8 ? decode_places<D, 8>() : decode_places<D, 16>();
+    switch (group <= kGqMaxGroup || n <= kClusterMaxSlabs ? decode_ctas(D, n, slabs, G, c.max_cap, places) : 0) {
       case 1: return cluster(std::integral_constant<int, 1>{}, n, G);
       case 2: return cluster(std::integral_constant<int, 2>{}, n, G);
       case 4: return cluster(std::integral_constant<int, 4>{}, n, G);
       case 8: return cluster(std::integral_constant<int, 8>{}, n, G);
+      case kTenCluster: return cluster(std::integral_constant<int, kTenCluster>{}, n, G);
       case kWideCluster: return cluster(std::integral_constant<int, kWideCluster>{}, n, G);
     }
   } else {

@@ -6,7 +6,10 @@ namespace ag {
 
 constexpr int kClusterMaxSlabs = 64;    // float32, and groups of more than 16 heads: up to here one cluster per slab
 constexpr int kClusterSize = 8;
-constexpr int kWideCluster = 16, kWideMaxSlabs = 16;    // bf16, few slabs of many rows (see decode_ctas)
+constexpr int kWideCluster = 16, kTenCluster = 10, kWideMaxSlabs = 16;    // bf16, few slabs of many rows (see decode_ctas)
+// What the device has room for: clusters of sixteen CTAs at the same time (0: it cannot place one; eight is the portable size), and
+// clusters of sixteen and of ten without a shared SM.
+struct DecodePlaces { int wide, wide_apart, ten_apart; };
 
 // CTAs per slab of the bf16 cluster form for groups of G heads; 0: the split form.  From a sweep over 8 .. 1024 slabs of 100 ..
 // 16,000 rows, head_dim 64 and 128 (us per step, CTAs per slab 1 | 2 | 4 | 8, split form last; "of" a capacity: 1 - 3 % full):
@@ -22,27 +25,29 @@ constexpr int kWideCluster = 16, kWideMaxSlabs = 16;    // bf16, few slabs of ma
 // so that long slabs do not end alone, but of eight CTAs no more than five waves: slabs may hold far less than their capacity.
 // Only few slabs of very many rows need more CTAs than a cluster has, and only with more than kClusterMaxSlabs query slabs
 // (query_slabs) may they have them: up to there the scratch stays untouched, which callers without scratch of their own count on.
-// wide_at_once: clusters of sixteen CTAs that the device holds at the same time (0: none; eight is the portable size),
-// wide_apart: as many with no more than one CTA on any SM (7 on a B200, whatever the kernel).
-inline int decode_ctas(int D, int slabs, int query_slabs, int G, int max_cap, int wide_at_once, int wide_apart) {
+inline int decode_ctas(int D, int slabs, int query_slabs, int G, int max_cap, const DecodePlaces &places) {
   constexpr int kSms = 148;
   const int wave_ctas = kSms * (D == 128 ? (G <= 8 ? 3 : 2) : (G <= 8 ? 4 : 3));
   if (query_slabs > kClusterMaxSlabs && slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
-  // A cluster of sixteen takes its place later and merges more triples, but streams a long slab in half the time.  How full
-  // the cache is, is not known here.  What it costs beside a short cache depends on whether every cluster has sixteen SMs to
-  // itself (wide_apart of them do: one per GPC of 16 SMs or more).  us per step, 8 | 16 CTAs per slab, lengths 2 - 5 %, 15 - 30 %
-  // and 38 - 100 % of the capacity; steps with another kernel between them:
-  //   7 slabs   cap 2200 3.48 | 3.58 (2 - 5 %), 4400 4.26 | 3.90, 6.26 | 5.11      of 64   3.24 | 3.28, 3.74 | 3.53, 5.22 | 4.33
-  //   7 slabs, 8 heads   4.37 | 4.49, 5.21 | 4.89, 7.60 | 5.92      16 heads   6.13 | 5.84, 7.27 | 6.46, 10.4 | 7.95
-  //   8 slabs   3.40 | 3.71, 4.11 | 4.28, 6.44 | 5.28      4 heads   3.91 | 4.40, 4.73 | 4.96, 6.75 | 6.13      8 heads   4.42 | 5.04, 5.22 | 5.75, 7.57 | 6.99
-  //   16 slabs   3.59 | 4.21, 4.63 | 4.83, 6.75 | 6.36      4 heads   4.30 | 5.13, 5.29 | 5.93, 7.49 | 7.61      16 heads   7.49 | 13.6, 9.01 | 14.4, 12.2 | 17.4
-  // and back to back: 2 slabs, cap 600 3.02 | 3.12, 3.04 | 3.16, 3.36 | 3.10; 16 heads 5.72 | 5.32, 5.82 | 5.39, 6.23 | 5.46.
-  // Up to there, from 2048 rows of capacity (512 for more than 8 heads), they are taken: at most 3 % lost, up to 30 % gained.  Beyond
-  // it short caches lose 10 - 20 %, so only where a long one has far more to gain, with few heads (back to back, cap 13,000):
-  //   8 slabs   3.57 | 3.73, 5.96 | 5.41, 12.4 | 9.55      4 heads   4.07 | 4.56, 6.48 | 6.33, 12.9 | 10.4      8 heads   4.50 | 5.62, 7.06 | 7.68, 13.7 | 12.3
-  //   16 slabs   3.65 | 3.99, 6.46 | 6.01, 14.8 | 11.0      4 heads   4.40 | 5.00, 7.25 | 7.02, 15.3 | 12.0      of 64, 4 heads   3.65 | 3.98, 5.63 | 5.33, 11.1 | 8.81
-  if (slabs <= wide_apart ? max_cap > (G > 8 ? 512 : 2048) : slabs <= wide_at_once && slabs <= kWideMaxSlabs && G <= 4 && max_cap > 8192)
+  // A larger cluster takes its place later and merges more triples, but streams a long slab in less time.  How full the cache
+  // is, is not known here.  What the cluster costs beside a short cache depends on whether its CTAs have an SM each: then
+  // they gain up to 30 % and lose up to 3 % (5 % where nothing runs between two steps); else short caches lose 10 - 20 %, and
+  // twice the time where sixteen do not run at once.  us per step, 8 | 10 | 16 CTAs per slab, another kernel between steps;
+  // capacity 2200, lengths 2 - 5 % of it, 15 - 30 %, 38 - 100 %; capacity 4400, 38 - 100 %:
+  //   7 slabs             3.48 | 3.55 | 3.56    3.88 | 3.55 | 3.57    4.81 | 4.72 | 4.03    6.33 | 5.81 | 4.87
+  //   7 slabs, 16 heads   6.21 | 6.36 | 5.92    6.74 | 6.47 | 6.02    8.24 | 8.06 | 6.89    10.4 | 9.74 | 8.03
+  //   8 slabs             3.45 | 3.46 | 3.79    3.77 | 3.45 | 3.79    4.96 | 4.59 | 4.36    6.52 | 5.80 | 5.36
+  //   8 slabs, 4 heads    3.97 | 3.99 | 4.48    4.28 | 4.09 | 4.58    5.32 | 5.11 | 5.13    6.85 | 6.32 | 6.15
+  //   8 slabs, 8 heads    4.41 | 4.50 | 5.09    4.88 | 4.57 | 5.22    6.05 | 5.85 | 5.87    7.65 | 7.08 | 7.06
+  //   9 slabs of 64       3.17 | 3.22 | 3.39    3.45 | 3.25 | 3.36    4.27 | 4.01 | 3.78    5.43 | 4.89 | 4.51
+  //   12 slabs, 4 heads   4.06 | 4.50 | 4.50    4.39 | 4.67 | 4.61    5.35 | 5.42 | 5.21    6.96 | 6.65 | 6.25
+  //   16 slabs, 16 heads  7.55 | 7.79 | 13.6    7.96 | 7.95 | 13.9    9.89 | 9.42 | 15.6    12.3 | 11.6 | 17.5
+  // So sixteen up to wide_apart slabs, from 2048 rows of capacity (512 for more than 8 heads), then ten up to ten_apart for up to 8
+  // heads; sixteen that share SMs only where a long cache has far more to gain than a short one loses (back to back,
+  // cap 13,000: 8 slabs 3.57 | 3.73 of 8 | 16, 5.96 | 5.41, 12.4 | 9.55; 16 slabs, 4 heads 4.40 | 5.00, 7.25 | 7.02, 15.3 | 12.0).
+  if (slabs <= places.wide_apart ? max_cap > (G > 8 ? 512 : 2048) : slabs <= places.wide && slabs <= kWideMaxSlabs && G <= 4 && max_cap > 8192)
     return kWideCluster;
+  if (slabs <= places.ten_apart && slabs > places.wide_apart && slabs <= kWideMaxSlabs && G <= 8 && max_cap > 2048) return kTenCluster;
   int wave = max_cap <= 128 ? 1 : max_cap <= 512 ? 4 : kClusterSize;
   while (wave > 1 && (int64_t)slabs * wave > wave_ctas) wave /= 2;
   if (wave == 2 && max_cap <= 512) wave = 1;
