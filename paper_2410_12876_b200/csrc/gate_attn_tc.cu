@@ -16,7 +16,7 @@
 // (a panel of 64 columns of both parts, or one part of 64-wide heads, the part with the fewest products
 // first), so that the next pair's arrive while the rest of the scores and two P V run.
 // Gate call, scores of one tile at a time | of pairs, us: 4 heads of 128, 333 tokens 31.0 | 31.0, 1500 50.1 | 48.6, 4096 102.3 |
-// 95.7, 8192 265 | 247, 4 x 1999 155 | 149; 4 heads of 64, 4 x 1500 65.0 | 60.1, 8192 205 | 175.  A pair takes 3,072
+// 95.7, 8192 265 | 247, 4 x 1999 155 | 149; 4 heads of 64, 4 x 1500 65.0 | 60.1, 8192 205 | 175.  A pair of 128-wide heads takes 3,072
 // cycles of the tensor cores, which were busy 51 % of the time at 4096 tokens and are 60 %.  (The first tile's
 // scores on their own, as a branch of the issuing warp: 8192 tokens of 64-wide heads 175 -> 213.)
 //
@@ -57,8 +57,8 @@ struct GaCfg {
   static constexpr int kSlices = D == 64 ? kParts : kPanels;
   static constexpr int kSliceParts = D == 64 ? 1 : kParts;
   static constexpr int kSliceBytes = kSliceParts * kGaPanel;
-  static_assert(kSlices * kSliceBytes == 2 * kKvStage, "K of a pair takes two stages");
-  static constexpr int kUsedBytes = kParts * kTile + 4 * kKvStage + 1024 + 256;   // Q + 2 K stages + 2 V stages
+  static_assert(kSlices * kSliceBytes == 2 * kKvStage, "K of a pair takes what two tiles of V do");
+  static constexpr int kUsedBytes = kParts * kTile + 4 * kKvStage + 1024 + 256;   // Q + K of a pair + 2 V stages
   static constexpr uint32_t kColO = 256, kColP = kColO + D;
   static_assert(kColP + 64 * kParts <= 512, "tensor memory");
   // parts of the first and of the second operand of product t
@@ -219,7 +219,8 @@ gate_attn_tc_kernel(const __grid_constant__ GateAttnMaps tm, const __grid_consta
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sQ = smem;                    // [part]
-  uint8_t *sK = sQ + C::kParts * kGaTile;      // [stage][part]
+  // [slice][part of the slice][128 keys][64 columns]; of 64-wide heads slice s holds part kParts - 1 - s
+  uint8_t *sK = sQ + C::kParts * kGaTile;
   uint8_t *sV = sK + 2 * kGaKvStage;
   uint64_t *bars = reinterpret_cast<uint64_t *>(sV + 2 * kGaKvStage);
   uint64_t *q_empty = bars, *o_free = bars + 1;

@@ -23,8 +23,10 @@ struct DecodePlaces { int wide, wide_apart, ten_apart; };
 // While a step waits for latency: as many CTAs per slab as one wave holds (the registers allow 3 per SM at 128, 2 with more
 // than 8 heads; 4 and 3 at 64), unless the slab has too few rows for them.  Where it waits for HBM: 1024 rows per CTA or fewer,
 // so that long slabs do not end alone, but of eight CTAs no more than five waves: slabs may hold far less than their capacity.
-// Only few slabs of very many rows need more CTAs than a cluster has, and only with more than kClusterMaxSlabs query slabs
-// (query_slabs) may they have them: up to there the scratch stays untouched, which callers without scratch of their own count on.
+// Few slabs of very many rows with more than kClusterMaxSlabs query slabs (query_slabs) take the split form, which may have more CTAs
+// per slab than a cluster (up to there the scratch stays untouched, which callers without scratch of their own count on).  Its line
+// dates from clusters of eight; it is behind the larger ones: 38 - 100 % full, split | 8 | 16, 9 slabs of 8 heads, cap 8200 12.8 | 11.7 |
+// 10.5, 16,000 15.9 | 19.2 | 15.1; 16 slabs of 16 heads 22.96 | 26.1 | 26.6; 2 - 5 % full, 9 slabs of 8 heads, 16,000 9.9 | 5.2 | 5.8.
 inline int decode_ctas(int D, int slabs, int query_slabs, int G, int max_cap, const DecodePlaces &places) {
   constexpr int kSms = 148;
   const int wave_ctas = kSms * (D == 128 ? (G <= 8 ? 3 : 2) : (G <= 8 ? 4 : 3));
