@@ -758,7 +758,7 @@ static DecodePlaces decode_places() {
     a.places.wide = clusters_at_once(reinterpret_cast<const void *>(&decode_cluster_mma_kernel<D, kMaxG, kWideCluster>), cfg, attr, kWideCluster, smem);
     a.places.wide_apart = a.places.wide > 0 ? clusters_at_once(alone, cfg, attr, kWideCluster, kAloneSmem) : 0;
     a.places.ten_apart = 0;
-    if constexpr (kMaxG <= 8)
+    if constexpr (kMaxG <= 4)
       if (clusters_at_once(reinterpret_cast<const void *>(&decode_cluster_mma_kernel<D, kMaxG, kTenCluster>), cfg, attr, kTenCluster, smem) > 0)
         a.places.ten_apart = clusters_at_once(alone, cfg, attr, kTenCluster, kAloneSmem);
     a.context = context;
@@ -833,9 +833,9 @@ static int run_decode(const ag_layer_desc &d, const void *q, const void *k_new, 
     // grouped-query attention: one cluster per key/value slab reads it for all its query heads
     auto cluster = [&](auto ctas, int groups, int G) {
       constexpr int kCtas = decltype(ctas)::value;
-      constexpr int kMost = kCtas == kTenCluster ? 8 : 16;             // heads
+      constexpr int kMost = kCtas == kTenCluster ? 4 : 16;             // heads
       return (G == 1 ? launch_decode_cluster_mma<D, 1, kCtas> : G <= 4 ? launch_decode_cluster_mma<D, 4, kCtas> :
-              G <= 8 ? launch_decode_cluster_mma<D, 8, kCtas> : launch_decode_cluster_mma<D, kMost, kCtas>)(groups, G, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
+              G <= 8 ? launch_decode_cluster_mma<D, kMost < 8 ? kMost : 8, kCtas> : launch_decode_cluster_mma<D, kMost, kCtas>)(groups, G, q, k_new, v_new, c, scale_log2, o, ap, hm, rg, st);
     };
     const int n = group <= kGqMaxGroup ? kv_slabs : slabs, G = group <= kGqMaxGroup ? group : 1;
     // (clusters of one query head each never carry the append: see decode_carries_append)

@@ -33,7 +33,7 @@ inline int decode_ctas(int D, int slabs, int query_slabs, int G, int max_cap, co
   if (query_slabs > kClusterMaxSlabs && slabs * kClusterSize <= kSms && max_cap > 8192) return 0;
   // A larger cluster takes its place later and merges more triples, but streams a long slab in less time.  How full the cache
   // is, is not known here.  What the cluster costs beside a short cache depends on whether its CTAs have an SM each: then
-  // they gain up to 30 % and lose up to 3 % (5 % where nothing runs between two steps); else short caches lose 10 - 20 %, and
+  // they gain up to 30 % and lose up to 3 % (6 % where nothing runs between two steps); else short caches lose 10 - 20 %, and
   // twice the time where sixteen do not run at once.  us per step, 8 | 10 | 16 CTAs per slab, another kernel between steps;
   // capacity 2200, lengths 2 - 5 % of it, 15 - 30 %, 38 - 100 %; capacity 4400, 38 - 100 %:
   //   7 slabs             3.48 | 3.55 | 3.56    3.88 | 3.55 | 3.57    4.81 | 4.72 | 4.03    6.33 | 5.81 | 4.87
@@ -44,12 +44,12 @@ inline int decode_ctas(int D, int slabs, int query_slabs, int G, int max_cap, co
   //   9 slabs of 64       3.17 | 3.22 | 3.39    3.45 | 3.25 | 3.36    4.27 | 4.01 | 3.78    5.43 | 4.89 | 4.51
   //   12 slabs, 4 heads   4.06 | 4.50 | 4.50    4.39 | 4.67 | 4.61    5.35 | 5.42 | 5.21    6.96 | 6.65 | 6.25
   //   16 slabs, 16 heads  7.55 | 7.79 | 13.6    7.96 | 7.95 | 13.9    9.89 | 9.42 | 15.6    12.3 | 11.6 | 17.5
-  // So sixteen up to wide_apart slabs, from 2048 rows of capacity (512 for more than 8 heads), then ten up to ten_apart for up to 8
-  // heads; sixteen that share SMs only where a long cache has far more to gain than a short one loses (back to back,
+  // So sixteen up to wide_apart slabs, from 2048 rows of capacity (512 for more than 8 heads), then ten up to ten_apart for up to 4
+  // heads (8 heads back to back, 2 - 5 % full: 8 slabs 4.02 | 4.30, 11 slabs 4.49 | 4.90); sixteen that share SMs only where a long cache has far more to gain than a short one loses (back to back,
   // cap 13,000: 8 slabs 3.57 | 3.73 of 8 | 16, 5.96 | 5.41, 12.4 | 9.55; 16 slabs, 4 heads 4.40 | 5.00, 7.25 | 7.02, 15.3 | 12.0).
   if (slabs <= places.wide_apart ? max_cap > (G > 8 ? 512 : 2048) : slabs <= places.wide && slabs <= kWideMaxSlabs && G <= 4 && max_cap > 8192)
     return kWideCluster;
-  if (slabs <= places.ten_apart && slabs > places.wide_apart && slabs <= kWideMaxSlabs && G <= 8 && max_cap > 2048) return kTenCluster;
+  if (slabs <= places.ten_apart && slabs > places.wide_apart && slabs <= kWideMaxSlabs && G <= 4 && max_cap > 2048) return kTenCluster;
   int wave = max_cap <= 128 ? 1 : max_cap <= 512 ? 4 : kClusterSize;
   while (wave > 1 && (int64_t)slabs * wave > wave_ctas) wave /= 2;
   if (wave == 2 && max_cap <= 512) wave = 1;

@@ -48,7 +48,7 @@ def test_lengths_at_the_edges_of_sixteen_blocks(D, h, hk):
     test_lengths_at_the_edges_of_blocks(D, h, hk, lens=(16, 17, 1024, 1039, 1040, 1041, 2063))
 
 
-@pytest.mark.parametrize("D,h,hk", [(128, 8, 8), (64, 32, 8), (128, 64, 8)])
+@pytest.mark.parametrize("D,h,hk", [(128, 8, 8), (64, 8, 8), (64, 32, 8), (128, 24, 8)])
 def test_lengths_at_the_edges_of_ten_blocks(D, h, hk):
     test_lengths_at_the_edges_of_blocks(D, h, hk, lens=(1, 17, 640, 655, 656, 657, 1281, 2063))
 
@@ -89,7 +89,7 @@ def test_ctas_per_slab(B, h, hk, D, longest):
 
 
 @pytest.mark.parametrize("B,h,hk,D,longest", [
-    (1, 4, 4, 128, 2060), (2, 20, 4, 64, 2060),          # up to seven slabs, from 2048 rows; eight of five heads: ten CTAs
+    (1, 4, 4, 128, 2060), (2, 20, 4, 64, 2060),          # up to seven slabs, from 2048 rows; eight of five heads: eight CTAs
     (4, 4, 4, 128, 4100), (2, 64, 8, 64, 4100),          # sixteen slabs, too few rows for it
     (1, 64, 4, 128, 520), (1, 48, 3, 64, 1040),          # 16 heads per slab, from 512; a second tile for one rank
 ])
@@ -99,7 +99,7 @@ def test_sixteen_ctas_per_slab(B, h, hk, D, longest):
 
 @pytest.mark.parametrize("B,h,hk,D,longest", [
     (4, 4, 4, 128, 8300), (4, 16, 4, 64, 8300), (1, 28, 7, 128, 2060),    # sixteen CTAs: up to 16 slabs beyond 8192 rows, seven
-    (1, 8, 8, 128, 2060), (2, 16, 4, 128, 2060), (1, 64, 8, 64, 4100),    # ten: eight slabs of 1, 4 and 8 heads
+    (1, 8, 8, 128, 2060), (2, 16, 4, 128, 2060), (1, 27, 9, 64, 4100),    # ten: eight and nine slabs of 1, 4 and 3 heads
     (20, 16, 1, 128, 1100), (9, 18, 2, 64, 1100),        # 16 and 9 heads, eight CTAs: two heads for a rank
     (20, 16, 1, 128, 400), (17, 12, 1, 64, 500),         # four CTAs, four and three heads for a rank
     (80, 16, 1, 128, 700), (120, 10, 1, 64, 700),        # two CTAs, eight and five

@@ -36,7 +36,7 @@ def test_larger_clusters_only_where_the_device_places_them(rules, D, slabs, G):
             ctas = rules.decode_ctas(D, slabs, slabs * G, G, cap, wide, apart, ten)
             assert ctas in (0, 1, 2, 4, 8, 10, 16)
             assert ctas != 16 or slabs <= wide
-            assert ctas != 10 or slabs <= ten and G <= 8
+            assert ctas != 10 or slabs <= ten and G <= 4
             # whether the split form is taken does not depend on it: a step's append is routed before the device is asked
             assert (ctas == 0) == (rules.decode_ctas(D, slabs, slabs * G, G, cap, 0, 0, 0) == 0)
 
@@ -44,7 +44,7 @@ def test_larger_clusters_only_where_the_device_places_them(rules, D, slabs, G):
 @pytest.mark.parametrize("D,slabs,G,cap,wide,want", [
     # clusters that share SMs lost 80 - 100 % (16 heads, two CTAs per SM: 14 at once) and 20 - 35 % (8 heads)
     (128, 16, 16, 2200, 14, 8), (128, 16, 16, 16000, 14, 8), (128, 14, 16, 2200, 14, 8), (64, 16, 16, 2200, 21, 8),
-    (128, 8, 8, 2200, 21, 10), (128, 8, 8, 16000, 21, 10), (64, 9, 8, 4400, 31, 10), (128, 8, 16, 4400, 14, 8), (128, 10, 4, 4400, 21, 8),
+    (128, 8, 8, 2200, 21, 8), (128, 8, 8, 16000, 21, 8), (64, 9, 8, 4400, 31, 8), (64, 9, 4, 4400, 31, 10), (128, 8, 16, 4400, 14, 8), (128, 10, 4, 4400, 21, 8),
     # few heads: 10 - 20 % lost in short caches, which a capacity of a few thousand rows does not outweigh
     (128, 8, 4, 2200, 21, 10), (128, 16, 1, 4400, 21, 8), (128, 8, 4, 8300, 21, 16), (64, 16, 1, 8300, 31, 16), (128, 8, 4, 2000, 21, 8),
     # an SM to each CTA: never more than 3 % behind, up to 30 % ahead
