@@ -17,8 +17,7 @@
 //   the heads shared among the ranks, one CTA of eight stages  6.5 | 12.2 | 11.7 | 16.2 | 25.9 | 53.0
 //   two of four stages                                         6.5 | 7.9 | 10.9 | 14.8 | 23.6 | 38.7
 //   three of three                                             6.4 | 7.9 | 11.2 | 13.6 | 21.7 | 34.6
-// and calls back to back, X in L2 where it fits: three of three 6.6 | 7.9 | 9.7 | 10.9 | 17.0 | 34.0; heads added up by loops of as many
-// ranks as there are, CTAs to a tile by gate_linear_split  5.8 | 7.3 | 9.4 | 10.5 | 15.5 | 31.0   (5.3 TB/s)
+//   with a loop of as many ranks as there are                  5.7 | 7.3 | 10.9 | 13.4 | 20.0 | 31.4   (5.2 TB/s)
 //   A = X      [B n, d]  row-major -> K-major operand, 128-byte swizzled rows
 //   B = W_lin  [d, h]    row-major -> MN-major operand: one panel of [64 k][64 n],
 //                                     columns past h filled with zeros by TMA
