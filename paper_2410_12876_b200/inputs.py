@@ -2,7 +2,7 @@
 
 This module only draws random tensors and lays out buffers.  It contains none
 of the layer's arithmetic (no gate, no mask, no softmax): both the CUDA path
-and the CPU checker are fed from here, so nothing in it may be something
+and the CPU oracle are fed from here, so nothing in it may be something
 either of them is meant to verify.  The only linear algebra is the upstream
 Q/K/V projection X W (Eq. 2's inputs), which lies outside the layer.
 
